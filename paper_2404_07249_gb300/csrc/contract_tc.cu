@@ -1,4 +1,4 @@
-// Tensor-core (tcgen05, sm_103a) triplet contraction with 3-term split-TF32 products.
+// Tensor-core (tcgen05, sm_103a) triplet contraction with two-term split products.
 //
 // Computes sums M[(j, k)][i] = sum_x g_j(x) g_k(x) h_i(x) over the cells x (Sec. 4.3.1, eq. beta-def: the
 // real-space sum of the separable bispectrum; with h = g the entry of pair (b, c) and single a is S_abc).  The work
@@ -7,37 +7,41 @@
 // the triplet a <= b <= c is read from pair (b, c) and single a, which prunes the 465 pairs x 30 singles of a
 // 30-bin binning to 255 pairs in two tiles with windows of 16 and 32 singles.
 //
-// Arithmetic: A = pair products g_j g_k (FP32), split as A = A_hi + A_lo with A_hi = A rounded to TF32 (nearest,
-// ties away from zero) and A_lo = A - A_hi in FP32 (read by the MMA as TF32).  B = singles: the tensor core reads an
-// FP32 operand as TF32 by truncation (measured: the 13 low bits are dropped toward zero), so the raw maps in the TMA
-// ring serve as B_hi = trunc(g) directly, and B_lo = g - trunc(g), rounded to TF32, is made per stage.  Per tile
-// and K = 8 cells three MMAs of N = W run:  D[:, 0:W] += A_hi . B_hi^T  and  D[:, W:2W] += A_hi . B_lo^T +
-// A_lo . B_hi^T  (both corrections in one accumulator); the lo*lo term (~2^-21 relative, unbiased) is dropped.  The
-// tensor core's internal accumulation is not round-to-nearest, so D restarts every 64 cells (8 MMAs per hi*hi
-// column); the epilogue adds D into FP32 registers (round-to-nearest) and those into FP64 shared memory every 2048
-// cells.  Cross-CTA sums are FP64 in a fixed order (deterministic).
+// Arithmetic: the pair products A = g_j g_k (FP32) and the singles B are split as hi + lo with hi the value rounded to
+// 11 bits and lo the rounded remainder, 22 bits in all.  Both parts are FP16, which has TF32's 11 bits at twice its
+// tensor rate and half its storage.  FP16's short exponent is met by powers of two taken from the maps' maxima
+// (k_absmax): a row's products are scaled below 2^15, a single's values below 2^15, and the final FP64 sums scaled
+// back.  Values far below a map's maximum lose bits only below 2^-40 of it.  Per tile and K = 16 cells two MMAs of
+// N = 2W run, D[:, hi | lo] += A_lo . [B_hi | B_lo]^T and then A_hi . [B_hi | B_lo]^T: all four partial products.  The
+// tensor core's internal accumulation is not round-to-nearest, so D restarts every 64 cells, the A_lo terms first
+// (they add to a small sum); the epilogue adds D into FP32 registers (round-to-nearest) and those into FP64 shared
+// memory every 2048 cells.  Cross-CTA sums are FP64 in a fixed order (deterministic).
 //
 // Measured on this part (and shaping the design): an MMA issued from warp-uniform code with its operands in uniform
 // registers costs ~16-20 cycles at N = 32 (the tensor pipe's rate), but ~200 cycles from a one-lane branch, so the
-// issuing loops are warp-uniform (elect.sync inside the asm) and divide-free; MMAs into one accumulator back to back
-// run at full rate; tensor memory stores reach ~650 B/clk an SM; the producers' shared-memory gathers (~500
-// wavefronts a stage) and their latency set the stage time.  Tensor memory (512 columns) holds the accumulator
-// (2W columns a tile) and a ring of A stages (64 columns a tile a stage).
+// issuing loop is warp-uniform (elect.sync inside the asm) and divide-free; tensor memory stores reach ~650 B/clk an
+// SM.  What bounds the kernel is shared memory: the producers' gathers (two 16-byte loads for every four products) and the
+// B operand's conversion; before, with 32-cell stages and one accumulator buffer, it was the barrier round trips of its
+// stages.  A stage is therefore 64 cells and the accumulators are double-buffered, so that no MMA waits for the epilogue.
+// Measured at 30 maps of 288^3 cells (two tiles): 3.88 ms with TF32 parts, 2.81 ms (and 0.39 ms for the maxima where the
+// maps come without them).  Tensor memory (512 columns) holds two accumulator buffers (2W columns a tile) and a ring of A
+// stages (64 columns a tile a stage).
 //
-// One CTA per SM over a contiguous range of cells, in stages of 32 cells (one TMA ring slot).  Warp roles, by
+// One CTA per SM over a contiguous range of cells, in stages of 64 cells (two TMA ring slots).  Warp roles, by
 // warpgroup (setmaxnreg moves registers from warpgroup 0 to the producers):
 //   warp 0       TMEM allocation; lane 0 streams the maps with TMA (cp.async.bulk.tensor, 32 cells x all maps per
 //                load, 128-byte swizzle) into an 8-slot shared-memory ring.
-//   warps 1-3    MMA issue: warp 1 + t waits for the stage (converged) and issues tile t's MMAs, commits them to the
-//                stage's release barriers (A stage, ring slot) and, at a period's end, to the accumulator barrier.
-//   warps 4-11   producers, two groups of four warps; group g makes cells 16g..16g+15 of every stage.  A thread owns
-//                one TMEM lane, i.e. one row of every tile: it forms the pair products, splits them (packed FP32
-//                pairs) and writes hi / lo straight into tensor memory (tcgen05.st: the A operand never touches
-//                shared memory), loading the next tile's operands before forming the current tile's products; each
-//                thread also makes one 16-byte chunk of the stage's B_lo.
-//   warps 12-15  epilogue: after every period read D with tcgen05.ld (each warp its TMEM lane quarter), release
-//                it to the issuers, accumulate.
+//   warp 1       MMA issue: waits for the stage (converged), issues every tile's MMAs and commits them to the A
+//                stage's release barrier and the accumulator barrier.
+//   warps 4-7    the B operand: scale and split the singles of every stage into FP16 rows of 64 cells (128-byte swizzle),
+//                8 rows of hi and 8 of lo alternating.
+//   producers    groups of four warps; group g makes the 32 cells of slots g, g + kProdGroups, ..  A thread owns one TMEM
+//                lane, i.e. one row of every tile: it forms the pair products, splits them and writes hi / lo straight
+//                into tensor memory (tcgen05.st: the A operand never touches shared memory).
+//   epilogue     four warps: after every stage read D with tcgen05.ld (each warp its TMEM lane quarter), release it to
+//                the issuer, accumulate.
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -56,31 +60,32 @@ namespace tc {
 
 constexpr int kSlotCells = 32;     // cells per TMA box row (128 bytes)
 constexpr int kRingSlots = 8;
-constexpr int kKC = 32;            // cells per A stage = one ring slot (four K = 8 MMA steps)
+constexpr int kKC = 64;            // cells per A stage = two ring slots (four K = 16 MMA steps)
 constexpr int kMaxAStages = 6;
-constexpr int kPeriod = 2;         // A stages per TMEM accumulation period (64 cells)
-constexpr int kSpill = 32;         // periods per FP32 register sum (2048 cells)
-constexpr int kDBuf = 1;           // accumulator buffers (1: the issuers wait for the epilogue between periods)
-static_assert(kDBuf == 1, "the MMA issue loop assumes one accumulator buffer");
+constexpr int kSpill = 32;         // stages per FP32 register sum (2048 cells)
+constexpr int kDBuf = 2;           // accumulator buffers (the epilogue reads one while the MMAs fill the other)
+constexpr int kAcols = 64;         // tensor memory columns of a tile's A stage: hi and lo of 64 cells, two a column
+constexpr int kMaxRows = 128;      // map rows of a slot: <= 64 g rows and <= 64 h rows
 constexpr int kMaxTiles = 3;       // tiles per CTA
 constexpr int kMaxUnits = 3;       // 16-column output units per CTA (16 FP32 sums each, in registers)
 constexpr int kMaxGroups = 4;      // row groups (grid.y)
-constexpr int kProdGroups = 2;     // producer warp groups; group g makes half g (16 cells) of every stage
+constexpr int kProdGroups = 2;     // producer warp groups; group g makes slots g, g + kProdGroups, .. (32 cells each)
 constexpr int kProdWarps = 4 * kProdGroups;
 constexpr int kEpiWarps = 4;
-// Warpgroup 0: TMA (warp 0), MMA issue (warp 1), two idle warps; warpgroups 1-2: producers; warpgroup 3: epilogue.
-constexpr int kProdWarp0 = 4;
-constexpr int kWarps = 16;
-// Register split (setmaxnreg, per warpgroup): the CTA is launched with 128 registers a thread (65536 in all);
-// warpgroup 0 gives registers back, the producers take them, the epilogue keeps 128:
-// 48 * 128 + 168 * 256 + 128 * 128 = 65536.
-constexpr int kRegsLaunch = 128, kRegsCtl = 48, kRegsProd = 168;
-static_assert(kRegsCtl * 128 + kRegsProd * 256 + kRegsLaunch * 128 <= kRegsLaunch * 32 * kWarps,
+// Warpgroup 0: TMA (warp 0), MMA issue (warp 1), two idle warps; then the B operand (four warps), the producers and the
+// epilogue, a warpgroup each (producers: kProdGroups).
+constexpr int kBWarp0 = 4, kBWarps = 4;
+constexpr int kProdWarp0 = kBWarp0 + kBWarps;
+constexpr int kWarps = kProdWarp0 + kProdWarps + kEpiWarps;
+// Register split (setmaxnreg, per warpgroup): the CTA is launched with kRegsLaunch registers a thread; warpgroup 0 gives
+// registers back, the producers take them, the B warps and the epilogue keep what they have.
+constexpr int kRegsLaunch = 96, kRegsCtl = 40, kRegsB = 96, kRegsProd = 120;
+static_assert((kRegsCtl + kRegsB) * 128 + kRegsProd * 32 * kProdWarps + kRegsLaunch * 32 * kEpiWarps <= kRegsLaunch * 32 * kWarps,
               "register split exceeds the launch allocation");
 constexpr int kThreads = 32 * kWarps;
 constexpr int kMinSmem = 120 * 1024;   // one CTA per SM (the CTA allocates all 512 TMEM columns)
 constexpr unsigned kSpinLimit = 1u << 22;
-constexpr int kBloItems = 2;       // B_lo chunks per producer thread: <= 64 singles rows x 8 chunks / 256 threads
+constexpr int kBloItems = 2;       // 16-byte chunks of a slot's singles region a thread of 256: <= 64 rows x 8 chunks
 
 struct GroupDesc {
     int tile0;                 // first tile (row table index / 128)
@@ -88,9 +93,9 @@ struct GroupDesc {
     int unit_base;             // first unit of this group in the partial layout
     int d_cols;                // TMEM columns of one accumulator buffer (kDBuf buffers at 0, d_cols, ...)
     int a_col0;                // first TMEM column of the A ring
-    int bstage_bytes;          // B_lo bytes per A stage (the singles region of a slot)
+    int bstage_bytes;          // bytes of one part (hi or lo) of a B stage: 128 for each row of the singles region
     int tile_w[kMaxTiles];
-    int dm_col[kMaxTiles];     // TMEM column of tile t's accumulator: [hi*hi | hi*lo + lo*hi] (2W columns)
+    int dm_col[kMaxTiles];     // TMEM column of tile t's accumulator: [B_hi 8 | B_lo 8] for every 8 singles (2W columns)
     int tile_s0[kMaxTiles];    // first single of tile t's window
     int unit_tile[kMaxUnits], unit_c[kMaxUnits];
 };
@@ -99,7 +104,8 @@ struct Params {
     long ncell, cells_cta;
     int ng, nh, hsep, h_row0;  // maps in the slot; singles; singles from the h part; first h row in a slot
     int slot_bytes, off_b, off_acc, off_bar;
-    int s_off, s_chunks;       // singles region of a slot: byte offset and 16-byte chunks (B_lo is made for all)
+    int s_off, s_chunks;       // singles region of a slot: byte offset and 16-byte chunks (B is made for all)
+    const uint32_t* absmax;    // max |map| bit patterns by slot row (the scale factors)
     int total_units;
     const short2* rows;        // [tiles][128] pairs (j, k); (-1, -1) pads
     double* partial;           // [gridDim.x][total_units][16][128]
@@ -192,15 +198,35 @@ __device__ __forceinline__ uint64_t sub_x2(uint64_t a, uint64_t b) {
 }
 // Two values at once: v = hi + lo with hi = v rounded to TF32 (nearest, ties away from zero: add half a unit of the
 // 10-bit mantissa, bit 12, and clear the 13 low bits; a carry moves into the exponent as it should) and lo = v - hi
-// in FP32.  lo is symmetric about zero, so the tensor core's truncation of lo to TF32 is unbiased.  (When v is a
-// product, the compiler may fuse the multiply into the subtraction; lo then also carries the product's rounding
-// error, which only makes hi + lo closer to the exact product.)
+// in FP32.  lo is symmetric about zero, so the tensor core's truncation of lo to TF32 is unbiased.  (Used by the Gram.)
 __device__ __forceinline__ void split_x2(uint64_t v, uint64_t& hi, uint64_t& lo) {
     const uint32_t h0 = ((uint32_t)v + 0x1000u) & 0xFFFFE000u;
     const uint32_t h1 = ((uint32_t)(v >> 32) + 0x1000u) & 0xFFFFE000u;
     hi = (uint64_t)h0 | ((uint64_t)h1 << 32);
     lo = sub_x2(v, hi);
 }
+// Two values at once: v = hi + lo + (a remainder below 2^-22 |v|), hi and lo packed FP16 pairs rounded to nearest (the
+// first value in the low half); hi is 11 bits of v and v - hi is exact in FP32.
+__device__ __forceinline__ void split_h2(uint64_t v, uint32_t& hi, uint32_t& lo) {
+    const float v0 = __uint_as_float((uint32_t)v), v1 = __uint_as_float((uint32_t)(v >> 32));
+    const __half2 h = __floats2half2_rn(v0, v1);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    const float2 f = __half22float2(h);
+    const uint64_t r = sub_x2(v, f2pack(f.x, f.y));
+    const __half2 l = __floats2half2_rn(__uint_as_float((uint32_t)r), __uint_as_float((uint32_t)(r >> 32)));
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+// Scale exponents.  map_exp(m): the smallest e with m < 2^e for a map's largest magnitude m (bit pattern; 0 for a map
+// with infinities or NaN, whose sums are not finite at any scale).  A row (j, k) is scaled by 2^row_exp, a single by
+// 2^single_exp, which puts every product and every single below 2^15 (half the largest FP16 number).
+__host__ __device__ inline int map_exp(uint32_t m) {
+    const int e = (int)((m >> 23) & 255u);
+    return e == 255 ? 0 : (e < 1 ? 1 : e) - 126;
+}
+__host__ __device__ inline int clamp_exp(int e) { return e < -126 ? -126 : (e > 127 ? 127 : e); }
+__host__ __device__ inline int row_exp(uint32_t mj, uint32_t mk) { return clamp_exp(15 - map_exp(mj) - map_exp(mk)); }
+__host__ __device__ inline int single_exp(uint32_t ma) { return clamp_exp(15 - map_exp(ma)); }
+__device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }   // -126 <= e <= 127
 
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* v) {
     asm volatile(
@@ -249,6 +275,11 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// The same for kind::f16 with FP16 operands (D = F32, A = B = F16, both K-major).
+__host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
+    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
 // The MMA and its commit are executed by a whole converged warp and issued by the one lane that elect.sync picks
 // (the same lane every time with all 32 active, so the commit tracks the MMAs of the issuing thread).  Keeping the
 // issuing code warp-uniform, rather than inside a one-lane branch, lets the compiler hold the operands in uniform
@@ -259,6 +290,14 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint32_t a_tmem, uint6
     asm volatile(
         "{\n\t.reg .pred p, q;\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accum)
+        : "memory");
+}
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                        uint32_t accum) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
         "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accum)
         : "memory");
 }
@@ -283,25 +322,20 @@ __device__ __forceinline__ const float4* ring_chunk(const unsigned char* slot, i
     return reinterpret_cast<const float4*>(slot + r * 128 + ((ch ^ (r & 7)) << 4));
 }
 
-// Epilogue of NU output units (a compile-time count keeps the FP32 sums in registers): halfway through every
-// period read this warp's TMEM lane quarter of the previous period's accumulators with tcgen05.ld, release the D
-// buffer, add into the FP32 sums; every kSpill periods add those into the FP64 sums in shared memory (FP64 is slow
-// on this part, so only there); finally write this CTA's FP64 partials.
+// Epilogue of NU output units (a compile-time count keeps the FP32 sums in registers): after every stage read this
+// warp's TMEM lane quarter of the stage's accumulators with tcgen05.ld, release the D buffer, add into the FP32 sums;
+// every kSpill stages add those into the FP64 sums in shared memory (FP64 is slow on this part, so only there);
+// finally write this CTA's FP64 partials.
 template <int NU>
 __device__ __forceinline__ void epilogue(const GroupDesc& G, const Params& P, uint32_t tmem, double* acc64,
-                                         uint64_t* d_full, uint64_t* d_empty, volatile int* abort_flag, int nper,
+                                         uint64_t* d_full, uint64_t* d_empty, volatile int* abort_flag, int nstages,
                                          int warp, int lane) {
     const int q = warp & 3;
     const int row = 32 * q + lane;
     const uint32_t lane_base = (uint32_t)(32 * q) << 16;
-    const int ntiles = G.ntiles;
-    uint32_t cols[NU][2];     // hi*hi and the corrections (hi*lo + lo*hi) of unit u
+    uint32_t cols[NU];        // unit u: 32 columns [hi 8 | lo 8 | hi 8 | lo 8]
 #pragma unroll
-    for (int u = 0; u < NU; ++u) {
-        const int t = G.unit_tile[u], cu = G.unit_c[u];
-        cols[u][0] = (uint32_t)(G.dm_col[t] + cu);
-        cols[u][1] = (uint32_t)(G.dm_col[t] + G.tile_w[t] + cu);
-    }
+    for (int u = 0; u < NU; ++u) cols[u] = (uint32_t)(G.dm_col[G.unit_tile[u]] + 2 * G.unit_c[u]);
     const uint32_t d_cols = (uint32_t)G.d_cols;
     int* const err = P.err;
     double* const out = P.partial + ((size_t)blockIdx.x * P.total_units + G.unit_base) * 2048;
@@ -311,29 +345,28 @@ __device__ __forceinline__ void epilogue(const GroupDesc& G, const Params& P, ui
     for (int u = 0; u < NU; ++u)
 #pragma unroll
         for (int j = 0; j < 16; ++j) acc[u][j] = 0.f;
-    bool ok = true;
-    for (int per = 0; per < nper && ok; ++per) {
-        const int db = per % kDBuf;
-        for (int t = 0; t < ntiles && ok; ++t)
-            ok = warp_wait(&d_full[db * kMaxTiles + t], (uint32_t)((per / kDBuf) & 1), abort_flag, err);
-        if (!ok) break;
+    for (int st = 0; st < nstages; ++st) {
+        const int db = st & 1;
+        if (!warp_wait(&d_full[db], (uint32_t)((st >> 1) & 1), abort_flag, err)) break;
         tc_fence_after();
         const uint32_t dbase = tmem + lane_base + (uint32_t)db * d_cols;
 #pragma unroll
-        for (int u = 0; u < NU; ++u)
-            {
-                // both pieces in flight together, one wait
-                uint32_t v0[16], v1[16];
-                tmem_ld16(dbase + cols[u][0], v0);
-                tmem_ld16(dbase + cols[u][1], v1);
-                tmem_wait_ld32(v0, v1);
+        for (int u = 0; u < NU; ++u) {
+            // both halves in flight together, one wait
+            uint32_t v0[16], v1[16];
+            tmem_ld16(dbase + cols[u], v0);
+            tmem_ld16(dbase + cols[u] + 16u, v1);
+            tmem_wait_ld32(v0, v1);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) acc[u][j] += __uint_as_float(v0[j]) + __uint_as_float(v1[j]);
+            for (int j = 0; j < 8; ++j) {
+                acc[u][j] += __uint_as_float(v0[j]) + __uint_as_float(v0[8 + j]);
+                acc[u][8 + j] += __uint_as_float(v1[j]) + __uint_as_float(v1[8 + j]);
             }
+        }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&d_empty[db]);   // one arrival a warp (the warp's loads are done)
-        if ((per + 1) % kSpill == 0) {
+        if ((st + 1) % kSpill == 0) {
 #pragma unroll
             for (int u = 0; u < NU; ++u)
 #pragma unroll
@@ -351,137 +384,140 @@ __device__ __forceinline__ void epilogue(const GroupDesc& G, const Params& P, ui
 }
 
 
-// Producer warp of group gp = (warp - 1) / 4: cells 16 gp .. 16 gp + 15 of every 32-cell stage, for NT tiles (a
-// compile-time count: every tile's products live in their own registers, so the next tile's arithmetic does not
-// wait for the previous tile's TMEM store to read its registers).  A thread owns TMEM lane 32 (warp % 4) + lane,
-// i.e. row `row` of every tile.  The 64 columns of a tile's stage block are [hi 16 | lo 16] of half 0, then of half
-// 1; a thread writes its half with one 32-column TMEM store per tile.  (The B operand is made by warp 0.)
+// Producer warp of group gp: the 32 cells of slots gp, gp + 3, .. (two slots a 64-cell stage), for NT tiles.  A thread owns TMEM
+// lane 32 (warp % 4) + lane, i.e. row `row` of every tile.  The 64 columns of a tile's stage block are [hi 16 | lo 16]
+// of slot 0, then of slot 1 (two cells a column); a thread writes its slot's part with one 32-column TMEM store per
+// tile.
 template <int NT>
 __device__ __forceinline__ void producer(const GroupDesc& G, const Params& P, uint32_t tmem, const unsigned char* ring,
-                                         unsigned char* bst, uint64_t* slot_full, uint64_t* slot_empty,
-                                         uint64_t* a_full, uint64_t* a_empty, volatile int* abort_flag, int nstages,
-                                         int warp, int lane) {
+                                         uint64_t* slot_full, uint64_t* slot_empty, uint64_t* a_full, uint64_t* a_empty,
+                                         volatile int* abort_flag, int nstages, int warp, int lane) {
     const int gp = (warp - kProdWarp0) >> 2;
     const int q = warp & 3;
     const int row = 32 * q + lane;
     const uint32_t lane_base = (uint32_t)(32 * q) << 16;
-    const int nA = G.nA, a_col0 = G.a_col0, slot_bytes = P.slot_bytes, bstage_bytes = G.bstage_bytes;
-    const int s_off = P.s_off, s_chunks = P.s_chunks;
-    const int ptid = 32 * (warp - kProdWarp0) + lane;   // 0 .. 255 over both groups
+    const int nA = G.nA, a_col0 = G.a_col0, slot_bytes = P.slot_bytes;
     int* const err = P.err;
-    int pj[NT], pk[NT];
+    int oj[NT], ok_[NT];          // byte offsets of the rows' maps in a slot, and their swizzle phases
+    int xj[NT], xk[NT];
+    bool pad[NT];
+    uint64_t scale[NT];           // the row's power of two, twice
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
         const short2 jk = P.rows[(size_t)(G.tile0 + t) * 128 + row];
-        pj[t] = jk.x;
-        pk[t] = jk.y;
+        pad[t] = jk.x < 0;
+        const int j = max((int)jk.x, 0), k = max((int)jk.y, 0);
+        oj[t] = j * 128; xj[t] = (j & 7) << 4;
+        ok_[t] = k * 128; xk[t] = (k & 7) << 4;
+        const float f = pad[t] ? 0.f : pow2f(row_exp(P.absmax[j], P.absmax[k]));
+        scale[t] = f2pack(f, f);
     }
-    // Rolling prefetch: the operands of the next tile (the next stage's first tile after the last one) are loaded
-    // before the current tile's products are formed, so shared-memory latency overlaps the arithmetic.  Padding rows
-    // (j < 0) read row 0 and store zeros.
-    float4 xc[4], yc[4], xn[4], yn[4];
-    uint4 bl[kBloItems];
-    // with two tiles warp 3 (idle otherwise) makes B_lo; with one tile the producers have the time for it (one warp
-    // would be the slower path: measured), with three warp 3 issues tile 2's MMAs
-    constexpr bool kBloByProducers = NT != 2;
-    auto load_tile = [&](const unsigned char* slot, int t, float4 (&x)[4], float4 (&y)[4]) {
-        const int j = max(pj[t], 0), k = max(pk[t], 0);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            x[c] = *ring_chunk(slot, j, 4 * gp + c);
-            y[c] = *ring_chunk(slot, k, 4 * gp + c);
-        }
-    };
-    auto load_blo = [&](const unsigned char* slot, uint4 (&b)[kBloItems]) {
-#pragma unroll
-        for (int m = 0; m < kBloItems; ++m)
-            if (ptid + 256 * m < s_chunks) b[m] = *reinterpret_cast<const uint4*>(slot + s_off + 16 * (ptid + 256 * m));
-    };
     // tensor-memory addresses from warp-uniform, divide-free values (the base is 0: the CTA holds all 512
-    // columns; the issuing warps check it), so that the compiler keeps the store addresses in uniform registers
-    if (nstages <= 0 || tmem != 0u) return;
-    if (!warp_wait(&slot_full[0], 0u, abort_flag, err)) return;
-    load_tile(ring, 0, xc, yc);
-    if (kBloByProducers) load_blo(ring, bl);
-    int s = 0, as = 0, s1 = 1 % kRingSlots;
-    uint32_t aph = 1u, s1ph = 0u;                        // a_empty parity of round st / nA - 1; slot_full of st + 1
-    uint32_t a_stage = (uint32_t)a_col0;
-    const uint32_t a_step = 64u * NT;
-    for (int st = 0; st < nstages; ++st) {
+    // columns; the issuing warp checks it), so that the compiler keeps the store addresses in uniform registers
+    if (tmem != 0u) return;
+    // slot sl: half sl % 2 of stage st = sl / 2, ring slot s = sl % kRingSlots, A stage as = st % nA
+    int s = gp, st = gp >> 1, as = st;
+    while (as >= nA) as -= nA;
+    uint32_t sph = 0u, aph = st >= nA ? 0u : 1u;        // slot_full parity; a_empty parity of round st / nA - 1
+    const uint32_t a_step = (uint32_t)kAcols * NT;
+    uint32_t a_stage = (uint32_t)a_col0 + a_step * (uint32_t)as;
+    const int nslots = 2 * nstages;
+    for (int sl = gp; sl < nslots; sl += kProdGroups) {
+        const uint32_t half = (uint32_t)(sl & 1);
+        if (!warp_wait(&slot_full[s], sph, abort_flag, err)) break;
         const unsigned char* slot = ring + (size_t)s * slot_bytes;
         bool ok = true;
 #pragma unroll
         for (int t = 0; t < NT; ++t) {
-            // (no break inside this unrolled loop: a failed wait clears ok, the rest of the stage is skipped)
-            if (t + 1 < NT) {
-                load_tile(slot, t + 1, xn, yn);
-            } else if (st + 1 < nstages) {
-                ok = ok && warp_wait(&slot_full[s1], s1ph, abort_flag, err);
-                if (ok) load_tile(ring + (size_t)s1 * slot_bytes, 0, xn, yn);
-            }
-            if (t == 0) {
-                // tensor memory A stage and B_lo stage `as` are free once the MMAs of stage st - nA completed
-                if (st >= nA) ok = ok && warp_wait(&a_empty[as], aph, abort_flag, err);
-                tc_fence_after();
-            }
-            if (!ok) continue;
             uint32_t v[32];
+            const unsigned char* rj = slot + oj[t];
+            const unsigned char* rk = slot + ok_[t];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                uint64_t h0, l0, h1, l1;
-                split_x2(mul_x2(f2pack(xc[c].x, xc[c].y), f2pack(yc[c].x, yc[c].y)), h0, l0);
-                split_x2(mul_x2(f2pack(xc[c].z, xc[c].w), f2pack(yc[c].z, yc[c].w)), h1, l1);
-                v[4 * c + 0] = (uint32_t)h0;
-                v[4 * c + 1] = (uint32_t)(h0 >> 32);
-                v[4 * c + 2] = (uint32_t)h1;
-                v[4 * c + 3] = (uint32_t)(h1 >> 32);
-                v[16 + 4 * c + 0] = (uint32_t)l0;
-                v[16 + 4 * c + 1] = (uint32_t)(l0 >> 32);
-                v[16 + 4 * c + 2] = (uint32_t)l1;
-                v[16 + 4 * c + 3] = (uint32_t)(l1 >> 32);
+            for (int c = 0; c < 8; ++c) {
+                const float4 x = *reinterpret_cast<const float4*>(rj + ((c << 4) ^ xj[t]));
+                const float4 y = *reinterpret_cast<const float4*>(rk + ((c << 4) ^ xk[t]));
+                split_h2(mul_x2(mul_x2(f2pack(x.x, x.y), f2pack(y.x, y.y)), scale[t]), v[2 * c], v[16 + 2 * c]);
+                split_h2(mul_x2(mul_x2(f2pack(x.z, x.w), f2pack(y.z, y.w)), scale[t]), v[2 * c + 1], v[16 + 2 * c + 1]);
             }
-            if (pj[t] < 0) {
+            if (pad[t]) {
 #pragma unroll
                 for (int c = 0; c < 32; ++c) v[c] = 0u;
             }
-            tmem_st32(lane_base + a_stage + (uint32_t)(64 * t + 32 * gp), v);
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                xc[c] = xn[c];
-                yc[c] = yn[c];
+            if (t == 0) {
+                // tensor memory A stage `as` is free once the MMAs of stage st - nA completed
+                if (st >= nA) ok = warp_wait(&a_empty[as], aph, abort_flag, err);
+                tc_fence_after();
             }
+            if (ok) tmem_st32(lane_base + a_stage + (uint32_t)(kAcols * t) + 32u * half, v);
         }
         if (!ok) break;
-        // B_lo = (g - trunc(g)) rounded to TF32 (nearest, ties away), at the same byte offset as g (same swizzle)
-        unsigned char* bs = bst + (size_t)as * bstage_bytes;
-#pragma unroll
-        for (int m = 0; m < kBloItems; ++m) {
-            if (kBloByProducers && ptid + 256 * m < s_chunks) {
-                uint32_t* w = reinterpret_cast<uint32_t*>(&bl[m]);
-                const uint64_t g01 = (uint64_t)w[0] | ((uint64_t)w[1] << 32);
-                const uint64_t g23 = (uint64_t)w[2] | ((uint64_t)w[3] << 32);
-                const uint64_t t01 = g01 & 0xFFFFE000FFFFE000ull, t23 = g23 & 0xFFFFE000FFFFE000ull;
-                const uint64_t l01 = sub_x2(g01, t01), l23 = sub_x2(g23, t23);
-                *reinterpret_cast<uint4*>(bs + 16 * (ptid + 256 * m)) =
-                    make_uint4(((uint32_t)l01 + 0x1000u) & 0xFFFFE000u, ((uint32_t)(l01 >> 32) + 0x1000u) & 0xFFFFE000u,
-                               ((uint32_t)l23 + 0x1000u) & 0xFFFFE000u, ((uint32_t)(l23 >> 32) + 0x1000u) & 0xFFFFE000u);
-            }
-        }
-        // the next stage's B_lo chunks (its slot is already full: waited for the first tile's prefetch)
-        if (kBloByProducers && st + 1 < nstages) load_blo(ring + (size_t)s1 * slot_bytes, bl);
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // B_lo stores -> tensor core
         tc_fence_before();
         // one arrival a warp on each barrier: __syncwarp orders the other lanes' stores and reads before lane 0's
-        // release (256 single-thread arrivals were 512 shared-memory atomics on two words every stage)
+        // release
         __syncwarp();
         if (lane == 0) {
             mbar_arrive(&a_full[as]);
             mbar_arrive(&slot_empty[s]);
         }
-        s = s1;
-        if (++s1 == kRingSlots) { s1 = 0; s1ph ^= 1u; }
-        if (++as == nA) { as = 0; aph ^= 1u; a_stage = (uint32_t)a_col0; } else { a_stage += a_step; }
+        s += kProdGroups;
+        if (s >= kRingSlots) { s -= kRingSlots; sph ^= 1u; }
+        // kProdGroups slots on
+        const int adv = ((int)half + kProdGroups) >> 1;
+        st += adv;
+        as += adv;
+        a_stage += a_step * (uint32_t)adv;
+        if (as >= nA) { as -= nA; aph ^= 1u; a_stage -= a_step * (uint32_t)nA; }
+    }
+}
+
+// B warp w (0 .. 3): half of the singles (8-row groups w / 2, w / 2 + 2, ..) of ring slot b = w % 2 of every stage -> FP16
+// hi and lo rows of 64 cells (128 bytes, 128-byte swizzle), cells 32 b .. 32 b + 31.  Rows r of the singles region, in
+// groups of eight: hi rows of group i at 2 i x 1024 bytes, lo rows at (2 i + 1) x 1024, so that a window of W singles is
+// 2W consecutive B rows.  A warp makes a group of eight rows at a time, lane (r, piece) = (lane / 4, lane % 4) eight cells
+// of row r; the rows' scales wait in shared memory.  (Two warps with the scales read from global memory set the pace of the
+// whole kernel.)
+__device__ __forceinline__ void make_b(const GroupDesc& G, const Params& P, const unsigned char* ring,
+                                       unsigned char* bst, const float* bscale, uint64_t* slot_full, uint64_t* slot_empty,
+                                       uint64_t* a_full, uint64_t* a_empty, volatile int* abort_flag, int nstages, int w,
+                                       int lane) {
+    const int b = w & 1;
+    const int nA = G.nA, slot_bytes = P.slot_bytes, stage_bytes = 2 * G.bstage_bytes;
+    const int ngrp = P.s_chunks / 64;               // groups of eight rows (eight chunks a row)
+    int* const err = P.err;
+    const int r = lane >> 2, pc = lane & 3, x = r << 4;
+    const int src0 = P.s_off + r * 128 + ((pc << 5) ^ x), src1 = P.s_off + r * 128 + (((pc << 5) + 16) ^ x);
+    const int dst0 = r * 128 + (((4 * b + pc) << 4) ^ x);
+    int s = b, as = 0;
+    uint32_t sph = 0u, aph = 1u;
+    for (int st = 0; st < nstages; ++st) {
+        if (!warp_wait(&slot_full[s], sph, abort_flag, err)) break;
+        if (st >= nA && !warp_wait(&a_empty[as], aph, abort_flag, err)) break;
+        const unsigned char* src = ring + (size_t)s * slot_bytes;
+        unsigned char* dst = bst + (size_t)as * stage_bytes + dst0;
+#pragma unroll 2
+        for (int g = w >> 1; g < ngrp; g += 2) {
+            const float f = bscale[8 * g + r];
+            const uint64_t f2 = f2pack(f, f);
+            const float4 u = *reinterpret_cast<const float4*>(src + src0 + g * 1024);
+            const float4 v = *reinterpret_cast<const float4*>(src + src1 + g * 1024);
+            uint4 h, l;
+            split_h2(mul_x2(f2pack(u.x, u.y), f2), h.x, l.x);
+            split_h2(mul_x2(f2pack(u.z, u.w), f2), h.y, l.y);
+            split_h2(mul_x2(f2pack(v.x, v.y), f2), h.z, l.z);
+            split_h2(mul_x2(f2pack(v.z, v.w), f2), h.w, l.w);
+            *reinterpret_cast<uint4*>(dst + g * 2048) = h;
+            *reinterpret_cast<uint4*>(dst + g * 2048 + 1024) = l;
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // B stores -> tensor core
+        __syncwarp();
+        if (lane == 0) {
+            mbar_arrive(&a_full[as]);
+            mbar_arrive(&slot_empty[s]);
+        }
+        s += 2;
+        if (s >= kRingSlots) { s = b; sph ^= 1u; }
+        if (++as == nA) { as = 0; aph ^= 1u; }
     }
 }
 
@@ -495,15 +531,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     unsigned char* bst = smem + P.off_b;
     double* acc64 = reinterpret_cast<double*>(smem + P.off_acc);                 // [unit][16][128]
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P.off_bar);
-    uint64_t* slot_full = bars;                        // [kRingSlots]  TMA -> producers
-    uint64_t* slot_empty = bars + kRingSlots;          // [kRingSlots]  producers -> TMA
-    uint64_t* a_full = bars + 2 * kRingSlots;          // [kMaxAStages] producers -> issuers
-    uint64_t* a_empty = a_full + kMaxAStages;          // [kMaxAStages] MMA commit -> producers
-    uint64_t* d_full = a_empty + kMaxAStages;          // [2][kMaxTiles] MMA commit -> epilogue (D buffer, tile)
-    uint64_t* d_empty = d_full + 2 * kMaxTiles;        // [2]            epilogue -> issuers (D buffer)
-    uint64_t* fin = d_empty + 2;                       // [kMaxTiles]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + kMaxTiles);
+    uint64_t* slot_full = bars;                        // [kRingSlots]  TMA -> producers, B warps
+    uint64_t* slot_empty = bars + kRingSlots;          // [kRingSlots]  producers, B warps -> TMA
+    uint64_t* a_full = bars + 2 * kRingSlots;          // [kMaxAStages] producers, B warps -> issuer
+    uint64_t* a_empty = a_full + kMaxAStages;          // [kMaxAStages] MMA commit -> producers, B warps
+    uint64_t* d_full = a_empty + kMaxAStages;          // [kDBuf]       MMA commit -> epilogue
+    uint64_t* d_empty = d_full + kDBuf;                // [kDBuf]       epilogue -> issuer
+    uint64_t* fin = d_empty + kDBuf;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    float* bscale = reinterpret_cast<float*>(tmem_slot + 2);                    // [64] scales of the singles region's rows
 
     // warp index through a shuffle from lane 0: the compiler then knows it is warp-uniform, so role branches and
     // the tensor-memory addresses derived from it stay in uniform registers
@@ -511,28 +548,29 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const long c0 = (long)blockIdx.x * P.cells_cta;
     const long c1 = min(P.ncell, c0 + P.cells_cta);
-    const int nslots = c0 < c1 ? (int)((c1 - c0 + kSlotCells - 1) / kSlotCells) : 0;
-    const int nstages = nslots;                 // one A stage per ring slot
+    const int nstages = c0 < c1 ? (int)((c1 - c0 + kKC - 1) / kKC) : 0;
+    const int nslots = 2 * nstages;             // cells beyond the maps read as zero (TMA out-of-bounds fill)
     // plan fields used in the loops, in registers
-    const int nA = G.nA, ntiles = G.ntiles, a_col0 = G.a_col0, bstage_bytes = G.bstage_bytes;
+    const int nA = G.nA, ntiles = G.ntiles, a_col0 = G.a_col0;
     const int slot_bytes = P.slot_bytes;
     int* const err = P.err;
 
     for (int i = tid; i < G.nunits * 16 * 128; i += kThreads) acc64[i] = 0.0;
+    if (tid < P.s_chunks / 8) bscale[tid] = pow2f(single_exp(P.absmax[P.s_off / 128 + tid]));
     if (tid == 0) {
         for (int s = 0; s < kRingSlots; ++s) {
             mbar_init(&slot_full[s], 1);
-            // producer warps read a slot, the MMAs read B_hi, warp 3 (two tiles) reads it for B_lo
-            mbar_init(&slot_empty[s], kProdWarps + ntiles + (ntiles == 2 ? 1 : 0));
+            mbar_init(&slot_empty[s], 4 + 2);          // the slot's producer group and its two B warps
         }
         for (int s = 0; s < kMaxAStages; ++s) {
-            // both producer groups make a stage's A (and B_lo, except with two tiles: then warp 3 makes it)
-            mbar_init(&a_full[s], kProdWarps + (ntiles == 2 ? 1 : 0));
-            mbar_init(&a_empty[s], ntiles);        // one commit per issuing thread (tile)
+            mbar_init(&a_full[s], 4 * 2 + kBWarps);    // four producer warps a slot, two slots; the B warps
+            mbar_init(&a_empty[s], 1);
         }
-        for (int i = 0; i < 2 * kMaxTiles; ++i) mbar_init(&d_full[i], 1);
-        for (int i = 0; i < 2; ++i) mbar_init(&d_empty[i], kEpiWarps);
-        for (int i = 0; i < kMaxTiles; ++i) mbar_init(&fin[i], 1);
+        for (int i = 0; i < kDBuf; ++i) {
+            mbar_init(&d_full[i], 1);
+            mbar_init(&d_empty[i], kEpiWarps);
+        }
+        mbar_init(fin, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -545,7 +583,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp < kProdWarp0) {
+    if (warp < kBWarp0) {
         // warpgroup 0 hands registers to the producers (all four warps, one instruction)
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCtl));
         if (warp == 0) {
@@ -572,120 +610,83 @@ __global__ void __launch_bounds__(kThreads, 1)
                     drain_wait(&slot_full[sl % kRingSlots], (uint32_t)((sl / kRingSlots) & 1), err);
             }
             __syncwarp();
-        } else if (warp == 3 && ntiles == 2) {
-            // ------------------------------------------------------------------ B_lo (two tiles)
-            // every 16-byte chunk of a slot's singles region -> (g - trunc(g)) rounded to TF32, same offset in the
-            // B_lo stage; released to the issuers with one arrival on the stage barrier
-            const int s_off = P.s_off, s_chunks = P.s_chunks;
-            int s = 0, as = 0;
-            uint32_t sph = 0u, aph = 1u;
-            for (int st = 0; st < nstages; ++st) {
-                if (!warp_wait(&slot_full[s], sph, abort_flag, err)) break;
-                if (st >= nA && !warp_wait(&a_empty[as], aph, abort_flag, err)) break;
-                const unsigned char* src = ring + (size_t)s * slot_bytes + s_off;
-                unsigned char* dst = bst + (size_t)as * bstage_bytes;
-                for (int i0 = 0; i0 < s_chunks; i0 += 128) {
-                    uint4 g[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int i = i0 + 32 * u + lane;
-                        if (i < s_chunks) g[u] = *reinterpret_cast<const uint4*>(src + 16 * i);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int i = i0 + 32 * u + lane;
-                        if (i < s_chunks) {
-                            const uint64_t g01 = (uint64_t)g[u].x | ((uint64_t)g[u].y << 32);
-                            const uint64_t g23 = (uint64_t)g[u].z | ((uint64_t)g[u].w << 32);
-                            const uint64_t l01 = sub_x2(g01, g01 & 0xFFFFE000FFFFE000ull);
-                            const uint64_t l23 = sub_x2(g23, g23 & 0xFFFFE000FFFFE000ull);
-                            *reinterpret_cast<uint4*>(dst + 16 * i) = make_uint4(
-                                ((uint32_t)l01 + 0x1000u) & 0xFFFFE000u, ((uint32_t)(l01 >> 32) + 0x1000u) & 0xFFFFE000u,
-                                ((uint32_t)l23 + 0x1000u) & 0xFFFFE000u, ((uint32_t)(l23 >> 32) + 0x1000u) & 0xFFFFE000u);
-                        }
-                    }
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // B_lo stores -> tensor core
-                __syncwarp();
-                if (lane == 0) {
-                    mbar_arrive(&a_full[as]);
-                    mbar_arrive(&slot_empty[s]);
-                }
-                if (++s == kRingSlots) { s = 0; sph ^= 1u; }
-                if (++as == nA) { as = 0; aph ^= 1u; }
-            }
-        } else if (warp - 1 < ntiles) {
-            // ------------------------------------------------------------------ MMA issue (warp 1 + t: tile t)
+        } else if (warp == 1) {
+            // ------------------------------------------------------------------ MMA issue
             // The whole warp runs the loop (converged; every lane polls the barriers); the elected lane issues and
-            // commits inside mma_tf32 / mma_commit.
-            // tile t's window of singles: rows s0 .. s0 + W - 1 of a slot's singles region (B_hi: the slot itself, read
-            // as TF32, i.e. truncated) and of the B_lo stage (same layout)
-            const uint32_t ring_s = smem_u32(ring) + (uint32_t)P.s_off, bst_s = smem_u32(bst);
-            const int t = warp - 1;
-            const int W = G.tile_w[t];
-            const uint32_t idesc_w = idesc_tf32(128, W);
-            // Every operand below is built from warp-uniform values (parameters, constants, loop-carried counters;
-            // no division) so that the compiler keeps it in uniform registers: the tensor memory base is the
-            // constant 0, which is what a CTA allocating all 512 columns receives (lane 0, column 0).
+            // commits inside mma_f16 / mma_commit.  Every operand is built from warp-uniform values (parameters,
+            // constants, loop-carried counters; no division) so that the compiler keeps it in uniform registers: the
+            // tensor memory base is the constant 0, which is what a CTA allocating all 512 columns receives.
             const bool tmem_ok = tmem == 0u;
             if (!tmem_ok && lane == 0) {
                 *abort_flag = 1;
                 atomicExch(err, 1);
             }
-            const uint32_t dm = (uint32_t)G.dm_col[t], dc = dm + (uint32_t)W;
-            const uint32_t a_first = (uint32_t)(a_col0 + 64 * t), a_step = (uint32_t)(64 * ntiles);
-            const uint64_t bh_first = sdesc_sw128(ring_s + (uint32_t)(128 * G.tile_s0[t]));
-            const uint64_t bl_first = sdesc_sw128(bst_s + (uint32_t)(128 * G.tile_s0[t]));
-            // descriptor address steps (16-byte units; no carry out of the 14-bit field: shared memory < 2^18 bytes)
-            const uint64_t bh_step = (uint64_t)(slot_bytes >> 4), bl_step = (uint64_t)(bstage_bytes >> 4);
-            int s = 0, as = 0, pos = 0, per = 0;
-            uint32_t sph = 0, aph = 0;
-            uint32_t aa = a_first;
-            uint64_t bh = bh_first, bl = bl_first;
+            // tile t's window of singles: 2W rows of the B stage from group s0 / 8 (2048 bytes a group of eight)
+            uint32_t idesc[kMaxTiles], dcol[kMaxTiles];
+            uint64_t bwin[kMaxTiles];
+#pragma unroll
+            for (int t = 0; t < kMaxTiles; ++t) {
+                const int tt = t < ntiles ? t : 0;
+                idesc[t] = idesc_f16(128, 2 * G.tile_w[tt]);
+                dcol[t] = (uint32_t)G.dm_col[tt];
+                bwin[t] = sdesc_sw128(smem_u32(bst) + (uint32_t)(256 * G.tile_s0[tt]));
+            }
+            const uint32_t a_step = (uint32_t)(kAcols * ntiles), d_cols = (uint32_t)G.d_cols;
+            // descriptor address step (16-byte units; no carry out of the 14-bit field: shared memory < 2^18 bytes)
+            const uint64_t b_step = (uint64_t)(2 * G.bstage_bytes >> 4);
+            int as = 0;
+            uint32_t aph = 0, aa = (uint32_t)a_col0, db = 0, dph = 1;
+            uint64_t bo = 0;
             for (int st = 0; st < nstages && tmem_ok; ++st) {
-                const bool pstart = pos == 0;
-                // one accumulator buffer: a period's first MMAs wait until the epilogue has read the previous one
-                if (pstart && per >= 1 && !warp_wait(&d_empty[0], (uint32_t)((per - 1) & 1), abort_flag, err)) break;
-                if (!warp_wait(&slot_full[s], sph, abort_flag, err)) break;
+                // the epilogue has read this accumulator buffer's previous sums
+                if (st >= kDBuf && !warp_wait(&d_empty[db], dph, abort_flag, err)) break;
                 if (!warp_wait(&a_full[as], aph, abort_flag, err)) break;
                 tc_fence_after();
 #pragma unroll
-                for (int ks = 0; ks < kKC / 8; ++ks) {
-                    // K step ks: cells 8 ks .. 8 ks + 7; A_hi at half (ks / 2), column 8 (ks % 2); A_lo at +16.  B
-                    // advances 32 bytes a step within the swizzle atom (2 in the descriptor's address field)
-                    const uint32_t ah = aa + 32u * (ks >> 1) + 8u * (ks & 1);
-                    const uint32_t acc = (pstart && ks == 0) ? 0u : 1u;
-                    mma_tf32(dm, ah, bh + (uint64_t)(2 * ks), idesc_w, acc);          // A_hi . B_hi
-                    mma_tf32(dc, ah, bl + (uint64_t)(2 * ks), idesc_w, acc);          // A_hi . B_lo
-                    mma_tf32(dc, ah + 16u, bh + (uint64_t)(2 * ks), idesc_w, 1u);     // + A_lo . B_hi
+                for (int t = 0; t < kMaxTiles; ++t) {
+                    if (t < ntiles) {
+                        const uint32_t d = dcol[t] + db * d_cols, a = aa + (uint32_t)(kAcols * t);
+                        const uint64_t bd = bwin[t] + bo;
+                        // K step ks: cells 16 ks .. 16 ks + 15; A_hi at slot block ks / 2, column 8 (ks % 2); A_lo at
+                        // +16.  B advances 32 bytes a step within the swizzle atom (2 in the descriptor)
+#pragma unroll
+                        for (int ks = 0; ks < kKC / 16; ++ks)
+                            mma_f16(d, a + 16u + 32u * (ks >> 1) + 8u * (ks & 1), bd + (uint64_t)(2 * ks), idesc[t],
+                                    ks ? 1u : 0u);
+#pragma unroll
+                        for (int ks = 0; ks < kKC / 16; ++ks)
+                            mma_f16(d, a + 32u * (ks >> 1) + 8u * (ks & 1), bd + (uint64_t)(2 * ks), idesc[t], 1u);
+                    }
                 }
                 mma_commit(&a_empty[as]);
-                mma_commit(&slot_empty[s]);
-                if (pos == kPeriod - 1 || st == nstages - 1) mma_commit(&d_full[t]);
-                if (++s == kRingSlots) { s = 0; sph ^= 1u; bh = bh_first; } else { bh += bh_step; }
-                if (++as == nA) { as = 0; aph ^= 1u; aa = a_first; bl = bl_first; } else { aa += a_step; bl += bl_step; }
-                if (++pos == kPeriod) { pos = 0; ++per; }
+                mma_commit(&d_full[db]);
+                if (++as == nA) { as = 0; aph ^= 1u; aa = (uint32_t)a_col0; bo = 0; } else { aa += a_step; bo += b_step; }
+                db ^= 1u;
+                if (db == 0) dph ^= 1u;
             }
             // every MMA issued by the elected thread has completed before TMEM is released
-            mma_commit(&fin[t]);
-            drain_wait(&fin[t], 0, err);
+            mma_commit(fin);
+            drain_wait(fin, 0, err);
             __syncwarp();
         }
+    } else if (warp < kProdWarp0) {
+        // ------------------------------------------------------------------ the B operand
+        if (kRegsB < kRegsLaunch) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsB));
+        make_b(G, P, ring, bst, bscale, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp - kBWarp0, lane);
     } else if (warp < kProdWarp0 + kProdWarps) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsProd));
         // ------------------------------------------------------------------ producers
         switch (ntiles) {
-            case 1: producer<1>(G, P, tmem, ring, bst, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
-            case 2: producer<2>(G, P, tmem, ring, bst, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
-            default: producer<3>(G, P, tmem, ring, bst, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
+            case 1: producer<1>(G, P, tmem, ring, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
+            case 2: producer<2>(G, P, tmem, ring, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
+            default: producer<3>(G, P, tmem, ring, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
         }
     } else {
         // ------------------------------------------------------------------ epilogue
-        const int nper = (nstages + kPeriod - 1) / kPeriod;
         switch (G.nunits) {
-            case 1: epilogue<1>(G, P, tmem, acc64, d_full, d_empty, abort_flag, nper, warp, lane); break;
-            case 2: epilogue<2>(G, P, tmem, acc64, d_full, d_empty, abort_flag, nper, warp, lane); break;
-            default: epilogue<3>(G, P, tmem, acc64, d_full, d_empty, abort_flag, nper, warp, lane); break;
+            case 1: epilogue<1>(G, P, tmem, acc64, d_full, d_empty, abort_flag, nstages, warp, lane); break;
+            case 2: epilogue<2>(G, P, tmem, acc64, d_full, d_empty, abort_flag, nstages, warp, lane); break;
+            default: epilogue<3>(G, P, tmem, acc64, d_full, d_empty, abort_flag, nstages, warp, lane); break;
         }
     }
     tc_fence_before();
@@ -694,15 +695,32 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-// out[o] = sum over CTAs of partial[cta][gidx[o]], in CTA order (deterministic).
+// absmax[row0 + r] = bit pattern of max |maps[r][x]| over the cells (blockIdx.y: map r; absmax zeroed before).  NaN and
+// infinity order above every finite value as bit patterns.
+__global__ void __launch_bounds__(256) k_absmax(const float4* __restrict__ maps, long n4, uint32_t* __restrict__ absmax) {
+    const float4* m = maps + (size_t)blockIdx.y * n4;
+    uint32_t a = 0;
+    for (long i = (long)blockIdx.x * 256 + threadIdx.x; i < n4; i += (long)gridDim.x * 256) {
+        const float4 v = m[i];
+        a = max(max(a, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu)),
+                max(__float_as_uint(v.z) & 0x7fffffffu, __float_as_uint(v.w) & 0x7fffffffu));
+    }
+    a = __reduce_max_sync(0xffffffffu, a);
+    if ((threadIdx.x & 31) == 0 && a) atomicMax(absmax + blockIdx.y, a);
+}
+
+// out[o] = 2^-(row and single exponents) sum over CTAs of partial[cta][gidx[o]], in CTA order (deterministic).  rows[o]
+// holds the slot rows (j, k, single) of output o.
 __global__ void k_reduce_gather(const double* __restrict__ partial, int ncta, long stride,
-                                const int* __restrict__ gidx, int n_out, double* __restrict__ out) {
+                                const int* __restrict__ gidx, const uchar4* __restrict__ rows,
+                                const uint32_t* __restrict__ absmax, int n_out, double* __restrict__ out) {
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= n_out) return;
     const long g = gidx[o];
     double s = 0.0;
     for (int c = 0; c < ncta; ++c) s += partial[(long)c * stride + g];
-    out[o] = s;
+    const uchar4 r = rows[o];
+    out[o] = ldexp(s, -row_exp(absmax[r.x], absmax[r.y]) - single_exp(absmax[r.z]));
 }
 
 // Self-test of the bounded waits: one thread waits on an mbarrier phase that nothing completes; the wait gives up
@@ -1041,8 +1059,10 @@ struct Plan {
     size_t smem = 0;
     short2* d_rows = nullptr;
     int* d_gidx = nullptr;
+    uchar4* d_orows = nullptr;   // slot rows (j, k, single) of every output
     double* d_partial = nullptr;
     ~Plan() {
+        if (d_orows) cudaFree(d_orows);
         if (d_rows) cudaFree(d_rows);
         if (d_gidx) cudaFree(d_gidx);
         if (d_partial) cudaFree(d_partial);
@@ -1075,6 +1095,33 @@ static std::vector<std::pair<int, int>> cut_tiles(const std::vector<NeedPair>& P
     return seg;
 }
 
+// Orders the rows [first, last) of a tile, sorted by (j, k), to avoid bank conflicts of the producers' gathers.  A
+// 16-byte load of a warp is served for eight lanes at a time; the slots' swizzle puts chunk c of map m into bank group
+// c ^ (m % 8), so eight consecutive rows are conflict-free when their maps j, and their maps k, are equal or distinct
+// modulo 8.  Greedy: every group of eight takes the first remaining rows that conflict least.
+static void order_rows(std::vector<NeedPair>& need, int first, int last) {
+    std::vector<NeedPair> rest(need.begin() + first, need.begin() + last), out;
+    std::vector<char> used(rest.size(), 0);
+    while (out.size() < rest.size()) {
+        std::set<int> mj[8], mk[8];          // the group's maps by bank group
+        for (int g = 0; g < 8 && out.size() < rest.size(); ++g) {
+            int best = -1, best_cost = 1 << 30;
+            for (size_t i = 0; i < rest.size(); ++i) {
+                if (used[i]) continue;
+                const std::set<int>&a = mj[rest[i].j & 7], &b = mk[rest[i].k & 7];
+                const int cost = (int)(a.size() - a.count(rest[i].j) + b.size() - b.count(rest[i].k));
+                if (cost < best_cost) { best_cost = cost; best = (int)i; }
+                if (cost == 0) break;
+            }
+            used[best] = 1;
+            mj[rest[best].j & 7].insert(rest[best].j);
+            mk[rest[best].k & 7].insert(rest[best].k);
+            out.push_back(rest[best]);
+        }
+    }
+    std::copy(out.begin(), out.end(), need.begin() + first);
+}
+
 // Pure host layout of a plan (no CUDA calls): tiles, row groups, TMEM / shared-memory layout, the row table and the
 // gather index of every output.  Returns nullptr or an error message.
 // sing_g = 1 with hsep = 1: the slot holds the g rows and the h rows (pairs may take one map from each, h rows at
@@ -1098,9 +1145,9 @@ static const char* layout_plan(Plan& pl, long ncell, int nsm, int ng, int nh, in
         int lo = 1 << 30, hi = -1;
         for (int i = sg.first; i < sg.second; ++i) { lo = std::min(lo, need[i].lo); hi = std::max(hi, need[i].hi); }
         const int s0 = lo / 8 * 8;
-        // within a tile, order rows by (j, k): lanes of a warp then share j and read consecutive k (no bank conflicts)
         std::stable_sort(need.begin() + sg.first, need.begin() + sg.second,
                          [](const NeedPair& a, const NeedPair& b) { return std::tie(a.j, a.k) < std::tie(b.j, b.k); });
+        order_rows(need, sg.first, sg.second);
         tiles.push_back({sg.first, sg.second, s0, round_w(hi + 1 - s0)});
     }
     if (tiles.empty()) tiles.push_back({0, 0, 0, 16});
@@ -1110,7 +1157,7 @@ static const char* layout_plan(Plan& pl, long ncell, int nsm, int ng, int nh, in
         int e = t, dcols = 0, units = 0;
         while (e < (int)tiles.size() && e - t < opts.group_cap) {
             const int nd = dcols + 2 * tiles[e].W, nu = units + tiles[e].W / 16, nt = e - t + 1;
-            if (nu > kMaxUnits || kDBuf * ((nd + 31) / 32 * 32) + 2 * 2 * kKC * nt > 512) break;
+            if (nu > kMaxUnits || kDBuf * ((nd + 31) / 32 * 32) + 2 * kAcols * nt > 512) break;
             dcols = nd; units = nu; ++e;
         }
         if (e == t) return "contract_tc: tile does not fit tensor memory";
@@ -1140,7 +1187,7 @@ static const char* layout_plan(Plan& pl, long ncell, int nsm, int ng, int nh, in
         D = GroupDesc{};
         const int t0 = groups[gi].first, nt = groups[gi].second - t0;
         D.tile0 = t0; D.ntiles = nt; D.unit_base = unit_base;
-        // accumulators: [hi*hi | corrections] (2W) of every tile, largest first, so each is aligned to its size
+        // accumulators (2W columns) of every tile, largest first, so each is aligned to its size
         std::vector<std::pair<int, int>> dl;   // (size, tile)
         for (int t = 0; t < nt; ++t) dl.push_back({2 * tiles[t0 + t].W, t});
         std::stable_sort(dl.begin(), dl.end(), [](auto& a, auto& b) { return a.first > b.first; });
@@ -1151,15 +1198,15 @@ static const char* layout_plan(Plan& pl, long ncell, int nsm, int ng, int nh, in
         }
         D.d_cols = (col + 31) / 32 * 32;
         D.a_col0 = kDBuf * D.d_cols;
-        D.nA = std::min(kMaxAStages, (512 - D.a_col0) / (2 * kKC * nt));
-        // windows of singles; B_lo stages hold a slot's whole singles region
+        D.nA = std::min(kMaxAStages, (512 - D.a_col0) / (kAcols * nt));
+        // windows of singles; B stages hold a slot's whole singles region, hi and lo
         for (int t = 0; t < nt; ++t) {
             const TileH& T = tiles[t0 + t];
             D.tile_w[t] = T.W;
             D.tile_s0[t] = T.s0;
         }
         D.bstage_bytes = srows * 128;
-        max_b = std::max(max_b, D.nA * D.bstage_bytes);
+        max_b = std::max(max_b, D.nA * 2 * D.bstage_bytes);
         // output units
         int u = 0;
         for (int t = 0; t < nt; ++t)
@@ -1190,17 +1237,34 @@ static const char* layout_plan(Plan& pl, long ncell, int nsm, int ng, int nh, in
     P.off_acc = P.off_b + max_b;
     P.off_bar = P.off_acc + kMaxUnits * 16 * 128 * 8;
     // + 1024: the kernel aligns the start of its dynamic shared memory to 1024 bytes (128-byte swizzle atoms)
-    pl.smem = std::max((size_t)kMinSmem, (size_t)P.off_bar + 64 * 8 + 64) + 1024;
+    pl.smem = std::max((size_t)kMinSmem, (size_t)P.off_bar + 64 * 8 + 64 * 4) + 1024;
     if (pl.smem > 227 * 1024) return "contract_tc: shared memory plan exceeds 227 KB";
 
-    const long nsl = (ncell + kSlotCells - 1) / kSlotCells;
+    const long nsl = (ncell + kKC - 1) / kKC;
     const long want = opts.cta_mode == 1 ? std::max(1L, (long)nsm / pl.ngroups) : (opts.cta_mode == 2 ? 2L * nsm : (long)nsm);
     pl.ncta = (int)std::max(1L, std::min(want, nsl));
-    pl.cells_cta = (nsl + pl.ncta - 1) / pl.ncta * kSlotCells;
+    pl.cells_cta = (nsl + pl.ncta - 1) / pl.ncta * kKC;
     pl.ncta = (int)((ncell + pl.cells_cta - 1) / pl.cells_cta);
     P.ncell = ncell;
     P.cells_cta = pl.cells_cta;
     return nullptr;
+}
+
+struct PlanCache {
+    std::map<std::tuple<int, int, int, int, long>, Plan*> plans;   // (ng, nh, hsep, kind, ncell)
+    double* gram_part = nullptr;                                   // Gram partials (K splits)
+    size_t gram_cap = 0;
+    uint32_t* d_absmax = nullptr;                                  // [kMaxRows] maxima of the maps by slot row
+    ~PlanCache() {
+        if (d_absmax) cudaFree(d_absmax);
+        for (auto& kv : plans) delete kv.second;
+        if (gram_part) cudaFree(gram_part);
+    }
+};
+
+static PlanCache* cache_of(polybin_ctx* ctx) {
+    if (!ctx->tc) ctx->tc = new PlanCache();
+    return static_cast<PlanCache*>(ctx->tc);
 }
 
 static int build_plan(polybin_ctx* ctx, Plan& pl, long ncell, int ng, int nh, int hsep, std::vector<NeedPair> need,
@@ -1214,27 +1278,26 @@ static int build_plan(polybin_ctx* ctx, Plan& pl, long ncell, int ng, int nh, in
     pl.need = need;
     pl.sing_g = sing_g;
     pl.ncell = ncell;
+    std::vector<uchar4> orows(std::max(n_out, 1), make_uchar4(0, 0, 0, 0));
+    const int srow0 = (hsep && !sing_g) ? (ng + 7) / 8 * 8 : 0;      // slot row of the first single
+    for (const NeedPair& p : need)
+        for (auto& so : p.outs)
+            orows[so.second] = make_uchar4((unsigned char)p.j, (unsigned char)p.k, (unsigned char)(srow0 + so.first), 0);
     const char* msg = layout_plan(pl, ncell, nsm, ng, nh, hsep, std::move(need), n_out, rows, gidx, sing_g, opts);
     if (msg) return quiet ? POLYBIN_EINVAL : fail(ctx, POLYBIN_EINVAL, "%s", msg);
+    PlanCache* pc = cache_of(ctx);
+    if (!pc->d_absmax) PB_CUDA_OK(cudaMalloc(&pc->d_absmax, sizeof(uint32_t) * kMaxRows));
     PB_CUDA_OK(cudaMalloc(&pl.d_rows, sizeof(short2) * rows.size()));
     PB_CUDA_OK(cudaMemcpy(pl.d_rows, rows.data(), sizeof(short2) * rows.size(), cudaMemcpyHostToDevice));
     PB_CUDA_OK(cudaMalloc(&pl.d_gidx, sizeof(int) * gidx.size()));
     PB_CUDA_OK(cudaMemcpy(pl.d_gidx, gidx.data(), sizeof(int) * gidx.size(), cudaMemcpyHostToDevice));
+    PB_CUDA_OK(cudaMalloc(&pl.d_orows, sizeof(uchar4) * orows.size()));
+    PB_CUDA_OK(cudaMemcpy(pl.d_orows, orows.data(), sizeof(uchar4) * orows.size(), cudaMemcpyHostToDevice));
     PB_CUDA_OK(cudaMalloc(&pl.d_partial, sizeof(double) * (size_t)pl.ncta * pl.total_units * 2048));
     pl.base.rows = pl.d_rows;
     pl.base.partial = pl.d_partial;
     return POLYBIN_OK;
 }
-
-struct PlanCache {
-    std::map<std::tuple<int, int, int, int, long>, Plan*> plans;   // (ng, nh, hsep, kind, ncell)
-    double* gram_part = nullptr;                                   // Gram partials (K splits)
-    size_t gram_cap = 0;
-    ~PlanCache() {
-        for (auto& kv : plans) delete kv.second;
-        if (gram_part) cudaFree(gram_part);
-    }
-};
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -1311,28 +1374,37 @@ static int launch(polybin_ctx* ctx, Plan& pl, const float* g, const float* h, do
             return fail(ctx, POLYBIN_ECUDA, "contract_tc: kernel built with %d registers a thread, %d expected", fa.numRegs,
                         kRegsLaunch);
     }
+    PlanCache* pc = cache_of(ctx);
     Params P = pl.base;
     P.err = ctx->d_err;
+    P.absmax = pc->d_absmax;
     {
         StageTimer timer(ctx, kStageContract);
+        // the maps' maxima (scale factors), by slot row
+        e = cudaMemsetAsync(pc->d_absmax, 0, sizeof(uint32_t) * kMaxRows, ctx->stream);
+        if (e != cudaSuccess) return fail_cuda(ctx, e, "cudaMemsetAsync", __FILE__, __LINE__);
+        const long n4 = pl.base.ncell / 4;
+        const unsigned nblk = (unsigned)std::min((n4 + 1023) / 1024, 64L);
+        k_absmax<<<dim3(nblk, pl.ng, 1), 256, 0, ctx->stream>>>(reinterpret_cast<const float4*>(g), n4, pc->d_absmax);
+        ctx->launches += 1;
+        if (pl.hsep) {
+            k_absmax<<<dim3(nblk, pl.nh, 1), 256, 0, ctx->stream>>>(reinterpret_cast<const float4*>(h), n4,
+                                                                     pc->d_absmax + pl.base.h_row0);
+            ctx->launches += 1;
+        }
         k_contract_tc<<<dim3(pl.ncta, pl.ngroups, 1), kThreads, pl.smem, ctx->stream>>>(mg, mh, P);
         ctx->launches += 1;
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail_cuda(ctx, e, "k_contract_tc", __FILE__, __LINE__);
         k_reduce_gather<<<(pl.n_out + 255) / 256, 256, 0, ctx->stream>>>(pl.d_partial, pl.ncta,
                                                                           (long)pl.total_units * 2048, pl.d_gidx,
-                                                                          pl.n_out, d_out);
+                                                                          pl.d_orows, pc->d_absmax, pl.n_out, d_out);
         ctx->launches += 1;
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail_cuda(ctx, e, "k_reduce_gather", __FILE__, __LINE__);
     }
     if (ctx->capturing) return POLYBIN_OK;   // the caller reads the error flags after the graph has run
     return read_err_flags(ctx, "contract_tc");
-}
-
-static PlanCache* cache_of(polybin_ctx* ctx) {
-    if (!ctx->tc) ctx->tc = new PlanCache();
-    return static_cast<PlanCache*>(ctx->tc);
 }
 
 // Autotuner.  On the first launch of a plan outside stream capture (unless POLYBIN_AUTOTUNE=0), every distinct valid
