@@ -299,33 +299,42 @@ int run_contract(polybin_ctx* ctx, const T* g, int ng, const T* h, int nh, doubl
     k_contract<T><<<grid, 256, sm, ctx->stream>>>(g, h, ncell, ctx->d_pairs + pairs_offset(ng), G, d_partial);
     if ((rc = launch_check(ctx, "k_contract"))) return rc;
     const long nout = (long)G.npairs * G.nh;
-    k_reduce_partials<<<(unsigned)((nout + 255) / 256), 256, 0, ctx->stream>>>(d_partial, G.ncb, nout, d_out);
+    k_reduce_partials<<<reduce_blocks(nout), dim3(32, kRedSlices), 0, ctx->stream>>>(d_partial, G.ncb, nout, d_out);
     return launch_check(ctx, "k_reduce_partials");
+}
+
+// Partials [nx][nb][nseg][nell] of the binned products of nx box spectra X + z x_stride with A.
+template <typename T>
+int launch_cross_bin(polybin_ctx* ctx, const C<T>* X, long x_stride, int nx, const C<T>* A, double* partial) {
+    k_cross_bin<T><<<dim3(ctx->nb, ctx->pk_nseg, nx), 256, 0, ctx->stream>>>(
+        X, A, x_stride, ctx->d_offs, ctx->d_coef, ctx->nmodes, ctx->d_bin_start, ctx->nell, ctx->pk_seg_len, partial);
+    return launch_check(ctx, "k_cross_bin");
+}
+template int launch_cross_bin<float>(polybin_ctx*, const float2*, long, int, const float2*, double*);
+template int launch_cross_bin<double>(polybin_ctx*, const double2*, long, int, const double2*, double*);
+
+// out[z][nell][nb] = the segments' sums (or, with counts, the normalised P_ell) of nx sets of partials.
+int launch_bin_sum(polybin_ctx* ctx, const double* partial, int nx, const double* counts, double scale, double* out) {
+    k_bin_sum<<<dim3(ctx->nb, ctx->nell, nx), 32, 0, ctx->stream>>>(partial, ctx->pk_nseg, ctx->nell, counts, scale, out);
+    return launch_check(ctx, "k_bin_sum");
 }
 
 // a4: P_ell binning partials [nb][nseg][nell] (device, ctx->d_pkpart) from the box spectrum.
 template <typename T>
 int run_pkbin_dev(polybin_ctx* ctx, const C<T>* box) {
     StageTimer timer(ctx, kStagePk);
-    k_pk_bin<T><<<dim3(ctx->nb, ctx->pk_nseg, 1), 256, 0, ctx->stream>>>(box, ctx->d_offs, ctx->d_coef, ctx->nmodes,
-                                                                         ctx->d_bin_start, ctx->nell, ctx->pk_seg_len,
-                                                                         ctx->d_pkpart);
-    return launch_check(ctx, "k_pk_bin");
+    return launch_cross_bin<T>(ctx, box, 0, 1, box, ctx->d_pkpart);
 }
 
-// a4: P_ell numerators num[ell][b] (host) from the box spectrum (segments summed in order on the host).
+// a4: P_ell numerators num[ell][b] (host) from the box spectrum.
 template <typename T>
 int run_pkbin(polybin_ctx* ctx, const C<T>* box, std::vector<double>& num) {
     int rc;
-    const int nb = ctx->nb, nell = ctx->nell;
     if ((rc = run_pkbin_dev<T>(ctx, box))) return rc;
-    std::vector<double> part((size_t)nb * ctx->pk_nseg * nell);
-    PB_CUDA_OK(cudaMemcpyAsync(part.data(), ctx->d_pkpart, part.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    if ((rc = launch_bin_sum(ctx, ctx->d_pkpart, 1, nullptr, 1.0, ctx->d_pkout))) return rc;
+    num.resize((size_t)ctx->nell * ctx->nb);
+    PB_CUDA_OK(cudaMemcpyAsync(num.data(), ctx->d_pkout, num.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
-    num.assign((size_t)nell * nb, 0.0);
-    for (int b = 0; b < nb; ++b)
-        for (int s = 0; s < ctx->pk_nseg; ++s)
-            for (int l = 0; l < nell; ++l) num[(size_t)l * nb + b] += part[((size_t)b * ctx->pk_nseg + s) * nell + l];
     return POLYBIN_OK;
 }
 
@@ -483,7 +492,8 @@ static int plan_pk(polybin_ctx* ctx) {
     }
     long maxlen = 1;
     for (int b = 0; b < nb; ++b) maxlen = std::max(maxlen, (long)offs[b].size());
-    ctx->pk_seg_len = 8192;
+    // about four segments of the mode lists an SM (a multiple of the CTA's 256 threads, at most 4096 modes)
+    ctx->pk_seg_len = (int)std::min(4096L, std::max(256L, (M / (4 * 152) + 255) / 256 * 256));
     ctx->pk_nseg = (int)((maxlen + ctx->pk_seg_len - 1) / ctx->pk_seg_len);
     polybin_ctx* c = ctx;
     PB_CUDA_OK_C(cudaMalloc(&c->d_offs, sizeof(int) * std::max(M, 1L)));

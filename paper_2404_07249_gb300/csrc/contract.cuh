@@ -135,43 +135,89 @@ __global__ void __launch_bounds__(256) k_contract(const T* __restrict__ g, const
     }
 }
 
-// Sum per-cell-block partials in a fixed order: out[o] = sum_cb partial[cb][o].
-static __global__ void k_reduce_partials(const double* __restrict__ partial, int ncb, long nout, double* __restrict__ out) {
-    const long o = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= nout) return;
+// Sum per-cell-block partials in a fixed order: out[o] = sum_cb partial[cb][o].  32 outputs x 16 slices of the blocks a
+// CTA (blockDim (32, 16)): slice q sums blocks q, q + 16, .. with coalesced loads that do not wait for one another, the
+// slices are then added in order.  Bound by load latency: one thread an output took 94 us for 559 blocks.
+constexpr int kRedSlices = 16;
+static __global__ void __launch_bounds__(32 * kRedSlices) k_reduce_partials(const double* __restrict__ partial, int ncb,
+                                                                            long nout, double* __restrict__ out) {
+    __shared__ double red[kRedSlices][33];
+    const long o = (long)blockIdx.x * 32 + threadIdx.x;
     double s = 0.0;
-    for (int cb = 0; cb < ncb; ++cb) s += partial[(size_t)cb * nout + o];
+    if (o < nout) {
+#pragma unroll 8
+        for (int cb = threadIdx.y; cb < ncb; cb += kRedSlices) s += partial[(size_t)cb * nout + o];
+    }
+    red[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y || o >= nout) return;
+    for (int q = 1; q < kRedSlices; ++q) s += red[q][threadIdx.x];
     out[o] = s;
 }
+inline unsigned reduce_blocks(long nout) { return (unsigned)((nout + 31) / 32); }
 
 // ------------------------------------------------------------------------------------------------
-// P_ell binning reduction (Sec. 3.4.1, eq. pk-limit): num[ell][b] = sum_{k in b} L_ell(mu) |D(k)|^2 over
-// the full k-grid, evaluated on the half spectrum with coefficient w_k L_ell (w_k = 1 on the kz = 0 and
-// Nyquist planes, 2 elsewhere) precomputed per mode in FP64.  One CTA per (bin, segment of that bin's
-// mode list); deterministic tree reduction in FP64.
+// Binned products over the half spectrum (Sec. 3.4.1, eq. pk-limit; Sec. 3.3.2, eq. fish-from-Q):
+//   partial[z][b][seg][ell] = sum_{modes of segment seg of bin b} coef_ell Re(conj X_z A),
+// coef_ell = w_k L_ell(mu) (w_k = 1 on the kz = 0 and Nyquist planes, 2 elsewhere) precomputed per mode in FP64; with
+// X = A it gives the sums of L_ell |D|^2 over the full k-grid.  X_z = X + z x_stride.  One CTA per (bin, segment of that
+// bin's mode list, z); deterministic tree reduction in FP64.  The FP64 pipe (two lanes a clock an SM on this part) bounds
+// it once every SM has work, so plan_pk cuts the lists into about four segments an SM: with 8192 modes a segment, 20
+// to 40 CTAs took 70 us for 64^3 and for 256^3 alike.
 template <typename T>
-__global__ void __launch_bounds__(256) k_pk_bin(const C<T>* __restrict__ spec, const int* __restrict__ offs,
-                                                const double* __restrict__ coef, long nmodes_total,
-                                                const int* __restrict__ bin_start, int nell, int seg_len,
-                                                double* __restrict__ partial /*[nb][nseg][nell]*/) {
-    __shared__ double red[256 * 3];
+__global__ void __launch_bounds__(256) k_cross_bin(const C<T>* __restrict__ X, const C<T>* __restrict__ A, long x_stride,
+                                                   const int* __restrict__ offs, const double* __restrict__ coef,
+                                                   long nmodes_total, const int* __restrict__ bin_start, int nell,
+                                                   int seg_len, double* __restrict__ partial) {
+    __shared__ double red[256];
     const int b = blockIdx.x, seg = blockIdx.y;
     const long beg = bin_start[b] + (long)seg * seg_len;
     const long end = min((long)bin_start[b + 1], beg + seg_len);
-    double s[3] = {0.0, 0.0, 0.0};
-    for (long m = beg + threadIdx.x; m < end; m += blockDim.x) {
-        const C<T> d = spec[offs[m]];
-        const double p = (double)d.x * (double)d.x + (double)d.y * (double)d.y;
-        for (int l = 0; l < nell; ++l) s[l] += coef[(long)l * nmodes_total + m] * p;
+    const C<T>* __restrict__ Xz = X + (long)blockIdx.z * x_stride;
+    double* out = partial + (((long)blockIdx.z * gridDim.x + b) * gridDim.y + seg) * nell;
+    if (beg >= end) {
+        if (threadIdx.x < nell) out[threadIdx.x] = 0.0;
+        return;
     }
-    for (int l = 0; l < 3; ++l) red[l * 256 + threadIdx.x] = s[l];
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int l = 0; l < 3; ++l) red[l * 256 + threadIdx.x] += red[l * 256 + threadIdx.x + w];
+    double s[3] = {0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (long m = beg + threadIdx.x; m < end; m += 256) {
+        const int o = offs[m];
+        const C<T> x = Xz[o], a = A[o];
+        const double p = (double)x.x * (double)a.x + (double)x.y * (double)a.y;
+#pragma unroll
+        for (int l = 0; l < 3; ++l)
+            if (l < nell) s[l] += coef[(long)l * nmodes_total + m] * p;
+    }
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+        if (l >= nell) break;
+        red[threadIdx.x] = s[l];
+        __syncthreads();
+        for (int w = 128; w > 0; w >>= 1) {
+            if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) out[l] = red[0];
         __syncthreads();
     }
-    if (threadIdx.x < nell) partial[((long)b * gridDim.y + seg) * nell + threadIdx.x] = red[threadIdx.x * 256];
+}
+
+// out[z][l][b] = sum_seg partial[z][b][seg][l] (one warp per (b, l, z); fixed order).  With counts: the normalised
+// P_ell, (4 l + 1) scale sum / counts[b], NaN for an empty bin.
+static __global__ void __launch_bounds__(32) k_bin_sum(const double* __restrict__ partial, int nseg, int nell,
+                                                       const double* __restrict__ counts, double scale,
+                                                       double* __restrict__ out) {
+    const int nb = gridDim.x, b = blockIdx.x, l = blockIdx.y, z = blockIdx.z;
+    const double* p = partial + ((long)z * nb + b) * nseg * nell + l;
+    double s = 0.0;
+#pragma unroll 4
+    for (int q = threadIdx.x; q < nseg; q += 32) s += p[(long)q * nell];
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) s += __shfl_down_sync(0xffffffffu, s, w);
+    if (threadIdx.x) return;
+    if (counts) s = counts[b] > 0 ? (4 * l + 1) * scale * s / counts[b] : __longlong_as_double(0x7ff8000000000000LL);
+    out[((long)z * nell + l) * nb + b] = s;
 }
 
 }  // namespace pb

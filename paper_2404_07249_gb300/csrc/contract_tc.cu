@@ -711,14 +711,25 @@ __global__ void __launch_bounds__(256) k_absmax(const float4* __restrict__ maps,
 
 // out[o] = 2^-(row and single exponents) sum over CTAs of partial[cta][gidx[o]], in CTA order (deterministic).  rows[o]
 // holds the slot rows (j, k, single) of output o.
-__global__ void k_reduce_gather(const double* __restrict__ partial, int ncta, long stride,
-                                const int* __restrict__ gidx, const uchar4* __restrict__ rows,
-                                const uint32_t* __restrict__ absmax, int n_out, double* __restrict__ out) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= n_out) return;
-    const long g = gidx[o];
+// 32 outputs x 16 slices of the CTAs a block (blockDim (32, 16)), as k_reduce_partials.
+constexpr int kSlices = 16;
+__global__ void __launch_bounds__(32 * kSlices) k_reduce_gather(const double* __restrict__ partial, int ncta, long stride,
+                                                                const int* __restrict__ gidx,
+                                                                const uchar4* __restrict__ rows,
+                                                                const uint32_t* __restrict__ absmax, int n_out,
+                                                                double* __restrict__ out) {
+    __shared__ double red[kSlices][33];
+    const int o = blockIdx.x * 32 + threadIdx.x;
     double s = 0.0;
-    for (int c = 0; c < ncta; ++c) s += partial[(long)c * stride + g];
+    if (o < n_out) {
+        const long g = gidx[o];
+#pragma unroll 4
+        for (int c = threadIdx.y; c < ncta; c += kSlices) s += partial[(long)c * stride + g];
+    }
+    red[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y || o >= n_out) return;
+    for (int q = 1; q < kSlices; ++q) s += red[q][threadIdx.x];
     const uchar4 r = rows[o];
     out[o] = ldexp(s, -row_exp(absmax[r.x], absmax[r.y]) - single_exp(absmax[r.z]));
 }
@@ -1396,9 +1407,8 @@ static int launch(polybin_ctx* ctx, Plan& pl, const float* g, const float* h, do
         ctx->launches += 1;
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail_cuda(ctx, e, "k_contract_tc", __FILE__, __LINE__);
-        k_reduce_gather<<<(pl.n_out + 255) / 256, 256, 0, ctx->stream>>>(pl.d_partial, pl.ncta,
-                                                                          (long)pl.total_units * 2048, pl.d_gidx,
-                                                                          pl.d_orows, pc->d_absmax, pl.n_out, d_out);
+        k_reduce_gather<<<(pl.n_out + 31) / 32, dim3(32, kSlices), 0, ctx->stream>>>(
+            pl.d_partial, pl.ncta, (long)pl.total_units * 2048, pl.d_gidx, pl.d_orows, pc->d_absmax, pl.n_out, d_out);
         ctx->launches += 1;
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail_cuda(ctx, e, "k_reduce_gather", __FILE__, __LINE__);

@@ -158,8 +158,8 @@ static int simt_triplet_sums(polybin_ctx* ctx, int kind, const T* g, const T* h,
             k_contract<T><<<dim3(G.ngroups, G.ncb, 1), 256, sm, ctx->stream>>>(g, hs, ncell, pl.d_pairs + Gp.pair_off, G,
                                                                              w.partial);
             const long nout = (long)G.npairs * G.nh;
-            k_reduce_partials<<<(unsigned)((nout + 255) / 256), 256, 0, ctx->stream>>>(w.partial, G.ncb, nout,
-                                                                                       pl.d_M + Gp.out_off);
+            k_reduce_partials<<<reduce_blocks(nout), dim3(32, kRedSlices), 0, ctx->stream>>>(w.partial, G.ncb, nout,
+                                                                                             pl.d_M + Gp.out_off);
             ctx->launches += 2;
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return fail_cuda(ctx, e, "k_contract (pruned)", __FILE__, __LINE__);
@@ -268,26 +268,9 @@ int run_bk_normalise(polybin_ctx* ctx, const double* d_S, double* d_B, double fa
     return POLYBIN_OK;
 }
 
-// P[l][b] = (4 l + 1) scale sum_seg part[b][seg][l] / counts[b] (segments summed in order; NaN for an empty bin).
-static __global__ void k_pk_normalise(const double* __restrict__ part, int nb, int nseg, int nell,
-                                      const double* __restrict__ counts, double scale, double* __restrict__ P) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nb * nell) return;
-    const int l = i / nb, b = i - l * nb;
-    double s = 0.0;
-    for (int q = 0; q < nseg; ++q) s += part[((long)b * nseg + q) * nell + l];
-    P[i] = counts[b] > 0 ? (4 * l + 1) * scale * s / counts[b] : __longlong_as_double(0x7ff8000000000000LL);
-}
-
 int run_pk_normalise(polybin_ctx* ctx, double* d_P) {
-    const int n = ctx->nb * ctx->nell;
     const double N = (double)ctx->ncell;
-    k_pk_normalise<<<(n + 127) / 128, 128, 0, ctx->stream>>>(ctx->d_pkpart, ctx->nb, ctx->pk_nseg, ctx->nell,
-                                                             ctx->d_counts, ctx->vol / (N * N), d_P);
-    ctx->launches += 1;
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fail_cuda(ctx, e, "k_pk_normalise", __FILE__, __LINE__);
-    return POLYBIN_OK;
+    return launch_bin_sum(ctx, ctx->d_pkpart, 1, ctx->d_counts, ctx->vol / (N * N), d_P);
 }
 
 }  // namespace pb

@@ -131,7 +131,7 @@ extern "C" int polybin_contract_noalloc(const float* g, int n_g, const float* h,
                                                                  slot->scratch);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(POLYBIN_ECUDA, std::string("polybin_contract_noalloc: ") + cudaGetErrorString(e));
-    k_reduce_partials<<<(unsigned)((per_cb + 255) / 256), 256, 0, st>>>(slot->scratch, G.ncb, per_cb, m_out_dev);
+    k_reduce_partials<<<reduce_blocks(per_cb), dim3(32, kRedSlices), 0, st>>>(slot->scratch, G.ncb, per_cb, m_out_dev);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(POLYBIN_ECUDA, std::string("polybin_contract_noalloc: ") + cudaGetErrorString(e));
     return POLYBIN_OK;

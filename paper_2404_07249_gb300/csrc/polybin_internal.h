@@ -94,6 +94,11 @@ template <typename T> int run_shells(polybin_ctx*, const C<T>*, C<T>*, C<T>*, T*
 template <typename T>
 int run_shells_m(polybin_ctx*, const C<T>*, C<T>*, C<T>*, T*, int ell, int m, const InvGrid& ig);
 template <typename T> int run_pkbin(polybin_ctx*, const C<T>*, std::vector<double>&);
+// Binned products of nx box spectra X + z x_stride with A (partials [nx][nb][nseg][nell]) and the sums over segments
+// out[nx][nell][nb] (counts given: P_ell normalised).
+template <typename T>
+int launch_cross_bin(polybin_ctx*, const C<T>* X, long x_stride, int nx, const C<T>* A, double* partial);
+int launch_bin_sum(polybin_ctx*, const double* partial, int nx, const double* counts, double scale, double* out);
 // Contractions over `ncell` cells (maps of the data grid or of the contraction grid).
 template <typename T> int run_contract(polybin_ctx*, const T*, int, const T*, int, double*, size_t, double*, long ncell);
 // Contraction dispatch: the tensor-core kernel in POLYBIN_SPLIT_TF32X3 mode, the SIMT kernel otherwise.

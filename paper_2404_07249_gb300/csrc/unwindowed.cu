@@ -70,32 +70,6 @@ __global__ void k_draw(T* __restrict__ out, long N, unsigned long long seed, uin
     }
 }
 
-// Binned cross products over the half spectrum: out[b][seg][ell] = sum_{modes m of bin b} coef_ell(m) Re(conj X A).
-template <typename T>
-__global__ void __launch_bounds__(256) k_cross_bin(const C<T>* __restrict__ X, const C<T>* __restrict__ A,
-                                                   const int* __restrict__ offs, const double* __restrict__ coef,
-                                                   long nmodes_total, const int* __restrict__ bin_start, int nell,
-                                                   int seg_len, double* __restrict__ partial) {
-    __shared__ double red[256 * 3];
-    const int b = blockIdx.x, seg = blockIdx.y;
-    const long beg = bin_start[b] + (long)seg * seg_len;
-    const long end = min((long)bin_start[b + 1], beg + seg_len);
-    double s[3] = {0.0, 0.0, 0.0};
-    for (long m = beg + threadIdx.x; m < end; m += blockDim.x) {
-        const C<T> x = X[offs[m]], a = A[offs[m]];
-        const double p = (double)x.x * (double)a.x + (double)x.y * (double)a.y;
-        for (int l = 0; l < nell; ++l) s[l] += coef[(long)l * nmodes_total + m] * p;
-    }
-    for (int l = 0; l < 3; ++l) red[l * 256 + threadIdx.x] = s[l];
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-            for (int l = 0; l < 3; ++l) red[l * 256 + threadIdx.x] += red[l * 256 + threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x < nell) partial[((long)b * gridDim.y + seg) * nell + threadIdx.x] = red[threadIdx.x * 256];
-}
-
 // Q-derivative spectrum of one triplet (a, b, c) from the pair spectra of two fields (eq. Q-bis-global):
 //   out(k) = fac [ Theta_c (P1_ab - P2_ab) + Theta_a (P1_bc - P2_bc) + Theta_b (P1_ac - P2_ac) ](k),
 // fac = 2 / Delta_abc, over every entry of the box (zero outside bins a, b, c).
@@ -347,6 +321,10 @@ __global__ void __launch_bounds__(256) k_cross_bin_local(const C<T>* __restrict_
     const int b = blockIdx.x, seg = blockIdx.y;
     const long beg = bin_start[b] + (long)seg * seg_len;
     const long end = min((long)bin_start[b + 1], beg + seg_len);
+    if (beg >= end) {
+        if (threadIdx.x < nell) partial[((long)b * gridDim.y + seg) * nell + threadIdx.x] = 0.0;
+        return;
+    }
     double s[3] = {0.0, 0.0, 0.0};
     for (long q = beg + threadIdx.x; q < end; q += blockDim.x) {
         const C<T> x = X[offs[q]];
@@ -394,6 +372,7 @@ struct UwState {
     void* v2 = nullptr;       //                                [N0][N1][Bz]
     double* dF = nullptr;     // device Fisher accumulator
     double* dpart = nullptr;  // cross-bin partials
+    double* dsum = nullptr;   // their sums over segments [nell][nb]
     double* dvec = nullptr;
     double* dvec2 = nullptr;
     int* dinfo = nullptr;
@@ -431,7 +410,7 @@ struct UwState {
 static void uw_free(UwState* u) {
     if (!u) return;
     void* ptrs[] = {u->g2, u->xmap, u->a[0], u->a[1], u->spec[0], u->spec[1], u->spec[2], u->spec[3], u->pairs, u->qbox,
-                    u->zc, u->yc, u->v1, u->v2, u->dF, u->dpart, u->dvec, u->dvec2, u->dinfo, u->dFp_inv, u->dFb_inv,
+                    u->zc, u->yc, u->v1, u->v2, u->dF, u->dpart, u->dsum, u->dvec, u->dvec2, u->dinfo, u->dFp_inv, u->dFb_inv,
                     u->ylc, u->hbox, u->g3, u->dFl_inv, u->dFo_inv, u->bmaps, u->bpart, u->bout,
                     u->dpart_all};
     for (void* p : ptrs)
@@ -470,6 +449,7 @@ static int uw_alloc(polybin_ctx* ctx, bool need_b) {
         if ((rc = need(&u->spec[f], sizeof(C<T>) * nbox))) return rc;
     if ((rc = need(&u->g2, sizeof(T) * (size_t)nb * N))) return rc;
     if ((rc = need((void**)&u->dpart, sizeof(double) * (size_t)nb * ctx->pk_nseg * 3))) return rc;
+    if ((rc = need((void**)&u->dsum, sizeof(double) * (size_t)nb * 3))) return rc;
     if ((rc = need((void**)&u->dinfo, sizeof(int)))) return rc;
     if ((rc = need((void**)&u->dvec, sizeof(double) * 4096))) return rc;
     if ((rc = need((void**)&u->dvec2, sizeof(double) * 4096))) return rc;
@@ -563,39 +543,26 @@ int run_inverse_box(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* ou
     return POLYBIN_OK;
 }
 
+// Host copy of the segment sums [nell][nb] of the partials dpart.
+static int read_bin_sums(polybin_ctx* ctx, const double* dpart, std::vector<double>& out) {
+    UwState* u = static_cast<UwState*>(ctx->ext);
+    int rc;
+    if ((rc = launch_bin_sum(ctx, dpart, 1, nullptr, 1.0, u->dsum))) return rc;
+    out.resize((size_t)ctx->nell * ctx->nb);
+    PB_CUDA_OK(cudaMemcpyAsync(out.data(), u->dsum, out.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
+    return POLYBIN_OK;
+}
+
 // Binned cross products (host result [nell][nb]) of two box spectra.
 template <typename T>
 static int run_cross_bin(polybin_ctx* ctx, const C<T>* X, const C<T>* A, double* dpart, std::vector<double>& out) {
-    const int nb = ctx->nb, nell = ctx->nell;
-    uw::k_cross_bin<T><<<dim3(nb, ctx->pk_nseg, 1), 256, 0, ctx->stream>>>(X, A, ctx->d_offs, ctx->d_coef, ctx->nmodes,
-                                                                            ctx->d_bin_start, nell, ctx->pk_seg_len, dpart);
-    ctx->launches++;
-    std::vector<double> part((size_t)nb * ctx->pk_nseg * nell);
-    PB_CUDA_OK(cudaGetLastError());
-    PB_CUDA_OK(cudaMemcpyAsync(part.data(), dpart, part.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
-    out.assign((size_t)nell * nb, 0.0);
-    for (int b = 0; b < nb; ++b)
-        for (int s = 0; s < ctx->pk_nseg; ++s)
-            for (int l = 0; l < nell; ++l) out[(size_t)l * nb + b] += part[((size_t)b * ctx->pk_nseg + s) * nell + l];
-    return POLYBIN_OK;
+    int rc;
+    if ((rc = launch_cross_bin<T>(ctx, X, 0, 1, A, dpart))) return rc;
+    return read_bin_sums(ctx, dpart, out);
 }
 
 // ---------------------------------------------------------------------------------------------- P Fisher
-
-// The binned cross products of alpha's spectrum X with A into slot alpha of dpart_all (no read-back).
-template <typename T>
-static int launch_cross_bin(polybin_ctx* ctx, const C<T>* X, const C<T>* A, int alpha) {
-    UwState* u = static_cast<UwState*>(ctx->ext);
-    const int nb = ctx->nb, nell = ctx->nell;
-    const size_t per = (size_t)nb * ctx->pk_nseg * nell;
-    uw::k_cross_bin<T><<<dim3(nb, ctx->pk_nseg, 1), 256, 0, ctx->stream>>>(X, A, ctx->d_offs, ctx->d_coef, ctx->nmodes,
-                                                                            ctx->d_bin_start, nell, ctx->pk_seg_len,
-                                                                            u->dpart_all + (size_t)alpha * per);
-    ctx->launches++;
-    PB_CUDA_OK(cudaGetLastError());
-    return POLYBIN_OK;
-}
 
 // One Monte Carlo term of the P Fisher matrix (eq. fish-from-Q, global line of sight), host [na][na], na = nell*nb:
 // F[(l,b)][(l',b')] = 1/2 (1/N) sum_k conj(FT[s IFT[Theta_b L_l FT[s a]]]) Theta_b' L_l' FT[a],  s = w n.
@@ -617,13 +584,14 @@ static int pk_fisher_draw(polybin_ctx* ctx, const float* n, const float* w, unsi
     if ((rc = run_forward<T, T, float>(ctx, a, w, n, (C<T>*)W.t1, (C<T>*)W.t2, SA))) return rc;
     F.assign((size_t)na * na, 0.0);
     const size_t per = (size_t)nb * ctx->pk_nseg * nell;
-    if (u->dpart_all_cap < (size_t)na * per) {
+    if (u->dpart_all_cap < (size_t)na * (per + na)) {
         if (u->dpart_all) cudaFree(u->dpart_all);
         u->dpart_all = nullptr;
         u->dpart_all_cap = 0;
-        PB_CUDA_OK(cudaMalloc((void**)&u->dpart_all, sizeof(double) * (size_t)na * per));
-        u->dpart_all_cap = (size_t)na * per;
+        PB_CUDA_OK(cudaMalloc((void**)&u->dpart_all, sizeof(double) * (size_t)na * (per + na)));
+        u->dpart_all_cap = (size_t)na * (per + na);
     }
+    double* const dsums = u->dpart_all + (size_t)na * per;      // [na][nell][nb]
     T* q = (T*)u->g2;
     for (int il = 0; il < nell; ++il) {
         if ((rc = ensure_fine_inv<T>(ctx))) return rc;
@@ -631,21 +599,13 @@ static int pk_fisher_draw(polybin_ctx* ctx, const float* n, const float* w, unsi
         for (int b = 0; b < nb; ++b) {
             C<T>* X = (C<T>*)u->spec[2];
             if ((rc = run_forward<T, T, float>(ctx, q + (size_t)b * N, w, n, (C<T>*)W.t1, (C<T>*)W.t2, X))) return rc;
-            if ((rc = launch_cross_bin<T>(ctx, X, A, il * nb + b))) return rc;
+            if ((rc = launch_cross_bin<T>(ctx, X, 0, 1, A, u->dpart_all + (size_t)(il * nb + b) * per))) return rc;
         }
     }
-    std::vector<double> part((size_t)na * per);
-    PB_CUDA_OK(cudaMemcpyAsync(part.data(), u->dpart_all, part.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    if ((rc = launch_bin_sum(ctx, u->dpart_all, na, nullptr, 1.0, dsums))) return rc;
+    PB_CUDA_OK(cudaMemcpyAsync(F.data(), dsums, F.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
-    for (int alpha = 0; alpha < na; ++alpha) {
-        const double* pa = part.data() + (size_t)alpha * per;
-        for (int b2 = 0; b2 < nb; ++b2)
-            for (int jl = 0; jl < nell; ++jl) {
-                double acc = 0.0;
-                for (int sg = 0; sg < ctx->pk_nseg; ++sg) acc += pa[((size_t)b2 * ctx->pk_nseg + sg) * nell + jl];
-                F[(size_t)alpha * na + jl * nb + b2] = 0.5 * acc / (double)N;
-            }
-    }
+    for (double& f : F) f = 0.5 * f / (double)N;
     return POLYBIN_OK;
 }
 
@@ -901,14 +861,7 @@ static int run_cross_local(polybin_ctx* ctx, const C<T>* X, std::vector<double>&
         X, u->ylc, ctx->d_offs, ctx->d_coef, ctx->nmodes, ctx->d_bin_start, nell, ctx->pk_seg_len, u->dpart);
     ctx->launches++;
     PB_CUDA_OK(cudaGetLastError());
-    std::vector<double> part((size_t)nb * ctx->pk_nseg * nell);
-    PB_CUDA_OK(cudaMemcpyAsync(part.data(), u->dpart, part.size() * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
-    out.assign((size_t)nell * nb, 0.0);
-    for (int b = 0; b < nb; ++b)
-        for (int sg = 0; sg < ctx->pk_nseg; ++sg)
-            for (int l = 0; l < nell; ++l) out[(size_t)l * nb + b] += part[((size_t)b * ctx->pk_nseg + sg) * nell + l];
-    return POLYBIN_OK;
+    return read_bin_sums(ctx, u->dpart, out);
 }
 
 // Numerator with a local line of sight (Sec. 3.3.1, eq. pk-num-fft), pixel units:
