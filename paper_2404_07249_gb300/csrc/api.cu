@@ -269,21 +269,7 @@ int run_bulk_wait_selftest(polybin_ctx* ctx, unsigned limit) {
     return launch_check(ctx, "k_bulk_wait_selftest");
 }
 
-ContractGeom contract_geom(int nb, int nh, long ncell) {
-    ContractGeom G;
-    G.nb = nb; G.nh = nh; G.npairs = nb * (nb + 1) / 2;
-    G.ct = (nh + kTN - 1) / kTN;
-    G.rt = 256 / G.ct;
-    const int need = (G.npairs + kTM - 1) / kTM * kTM;
-    G.rows_cta = std::min(G.rt * kTM, need);
-    G.nhp = G.ct * kTN;
-    G.ngroups = (G.npairs + G.rows_cta - 1) / G.rows_cta;
-    const long nchunks = (ncell + kCH - 1) / kCH;
-    long ncb = std::max(1L, std::min(nchunks, (long)(4 * 152 / G.ngroups)));
-    G.cells_cta = ((ncell + ncb - 1) / ncb + kCH - 1) / kCH * kCH;
-    G.ncb = (int)((ncell + G.cells_cta - 1) / G.cells_cta);
-    return G;
-}
+ContractGeom contract_geom(int nb, int nh, long ncell) { return contract_geom_rows(nb, nb * (nb + 1) / 2, nh, ncell); }
 
 // a3: contraction; result (device, [npairs][nh] doubles) in d_out.
 template <typename T>
@@ -293,10 +279,10 @@ int run_contract(polybin_ctx* ctx, const T* g, int ng, const T* h, int nh, doubl
     StageTimer timer(ctx, kStageContract);
     ContractGeom G = contract_geom(ng, nh, ncell);
     if ((size_t)G.ncb * G.npairs * G.nh > partial_cap) return fail(ctx, POLYBIN_EINVAL, "contract: partial buffer too small");
-    const size_t sm = ((size_t)kCH * G.rows_cta + (size_t)kCH * G.nhp + (size_t)ng * (kCH + 1)) * sizeof(T) + 16;
+    const size_t sm = contract_smem<T>(G);
     if ((rc = set_smem<T>(ctx, (const void*)k_contract<T>, sm))) return rc;
     dim3 grid(G.ngroups, G.ncb, 1);
-    k_contract<T><<<grid, 256, sm, ctx->stream>>>(g, h, ncell, ctx->d_pairs + pairs_offset(ng), G, d_partial);
+    k_contract<T><<<grid, 256, sm, ctx->stream>>>(g, h, 0, ncell, ctx->d_pairs + pairs_offset(ng), G, d_partial);
     if ((rc = launch_check(ctx, "k_contract"))) return rc;
     const long nout = (long)G.npairs * G.nh;
     k_reduce_partials<<<reduce_blocks(nout), dim3(32, kRedSlices), 0, ctx->stream>>>(d_partial, G.ncb, nout, d_out);

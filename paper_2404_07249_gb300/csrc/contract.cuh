@@ -4,33 +4,74 @@
 // pair rows; per chunk of CH cells it stages the maps in shared memory, forms the pair products once,
 // and every thread accumulates a TM x TN register tile of outputs.
 //
-// Precision (float): products and chunk sums in FP32, flushed every FLUSH chunks into FP64 registers;
-// per-CTA FP64 partials are reduced across CTAs in a fixed order (deterministic).
+// Few rows leave most of a CTA without a tile (36 pairs x 8 singles are nine tiles of 4 x 8), so the tiles are
+// replicated kg times over the threads, replica q taking the cells q, q + kg, .. of every chunk; the replicas are added
+// in order at the end.  The next chunk's maps are loaded into registers while the current one is worked on, and
+// products and singles are written as 16-byte pieces with row strides of an odd number of pieces (no bank conflicts, no
+// division by run-time sizes per element).
+//
+// Precision (float): products and chunk sums in FP32, flushed every FLUSH chunks into FP64 registers (double: FP64
+// throughout); per-CTA FP64 partials are reduced across CTAs in a fixed order (deterministic).
 #pragma once
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace pb {
 
-constexpr int kCH = 32;       // cells per chunk
+constexpr int kCH = 32;       // cells per chunk (one a lane when products are formed)
 constexpr int kTM = 4;        // pair rows per thread
 constexpr int kTN = 8;        // singles per thread
 constexpr int kFlush = 16;    // chunks per FP32 partial sum (512 cells)
+constexpr int kGS = kCH + 1;  // row stride of the staged maps
 
 struct ContractGeom {
     int nb, nh, npairs;
     int rt, ct;        // thread tile grid (rt * ct <= 256)
+    int kg;            // replicas of the tile grid over the cells of a chunk (rt * ct * kg <= 256)
     int rows_cta;      // pair rows per CTA (multiple of kTM)
-    int nhp;           // padded singles (ct * kTN)
+    int rps;           // row stride of the product array (elements; an odd multiple of 4, >= rows_cta)
+    int nhp;           // row stride of the singles array (an odd multiple of 4, >= ct * kTN)
     int ngroups;       // row groups
     int ncb;           // cell blocks
     long cells_cta;    // cells per CTA (multiple of kCH)
 };
+
+// Geometry of npairs rows against nh singles out of nb staged maps over ncell cells.
+inline ContractGeom contract_geom_rows(int nb, int npairs, int nh, long ncell) {
+    ContractGeom G;
+    G.nb = nb; G.nh = nh; G.npairs = npairs;
+    G.ct = (nh + kTN - 1) / kTN;
+    const int need = (npairs + kTM - 1) / kTM * kTM;
+    G.rows_cta = std::min(256 / G.ct * kTM, need);
+    G.rt = G.rows_cta / kTM;
+    G.kg = std::min(256 / (G.rt * G.ct), kCH);
+    G.rps = G.rows_cta / 4 % 2 ? G.rows_cta : G.rows_cta + 4;
+    G.nhp = G.ct * kTN + 4;
+    G.ngroups = (npairs + G.rows_cta - 1) / G.rows_cta;
+    const long nchunks = (ncell + kCH - 1) / kCH;
+    long ncb = std::max(1L, std::min(nchunks, (long)(4 * 152 / G.ngroups)));
+    G.cells_cta = ((ncell + ncb - 1) / ncb + kCH - 1) / kCH * kCH;
+    G.ncb = (int)((ncell + G.cells_cta - 1) / G.cells_cta);
+    return G;
+}
+
+// Dynamic shared memory: products [kCH][rps], singles [kCH][nhp], maps [nb][kGS]; at the end the tiles' sums of one
+// replica (FP64; only with replicas, then at most 128 tiles) in the place of the products.
+template <typename T> inline size_t contract_smem(const ContractGeom& G) {
+    const size_t work = ((size_t)kCH * G.rps + (size_t)kCH * G.nhp + (size_t)G.nb * kGS) * sizeof(T);
+    const size_t sums = G.kg > 1 ? (size_t)G.rt * G.ct * kTM * kTN * sizeof(double) : 0;
+    return std::max(work, sums) + 16;
+}
 
 template <typename T> struct Vec4;
 template <> struct Vec4<float> {
     __device__ __forceinline__ static void load(const float* p, float* v) {
         float4 a = *reinterpret_cast<const float4*>(p);
         v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    }
+    __device__ __forceinline__ static void store(float* p, const float* v) {
+        *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
     }
 };
 template <> struct Vec4<double> {
@@ -39,27 +80,31 @@ template <> struct Vec4<double> {
         double2 b = *reinterpret_cast<const double2*>(p + 2);
         v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
     }
+    __device__ __forceinline__ static void store(double* p, const double* v) {
+        *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+        *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
+    }
 };
 
+// Singles: rows hsub .. hsub + nh - 1 of g when h is null, else the maps h.
 template <typename T>
-__global__ void __launch_bounds__(256) k_contract(const T* __restrict__ g, const T* __restrict__ h, long ncell,
+__global__ void __launch_bounds__(256, 2) k_contract(const T* __restrict__ g, const T* __restrict__ h, int hsub, long ncell,
                                                   const short2* __restrict__ pairs, ContractGeom G,
                                                   double* __restrict__ partial) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x;
-    const int RP = G.rows_cta;
-    const int NHP = G.nhp;
-    const int GS = kCH + 1;
-    T* sP = reinterpret_cast<T*>(smem_raw);          // [kCH][RP]
-    T* sH = sP + (size_t)kCH * RP;                    // [kCH][NHP]
-    T* sG = sH + (size_t)kCH * NHP;                   // [nb][GS]
-    const int r0 = blockIdx.x * RP;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int RPS = G.rps, NHP = G.nhp;
+    T* sP = reinterpret_cast<T*>(smem_raw);          // [kCH][RPS]
+    T* sH = sP + (size_t)kCH * RPS;                   // [kCH][NHP]
+    T* sG = sH + (size_t)kCH * NHP;                   // [nb][kGS]
+    const int r0 = blockIdx.x * G.rows_cta;
     const long cbeg = (long)blockIdx.y * G.cells_cta;
     const long cend = min(ncell, cbeg + G.cells_cta);
-    const int rt = tid % G.rt, ct = tid / G.rt;
-    const bool active = ct < G.ct && rt * kTM < RP;
-
-    for (int idx = tid; idx < kCH * NHP; idx += blockDim.x) sH[idx] = T(0);
+    // tile (rt, ct) of replica kq; threads beyond the last replica only stage
+    const int ntile = G.rt * G.ct;
+    const int kq = tid / ntile, tt = tid - kq * ntile;
+    const int ct = tt / G.rt, rt = tt - ct * G.rt;
+    const bool active = kq < G.kg;
 
     T acc[kTM][kTN];
     double acc64[kTM][kTN];
@@ -68,52 +113,76 @@ __global__ void __launch_bounds__(256) k_contract(const T* __restrict__ g, const
 #pragma unroll
         for (int v = 0; v < kTN; ++v) { acc[u][v] = T(0); acc64[u][v] = 0.0; }
 
-    int chunk = 0;
-    for (long c0 = cbeg; c0 < cend; c0 += kCH, ++chunk) {
-        __syncthreads();
-        for (int idx = tid; idx < G.nb * kCH; idx += blockDim.x) {
-            const int b = idx / kCH, x = idx - b * kCH;
-            const long cell = c0 + x;
-            sG[b * GS + x] = cell < cend ? g[(long)b * ncell + cell] : T(0);
+    // warp w stages maps w, w + 8, .. (at most 8 of g, 8 of h), lane = cell
+    T pre[8], preh[8];
+    auto fetch = [&](long c0) {
+        const long cell = c0 + lane;
+        const bool in = cell < cend;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int b = warp + 8 * i;
+            pre[i] = in && b < G.nb ? g[(long)b * ncell + cell] : T(0);
         }
         if (h) {
-            for (int idx = tid; idx < G.nh * kCH; idx += blockDim.x) {
-                const int i = idx / kCH, x = idx - i * kCH;
-                const long cell = c0 + x;
-                sH[x * NHP + i] = cell < cend ? h[(long)i * ncell + cell] : T(0);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int b = warp + 8 * i;
+                preh[i] = in && b < G.nh ? h[(long)b * ncell + cell] : T(0);
             }
+        }
+    };
+    int chunk = 0;
+    fetch(cbeg);
+    for (long c0 = cbeg; c0 < cend; c0 += kCH, ++chunk) {
+        __syncthreads();                              // the previous chunk's products and singles have been read
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (warp + 8 * i < G.nb) sG[(warp + 8 * i) * kGS + lane] = pre[i];
+        if (h) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (warp + 8 * i < G.nh) sH[lane * NHP + warp + 8 * i] = preh[i];
         }
         __syncthreads();
-        if (!h) {
-            for (int idx = tid; idx < G.nh * kCH; idx += blockDim.x) {
-                const int x = idx % kCH, i = idx / kCH;
-                sH[x * NHP + i] = sG[i * GS + x];
+        if (c0 + kCH < cend) fetch(c0 + kCH);
+        for (int q = warp; q < G.rows_cta / 4; q += 8) {
+            T v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int gp = r0 + 4 * q + u;
+                v[u] = T(0);
+                if (gp < G.npairs) {
+                    const short2 jk = pairs[gp];
+                    v[u] = sG[jk.x * kGS + lane] * sG[jk.y * kGS + lane];
+                }
             }
+            Vec4<T>::store(sP + lane * RPS + 4 * q, v);
         }
-        for (int idx = tid; idx < RP * kCH; idx += blockDim.x) {
-            const int p = idx % RP, x = idx / RP;
-            const int gp = r0 + p;
-            T v = T(0);
-            if (gp < G.npairs) {
-                const short2 jk = pairs[gp];
-                v = sG[jk.x * GS + x] * sG[jk.y * GS + x];
+        if (!h) {
+            for (int q = warp; q < G.ct * (kTN / 4); q += 8) {
+                T v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = 4 * q + u < G.nh ? sG[(hsub + 4 * q + u) * kGS + lane] : T(0);
+                Vec4<T>::store(sH + lane * NHP + 4 * q, v);
             }
-            sP[x * RP + p] = v;
         }
         __syncthreads();
         if (active) {
-#pragma unroll 4
-            for (int x = 0; x < kCH; ++x) {
+#pragma unroll 2
+            for (int x = kq; x < kCH; x += G.kg) {
                 T a[kTM], b[kTN];
-                Vec4<T>::load(sP + x * RP + rt * kTM, a);
+                Vec4<T>::load(sP + x * RPS + rt * kTM, a);
                 Vec4<T>::load(sH + x * NHP + ct * kTN, b);
                 Vec4<T>::load(sH + x * NHP + ct * kTN + 4, b + 4);
 #pragma unroll
                 for (int u = 0; u < kTM; ++u)
 #pragma unroll
-                    for (int v = 0; v < kTN; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
+                    for (int v = 0; v < kTN; ++v) {
+                        if constexpr (sizeof(T) == 8) acc64[u][v] = fma(a[u], b[v], acc64[u][v]);
+                        else acc[u][v] = fma(a[u], b[v], acc[u][v]);
+                    }
             }
-            if ((chunk + 1) % kFlush == 0) {
+            if (sizeof(T) == 4 && (chunk + 1) % kFlush == 0) {
 #pragma unroll
                 for (int u = 0; u < kTM; ++u)
 #pragma unroll
@@ -121,7 +190,31 @@ __global__ void __launch_bounds__(256) k_contract(const T* __restrict__ g, const
             }
         }
     }
-    if (!active) return;
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int u = 0; u < kTM; ++u)
+#pragma unroll
+            for (int v = 0; v < kTN; ++v) acc64[u][v] += (double)acc[u][v];
+    }
+    // replicas 1, 2, .. are added to replica 0 in order
+    double* red = reinterpret_cast<double*>(smem_raw);   // [kTM * kTN][ntile]
+    for (int q = 1; q < G.kg; ++q) {
+        __syncthreads();
+        if (kq == q) {
+#pragma unroll
+            for (int u = 0; u < kTM; ++u)
+#pragma unroll
+                for (int v = 0; v < kTN; ++v) red[(u * kTN + v) * ntile + tt] = acc64[u][v];
+        }
+        __syncthreads();
+        if (kq == 0) {
+#pragma unroll
+            for (int u = 0; u < kTM; ++u)
+#pragma unroll
+                for (int v = 0; v < kTN; ++v) acc64[u][v] += red[(u * kTN + v) * ntile + tt];
+        }
+    }
+    if (kq != 0) return;
     double* out = partial + (size_t)blockIdx.y * G.npairs * G.nh;
 #pragma unroll
     for (int u = 0; u < kTM; ++u) {
@@ -130,7 +223,7 @@ __global__ void __launch_bounds__(256) k_contract(const T* __restrict__ g, const
 #pragma unroll
         for (int v = 0; v < kTN; ++v) {
             const int i = ct * kTN + v;
-            if (i < G.nh) out[(size_t)gp * G.nh + i] = acc64[u][v] + (double)acc[u][v];
+            if (i < G.nh) out[(size_t)gp * G.nh + i] = acc64[u][v];
         }
     }
 }

@@ -108,23 +108,6 @@ static int build_simt_plan(polybin_ctx* ctx, int kind, SimtPlan& pl) {
     return POLYBIN_OK;
 }
 
-// SIMT geometry for an explicit pair table of npairs rows against nh singles over ncell cells.
-static ContractGeom geom_rows(int nb, int npairs, int nh, long ncell) {
-    ContractGeom G;
-    G.nb = nb; G.nh = nh; G.npairs = npairs;
-    G.ct = (nh + kTN - 1) / kTN;
-    G.rt = 256 / G.ct;
-    const int need = (npairs + kTM - 1) / kTM * kTM;
-    G.rows_cta = std::min(G.rt * kTM, need);
-    G.nhp = G.ct * kTN;
-    G.ngroups = (npairs + G.rows_cta - 1) / G.rows_cta;
-    const long nchunks = (ncell + kCH - 1) / kCH;
-    long ncb = std::max(1L, std::min(nchunks, (long)(4 * 152 / G.ngroups)));
-    G.cells_cta = ((ncell + ncb - 1) / ncb + kCH - 1) / kCH * kCH;
-    G.ncb = (int)((ncell + G.cells_cta - 1) / G.cells_cta);
-    return G;
-}
-
 __global__ void k_gather_triplets(const double* __restrict__ M, const int* __restrict__ m, int nt,
                                   double* __restrict__ S);
 
@@ -145,18 +128,19 @@ static int simt_triplet_sums(polybin_ctx* ctx, int kind, const T* g, const T* h,
     {
         StageTimer timer(ctx, kStageContract);
         for (const SimtGroup& Gp : pl.groups) {
-            ContractGeom G = geom_rows(nb, Gp.npairs, Gp.W, ncell);
+            const ContractGeom G = contract_geom_rows(nb, Gp.npairs, Gp.W, ncell);
             if ((size_t)G.ncb * G.npairs * G.nh > w.partial_cap)
                 return fail(ctx, POLYBIN_EINVAL, "contract: partial buffer too small");
-            const size_t sm = ((size_t)kCH * G.rows_cta + (size_t)kCH * G.nhp + (size_t)nb * (kCH + 1)) * sizeof(T) + 16;
+            const size_t sm = contract_smem<T>(G);
             if (sm > 48 * 1024) {
                 cudaError_t e = cudaFuncSetAttribute((const void*)k_contract<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                      (int)sm);
                 if (e != cudaSuccess) return fail_cuda(ctx, e, "cudaFuncSetAttribute", __FILE__, __LINE__);
             }
-            const T* hs = (kind == 0 ? g : h) + (size_t)Gp.s0 * ncell;
-            k_contract<T><<<dim3(G.ngroups, G.ncb, 1), 256, sm, ctx->stream>>>(g, hs, ncell, pl.d_pairs + Gp.pair_off, G,
-                                                                             w.partial);
+            // kind 0: the singles are rows of g, staged once
+            const T* hs = kind == 0 ? nullptr : h + (size_t)Gp.s0 * ncell;
+            k_contract<T><<<dim3(G.ngroups, G.ncb, 1), 256, sm, ctx->stream>>>(g, hs, Gp.s0, ncell,
+                                                                             pl.d_pairs + Gp.pair_off, G, w.partial);
             const long nout = (long)G.npairs * G.nh;
             k_reduce_partials<<<reduce_blocks(nout), dim3(32, kRedSlices), 0, ctx->stream>>>(w.partial, G.ncb, nout,
                                                                                              pl.d_M + Gp.out_off);

@@ -122,12 +122,12 @@ extern "C" int polybin_contract_noalloc(const float* g, int n_g, const float* h,
             slot->ready = true;
         }
     }
-    const size_t sm = ((size_t)kCH * G.rows_cta + (size_t)kCH * G.nhp + (size_t)n_g * (kCH + 1)) * sizeof(float) + 16;
+    const size_t sm = contract_smem<float>(G);
     if (sm > 48 * 1024) {
         e = cudaFuncSetAttribute((const void*)k_contract<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return set_error(POLYBIN_ECUDA, std::string("polybin_contract_noalloc: ") + cudaGetErrorString(e));
     }
-    k_contract<float><<<dim3(G.ngroups, G.ncb, 1), 256, sm, st>>>(g, h, (long)ncell, slot->pairs + pairs_offset(n_g), G,
+    k_contract<float><<<dim3(G.ngroups, G.ncb, 1), 256, sm, st>>>(g, h, 0, (long)ncell, slot->pairs + pairs_offset(n_g), G,
                                                                  slot->scratch);
     e = cudaGetLastError();
     if (e != cudaSuccess) return set_error(POLYBIN_ECUDA, std::string("polybin_contract_noalloc: ") + cudaGetErrorString(e));
