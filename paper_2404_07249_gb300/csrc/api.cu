@@ -9,11 +9,13 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
 #include "contract.cuh"
 #include "fft.cuh"
+#include "fft2.h"
 #include "polybin.h"
 #include "polybin_internal.h"
 
@@ -94,7 +96,17 @@ int run_forward(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T
     auto tw = [&](int a) { return (const C<T>*)(sizeof(T) == 4 ? ig.tw_f[a] : ig.tw_d[a]); };
     int rc = POLYBIN_OK;
     StageTimer timer(ctx, kStageForward);
-    {
+    // FP32 passes of the two-stage lengths (fft2.cuh); the staged passes take FP64 and the other lengths
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value && std::is_same<TIN, float>::value && std::is_same<TM, float>::value) {
+        if (f2::has(N2)) {
+            f2::ZFwdBatch b;
+            b.it[0] = {in, m1 ? m1 : m2, m1 ? m2 : nullptr, nullptr, nullptr, t1};
+            done = f2::fwd_z(N2, b, 1, nlines, Bz, ctx->stream);
+            if ((rc = launch_check(ctx, "f2::fwd_z"))) return rc;
+        }
+    }
+    if (!done) {
         const int LP = lines_per_cta<T>(N2);
         const size_t sm = (2 * (size_t)N2 * (LP + 1) + N2) * sizeof(C<T>);
         const unsigned nblk = (unsigned)((nlines + 2 * LP - 1) / (2 * LP));
@@ -112,11 +124,13 @@ int run_forward(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T
         it.in = t1; it.out = t2;
         it.in_os = (long)N1 * Bz; it.in_es = Bz; it.out_os = (long)By * Bz; it.out_es = Bz;
         it.ncols = Bz; it.nouter = N0; it.rng = ctx->gy;
-        dim3 grid((Bz + TK - 1) / TK, N0, 1);
-        PB_WITH_NT(N1, NT, {
-            if ((rc = set_smem<T>(ctx, (const void*)k_col<T, -1, NT>, sm))) return rc;
-            k_col<T, -1, NT><<<grid, 256, sm, ctx->stream>>>(b, ig.plan[1], tw(1), TK);
-        })
+        if (!(sizeof(T) == 4 && f2::col(N1, -1, b, 1, Bz, N0, ctx->stream))) {
+            dim3 grid((Bz + TK - 1) / TK, N0, 1);
+            PB_WITH_NT(N1, NT, {
+                if ((rc = set_smem<T>(ctx, (const void*)k_col<T, -1, NT>, sm))) return rc;
+                k_col<T, -1, NT><<<grid, 256, sm, ctx->stream>>>(b, ig.plan[1], tw(1), TK);
+            })
+        }
         if ((rc = launch_check(ctx, "k_col fwd y"))) return rc;
     }
     {
@@ -128,11 +142,13 @@ int run_forward(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T
         it.in = t2; it.out = box;
         it.in_os = 0; it.in_es = ncols; it.out_os = 0; it.out_es = ncols;
         it.ncols = ncols; it.nouter = 1; it.rng = ctx->gx;
-        dim3 grid((ncols + TK - 1) / TK, 1, 1);
-        PB_WITH_NT(N0, NT, {
-            if ((rc = set_smem<T>(ctx, (const void*)k_col<T, -1, NT>, sm))) return rc;
-            k_col<T, -1, NT><<<grid, 256, sm, ctx->stream>>>(b, ig.plan[0], tw(0), TK);
-        })
+        if (!(sizeof(T) == 4 && f2::col(N0, -1, b, 1, ncols, 1, ctx->stream))) {
+            dim3 grid((ncols + TK - 1) / TK, 1, 1);
+            PB_WITH_NT(N0, NT, {
+                if ((rc = set_smem<T>(ctx, (const void*)k_col<T, -1, NT>, sm))) return rc;
+                k_col<T, -1, NT><<<grid, 256, sm, ctx->stream>>>(b, ig.plan[0], tw(0), TK);
+            })
+        }
         if ((rc = launch_check(ctx, "k_col fwd x"))) return rc;
     }
     return POLYBIN_OK;
@@ -143,16 +159,49 @@ int run_forward(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T
     return run_forward<T, TIN, TM>(ctx, in, m1, m2, t1, t2, box, ctx->fg);
 }
 
+// C2R z-pass of nitem items on the staged and the FP64 register-resident passes.
+template <typename T>
+int launch_inv_z(polybin_ctx* ctx, const ZInvBatch& b, int nitem, long nlines, T scale, const T* mulout, const FftPlan& plan,
+                 const C<T>* tw) {
+    const int n = plan.n;
+    int rc;
+    if constexpr (sizeof(T) == 8) {
+        const int lpc = 16;                           // line pairs a CTA
+        const dim3 grid((unsigned)(((nlines + 1) / 2 + lpc - 1) / lpc), nitem, 1);
+        if (n == 512) {
+            k_inv_z512<T><<<grid, 256, 0, ctx->stream>>>(b, nlines, scale, mulout, tw, lpc);
+            return POLYBIN_OK;
+        }
+        if (n == 256) {
+            k_inv_z256<T><<<grid, 256, 0, ctx->stream>>>(b, nlines, scale, mulout, tw, lpc);
+            return POLYBIN_OK;
+        }
+    }
+    const int LP = lines_per_cta<T>(n);
+    const size_t sm = (2 * (size_t)n * (LP + 1) + n) * sizeof(C<T>);
+    const dim3 grid((unsigned)((nlines + 2 * LP - 1) / (2 * LP)), nitem, 1);
+    PB_WITH_NT_INV(n, NT, {
+        if ((rc = set_smem<T>(ctx, (const void*)k_inv_z<T, NT>, sm))) return rc;
+        k_inv_z<T, NT><<<grid, 256, sm, ctx->stream>>>(b, nlines, scale, mulout, plan, tw, LP);
+    })
+    return POLYBIN_OK;
+}
+template int launch_inv_z<float>(polybin_ctx*, const ZInvBatch&, int, long, float, const float*, const FftPlan&, const float2*);
+template int launch_inv_z<double>(polybin_ctx*, const ZInvBatch&, int, long, double, const double*, const FftPlan&,
+                                  const double2*);
+
 // a2: shell maps g_b = IFT[Theta_b L_ell D] for all bins on grid ig (box == nullptr: unit spectrum, giving t_b).
 // The inverse DFT is normalised by the data grid's 1/N on either grid, so a map on the contraction grid holds the
 // same band-limited function as on the data grid, sampled at fewer points.
 template <typename T>
-int run_shells(polybin_ctx* ctx, const C<T>* box, C<T>* u1, C<T>* u2, T* g, int ell, const InvGrid& ig) {
-    return run_shells_m<T>(ctx, box, u1, u2, g, ell, kLegendreM, ig);
+int run_shells(polybin_ctx* ctx, const C<T>* box, C<T>* u1, C<T>* u2, T* g, int ell, const InvGrid& ig,
+               uint32_t* absmax) {
+    return run_shells_m<T>(ctx, box, u1, u2, g, ell, kLegendreM, ig, absmax);
 }
 
 template <typename T>
-int run_shells_m(polybin_ctx* ctx, const C<T>* box, C<T>* u1, C<T>* u2, T* g, int ell, int m, const InvGrid& ig) {
+int run_shells_m(polybin_ctx* ctx, const C<T>* box, C<T>* u1, C<T>* u2, T* g, int ell, int m, const InvGrid& ig,
+                 uint32_t* absmax) {
     const int N0 = ig.N[0], N1 = ig.N[1], N2 = ig.N[2];
     const int nb = ctx->nb;
     int rc = POLYBIN_OK;
@@ -174,12 +223,11 @@ int run_shells_m(polybin_ctx* ctx, const C<T>* box, C<T>* u1, C<T>* u2, T* g, in
             b.it[i].m = m;
             maxcols = std::max(maxcols, bb.ry.cnt * bb.rz.cnt);
         }
-        if (N0 == 288 && sizeof(T) == 4) {
-            // register-resident 288-point x lines, 16 columns of the bin's box a CTA
-            dim3 grid288((maxcols + kY288Cols - 1) / kY288Cols, nb, 1);
-            k_inv_x288_filter<<<grid288, kY288Threads, y288_smem(), ctx->stream>>>(
-                b, (const float2*)box, ctx->gx, ctx->gy, ctx->gz, (float)(1.0 / (double)ctx->ncell), (const float2*)tw(0));
-        } else {
+        bool done = false;
+        if constexpr (std::is_same<T, float>::value)
+            done = f2::xfilter(N0, b, nb, maxcols, box, ctx->gx, ctx->gy, ctx->gz, (float)(1.0 / (double)ctx->ncell),
+                               ctx->stream);
+        if (!done) {
             dim3 grid((maxcols + TK - 1) / TK, nb, 1);
             PB_WITH_NT_INV(N0, NT, {
                 if ((rc = set_smem<T>(ctx, (const void*)k_inv_x_filter<T, NT>, sm))) return rc;
@@ -203,11 +251,7 @@ int run_shells_m(polybin_ctx* ctx, const C<T>* box, C<T>* u1, C<T>* u2, T* g, in
             it.ncols = bb.rz.cnt; it.nouter = N0; it.rng = bb.ry;
             maxc = std::max(maxc, bb.rz.cnt);
         }
-        if (N1 == 288 && sizeof(T) == 4) {
-            // register-resident 288-point columns, 16 wave numbers kz a CTA
-            dim3 grid288((maxc + kY288Cols - 1) / kY288Cols, N0, nb);
-            k_inv_y288<<<grid288, kY288Threads, y288_smem(), ctx->stream>>>(b, (const float2*)tw(1));
-        } else {
+        if (!(sizeof(T) == 4 && f2::col(N1, +1, b, nb, maxc, N0, ctx->stream))) {
             dim3 grid((maxc + TK - 1) / TK, N0, nb);
             PB_WITH_NT_INV(N1, NT, {
                 if ((rc = set_smem<T>(ctx, (const void*)k_col<T, +1, NT>, sm))) return rc;
@@ -217,8 +261,6 @@ int run_shells_m(polybin_ctx* ctx, const C<T>* box, C<T>* u1, C<T>* u2, T* g, in
         if ((rc = launch_check(ctx, "k_col inv y"))) return rc;
     }
     {
-        const int LP = lines_per_cta<T>(N2);
-        const size_t sm = (2 * (size_t)N2 * (LP + 1) + N2) * sizeof(C<T>);
         ZInvBatch b;
         for (int i = 0; i < nb; ++i) {
             const BinBox& bb = ig.bbox[i];
@@ -227,36 +269,16 @@ int run_shells_m(polybin_ctx* ctx, const C<T>* box, C<T>* u1, C<T>* u2, T* g, in
             b.it[i].kin = bb.rz.cnt;
         }
         const long nlines = (long)N0 * N1;
-        if (N2 == 512) {
-            // register-resident 512-point transform, 16 line pairs per CTA
-            const int lpc = 16;
-            dim3 grid512((unsigned)(((nlines + 1) / 2 + lpc - 1) / lpc), nb, 1);
-            k_inv_z512<T><<<grid512, 256, 0, ctx->stream>>>(b, nlines, T(1), (const T*)nullptr, tw(2), lpc);
-        } else if (N2 == 256) {
-            // register-resident 256-point transform, one warp a line pair, 16 line pairs per CTA
-            const int lpc = 16;
-            dim3 grid256((unsigned)(((nlines + 1) / 2 + lpc - 1) / lpc), nb, 1);
-            k_inv_z256<T><<<grid256, 256, 0, ctx->stream>>>(b, nlines, T(1), (const T*)nullptr, tw(2), lpc);
-        } else if (N2 == 288 && sizeof(T) == 4) {
-            // register-resident 288-point transform, 128 line pairs per CTA (8 rounds of 16, each round's input
-            // staged one round ahead by one bulk copy of the TMA engine; a copy that never lands raises the
-            // staging error flag, reported at the next read of the flags)
-            if ((rc = ensure_err_flag(ctx))) return rc;
-            const int ppc = 128;
-            int kin_max = 1;
-            for (int i = 0; i < nb; ++i) kin_max = std::max(kin_max, b.it[i].kin);
-            const size_t smz = z288_smem(kin_max);
-            dim3 grid288((unsigned)(((nlines + 1) / 2 + ppc - 1) / ppc), nb, 1);
-            if ((rc = set_smem<T>(ctx, (const void*)k_inv_z288, smz))) return rc;
-            k_inv_z288<<<grid288, kZ288Threads, smz, ctx->stream>>>(b, nlines, 1.f, (const float*)nullptr,
-                                                                    (const float2*)tw(2), ppc,
-                                                                    ctx->d_err + kErrStaging);
-        } else {
-            dim3 grid((unsigned)((nlines + 2 * LP - 1) / (2 * LP)), nb, 1);
-            PB_WITH_NT_INV(N2, NT, {
-                if ((rc = set_smem<T>(ctx, (const void*)k_inv_z<T, NT>, sm))) return rc;
-                k_inv_z<T, NT><<<grid, 256, sm, ctx->stream>>>(b, nlines, T(1), (const T*)nullptr, ig.plan[2], tw(2), LP);
-            })
+        bool done = false;
+        if constexpr (std::is_same<T, float>::value) {
+            if (absmax) PB_CUDA_OK(cudaMemsetAsync(absmax, 0, sizeof(uint32_t) * kMaxItems, ctx->stream));
+            // (16-byte stores: a caller's maps may lie at any float)
+            done = reinterpret_cast<uintptr_t>(g) % 16 == 0 &&
+                   f2::inv_z(N2, b, nb, nlines, 1.f, nullptr, absmax, ctx->stream);
+        }
+        if (!done) {
+            if ((rc = launch_inv_z<T>(ctx, b, nb, nlines, T(1), (const T*)nullptr, ig.plan[2], tw(2)))) return rc;
+            if (absmax && (rc = run_absmax(ctx, (const float*)g, nb, ig.ncell, absmax))) return rc;
         }
         if ((rc = launch_check(ctx, "k_inv_z"))) return rc;
     }
@@ -336,16 +358,17 @@ template int run_pkbin<float>(polybin_ctx*, const float2*, std::vector<double>&)
 template int run_pkbin<double>(polybin_ctx*, const double2*, std::vector<double>&);
 template int run_pkbin_dev<float>(polybin_ctx*, const float2*);
 template int run_pkbin_dev<double>(polybin_ctx*, const double2*);
-template int run_shells<float>(polybin_ctx*, const float2*, float2*, float2*, float*, int, const InvGrid&);
-template int run_shells<double>(polybin_ctx*, const double2*, double2*, double2*, double*, int, const InvGrid&);
-template int run_shells_m<float>(polybin_ctx*, const float2*, float2*, float2*, float*, int, int, const InvGrid&);
-template int run_shells_m<double>(polybin_ctx*, const double2*, double2*, double2*, double*, int, int, const InvGrid&);
+template int run_shells<float>(polybin_ctx*, const float2*, float2*, float2*, float*, int, const InvGrid&, uint32_t*);
+template int run_shells<double>(polybin_ctx*, const double2*, double2*, double2*, double*, int, const InvGrid&, uint32_t*);
+template int run_shells_m<float>(polybin_ctx*, const float2*, float2*, float2*, float*, int, int, const InvGrid&, uint32_t*);
+template int run_shells_m<double>(polybin_ctx*, const double2*, double2*, double2*, double*, int, int, const InvGrid&,
+                                  uint32_t*);
 template int run_contract<float>(polybin_ctx*, const float*, int, const float*, int, double*, size_t, double*, long);
 template int run_contract<double>(polybin_ctx*, const double*, int, const double*, int, double*, size_t, double*, long);
 
 template <>
 int run_contract_any<double>(polybin_ctx* ctx, const double* g, int ng, const double* h, int nh, double* part,
-                             size_t cap, double* out, long ncell) {
+                             size_t cap, double* out, long ncell, const uint32_t*, const uint32_t*) {
     return run_contract<double>(ctx, g, ng, h, nh, part, cap, out, ncell);
 }
 
@@ -782,6 +805,10 @@ extern "C" int polybin_init(polybin_ctx** out, const int grid[3], const double b
     if (!rc) rc = plan_pk(ctx);
     // the device error flags exist from the start (kernels captured into CUDA graphs write them)
     if (!rc) rc = ensure_err_flag(ctx);
+    if (!rc && prec == POLYBIN_SPLIT_TF32X3) {
+        cudaError_t e = cudaMalloc(&ctx->d_mapmax, sizeof(uint32_t) * 2 * kMaxItems);
+        if (e != cudaSuccess) rc = fail_cuda(ctx, e, "map maxima", __FILE__, __LINE__);
+    }
     if (!rc) rc = (prec == POLYBIN_FP64) ? alloc_work<double>(ctx, ctx->w) : alloc_work<float>(ctx, ctx->w);
     if (!rc && prec == POLYBIN_SPLIT_TF32X3) rc = tf32_selfcheck(ctx);
     if (rc) {
@@ -798,7 +825,7 @@ extern "C" void polybin_destroy(polybin_ctx* ctx) {
     free_work(ctx->w);
     if (ctx->cstream) cudaStreamSynchronize(ctx->cstream);
     void* ptrs[] = {ctx->d_lut, ctx->d_pairs, ctx->d_offs, ctx->d_coef, ctx->d_bin_start, ctx->d_pkpart, ctx->d_in,
-                    ctx->d_stage[0], ctx->d_stage[1], ctx->d_pkout, ctx->d_counts,
+                    ctx->d_stage[0], ctx->d_stage[1], ctx->d_mapmax, ctx->d_pkout, ctx->d_counts,
                     ctx->d_tw_f[0], ctx->d_tw_f[1], ctx->d_tw_f[2], ctx->d_tw_d[0], ctx->d_tw_d[1], ctx->d_tw_d[2],
                     ctx->d_ctw[0], ctx->d_ctw[1], ctx->d_ctw[2], ctx->d_ctw[3], ctx->d_ctw[4], ctx->d_ctw[5]};
     for (void* p : ptrs)
@@ -861,8 +888,8 @@ static int bk_pk_t(polybin_ctx* ctx, const float* delta, int batch, double* bk_o
                                        cudaMemcpyDeviceToHost, ctx->stream));
         }
         if (bk_out && nt > 0) {
-            if ((rc = run_shells<T>(ctx, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g, 0, ctx->cg))) return rc;
-            if ((rc = run_triplet_sums<T>(ctx, (const T*)w.g, ctx->d_S))) return rc;
+            if ((rc = run_shells<T>(ctx, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g, 0, ctx->cg, map_max(ctx, 0)))) return rc;
+            if ((rc = run_triplet_sums<T>(ctx, (const T*)w.g, ctx->d_S, map_max(ctx, 0)))) return rc;
             if ((rc = run_bk_normalise(ctx, ctx->d_S, ctx->d_B))) return rc;
             PB_CUDA_OK(cudaMemcpyAsync(bk_out + (size_t)f * nt, ctx->d_B, sizeof(double) * nt, cudaMemcpyDeviceToHost,
                                        ctx->stream));
@@ -890,14 +917,14 @@ static int bk_multipoles_t(polybin_ctx* ctx, const float* delta, int batch, int 
         if ((rc = run_forward<T, float, float>(ctx, in, (const float*)nullptr, (const float*)nullptr, (C<T>*)w.t1, (C<T>*)w.t2, (C<T>*)w.box))) return rc;
         if ((rc = st.done(f))) return rc;
         if (nt == 0) continue;
-        if ((rc = run_shells<T>(ctx, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g, 0, ctx->cg))) return rc;
+        if ((rc = run_shells<T>(ctx, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g, 0, ctx->cg, map_max(ctx, 0)))) return rc;
         for (int il = 0; il < nl; ++il) {
             const int ell = 2 * il;
             if (ell == 0) {
-                if ((rc = run_triplet_sums<T>(ctx, (const T*)w.g, ctx->d_S))) return rc;
+                if ((rc = run_triplet_sums<T>(ctx, (const T*)w.g, ctx->d_S, map_max(ctx, 0)))) return rc;
             } else {
-                if ((rc = run_shells<T>(ctx, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g2, ell, ctx->cg))) return rc;
-                if ((rc = run_triplet_sums_ell<T>(ctx, (const T*)w.g, (const T*)w.g2, ctx->d_S))) return rc;
+                if ((rc = run_shells<T>(ctx, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g2, ell, ctx->cg, map_max(ctx, 1)))) return rc;
+                if ((rc = run_triplet_sums_ell<T>(ctx, (const T*)w.g, (const T*)w.g2, ctx->d_S, map_max(ctx, 0), map_max(ctx, 1)))) return rc;
             }
             if ((rc = run_bk_normalise(ctx, ctx->d_S, ctx->d_B, 2.0 * ell + 1.0))) return rc;
             PB_CUDA_OK(cudaMemcpyAsync(bk_out + ((size_t)f * nl + il) * nt, ctx->d_B, sizeof(double) * nt,

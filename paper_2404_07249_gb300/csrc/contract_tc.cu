@@ -10,7 +10,7 @@
 // Arithmetic: the pair products A = g_j g_k (FP32) and the singles B are split as hi + lo with hi the value rounded to
 // 11 bits and lo the rounded remainder, 22 bits in all.  Both parts are FP16, which has TF32's 11 bits at twice its
 // tensor rate and half its storage.  FP16's short exponent is met by powers of two taken from the maps' maxima
-// (k_absmax): a row's products are scaled below 2^15, a single's values below 2^15, and the final FP64 sums scaled
+// (found by the z-pass that writes them, or by k_absmax): a row's products are scaled below 2^15, a single's values below 2^15, and the final FP64 sums scaled
 // back.  Values far below a map's maximum lose bits only below 2^-40 of it.  Per tile and K = 16 cells two MMAs of
 // N = 2W run, D[:, hi | lo] += A_lo . [B_hi | B_lo]^T and then A_hi . [B_hi | B_lo]^T: all four partial products.  The
 // tensor core's internal accumulation is not round-to-nearest, so D restarts every 64 cells, the A_lo terms first
@@ -65,7 +65,6 @@ constexpr int kMaxAStages = 6;
 constexpr int kSpill = 32;         // stages per FP32 register sum (2048 cells)
 constexpr int kDBuf = 2;           // accumulator buffers (the epilogue reads one while the MMAs fill the other)
 constexpr int kAcols = 64;         // tensor memory columns of a tile's A stage: hi and lo of 64 cells, two a column
-constexpr int kMaxRows = 128;      // map rows of a slot: <= 64 g rows and <= 64 h rows
 constexpr int kMaxTiles = 3;       // tiles per CTA
 constexpr int kMaxUnits = 3;       // 16-column output units per CTA (16 FP32 sums each, in registers)
 constexpr int kMaxGroups = 4;      // row groups (grid.y)
@@ -105,7 +104,7 @@ struct Params {
     int ng, nh, hsep, h_row0;  // maps in the slot; singles; singles from the h part; first h row in a slot
     int slot_bytes, off_b, off_acc, off_bar;
     int s_off, s_chunks;       // singles region of a slot: byte offset and 16-byte chunks (B is made for all)
-    const uint32_t* absmax;    // max |map| bit patterns by slot row (the scale factors)
+    const uint32_t *gmax, *hmax;   // max |map| bit patterns of the g rows and of the h rows (the scale factors)
     int total_units;
     const short2* rows;        // [tiles][128] pairs (j, k); (-1, -1) pads
     double* partial;           // [gridDim.x][total_units][16][128]
@@ -222,6 +221,10 @@ __device__ __forceinline__ void split_h2(uint64_t v, uint32_t& hi, uint32_t& lo)
 __host__ __device__ inline int map_exp(uint32_t m) {
     const int e = (int)((m >> 23) & 255u);
     return e == 255 ? 0 : (e < 1 ? 1 : e) - 126;
+}
+// Largest magnitude of the map at slot row r (h rows start at h_row0).
+__device__ __forceinline__ uint32_t row_max(const uint32_t* gmax, const uint32_t* hmax, int h_row0, int r) {
+    return r < h_row0 ? gmax[r] : hmax[r - h_row0];
 }
 __host__ __device__ inline int clamp_exp(int e) { return e < -126 ? -126 : (e > 127 ? 127 : e); }
 __host__ __device__ inline int row_exp(uint32_t mj, uint32_t mk) { return clamp_exp(15 - map_exp(mj) - map_exp(mk)); }
@@ -409,7 +412,7 @@ __device__ __forceinline__ void producer(const GroupDesc& G, const Params& P, ui
         const int j = max((int)jk.x, 0), k = max((int)jk.y, 0);
         oj[t] = j * 128; xj[t] = (j & 7) << 4;
         ok_[t] = k * 128; xk[t] = (k & 7) << 4;
-        const float f = pad[t] ? 0.f : pow2f(row_exp(P.absmax[j], P.absmax[k]));
+        const float f = pad[t] ? 0.f : pow2f(row_exp(row_max(P.gmax, P.hmax, P.h_row0, j), row_max(P.gmax, P.hmax, P.h_row0, k)));
         scale[t] = f2pack(f, f);
     }
     // tensor-memory addresses from warp-uniform, divide-free values (the base is 0: the CTA holds all 512
@@ -556,7 +559,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int* const err = P.err;
 
     for (int i = tid; i < G.nunits * 16 * 128; i += kThreads) acc64[i] = 0.0;
-    if (tid < P.s_chunks / 8) bscale[tid] = pow2f(single_exp(P.absmax[P.s_off / 128 + tid]));
+    if (tid < P.s_chunks / 8) bscale[tid] = pow2f(single_exp(row_max(P.gmax, P.hmax, P.h_row0, P.s_off / 128 + tid)));
     if (tid == 0) {
         for (int s = 0; s < kRingSlots; ++s) {
             mbar_init(&slot_full[s], 1);
@@ -716,7 +719,8 @@ constexpr int kSlices = 16;
 __global__ void __launch_bounds__(32 * kSlices) k_reduce_gather(const double* __restrict__ partial, int ncta, long stride,
                                                                 const int* __restrict__ gidx,
                                                                 const uchar4* __restrict__ rows,
-                                                                const uint32_t* __restrict__ absmax, int n_out,
+                                                                const uint32_t* __restrict__ gmax,
+                                                                const uint32_t* __restrict__ hmax, int h_row0, int n_out,
                                                                 double* __restrict__ out) {
     __shared__ double red[kSlices][33];
     const int o = blockIdx.x * 32 + threadIdx.x;
@@ -731,7 +735,8 @@ __global__ void __launch_bounds__(32 * kSlices) k_reduce_gather(const double* __
     if (threadIdx.y || o >= n_out) return;
     for (int q = 1; q < kSlices; ++q) s += red[q][threadIdx.x];
     const uchar4 r = rows[o];
-    out[o] = ldexp(s, -row_exp(absmax[r.x], absmax[r.y]) - single_exp(absmax[r.z]));
+    out[o] = ldexp(s, -row_exp(row_max(gmax, hmax, h_row0, r.x), row_max(gmax, hmax, h_row0, r.y)) -
+                          single_exp(row_max(gmax, hmax, h_row0, r.z)));
 }
 
 // Self-test of the bounded waits: one thread waits on an mbarrier phase that nothing completes; the wait gives up
@@ -1265,7 +1270,7 @@ struct PlanCache {
     std::map<std::tuple<int, int, int, int, long>, Plan*> plans;   // (ng, nh, hsep, kind, ncell)
     double* gram_part = nullptr;                                   // Gram partials (K splits)
     size_t gram_cap = 0;
-    uint32_t* d_absmax = nullptr;                                  // [kMaxRows] maxima of the maps by slot row
+    uint32_t* d_absmax = nullptr;                                  // [2][64] maxima of g and h maps found here
     ~PlanCache() {
         if (d_absmax) cudaFree(d_absmax);
         for (auto& kv : plans) delete kv.second;
@@ -1297,7 +1302,7 @@ static int build_plan(polybin_ctx* ctx, Plan& pl, long ncell, int ng, int nh, in
     const char* msg = layout_plan(pl, ncell, nsm, ng, nh, hsep, std::move(need), n_out, rows, gidx, sing_g, opts);
     if (msg) return quiet ? POLYBIN_EINVAL : fail(ctx, POLYBIN_EINVAL, "%s", msg);
     PlanCache* pc = cache_of(ctx);
-    if (!pc->d_absmax) PB_CUDA_OK(cudaMalloc(&pc->d_absmax, sizeof(uint32_t) * kMaxRows));
+    if (!pc->d_absmax) PB_CUDA_OK(cudaMalloc(&pc->d_absmax, sizeof(uint32_t) * 2 * kMaxItems));
     PB_CUDA_OK(cudaMalloc(&pl.d_rows, sizeof(short2) * rows.size()));
     PB_CUDA_OK(cudaMemcpy(pl.d_rows, rows.data(), sizeof(short2) * rows.size(), cudaMemcpyHostToDevice));
     PB_CUDA_OK(cudaMalloc(&pl.d_gidx, sizeof(int) * gidx.size()));
@@ -1361,7 +1366,9 @@ static int make_map2(polybin_ctx* ctx, CUtensorMap* m, const float* base, long w
     return POLYBIN_OK;
 }
 
-static int launch(polybin_ctx* ctx, Plan& pl, const float* g, const float* h, double* d_out) {
+// gmax, hmax: the maps' maxima (kMaxItems entries each), or null: found here first.
+static int launch(polybin_ctx* ctx, Plan& pl, const float* g, const float* h, double* d_out, const uint32_t* gmax,
+                  const uint32_t* hmax) {
     CUtensorMap mg, mh;
     int rc = make_map(ctx, &mg, g, pl.ng, pl.base.ncell);
     if (rc) return rc;
@@ -1388,27 +1395,25 @@ static int launch(polybin_ctx* ctx, Plan& pl, const float* g, const float* h, do
     PlanCache* pc = cache_of(ctx);
     Params P = pl.base;
     P.err = ctx->d_err;
-    P.absmax = pc->d_absmax;
+    if (!gmax) {
+        if ((rc = run_absmax(ctx, g, pl.ng, pl.base.ncell, pc->d_absmax))) return rc;
+        gmax = pc->d_absmax;
+    }
+    if (pl.hsep && !hmax) {
+        if ((rc = run_absmax(ctx, h, pl.nh, pl.base.ncell, pc->d_absmax + kMaxItems))) return rc;
+        hmax = pc->d_absmax + kMaxItems;
+    }
+    P.gmax = gmax;
+    P.hmax = pl.hsep ? hmax : gmax;
     {
         StageTimer timer(ctx, kStageContract);
-        // the maps' maxima (scale factors), by slot row
-        e = cudaMemsetAsync(pc->d_absmax, 0, sizeof(uint32_t) * kMaxRows, ctx->stream);
-        if (e != cudaSuccess) return fail_cuda(ctx, e, "cudaMemsetAsync", __FILE__, __LINE__);
-        const long n4 = pl.base.ncell / 4;
-        const unsigned nblk = (unsigned)std::min((n4 + 1023) / 1024, 64L);
-        k_absmax<<<dim3(nblk, pl.ng, 1), 256, 0, ctx->stream>>>(reinterpret_cast<const float4*>(g), n4, pc->d_absmax);
-        ctx->launches += 1;
-        if (pl.hsep) {
-            k_absmax<<<dim3(nblk, pl.nh, 1), 256, 0, ctx->stream>>>(reinterpret_cast<const float4*>(h), n4,
-                                                                     pc->d_absmax + pl.base.h_row0);
-            ctx->launches += 1;
-        }
         k_contract_tc<<<dim3(pl.ncta, pl.ngroups, 1), kThreads, pl.smem, ctx->stream>>>(mg, mh, P);
         ctx->launches += 1;
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail_cuda(ctx, e, "k_contract_tc", __FILE__, __LINE__);
         k_reduce_gather<<<(pl.n_out + 31) / 32, dim3(32, kSlices), 0, ctx->stream>>>(
-            pl.d_partial, pl.ncta, (long)pl.total_units * 2048, pl.d_gidx, pl.d_orows, pc->d_absmax, pl.n_out, d_out);
+            pl.d_partial, pl.ncta, (long)pl.total_units * 2048, pl.d_gidx, pl.d_orows, P.gmax, P.hmax,
+            pl.base.h_row0, pl.n_out, d_out);
         ctx->launches += 1;
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail_cuda(ctx, e, "k_reduce_gather", __FILE__, __LINE__);
@@ -1422,7 +1427,8 @@ static int launch(polybin_ctx* ctx, Plan& pl, const float* g, const float* h, do
 // caller's own inputs, timed with CUDA events on the context stream (one launch to warm up, two timed); the fastest
 // replaces the plan in the cache.  Candidates differ only in how cells and rows are split, so their results agree to
 // FP32 rounding of the partial sums; after tuning every call takes the chosen plan.
-static int tune_plan(polybin_ctx* ctx, Plan** pl_io, const float* g, const float* h, double* d_out) {
+static int tune_plan(polybin_ctx* ctx, Plan** pl_io, const float* g, const float* h, double* d_out, const uint32_t* gmax,
+                     const uint32_t* hmax) {
     Plan* pl = *pl_io;
     if (pl->tuned) return POLYBIN_OK;
     if (ctx->capturing) {   // a captured graph keeps this plan's buffers: it must never be replaced
@@ -1437,10 +1443,10 @@ static int tune_plan(polybin_ctx* ctx, Plan** pl_io, const float* g, const float
     PB_CUDA_OK(cudaEventCreate(&e1));
     auto time_plan = [&](Plan& c, float* ms) -> int {
         int rc;
-        if ((rc = launch(ctx, c, g, h, d_out))) return rc;
+        if ((rc = launch(ctx, c, g, h, d_out, gmax, hmax))) return rc;
         PB_CUDA_OK(cudaEventRecord(e0, ctx->stream));
         for (int i = 0; i < 2; ++i)
-            if ((rc = launch(ctx, c, g, h, d_out))) return rc;
+            if ((rc = launch(ctx, c, g, h, d_out, gmax, hmax))) return rc;
         PB_CUDA_OK(cudaEventRecord(e1, ctx->stream));
         PB_CUDA_OK(cudaEventSynchronize(e1));
         PB_CUDA_OK(cudaEventElapsedTime(ms, e0, e1));
@@ -1494,10 +1500,11 @@ static int tune_plan(polybin_ctx* ctx, Plan** pl_io, const float* g, const float
     return rc;
 }
 
-static int launch_tuned(polybin_ctx* ctx, Plan* pl, const float* g, const float* h, double* d_out) {
+static int launch_tuned(polybin_ctx* ctx, Plan* pl, const float* g, const float* h, double* d_out, const uint32_t* gmax,
+                        const uint32_t* hmax) {
     int rc;
-    if ((rc = tune_plan(ctx, &pl, g, h, d_out))) return rc;
-    return launch(ctx, *pl, g, h, d_out);
+    if ((rc = tune_plan(ctx, &pl, g, h, d_out, gmax, hmax))) return rc;
+    return launch(ctx, *pl, g, h, d_out, gmax, hmax);
 }
 
 // Plan of all pairs (j <= k) of ng maps against the nh singles [0, nh), output M[(j, k)][i] pair-major.
@@ -1660,13 +1667,24 @@ bool tc_shape_ok(long ncell, const float* g, int ng, const float* h, int nh) {
 }
 
 // M[(j <= k)][i] (pair-major, device) of ng maps g against nh singles h (h == nullptr: h = g), over ncell cells.
-int run_contract_tc(polybin_ctx* ctx, const float* g, int ng, const float* h, int nh, double* d_out, long ncell) {
+int run_contract_tc(polybin_ctx* ctx, const float* g, int ng, const float* h, int nh, double* d_out, long ncell,
+                    const uint32_t* gmax, const uint32_t* hmax) {
     const int hsep = (h && h != g) ? 1 : 0;
     if (!hsep) nh = ng;
     tc::Plan* pl = nullptr;
     int rc = tc::full_plan(ctx, ncell, ng, nh, hsep, &pl);
     if (rc) return rc;
-    return tc::launch_tuned(ctx, pl, g, hsep ? h : g, d_out);
+    return tc::launch_tuned(ctx, pl, g, hsep ? h : g, d_out, gmax, hmax);
+}
+
+int run_absmax(polybin_ctx* ctx, const float* maps, int nmaps, long ncell, uint32_t* absmax) {
+    PB_CUDA_OK(cudaMemsetAsync(absmax, 0, sizeof(uint32_t) * kMaxItems, ctx->stream));
+    const long n4 = ncell / 4;
+    tc::k_absmax<<<dim3((unsigned)std::min((n4 + 1023) / 1024, 64L), nmaps, 1), 256, 0, ctx->stream>>>(
+        reinterpret_cast<const float4*>(maps), n4, absmax);
+    ctx->launches += 1;
+    PB_CUDA_OK(cudaGetLastError());
+    return POLYBIN_OK;
 }
 
 // Builds the closed-triplet plan ahead of time (before any stream capture).
@@ -1677,11 +1695,12 @@ int prepare_triplet_tc(polybin_ctx* ctx) {
 
 // S^ell'_abc = sum g_a g_b g_{c,ell} of every closed triplet (device, triplet order) from the shell maps g and the
 // Legendre-weighted maps gl on the contraction grid.
-int run_triplet_sums_ell_tc(polybin_ctx* ctx, const float* g, const float* gl, double* d_S) {
+int run_triplet_sums_ell_tc(polybin_ctx* ctx, const float* g, const float* gl, double* d_S, const uint32_t* gmax,
+                            const uint32_t* glmax) {
     tc::Plan* pl = nullptr;
     int rc = tc::ell_plan(ctx, &pl);
     if (rc) return rc;
-    return tc::launch_tuned(ctx, pl, g, gl, d_S);
+    return tc::launch_tuned(ctx, pl, g, gl, d_S, gmax, glmax);
 }
 
 // out[i][j] += scale sum_k A[i][k] B[j][k] for float32 rows A [nA][K], B [nB][K] (K a multiple of 4, 16-byte aligned
@@ -1735,11 +1754,11 @@ int run_gram_tc(polybin_ctx* ctx, const float* A, int nA, const float* B, int nB
 }
 
 // S'_abc of every closed triplet (device, triplet order) from the shell maps g on the contraction grid.
-int run_triplet_sums_tc(polybin_ctx* ctx, const float* g, double* d_S) {
+int run_triplet_sums_tc(polybin_ctx* ctx, const float* g, double* d_S, const uint32_t* gmax) {
     tc::Plan* pl = nullptr;
     int rc = tc::triplet_plan(ctx, &pl);
     if (rc) return rc;
-    return tc::launch_tuned(ctx, pl, g, g, d_S);
+    return tc::launch_tuned(ctx, pl, g, g, d_S, gmax, gmax);
 }
 
 }  // namespace pb

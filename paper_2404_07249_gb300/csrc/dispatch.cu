@@ -179,11 +179,11 @@ void destroy_extras(polybin_ctx* ctx) {
 // (polybin_last_path).
 template <>
 int run_contract_any<float>(polybin_ctx* ctx, const float* g, int ng, const float* h, int nh, double* part, size_t cap,
-                            double* out, long ncell) {
+                            double* out, long ncell, const uint32_t* gmax, const uint32_t* hmax) {
     const int nhh = h ? nh : ng;
     if (ctx->prec == POLYBIN_SPLIT_TF32X3 && tc_shape_ok(ncell, g, ng, h, nhh)) {
         ctx->last_path = POLYBIN_PATH_TENSOR_SPLIT_TF32X3;
-        return run_contract_tc(ctx, g, ng, h, nh, out, ncell);
+        return run_contract_tc(ctx, g, ng, h, nh, out, ncell, gmax, hmax);
     }
     ctx->last_path = POLYBIN_PATH_SIMT_FP32;
     return run_contract<float>(ctx, g, ng, h, nh, part, cap, out, ncell);
@@ -198,36 +198,38 @@ __global__ void k_gather_triplets(const double* __restrict__ M, const int* __res
 
 // The split-TF32 mode contracts only the pairs and singles of closed triplets on the tensor cores.
 template <>
-int run_triplet_sums<float>(polybin_ctx* ctx, const float* g, double* d_S) {
+int run_triplet_sums<float>(polybin_ctx* ctx, const float* g, double* d_S, const uint32_t* gmax) {
     if (ctx->Nabc.empty()) return POLYBIN_OK;
     if (ctx->prec == POLYBIN_SPLIT_TF32X3 && tc_shape_ok(ctx->cg.ncell, g, ctx->nb, nullptr, ctx->nb)) {
         ctx->last_path = POLYBIN_PATH_TENSOR_SPLIT_TF32X3;
-        return run_triplet_sums_tc(ctx, g, d_S);
+        return run_triplet_sums_tc(ctx, g, d_S, gmax);
     }
     ctx->last_path = POLYBIN_PATH_SIMT_FP32;
     return simt_triplet_sums<float>(ctx, 0, g, nullptr, d_S);
 }
 
 template <>
-int run_triplet_sums_ell<float>(polybin_ctx* ctx, const float* g, const float* gl, double* d_S) {
+int run_triplet_sums_ell<float>(polybin_ctx* ctx, const float* g, const float* gl, double* d_S, const uint32_t* gmax,
+                                const uint32_t* glmax) {
     if (ctx->Nabc.empty()) return POLYBIN_OK;
     if (ctx->prec == POLYBIN_SPLIT_TF32X3 && tc_shape_ok(ctx->cg.ncell, g, ctx->nb, gl, ctx->nb)) {
         ctx->last_path = POLYBIN_PATH_TENSOR_SPLIT_TF32X3;
-        return run_triplet_sums_ell_tc(ctx, g, gl, d_S);
+        return run_triplet_sums_ell_tc(ctx, g, gl, d_S, gmax, glmax);
     }
     ctx->last_path = POLYBIN_PATH_SIMT_FP32;
     return simt_triplet_sums<float>(ctx, 1, g, gl, d_S);
 }
 
 template <>
-int run_triplet_sums_ell<double>(polybin_ctx* ctx, const double* g, const double* gl, double* d_S) {
+int run_triplet_sums_ell<double>(polybin_ctx* ctx, const double* g, const double* gl, double* d_S, const uint32_t*,
+                                 const uint32_t*) {
     if (ctx->Nabc.empty()) return POLYBIN_OK;
     ctx->last_path = POLYBIN_PATH_SIMT_FP64;
     return simt_triplet_sums<double>(ctx, 1, g, gl, d_S);
 }
 
 template <>
-int run_triplet_sums<double>(polybin_ctx* ctx, const double* g, double* d_S) {
+int run_triplet_sums<double>(polybin_ctx* ctx, const double* g, double* d_S, const uint32_t*) {
     if (ctx->Nabc.empty()) return POLYBIN_OK;
     ctx->last_path = POLYBIN_PATH_SIMT_FP64;
     return simt_triplet_sums<double>(ctx, 0, g, nullptr, d_S);

@@ -1,0 +1,545 @@
+// Two-stage register FFTs (FP32) of the lengths N = P x Q listed in fft2.h and the pass kernels built on them.
+//
+// A transform of length N is shared by max(P, Q) threads.  With k = t + Q j and n = n1 + P n2 (w_m = e^{DIR 2 pi i / m})
+//   X[n1 + P n2] = sum_t w_Q^(t n2) [ w_N^(t n1) sum_j x[t + Q j] w_P^(j n1) ]:
+// thread t < Q takes the P-point DFT over j of its points in registers and multiplies by the twiddles, one exchange
+// through shared memory hands row n1 to thread n1 < P, which takes the Q-point DFT over t.  A staged Stockham pass of the
+// same length goes through shared memory once per radix (three to five times); these passes are bound by shared-memory
+// wavefronts and instruction issue, not by DRAM, so the single exchange is what they gain.  P and Q are as close as
+// they can be, so that neither stage idles many threads.  The points of a thread and all DFT coefficients are
+// compile-time indexed; twiddles come from a table laid out [n1][t], so that a warp reads consecutive entries.
+// Measured on cubic grids, forward transform and the maps of 4 bins (2 above n = 320), us, staged passes (with passes written
+// for one length at 256, 288 and 512) / these:
+//   n            64       96      128      180      216      256      300      320      360      400      480      512
+//   forward   16/17    35/17    24/21   118/34   192/44    85/58  413/100  347/112  710/146  956/185 1567/327  715/395
+//   maps      21/22    31/27    46/35   317/71  566/140  272/160 1295/349 579/398 1298/324 1764/417 2779/964  967/947
+#pragma once
+#include "fft.cuh"
+#include "fft2.h"
+
+namespace pb {
+namespace f2 {
+
+// ------------------------------------------------------------------------------------------------ roots of unity
+
+// cos and sin of x in [0, pi/4] by their Taylor series (the next terms are below 1e-19), evaluated at compile time.
+__host__ __device__ constexpr double taylor_cos(double x) {
+    double term = 1.0, sum = 1.0;
+    for (int i = 1; i <= 10; ++i) {
+        term *= -x * x / ((2 * i - 1) * (2 * i));
+        sum += term;
+    }
+    return sum;
+}
+__host__ __device__ constexpr double taylor_sin(double x) {
+    double term = x, sum = x;
+    for (int i = 1; i <= 10; ++i) {
+        term *= -x * x / ((2 * i) * (2 * i + 1));
+        sum += term;
+    }
+    return sum;
+}
+struct Root {
+    double c, s;
+};
+// e^{2 pi i m / n}, reduced exactly to an octant first.
+__host__ __device__ constexpr Root root(int m, int n) {
+    m %= n;
+    const int o = 8 * m / n;
+    const double q = 0.78539816339744830962;                       // pi / 4
+    double x = q * (double)(8 * m - o * n) / (double)n;            // angle within the octant
+    const bool odd = (o & 1) != 0;
+    if (odd) x = q * (double)((o + 1) * n - 8 * m) / (double)n;    // measured from the octant's end
+    const double c = taylor_cos(x), s = taylor_sin(x);
+    switch (o) {
+        case 0: return Root{c, s};
+        case 1: return Root{s, c};
+        case 2: return Root{-s, c};
+        case 3: return Root{-c, s};
+        case 4: return Root{-c, -s};
+        case 5: return Root{-s, -c};
+        case 6: return Root{s, -c};
+        default: return Root{c, -s};
+    }
+}
+template <int D> struct RootTab {
+    float c[D], s[D];
+    __host__ __device__ constexpr RootTab() : c(), s() {
+        for (int m = 0; m < D; ++m) {
+            const Root r = root(m, D);
+            c[m] = (float)r.c;
+            s[m] = (float)r.s;
+        }
+    }
+};
+// w_N^(t n1) as [n1][t].
+template <int P, int Q> struct TwTab {
+    float2 w[P * Q];
+    __host__ __device__ constexpr TwTab() : w() {
+        for (int a = 0; a < P; ++a)
+            for (int t = 0; t < Q; ++t) {
+                const Root r = root(a * t, P * Q);
+                w[a * Q + t].x = (float)r.c;
+                w[a * Q + t].y = (float)r.s;
+            }
+    }
+};
+template <int P, int Q> __device__ const TwTab<P, Q> kTw = TwTab<P, Q>();
+
+// ------------------------------------------------------------------------------------------------ codelets
+
+// Factors of a composite codelet R = A x B (B taken last).
+__host__ __device__ constexpr int codelet_b(int R) {
+    return R == 16 || R == 32 ? 4 : (R % 3 == 0 ? 3 : (R % 5 == 0 ? 5 : 2));
+}
+// a e^{DIR 2 pi i m / D} for constants m, D (after unrolling).
+template <int DIR, int D> __device__ __forceinline__ float2 rot(float2 a, int m) {
+    constexpr RootTab<D> tab{};
+    m %= D;
+    if (m == 0) return a;
+    if (4 * m == D) return muli<float>(a, DIR);
+    if (2 * m == D) return make_float2(-a.x, -a.y);
+    if (4 * m == 3 * D) return muli<float>(a, -DIR);
+    const float c = tab.c[m], s = DIR * tab.s[m];
+    return make_float2(a.x * c - a.y * s, a.x * s + a.y * c);
+}
+// X[n] = sum_j x[j] e^{DIR 2 pi i j n / R}, natural order in and out, in registers.
+template <int DIR, int R> __device__ __forceinline__ void codelet(float2* x) {
+    if constexpr (R == 1) {
+    } else if constexpr (R == 2 || R == 3 || R == 4 || R == 5 || R == 8) {
+        dft<float, DIR>(x, R);
+    } else {
+        constexpr int B = codelet_b(R), A = R / B;
+        float2 y[B][A];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+#pragma unroll
+            for (int a = 0; a < A; ++a) y[b][a] = x[B * a + b];
+            codelet<DIR, A>(y[b]);
+        }
+#pragma unroll
+        for (int c = 0; c < A; ++c) {
+            float2 z[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) z[b] = rot<DIR, R>(y[b][c], b * c);
+            codelet<DIR, B>(z);
+#pragma unroll
+            for (int d = 0; d < B; ++d) x[c + A * d] = z[d];
+        }
+    }
+}
+
+// Stage 1 of thread t: v[j] = x[t + Q j] -> the twiddled rows v[n1].
+template <int DIR, int P, int Q> __device__ __forceinline__ void stage1(float2* v, int t) {
+    codelet<DIR, P>(v);
+#pragma unroll
+    for (int n1 = 1; n1 < P; ++n1) {
+        const float2 w = kTw<P, Q>.w[n1 * Q + t];
+        v[n1] = DIR > 0 ? mul<float>(v[n1], w) : mulc<float>(v[n1], w);
+    }
+}
+
+// ------------------------------------------------------------------------------------------------ columns
+
+// CTAs per SM asked of the compiler: registers for about 2.5 max(P, Q) complex values a thread.
+__host__ __device__ constexpr int min_ctas(int threads, int pts) {
+    const int regs = pts <= 12 ? 56 : (pts <= 16 ? 64 : (pts <= 20 ? 80 : 128));
+    const int n = 65536 / (threads * regs);
+    return n < 1 ? 1 : n;
+}
+
+// Shared-memory wavefronts of the line exchanges of a CTA with TG threads a transform (8-byte accesses, half a warp at a
+// time): rows of stride `row`, transforms gs apart; the writes of `act_w` threads at consecutive places and the reads of
+// `act_r` threads one row apart.
+__host__ __device__ constexpr int exchange_cost(int threads, int TG, int gs, int row, int act_w, int act_r) {
+    int cost = 0;
+    for (int h = 0; h < threads; h += 16) {
+        int w[16] = {}, r[16] = {}, wm = 0, rm = 0;
+        for (int i = h; i < h + 16 && i < threads; ++i) {
+            const int g = i / TG, t = i % TG;
+            if (t < act_w) {
+                const int n = ++w[(g * gs + t) % 16];
+                wm = n > wm ? n : wm;
+            }
+            if (t < act_r) {
+                const int n = ++r[(g * gs + t * row) % 16];
+                rm = n > rm ? n : rm;
+            }
+        }
+        cost += wm + rm;
+    }
+    return cost;
+}
+// The same for the 4-byte stores of the real lines, transforms os numbers apart.
+__host__ __device__ constexpr int store_cost(int threads, int TG, int os, int act) {
+    int cost = 0;
+    for (int h = 0; h < threads; h += 32) {
+        int w[32] = {}, wm = 0;
+        for (int i = h; i < h + 32 && i < threads; ++i)
+            if (i % TG < act) {
+                const int n = ++w[((i / TG) * os + i % TG) % 32];
+                wm = n > wm ? n : wm;
+            }
+        cost += wm;
+    }
+    return cost;
+}
+
+template <int N> struct Geo {
+    static constexpr int P = stage_p(N), Q = N / P, TG = P > Q ? P : Q;
+    // columns: TC consecutive columns a CTA (128 or 64 bytes a row); with 64 bytes two rows share a half-warp, which an odd
+    // row count keeps apart.  64 bytes where the buffer of 16 columns would leave an SM too few CTAs (forward / maps at 360
+    // points 152 / 347 us with 16 columns, 146 / 324 with 8; at 400 193 / 451 and 185 / 417; at 324 no difference).
+    static constexpr int TC = TG > 20 || N >= 360 ? 8 : 16, kColThreads = TG * TC;
+    static constexpr int kColRow = TC == 8 ? (Q | 1) : Q;
+    static constexpr int kColSmem = P * kColRow * TC * (int)sizeof(float2);
+    // lines: G transforms a CTA
+    static constexpr int G = 256 / TG, kLineThreads = G * TG;
+    // odd row strides of the exchange buffers (P rows of Q, and Q rows of P for the masked pass) and the distance of the
+    // transforms: the one of sixteen with the fewest bank conflicts
+    static constexpr int QP = Q | 1, PP = P | 1;
+    static constexpr int kBuf0 = P * QP > Q * PP ? P * QP : Q * PP, kBuf = kBuf0 > N ? kBuf0 : N;
+    __host__ __device__ static constexpr int best_gs() {
+        int best = kBuf, bc = 1 << 30;
+        for (int gs = kBuf; gs < kBuf + 16; ++gs) {
+            const int c = exchange_cost(kLineThreads, TG, gs, QP, Q, P) * 2 + exchange_cost(kLineThreads, TG, gs, PP, P, Q);
+            if (c < bc) { bc = c; best = gs; }
+        }
+        return best;
+    }
+    static constexpr int GS = best_gs();
+    // real lines on their way out: V numbers a global store, transforms OS numbers apart
+    static constexpr int V = N % 4 == 0 ? 4 : 2;
+    __host__ __device__ static constexpr int best_os() {
+        int best = 2 * N, bc = 1 << 30;
+        for (int os = 2 * N; os < 2 * N + 32; os += V) {
+            const int c = store_cost(kLineThreads, TG, os, P);
+            if (c < bc) { bc = c; best = os; }
+        }
+        return best;
+    }
+    static constexpr int OS = best_os();
+    static constexpr int kLineSmem0 = G * GS * (int)sizeof(float2), kLineSmem1 = G * OS * (int)sizeof(float);
+    static constexpr int kLineSmem = kLineSmem0 > kLineSmem1 ? kLineSmem0 : kLineSmem1;
+};
+
+// One column (thread (t, c) of the CTA: column c of TC): load(k) gives point k, store(n, X) takes the results.
+template <int DIR, int N, class L, class S>
+__device__ __forceinline__ void col_fft(float2* buf, int t, int c, L load, S store) {
+    using E = Geo<N>;
+    constexpr int P = E::P, Q = E::Q, TC = E::TC, QR = E::kColRow;
+    if (t < Q) {
+        float2 v[P];
+#pragma unroll
+        for (int j = 0; j < P; ++j) v[j] = load(t + Q * j);
+        stage1<DIR, P, Q>(v, t);
+#pragma unroll
+        for (int n1 = 0; n1 < P; ++n1) buf[(n1 * QR + t) * TC + c] = v[n1];
+    }
+    __syncthreads();
+    if (t < P) {
+        float2 v[Q];
+#pragma unroll
+        for (int u = 0; u < Q; ++u) v[u] = buf[(t * QR + u) * TC + c];
+        codelet<DIR, Q>(v);
+#pragma unroll
+        for (int n2 = 0; n2 < Q; ++n2) store(t + P * n2, v[n2]);
+    }
+}
+
+// Strided column pass, the same items and results as k_col.
+template <int DIR, int N>
+__global__ void __launch_bounds__(Geo<N>::kColThreads, min_ctas(Geo<N>::kColThreads, Geo<N>::TG)) k_col(ColBatch batch) {
+    extern __shared__ __align__(16) float2 f2_smem[];
+    constexpr int TC = Geo<N>::TC;
+    const ColItem& item = batch.it[blockIdx.z];
+    const int c0 = blockIdx.x * TC, o = blockIdx.y;
+    if (c0 >= item.ncols || o >= item.nouter) return;   // uniform over the CTA
+    const int t = threadIdx.x / TC, c = threadIdx.x - t * TC;
+    const bool act = c0 + c < item.ncols;
+    const float2* __restrict__ in = static_cast<const float2*>(item.in) + (long)o * item.in_os + c0 + c;
+    float2* __restrict__ out = static_cast<float2*>(item.out) + (long)o * item.out_os + c0 + c;
+    const int lo = item.rng.lo, cnt = item.rng.cnt, in_es = (int)item.in_es, out_es = (int)item.out_es;
+    col_fft<DIR, N>(
+        f2_smem, t, c,
+        [&](int k) {
+            if (DIR < 0) return act ? in[(long)k * in_es] : make_float2(0.f, 0.f);
+            const int i = (k < N / 2 ? k : k - N) - lo;   // wave number of position k; zero outside the kept range
+            return act && i >= 0 && i < cnt ? in[(long)i * in_es] : make_float2(0.f, 0.f);
+        },
+        [&](int n, float2 v) {
+            if (!act) return;
+            if (DIR > 0) {
+                out[(long)n * out_es] = v;
+            } else {
+                const int i = (n < N / 2 ? n : n - N) - lo;
+                if (i >= 0 && i < cnt) out[(long)i * out_es] = v;
+            }
+        });
+}
+
+// First inverse pass with the shell filter, the same items and results as k_inv_x_filter.
+template <int N>
+__global__ void __launch_bounds__(Geo<N>::kColThreads, min_ctas(Geo<N>::kColThreads, Geo<N>::TG))
+    k_xfilter(XInvBatch batch, const float2* __restrict__ spec, AxisRange gx, AxisRange gy, AxisRange gz, float scale) {
+    extern __shared__ __align__(16) float2 f2_smem[];
+    constexpr int TC = Geo<N>::TC;
+    const XInvItem& item = batch.it[blockIdx.y];
+    const int ncols = item.ry.cnt * item.rz.cnt;
+    const int c0 = blockIdx.x * TC;
+    if (c0 >= ncols) return;                          // uniform over the CTA
+    const int t = threadIdx.x / TC, c = threadIdx.x - t * TC;
+    const int cc = c0 + c;
+    const bool act = cc < ncols;
+    const int fy = act ? item.ry.lo + cc / item.rz.cnt : 0;
+    const int fz = act ? item.rz.lo + cc % item.rz.cnt : 0;
+    float2* __restrict__ out = static_cast<float2*>(item.out) + cc;
+    col_fft<+1, N>(
+        f2_smem, t, c,
+        [&](int k) {
+            const int fx = k < N / 2 ? k : k - N;
+            const int i = fx - item.rx.lo;
+            float2 v = make_float2(0.f, 0.f);          // stays zero outside the bin
+            if (act && i >= 0 && i < item.rx.cnt) x_filter_value<float>(item, spec, gx, gy, gz, scale, fx, fy, fz, v);
+            return v;
+        },
+        [&](int n, float2 v) {
+            if (act) out[(long)n * ncols] = v;
+        });
+}
+
+// ------------------------------------------------------------------------------------------------ lines
+
+// Stage-1 input of thread t of an inverse transform: points k = t + Q j of the packed Hermitian pair Z = X1 + i X2
+// (kz < kin, zero above; imaginary parts of the kz = 0 and N/2 coefficients ignored).
+template <int N>
+__device__ __forceinline__ void load_hermitian(float2* v, const float2* __restrict__ in1, const float2* __restrict__ in2,
+                                               bool has2, int kin, int t) {
+    constexpr int P = Geo<N>::P, Q = Geo<N>::Q;
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+        const int k = t + Q * j;
+        float2 z = make_float2(0.f, 0.f);
+        if (k == 0 || 2 * k == N) {
+            if (k < kin) z = make_float2(in1[k].x, has2 ? in2[k].x : 0.f);
+        } else if (k < kin) {
+            const float2 a = in1[k];
+            const float2 b = has2 ? in2[k] : make_float2(0.f, 0.f);
+            z = make_float2(a.x - b.y, a.y + b.x);
+        } else if (N - k < kin) {
+            const float2 a = in1[N - k];
+            const float2 b = has2 ? in2[N - k] : make_float2(0.f, 0.f);
+            z = make_float2(a.x + b.y, b.x - a.y);
+        }
+        v[j] = z;
+    }
+}
+
+// The transform's kz < kout coefficients of the two real lines from the packed result Z (in buf): thread t of TG.
+template <int N>
+__device__ __forceinline__ void split_lines(const float2* buf, float2* __restrict__ o1, float2* __restrict__ o2, bool has2,
+                                            int kout, int t) {
+    for (int k = t; k < kout; k += Geo<N>::TG) {
+        const float2 zk = buf[k], zm = buf[k ? N - k : 0];
+        // X1 = (Z[k] + conj Z[N-k]) / 2 ;  X2 = (Z[k] - conj Z[N-k]) / (2i)
+        o1[k] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+        if (has2) o2[k] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+    }
+}
+
+// z-pass, forward (R2C), the same results as k_fwd_z: lines 2p and 2p + 1 packed as one complex line, multiplied on
+// load, kz < kout stored.  An item with sub holds differences of two products, in m1 - sub sub_m (m2 unused).
+template <int N>
+__global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineThreads, Geo<N>::TG))
+    k_fwd_z(ZFwdBatch batch, long nlines, int kout) {
+    extern __shared__ __align__(16) float2 f2_smem[];
+    using E = Geo<N>;
+    constexpr int P = E::P, Q = E::Q, QP = E::QP;
+    const ZFwdItem& item = batch.it[blockIdx.y];
+    const int g = threadIdx.x / E::TG, t = threadIdx.x - g * E::TG;
+    float2* buf = f2_smem + g * E::GS;
+    const long l1 = 2 * ((long)blockIdx.x * E::G + g);
+    const bool act = l1 < nlines, has2 = l1 + 1 < nlines;
+    float2 v[E::TG];
+    if (t < Q && act) {
+        const long i0 = l1 * N + t;
+        const float* __restrict__ in = item.in + i0;
+        const int d2 = has2 ? N : 0;                  // without a second line the first stands in for it, zeroed
+#pragma unroll
+        for (int j = 0; j < P; ++j) v[j] = make_float2(in[Q * j], in[Q * j + d2]);
+        if (item.m1) {
+            const float* __restrict__ m = item.m1 + i0;
+#pragma unroll
+            for (int j = 0; j < P; ++j) {
+                v[j].x *= m[Q * j];
+                v[j].y *= m[Q * j + d2];
+            }
+        }
+        if (item.sub) {
+            const float* __restrict__ a = item.sub + i0;
+            const float* __restrict__ b = item.sub_m + i0;
+#pragma unroll
+            for (int j = 0; j < P; ++j) {
+                v[j].x -= a[Q * j] * b[Q * j];
+                v[j].y -= a[Q * j + d2] * b[Q * j + d2];
+            }
+        } else if (item.m2) {
+            const float* __restrict__ m = item.m2 + i0;
+#pragma unroll
+            for (int j = 0; j < P; ++j) {
+                v[j].x *= m[Q * j];
+                v[j].y *= m[Q * j + d2];
+            }
+        }
+        if (!has2) {
+#pragma unroll
+            for (int j = 0; j < P; ++j) v[j].y = 0.f;
+        }
+        stage1<-1, P, Q>(v, t);
+#pragma unroll
+        for (int n1 = 0; n1 < P; ++n1) buf[n1 * QP + t] = v[n1];
+    }
+    __syncthreads();
+    if (t < P && act) {
+#pragma unroll
+        for (int u = 0; u < Q; ++u) v[u] = buf[t * QP + u];
+        codelet<-1, Q>(v);
+    }
+    __syncthreads();
+    if (t < P && act) {
+#pragma unroll
+        for (int n2 = 0; n2 < Q; ++n2) {
+            const int n = t + P * n2;
+            if (n < kout || N - n < kout) buf[n] = v[n2];
+        }
+    }
+    __syncthreads();
+    if (act) split_lines<N>(buf, item.out + l1 * kout, item.out + (l1 + 1) * kout, has2, kout, t);
+}
+
+// z-pass, inverse (C2R), the same results as k_inv_z.  The real lines go through shared memory so that the CTA's 2G lines,
+// one contiguous block, are written in 16-byte pieces (4-byte stores of P consecutive numbers straight from the registers
+// took 1.54 ms for 30 maps of 288^3 cells).  With absmax, absmax[item] takes the largest magnitude written (bit pattern),
+// which the triplet contraction scales by.
+template <int N>
+__global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineThreads, Geo<N>::TG))
+    k_inv_z(ZInvBatch batch, long nlines, float scale, const float* __restrict__ mulout, uint32_t* __restrict__ absmax) {
+    extern __shared__ __align__(16) float2 f2_smem[];
+    using E = Geo<N>;
+    constexpr int P = E::P, Q = E::Q, QP = E::QP;
+    const ZInvItem& item = batch.it[blockIdx.y];
+    const int kin = item.kin;
+    const int g = threadIdx.x / E::TG, t = threadIdx.x - g * E::TG;
+    float2* buf = f2_smem + g * E::GS;
+    const long l0 = 2 * (long)blockIdx.x * E::G, l1 = l0 + 2 * g;
+    const bool act = l1 < nlines, has2 = l1 + 1 < nlines;
+    const float2* __restrict__ in = static_cast<const float2*>(item.in) + l1 * kin;
+    float2 v[E::TG];
+    if (t < Q && act) {
+        load_hermitian<N>(v, in, in + kin, has2, kin, t);
+        stage1<+1, P, Q>(v, t);
+#pragma unroll
+        for (int n1 = 0; n1 < P; ++n1) buf[n1 * QP + t] = v[n1];
+    }
+    __syncthreads();
+    if (t < P && act) {
+#pragma unroll
+        for (int u = 0; u < Q; ++u) v[u] = buf[t * QP + u];
+        codelet<+1, Q>(v);
+    }
+    __syncthreads();
+    if (t < P && act) {
+        float* re = reinterpret_cast<float*>(f2_smem) + g * E::OS + t;
+#pragma unroll
+        for (int n2 = 0; n2 < Q; ++n2) {
+            re[P * n2] = v[n2].x * scale;
+            re[P * n2 + N] = v[n2].y * scale;
+        }
+    }
+    __syncthreads();
+    // lines l0 .. of the CTA, V numbers a store
+    constexpr int V = E::V, NV = N / V;
+    using VT = typename std::conditional<V == 4, float4, float2>::type;
+    const int nl = (int)min((long)2 * E::G, nlines - l0);
+    VT* __restrict__ out = reinterpret_cast<VT*>(static_cast<float*>(item.out) + l0 * N);
+    uint32_t top = 0u;
+    for (int q = threadIdx.x; q < nl * NV; q += E::kLineThreads) {
+        const int l = q / NV, e = q - l * NV;
+        VT a = *reinterpret_cast<const VT*>(reinterpret_cast<const float*>(f2_smem) + (l >> 1) * E::OS + (l & 1) * N + V * e);
+        float* p = reinterpret_cast<float*>(&a);
+#pragma unroll
+        for (int i = 0; i < V; ++i) {
+            if (mulout) p[i] *= mulout[l0 * N + (long)q * V + i];
+            top = max(top, __float_as_uint(p[i]) & 0x7fffffffu);
+        }
+        out[q] = a;
+    }
+    if (absmax) {
+        const int lanes = E::kLineThreads - (int)(threadIdx.x & ~31u);     // of this warp (the last one may be partial)
+        top = __reduce_max_sync(lanes >= 32 ? 0xffffffffu : (1u << lanes) - 1u, top);
+        // (a look first: of the hundreds of thousands of warps few still raise the maximum)
+        if ((threadIdx.x & 31) == 0 && top > __ldcg(absmax + blockIdx.y)) atomicMax(absmax + blockIdx.y, top);
+    }
+}
+
+// C2R z-pass, product with the real map s (same grid, lines l1, l1 + 1) and R2C z-pass in one kernel: the real lines
+// never leave the registers.  The inverse transform leaves n = n1 + P n2 in thread n1, which is what the forward one with
+// P and Q exchanged starts from.
+template <int N>
+__global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineThreads, Geo<N>::TG))
+    k_mask_z(ZMaskBatch batch, long nlines, const float* __restrict__ s, int kout) {
+    extern __shared__ __align__(16) float2 f2_smem[];
+    using E = Geo<N>;
+    constexpr int P = E::P, Q = E::Q, QP = E::QP, PP = E::PP;
+    const ZMaskItem& item = batch.it[blockIdx.y];
+    const int kin = item.kin;
+    const int g = threadIdx.x / E::TG, t = threadIdx.x - g * E::TG;
+    float2* buf = f2_smem + g * E::GS;
+    const long l1 = 2 * ((long)blockIdx.x * E::G + g);
+    const bool act = l1 < nlines, has2 = l1 + 1 < nlines;
+    const float2* __restrict__ in = item.in + l1 * kin;
+    float2 v[E::TG];
+    if (t < Q && act) {
+        load_hermitian<N>(v, in, in + kin, has2, kin, t);
+        stage1<+1, P, Q>(v, t);
+#pragma unroll
+        for (int n1 = 0; n1 < P; ++n1) buf[n1 * QP + t] = v[n1];
+    }
+    __syncthreads();
+    if (t < P && act) {
+#pragma unroll
+        for (int u = 0; u < Q; ++u) v[u] = buf[t * QP + u];
+        codelet<+1, Q>(v);
+        const float* __restrict__ sm = s + l1 * N + t;
+#pragma unroll
+        for (int n2 = 0; n2 < Q; ++n2) {
+            v[n2].x *= sm[P * n2];
+            v[n2].y = has2 ? v[n2].y * sm[P * n2 + N] : 0.f;
+        }
+        stage1<-1, Q, P>(v, t);
+    }
+    __syncthreads();                                  // every row of the first exchange has been read
+    if (t < P && act) {
+#pragma unroll
+        for (int n1 = 0; n1 < Q; ++n1) buf[n1 * PP + t] = v[n1];
+    }
+    __syncthreads();
+    if (t < Q && act) {
+#pragma unroll
+        for (int u = 0; u < P; ++u) v[u] = buf[t * PP + u];
+        codelet<-1, P>(v);
+    }
+    __syncthreads();
+    if (t < Q && act) {
+#pragma unroll
+        for (int n2 = 0; n2 < P; ++n2) {
+            const int n = t + Q * n2;
+            if (n < kout || N - n < kout) buf[n] = v[n2];
+        }
+    }
+    __syncthreads();
+    if (act) split_lines<N>(buf, item.out + l1 * kout, item.out + (l1 + 1) * kout, has2, kout, t);
+}
+
+}  // namespace f2
+}  // namespace pb

@@ -1,0 +1,83 @@
+// Host interface of the two-stage FFT passes (fft2.cuh): the lengths, the batch items and the launchers.
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "common.cuh"
+
+namespace pb {
+struct ColBatch;
+struct XInvBatch;
+struct ZInvBatch;
+namespace f2 {
+
+// Stage-1 points P of a length N = P x Q (0: not a two-stage length).
+__host__ __device__ constexpr int stage_p(int n) {
+    switch (n) {
+        case 48: return 6;
+        case 54: return 6;
+        case 60: return 6;
+        case 64: return 8;
+        case 72: return 8;
+        case 80: return 8;
+        case 90: return 9;
+        case 96: return 8;
+        case 100: return 10;
+        case 108: return 9;
+        case 120: return 10;
+        case 128: return 8;
+        case 144: return 12;
+        case 150: return 10;
+        case 160: return 10;
+        case 180: return 12;
+        case 192: return 12;
+        case 200: return 10;
+        case 216: return 12;
+        case 240: return 15;
+        case 256: return 16;
+        case 270: return 15;
+        case 288: return 16;
+        case 300: return 15;
+        case 320: return 16;
+        case 324: return 18;
+        case 360: return 18;
+        case 384: return 16;
+        case 400: return 20;
+        case 432: return 18;
+        case 480: return 20;
+        case 512: return 16;
+        default: return 0;
+    }
+}
+inline bool has(int n) { return stage_p(n) != 0; }
+
+constexpr int kBatch = 64;   // items of one launch (kMaxItems)
+
+struct ZFwdItem {
+    const float *in, *m1, *m2;   // product on load (m1, m2 may be null)
+    const float *sub, *sub_m;    // subtracted product (then m2 is not used)
+    float2* out;                 // [nlines][kout]
+};
+struct ZFwdBatch {
+    ZFwdItem it[kBatch];
+};
+struct ZMaskItem {
+    const float2* in;            // [nlines][kin]
+    float2* out;                 // [nlines][kout]
+    int kin;
+};
+struct ZMaskBatch {
+    ZMaskItem it[kBatch];
+};
+
+// Launchers over nitem items; false when n is not a two-stage length (nothing is launched).
+bool col(int n, int dir, const ColBatch& b, int nitem, int max_cols, int max_outer, cudaStream_t st);
+bool xfilter(int n, const XInvBatch& b, int nitem, int max_cols, const float2* spec, AxisRange gx, AxisRange gy,
+             AxisRange gz, float scale, cudaStream_t st);
+bool fwd_z(int n, const ZFwdBatch& b, int nitem, long nlines, int kout, cudaStream_t st);
+bool inv_z(int n, const ZInvBatch& b, int nitem, long nlines, float scale, const float* mulout, uint32_t* absmax,
+           cudaStream_t st);
+bool mask_z(int n, const ZMaskBatch& b, int nitem, long nlines, const float* s, int kout, cudaStream_t st);
+
+}  // namespace f2
+}  // namespace pb

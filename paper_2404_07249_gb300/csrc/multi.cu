@@ -43,8 +43,8 @@ static int capture_field(polybin_ctx* c, const float* field, double* host_dst) {
     if ((rc = run_forward<T, float, float>(c, field, (const float*)nullptr, (const float*)nullptr, (C<T>*)w.t1, (C<T>*)w.t2,
                                            (C<T>*)w.box)))
         return rc;
-    if ((rc = run_shells<T>(c, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g, 0, c->cg))) return rc;
-    if ((rc = run_triplet_sums<T>(c, (const T*)w.g, c->d_S))) return rc;
+    if ((rc = run_shells<T>(c, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g, 0, c->cg, map_max(c, 0)))) return rc;
+    if ((rc = run_triplet_sums<T>(c, (const T*)w.g, c->d_S, map_max(c, 0)))) return rc;
     if ((rc = run_bk_normalise(c, c->d_S, c->d_B))) return rc;
     cudaError_t e = cudaMemcpyAsync(host_dst, c->d_B, sizeof(double) * nt, cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess) return fail_cuda(c, e, "capture copy", __FILE__, __LINE__);

@@ -89,10 +89,19 @@ template <typename T, typename TIN, typename TM>
 int run_forward(polybin_ctx*, const TIN*, const TM*, const TM*, C<T>*, C<T>*, C<T>*, const InvGrid& ig);
 // Shell maps of all bins on grid `ig` (the data grid ctx->fg or the contraction grid ctx->cg), normalised with the
 // 1/N of the data grid's inverse DFT, so that maps on either grid sample the same band-limited function.
-template <typename T> int run_shells(polybin_ctx*, const C<T>*, C<T>*, C<T>*, T*, int ell, const InvGrid& ig);
+// With absmax (FP32 only), absmax[b] takes the largest magnitude of map b as a bit pattern (kMaxItems entries).
+template <typename T>
+int run_shells(polybin_ctx*, const C<T>*, C<T>*, C<T>*, T*, int ell, const InvGrid& ig, uint32_t* absmax = nullptr);
 // The same with the weight Ybar_lm(k / |k|) of the local line of sight (m in [-ell, ell]; m = kLegendreM: L_ell(mu)).
 template <typename T>
-int run_shells_m(polybin_ctx*, const C<T>*, C<T>*, C<T>*, T*, int ell, int m, const InvGrid& ig);
+int run_shells_m(polybin_ctx*, const C<T>*, C<T>*, C<T>*, T*, int ell, int m, const InvGrid& ig,
+                 uint32_t* absmax = nullptr);
+// C2R z-pass of nitem items on the staged and the FP64 register-resident passes (no launch check).
+template <typename T>
+int launch_inv_z(polybin_ctx*, const ZInvBatch& b, int nitem, long nlines, T scale, const T* mulout, const FftPlan& plan,
+                 const C<T>* tw);
+// absmax[r] = largest magnitude (bit pattern) of map r of nmaps maps of ncell cells (ncell a multiple of 4).
+int run_absmax(polybin_ctx*, const float* maps, int nmaps, long ncell, uint32_t* absmax);
 template <typename T> int run_pkbin(polybin_ctx*, const C<T>*, std::vector<double>&);
 // Binned products of nx box spectra X + z x_stride with A (partials [nx][nb][nseg][nell]) and the sums over segments
 // out[nx][nell][nb] (counts given: P_ell normalised).
@@ -102,7 +111,10 @@ int launch_bin_sum(polybin_ctx*, const double* partial, int nx, const double* co
 // Contractions over `ncell` cells (maps of the data grid or of the contraction grid).
 template <typename T> int run_contract(polybin_ctx*, const T*, int, const T*, int, double*, size_t, double*, long ncell);
 // Contraction dispatch: the tensor-core kernel in POLYBIN_SPLIT_TF32X3 mode, the SIMT kernel otherwise.
-template <typename T> int run_contract_any(polybin_ctx*, const T*, int, const T*, int, double*, size_t, double*, long ncell);
+// gmax, hmax: the maps' largest magnitudes as run_shells leaves them, or null (the tensor-core kernel then finds them).
+template <typename T>
+int run_contract_any(polybin_ctx*, const T*, int, const T*, int, double*, size_t, double*, long ncell,
+                     const uint32_t* gmax = nullptr, const uint32_t* hmax = nullptr);
 template <typename T> int alloc_work(polybin_ctx*, Work&);
 // Data-grid intermediates of the inverse transforms (ctx->w.u1f, u2f), allocated on first use.
 template <typename T> int ensure_fine_inv(polybin_ctx*);
@@ -113,17 +125,21 @@ int ensure_triplets(polybin_ctx*);
 bool split_tc_available();
 int tf32_selfcheck(polybin_ctx*);
 bool tc_shape_ok(long ncell, const float* g, int ng, const float* h, int nh);
-int run_contract_tc(polybin_ctx*, const float*, int, const float*, int, double*, long ncell);
+int run_contract_tc(polybin_ctx*, const float*, int, const float*, int, double*, long ncell, const uint32_t* gmax,
+                    const uint32_t* hmax);
 int prepare_triplet_tc(polybin_ctx*);
-int run_triplet_sums_tc(polybin_ctx*, const float* g, double* d_S);
-int run_triplet_sums_ell_tc(polybin_ctx*, const float* g, const float* gl, double* d_S);
+int run_triplet_sums_tc(polybin_ctx*, const float* g, double* d_S, const uint32_t* gmax);
+int run_triplet_sums_ell_tc(polybin_ctx*, const float* g, const float* gl, double* d_S, const uint32_t* gmax,
+                            const uint32_t* glmax);
 int run_gram_tc(polybin_ctx*, const float* A, int nA, const float* B, int nB, long K, double scale, double* d_out);
 void destroy_tc(polybin_ctx*);
 // S'_abc of every closed triplet (device, triplet order) from the nb shell maps g on the contraction grid; the
 // data-grid sum is S_abc = cg_ratio S'_abc.
-template <typename T> int run_triplet_sums(polybin_ctx*, const T* g, double* d_S);
+template <typename T> int run_triplet_sums(polybin_ctx*, const T* g, double* d_S, const uint32_t* gmax = nullptr);
 // S^ell'_abc = sum_x g_a g_b g_{c,ell} (gl: the maps g_{c,ell} = IFT[Theta_c L_ell D]) on the contraction grid.
-template <typename T> int run_triplet_sums_ell(polybin_ctx*, const T* g, const T* gl, double* d_S);
+template <typename T>
+int run_triplet_sums_ell(polybin_ctx*, const T* g, const T* gl, double* d_S, const uint32_t* gmax = nullptr,
+                         const uint32_t* glmax = nullptr);
 // B_abc = fac scale S'_abc / T_abc on the device (FP64), scale = (V^2 / N^3) cg_ratio (fac = 2 ell + 1 for a
 // multipole).
 int run_bk_normalise(polybin_ctx*, const double* d_S, double* d_B, double fac = 1.0);
@@ -226,6 +242,9 @@ struct polybin_ctx {
     int tused = 0;        // slots recorded since the last read-back
     bool topen = false;   // a stage bracket is open (brackets do not nest)
 
+    // split mode: largest magnitudes of two sets of nb shell maps (bit patterns, [2][kMaxItems])
+    uint32_t* d_mapmax = nullptr;
+
     // observer of the local line of sight, box coordinates centred on the origin (Mpc/h)
     double observer[3] = {0.0, 0.0, 0.0};
     // the contraction kernel that ran last (polybin_contract_path values), -1 before the first contraction
@@ -244,6 +263,8 @@ struct polybin_ctx {
 };
 
 namespace pb {
+// The maxima of map set `set` (0: W.g, 1: the second set of a mixed sum); null outside the split mode.
+inline uint32_t* map_max(polybin_ctx* ctx, int set) { return ctx->d_mapmax ? ctx->d_mapmax + set * kMaxItems : nullptr; }
 enum Stage { kStageForward = 0, kStageShells = 1, kStageContract = 2, kStagePk = 3, kNumStages = 4 };
 // Adds the elapsed times of the recorded stage brackets to stage_ms / stage_calls (waits for their stop events).
 inline void harvest_stage_times(polybin_ctx* ctx) {

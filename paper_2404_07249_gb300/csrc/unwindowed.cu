@@ -17,8 +17,10 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
+#include "fft2.h"
 #include "polybin_internal.h"
 
 namespace pb {
@@ -492,11 +494,13 @@ int run_inverse_box(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* ou
         it.in = box; it.out = v1;
         it.in_os = 0; it.in_es = ncols; it.out_os = 0; it.out_es = ncols;
         it.ncols = ncols; it.nouter = 1; it.rng = ctx->gx;
-        PB_WITH_NT(N0, NT, {
-            e = cudaFuncSetAttribute((const void*)k_col<T, +1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return fail_cuda(ctx, e, "attr", __FILE__, __LINE__);
-            k_col<T, +1, NT><<<dim3((ncols + tk - 1) / tk, 1, 1), 256, sm, ctx->stream>>>(b, ctx->plan[0], tw0, tk);
-        })
+        if (!(sizeof(T) == 4 && f2::col(N0, +1, b, 1, ncols, 1, ctx->stream))) {
+            PB_WITH_NT(N0, NT, {
+                e = cudaFuncSetAttribute((const void*)k_col<T, +1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                if (e != cudaSuccess) return fail_cuda(ctx, e, "attr", __FILE__, __LINE__);
+                k_col<T, +1, NT><<<dim3((ncols + tk - 1) / tk, 1, 1), 256, sm, ctx->stream>>>(b, ctx->plan[0], tw0, tk);
+            })
+        }
         ctx->launches++;
     }
     {
@@ -507,34 +511,25 @@ int run_inverse_box(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* ou
         it.in = v1; it.out = v2;
         it.in_os = (long)By * Bz; it.in_es = Bz; it.out_os = (long)N1 * Bz; it.out_es = Bz;
         it.ncols = Bz; it.nouter = N0; it.rng = ctx->gy;
-        PB_WITH_NT(N1, NT, {
-            e = cudaFuncSetAttribute((const void*)k_col<T, +1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            if (e != cudaSuccess) return fail_cuda(ctx, e, "attr", __FILE__, __LINE__);
-            k_col<T, +1, NT><<<dim3((Bz + tk - 1) / tk, N0, 1), 256, sm, ctx->stream>>>(b, ctx->plan[1], tw1, tk);
-        })
+        if (!(sizeof(T) == 4 && f2::col(N1, +1, b, 1, Bz, N0, ctx->stream))) {
+            PB_WITH_NT(N1, NT, {
+                e = cudaFuncSetAttribute((const void*)k_col<T, +1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                if (e != cudaSuccess) return fail_cuda(ctx, e, "attr", __FILE__, __LINE__);
+                k_col<T, +1, NT><<<dim3((Bz + tk - 1) / tk, N0, 1), 256, sm, ctx->stream>>>(b, ctx->plan[1], tw1, tk);
+            })
+        }
         ctx->launches++;
     }
     {
-        const int lp = lines_per_cta_of<T>(N2);
-        const size_t sm = (2 * (size_t)N2 * (lp + 1) + N2) * sizeof(C<T>);
         ZInvBatch b;
         b.it[0].in = v2; b.it[0].out = out; b.it[0].kin = Bz;
         const long nlines = (long)N0 * N1;
-        if (N2 == 256) {
-            const int lpc = 16;
-            k_inv_z256<T><<<dim3((unsigned)(((nlines + 1) / 2 + lpc - 1) / lpc), 1, 1), 256, 0, ctx->stream>>>(
-                b, nlines, T(1.0 / (double)ctx->ncell), mulout, tw2, lpc);
-        } else if (N2 == 512) {
-            const int lpc = 16;
-            k_inv_z512<T><<<dim3((unsigned)(((nlines + 1) / 2 + lpc - 1) / lpc), 1, 1), 256, 0, ctx->stream>>>(
-                b, nlines, T(1.0 / (double)ctx->ncell), mulout, tw2, lpc);
-        } else {
-            PB_WITH_NT(N2, NT, {
-                e = cudaFuncSetAttribute((const void*)k_inv_z<T, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-                if (e != cudaSuccess) return fail_cuda(ctx, e, "attr", __FILE__, __LINE__);
-                k_inv_z<T, NT><<<dim3((unsigned)((nlines + 2 * lp - 1) / (2 * lp)), 1, 1), 256, sm, ctx->stream>>>(
-                    b, nlines, T(1.0 / (double)ctx->ncell), mulout, ctx->plan[2], tw2, lp);
-            })
+        bool done = false;
+        if constexpr (std::is_same<T, float>::value)
+            done = f2::inv_z(N2, b, 1, nlines, (float)(1.0 / (double)ctx->ncell), mulout, nullptr, ctx->stream);
+        if (!done) {
+            const int rc = launch_inv_z<T>(ctx, b, 1, nlines, T(1.0 / (double)ctx->ncell), mulout, ctx->plan[2], tw2);
+            if (rc) return rc;
         }
         ctx->launches++;
     }
@@ -1290,10 +1285,10 @@ static int bk_unwindowed_t(polybin_ctx* ctx, const float* d, const float* w, con
     const double rho = ctx->cg_ratio;
     const long cn = ctx->cg.ncell;
     if ((rc = run_forward<T, float, float>(ctx, d, w, (const float*)nullptr, (C<T>*)W.t1, (C<T>*)W.t2, (C<T>*)W.box))) return rc;
-    if ((rc = run_shells<T>(ctx, (const C<T>*)W.box, (C<T>*)W.u1, (C<T>*)W.u2, (T*)W.g, 0, ctx->cg))) return rc;
+    if ((rc = run_shells<T>(ctx, (const C<T>*)W.box, (C<T>*)W.u1, (C<T>*)W.u2, (T*)W.g, 0, ctx->cg, map_max(ctx, 0)))) return rc;
     std::vector<double> S(std::max(nt, 1), 0.0), lin(nt, 0.0), Mv((size_t)np * nb);
     if (nt > 0) {
-        if ((rc = run_triplet_sums<T>(ctx, (const T*)W.g, ctx->d_S))) return rc;
+        if ((rc = run_triplet_sums<T>(ctx, (const T*)W.g, ctx->d_S, map_max(ctx, 0)))) return rc;
         PB_CUDA_OK(cudaMemcpyAsync(S.data(), ctx->d_S, sizeof(double) * nt, cudaMemcpyDeviceToHost, ctx->stream));
         PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
         for (int t = 0; t < nt; ++t) S[t] *= rho;
@@ -1301,9 +1296,10 @@ static int bk_unwindowed_t(polybin_ctx* ctx, const float* d, const float* w, con
     for (int i = 0; i < n_mocks; ++i) {
         const float* mock = mocks + (size_t)i * N;
         if ((rc = run_forward<T, float, float>(ctx, mock, w, (const float*)nullptr, (C<T>*)W.t1, (C<T>*)W.t2, (C<T>*)W.box))) return rc;
-        if ((rc = run_shells<T>(ctx, (const C<T>*)W.box, (C<T>*)W.u1, (C<T>*)W.u2, (T*)u->g2, 0, ctx->cg))) return rc;
+        if ((rc = run_shells<T>(ctx, (const C<T>*)W.box, (C<T>*)W.u1, (C<T>*)W.u2, (T*)u->g2, 0, ctx->cg, map_max(ctx, 1)))) return rc;
         // M[(j<=k) over v][i over u] = sum_x g_j[v] g_k[v] g_i[u]
-        if ((rc = run_contract_any<T>(ctx, (const T*)u->g2, nb, (const T*)W.g, nb, W.partial, W.partial_cap, W.mout, cn)))
+        if ((rc = run_contract_any<T>(ctx, (const T*)u->g2, nb, (const T*)W.g, nb, W.partial, W.partial_cap, W.mout, cn,
+                                      map_max(ctx, 1), map_max(ctx, 0))))
             return rc;
         PB_CUDA_OK(cudaMemcpyAsync(Mv.data(), W.mout, sizeof(double) * Mv.size(), cudaMemcpyDeviceToHost, ctx->stream));
         PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
@@ -1359,11 +1355,11 @@ static int bk_multipoles_local_t(polybin_ctx* ctx, const float* delta, int batch
                                                (C<T>*)w.t2, (C<T>*)w.box)))
             return rc;
         if (nt == 0) continue;
-        if ((rc = run_shells<T>(ctx, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g, 0, ctx->cg))) return rc;
+        if ((rc = run_shells<T>(ctx, (const C<T>*)w.box, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g, 0, ctx->cg, map_max(ctx, 0)))) return rc;
         for (int il = 0; il < nl; ++il) {
             const int ell = 2 * il;
             if (ell == 0) {
-                if ((rc = run_triplet_sums<T>(ctx, (const T*)w.g, ctx->d_S))) return rc;
+                if ((rc = run_triplet_sums<T>(ctx, (const T*)w.g, ctx->d_S, map_max(ctx, 0)))) return rc;
             } else {
                 for (int m = -ell; m <= ell; ++m) {
                     uw::k_mul_ylm<T, float, float><<<grid1d(N), 256, 0, ctx->stream>>>(
@@ -1377,8 +1373,8 @@ static int bk_multipoles_local_t(polybin_ctx* ctx, const float* delta, int batch
                     ctx->launches++;
                 }
                 PB_CUDA_OK(cudaGetLastError());
-                if ((rc = run_shells<T>(ctx, H, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g2, 0, ctx->cg))) return rc;
-                if ((rc = run_triplet_sums_ell<T>(ctx, (const T*)w.g, (const T*)w.g2, ctx->d_S))) return rc;
+                if ((rc = run_shells<T>(ctx, H, (C<T>*)w.u1, (C<T>*)w.u2, (T*)w.g2, 0, ctx->cg, map_max(ctx, 1)))) return rc;
+                if ((rc = run_triplet_sums_ell<T>(ctx, (const T*)w.g, (const T*)w.g2, ctx->d_S, map_max(ctx, 0), map_max(ctx, 1)))) return rc;
             }
             if ((rc = run_bk_normalise(ctx, ctx->d_S, ctx->d_B, 2.0 * ell + 1.0))) return rc;
             PB_CUDA_OK(cudaMemcpyAsync(bk_out + ((size_t)f * nl + il) * nt, ctx->d_B, sizeof(double) * nt,
