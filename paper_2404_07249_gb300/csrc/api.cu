@@ -88,10 +88,10 @@ template <> const double2* twiddles<double>(polybin_ctx* ctx, int axis) { return
 // a1: pruned forward transform of one real field on grid ig (optionally times m1 * m2) into the box of the wave
 // numbers |n_i| <= m (the same box on every grid with more than 2m points per axis).
 template <typename T, typename TIN, typename TM>
-int run_forward(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T>* t1, C<T>* t2, C<T>* box,
-                const InvGrid& ig) {
+int run_forward_box(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T>* t1, C<T>* t2, C<T>* box,
+                    const InvGrid& ig, const Box3& keep) {
     const int N0 = ig.N[0], N1 = ig.N[1], N2 = ig.N[2];
-    const int Bz = ctx->gz.cnt, By = ctx->gy.cnt;
+    const int Bz = keep.z.cnt, By = keep.y.cnt;
     const long nlines = (long)N0 * N1;
     auto tw = [&](int a) { return (const C<T>*)(sizeof(T) == 4 ? ig.tw_f[a] : ig.tw_d[a]); };
     int rc = POLYBIN_OK;
@@ -123,7 +123,7 @@ int run_forward(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T
         ColItem& it = b.it[0];
         it.in = t1; it.out = t2;
         it.in_os = (long)N1 * Bz; it.in_es = Bz; it.out_os = (long)By * Bz; it.out_es = Bz;
-        it.ncols = Bz; it.nouter = N0; it.rng = ctx->gy;
+        it.ncols = Bz; it.nouter = N0; it.rng = keep.y;
         if (!(sizeof(T) == 4 && f2::col(N1, -1, b, 1, Bz, N0, ctx->stream))) {
             dim3 grid((Bz + TK - 1) / TK, N0, 1);
             PB_WITH_NT(N1, NT, {
@@ -141,7 +141,7 @@ int run_forward(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T
         const int ncols = By * Bz;
         it.in = t2; it.out = box;
         it.in_os = 0; it.in_es = ncols; it.out_os = 0; it.out_es = ncols;
-        it.ncols = ncols; it.nouter = 1; it.rng = ctx->gx;
+        it.ncols = ncols; it.nouter = 1; it.rng = keep.x;
         if (!(sizeof(T) == 4 && f2::col(N0, -1, b, 1, ncols, 1, ctx->stream))) {
             dim3 grid((ncols + TK - 1) / TK, 1, 1);
             PB_WITH_NT(N0, NT, {
@@ -152,6 +152,12 @@ int run_forward(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T
         if ((rc = launch_check(ctx, "k_col fwd x"))) return rc;
     }
     return POLYBIN_OK;
+}
+
+template <typename T, typename TIN, typename TM>
+int run_forward(polybin_ctx* ctx, const TIN* in, const TM* m1, const TM* m2, C<T>* t1, C<T>* t2, C<T>* box,
+                const InvGrid& ig) {
+    return run_forward_box<T, TIN, TM>(ctx, in, m1, m2, t1, t2, box, ig, Box3{ctx->gx, ctx->gy, ctx->gz});
 }
 
 template <typename T, typename TIN, typename TM>
@@ -354,6 +360,10 @@ template int run_forward<double, double, double>(polybin_ctx*, const double*, co
 template int run_forward<double, float, float>(polybin_ctx*, const float*, const float*, const float*, double2*, double2*, double2*);
 template int run_forward<double, double, double>(polybin_ctx*, const double*, const double*, const double*, double2*, double2*, double2*);
 template int run_forward<double, double, float>(polybin_ctx*, const double*, const float*, const float*, double2*, double2*, double2*);
+template int run_forward_box<float, float, float>(polybin_ctx*, const float*, const float*, const float*, float2*, float2*,
+                                                  float2*, const InvGrid&, const Box3&);
+template int run_forward_box<double, float, float>(polybin_ctx*, const float*, const float*, const float*, double2*, double2*,
+                                                   double2*, const InvGrid&, const Box3&);
 template int run_pkbin<float>(polybin_ctx*, const float2*, std::vector<double>&);
 template int run_pkbin<double>(polybin_ctx*, const double2*, std::vector<double>&);
 template int run_pkbin_dev<float>(polybin_ctx*, const float2*);
@@ -550,6 +560,29 @@ static int upload_twiddles(polybin_ctx* ctx) {
             ctx->cg.tw_d[a] = ctx->d_ctw[2 * a + 1];
         }
     }
+    return POLYBIN_OK;
+}
+
+int plan_product_grid(polybin_ctx* ctx, InvGrid& pg, Box3& keep, void* tw[6]) {
+    // largest wave number of the box on each axis
+    const int m[3] = {std::max(-ctx->gx.lo, ctx->gx.lo + ctx->gx.cnt - 1), std::max(-ctx->gy.lo, ctx->gy.lo + ctx->gy.cnt - 1),
+                      ctx->gz.cnt - 1};
+    AxisRange* k[3] = {&keep.x, &keep.y, &keep.z};
+    for (int a = 0; a < 3; ++a) {
+        const int n = ctx->N[a];
+        int L = fft_len_at_least(4 * m[a] + 1);
+        // FP32: a two-stage length where one is not much longer
+        for (int l = L; l > 0 && l <= n && l <= L + L / 8; l += 2)
+            if (f2::has(l)) { L = l; break; }
+        pg.N[a] = L > 0 && L < n ? L : n;
+        if (pg.N[a] < n) *k[a] = a < 2 ? axis_box(2 * m[a], n) : z_box(2 * m[a], n);
+        else *k[a] = a < 2 ? AxisRange{-n / 2, n} : AxisRange{0, n / 2 + 1};
+        const int rc = make_twiddles(ctx, pg.N[a], &tw[2 * a], &tw[2 * a + 1]);
+        if (rc) return rc;
+        pg.tw_f[a] = tw[2 * a];
+        pg.tw_d[a] = tw[2 * a + 1];
+    }
+    plan_inv_grid(ctx, pg);
     return POLYBIN_OK;
 }
 

@@ -162,6 +162,7 @@ void destroy_extras(polybin_ctx* ctx) {
     destroy_unwindowed(ctx);
     destroy_optimal(ctx);
     destroy_multi(ctx);
+    destroy_maskop(ctx);
     destroy_tc(ctx);
     if (ctx->d_err) cudaFree(ctx->d_err);
     ctx->d_err = nullptr;

@@ -9,6 +9,7 @@ namespace f2 {
     bool col_##G(int, int, const ColBatch&, int, int, int, cudaStream_t);                                              \
     bool xfilter_##G(int, const XInvBatch&, int, int, const float2*, AxisRange, AxisRange, AxisRange, float,           \
                      cudaStream_t);                                                                                    \
+    bool xq_##G(int, const XqBatch&, int, int, const float2*, AxisRange, AxisRange, AxisRange, cudaStream_t);          \
     bool fwd_z_##G(int, const ZFwdBatch&, int, long, int, cudaStream_t);                                               \
     bool inv_z_##G(int, const ZInvBatch&, int, long, float, const float*, uint32_t*, cudaStream_t);                    \
     bool mask_z_##G(int, const ZMaskBatch&, int, long, const float*, int, cudaStream_t);
@@ -27,6 +28,11 @@ bool xfilter(int n, const XInvBatch& b, int nitem, int mc, const float2* spec, A
              float scale, cudaStream_t st) {
     return xfilter_a(n, b, nitem, mc, spec, gx, gy, gz, scale, st) || xfilter_b(n, b, nitem, mc, spec, gx, gy, gz, scale, st) ||
            xfilter_c(n, b, nitem, mc, spec, gx, gy, gz, scale, st) || xfilter_d(n, b, nitem, mc, spec, gx, gy, gz, scale, st);
+}
+bool xq(int n, const XqBatch& b, int nitem, int mc, const float2* pairs, AxisRange gx, AxisRange gy, AxisRange gz,
+        cudaStream_t st) {
+    return xq_a(n, b, nitem, mc, pairs, gx, gy, gz, st) || xq_b(n, b, nitem, mc, pairs, gx, gy, gz, st) ||
+           xq_c(n, b, nitem, mc, pairs, gx, gy, gz, st) || xq_d(n, b, nitem, mc, pairs, gx, gy, gz, st);
 }
 bool fwd_z(int n, const ZFwdBatch& b, int nitem, long nl, int kout, cudaStream_t st) {
     return fwd_z_a(n, b, nitem, nl, kout, st) || fwd_z_b(n, b, nitem, nl, kout, st) || fwd_z_c(n, b, nitem, nl, kout, st) ||

@@ -308,6 +308,47 @@ __global__ void __launch_bounds__(Geo<N>::kColThreads, min_ctas(Geo<N>::kColThre
         });
 }
 
+// First inverse pass of a triplet's Q-derivative spectrum, combined from the pair spectra on load.
+template <int N>
+__global__ void __launch_bounds__(Geo<N>::kColThreads, min_ctas(Geo<N>::kColThreads, Geo<N>::TG))
+    k_xq(XqBatch batch, const float2* __restrict__ pairs, AxisRange gx, AxisRange gy, AxisRange gz) {
+    extern __shared__ __align__(16) float2 f2_smem[];
+    constexpr int TC = Geo<N>::TC;
+    const XqItem& item = batch.it[blockIdx.y];
+    const int ncols = item.ry.cnt * item.rz.cnt;
+    const int c0 = blockIdx.x * TC;
+    if (c0 >= ncols) return;                          // uniform over the CTA
+    const int t = threadIdx.x / TC, c = threadIdx.x - t * TC;
+    const int cc = c0 + c;
+    const bool act = cc < ncols;
+    const int fy = act ? item.ry.lo + cc / item.rz.cnt : 0;
+    const int fz = act ? item.rz.lo + cc % item.rz.cnt : 0;
+    const int syz = fy * fy + fz * fz;
+    const float2* __restrict__ p = pairs + (fy - gy.lo) * gz.cnt + (fz - gz.lo);
+    const int xs = gy.cnt * gz.cnt;
+    float2* __restrict__ out = item.out + cc;
+    col_fft<+1, N>(
+        f2_smem, t, c,
+        [&](int k) {
+            const int fx = k < N / 2 ? k : k - N;
+            const int i = fx - item.rx.lo;
+            float2 v = make_float2(0.f, 0.f);
+            if (act && i >= 0 && i < item.rx.cnt) {
+                const int s = fx * fx + syz;
+                const long o = (long)(fx - gx.lo) * xs;
+                if (s >= item.clo && s <= item.chi) v = add<float>(v, p[item.pab + o]);
+                if (s >= item.alo && s <= item.ahi) v = add<float>(v, p[item.pbc + o]);
+                if (s >= item.blo && s <= item.bhi) v = add<float>(v, p[item.pac + o]);
+                v.x *= item.fac;
+                v.y *= item.fac;
+            }
+            return v;
+        },
+        [&](int n, float2 v) {
+            if (act) out[(long)n * ncols] = v;
+        });
+}
+
 // ------------------------------------------------------------------------------------------------ lines
 
 // Stage-1 input of thread t of an inverse transform: points k = t + Q j of the packed Hermitian pair Z = X1 + i X2

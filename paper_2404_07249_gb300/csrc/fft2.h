@@ -69,6 +69,18 @@ struct ZMaskItem {
 struct ZMaskBatch {
     ZMaskItem it[kBatch];
 };
+// Q-derivative spectrum of a triplet (a, b, c) from pair spectra P (box layout): fac [Theta_c P_ab + Theta_a P_bc +
+// Theta_b P_ac], each Theta the bin's range of integer |n|^2.
+struct XqItem {
+    float2* out;                 // [N][ry.cnt * rz.cnt]
+    AxisRange rx, ry, rz;        // box of the modes of the three bins
+    long pab, pbc, pac;          // offsets of the pair spectra
+    int alo, ahi, blo, bhi, clo, chi;
+    float fac;
+};
+struct XqBatch {
+    XqItem it[kBatch];
+};
 
 // Launchers over nitem items; false when n is not a two-stage length (nothing is launched).
 bool col(int n, int dir, const ColBatch& b, int nitem, int max_cols, int max_outer, cudaStream_t st);
@@ -78,6 +90,10 @@ bool fwd_z(int n, const ZFwdBatch& b, int nitem, long nlines, int kout, cudaStre
 bool inv_z(int n, const ZInvBatch& b, int nitem, long nlines, float scale, const float* mulout, uint32_t* absmax,
            cudaStream_t st);
 bool mask_z(int n, const ZMaskBatch& b, int nitem, long nlines, const float* s, int kout, cudaStream_t st);
+
+// First inverse pass of the Q-derivative spectra of nitem triplets.
+bool xq(int n, const XqBatch& b, int nitem, int max_cols, const float2* pairs, AxisRange gx, AxisRange gy, AxisRange gz,
+        cudaStream_t st);
 
 }  // namespace f2
 }  // namespace pb

@@ -28,6 +28,11 @@ template <int N> struct Run {
         k_xfilter<N><<<dim3((max_cols + E::TC - 1) / E::TC, nitem), E::kColThreads, E::kColSmem, st>>>(b, spec, gx, gy, gz,
                                                                                                      scale);
     }
+    static void xq(const XqBatch& b, int nitem, int max_cols, const float2* pairs, AxisRange gx, AxisRange gy, AxisRange gz,
+                   cudaStream_t st) {
+        allow_smem(k_xq<N>, E::kColSmem);
+        k_xq<N><<<dim3((max_cols + E::TC - 1) / E::TC, nitem), E::kColThreads, E::kColSmem, st>>>(b, pairs, gx, gy, gz);
+    }
     static dim3 line_grid(long nlines, int nitem) {
         return dim3((unsigned)(((nlines + 1) / 2 + E::G - 1) / E::G), nitem);
     }
@@ -59,6 +64,11 @@ template <int N> struct Run {
     bool xfilter_##G(int n, const XInvBatch& b, int nitem, int mc, const float2* spec, AxisRange gx, AxisRange gy,     \
                      AxisRange gz, float scale, cudaStream_t st) {                                                     \
         switch (n) { LENGTHS(xfilter(b, nitem, mc, spec, gx, gy, gz, scale, st)) }                                     \
+        return false;                                                                                                  \
+    }                                                                                                                  \
+    bool xq_##G(int n, const XqBatch& b, int nitem, int mc, const float2* pairs, AxisRange gx, AxisRange gy,           \
+                AxisRange gz, cudaStream_t st) {                                                                       \
+        switch (n) { LENGTHS(xq(b, nitem, mc, pairs, gx, gy, gz, st)) }                                                \
         return false;                                                                                                  \
     }                                                                                                                  \
     bool fwd_z_##G(int n, const ZFwdBatch& b, int nitem, long nl, int kout, cudaStream_t st) {                         \

@@ -35,6 +35,11 @@ struct InvGrid {
     long u1_total = 0, u2_total = 0;
 };
 
+// A box of wave numbers.
+struct Box3 {
+    AxisRange x, y, z;
+};
+
 // Device workspace of one compute precision.
 struct Work {
     size_t elem = 0;
@@ -87,6 +92,13 @@ int run_forward(polybin_ctx*, const TIN*, const TM*, const TM*, C<T>*, C<T>*, C<
 // The same on grid ig (the data grid ctx->fg or the contraction grid ctx->cg; intermediates sized for it).
 template <typename T, typename TIN, typename TM>
 int run_forward(polybin_ctx*, const TIN*, const TM*, const TM*, C<T>*, C<T>*, C<T>*, const InvGrid& ig);
+// The same into the box `keep` of its own.
+template <typename T, typename TIN, typename TM>
+int run_forward_box(polybin_ctx*, const TIN*, const TM*, const TM*, C<T>*, C<T>*, C<T>*, const InvGrid& ig, const Box3& keep);
+// The product grid of the masked operator FT[s IFT[.]] on the box |n_i| <= m: the smallest grid with more than 4m points
+// an axis (the data grid's length where that has no more), and the wave numbers of s that reach the box, |n_i| <= 2m
+// (all of them on an axis that keeps its length).  tw: six twiddle tables owned by the caller.
+int plan_product_grid(polybin_ctx*, InvGrid& pg, Box3& keep, void* tw[6]);
 // Shell maps of all bins on grid `ig` (the data grid ctx->fg or the contraction grid ctx->cg), normalised with the
 // 1/N of the data grid's inverse DFT, so that maps on either grid sample the same band-limited function.
 // With absmax (FP32 only), absmax[b] takes the largest magnitude of map b as a bit pattern (kMaxItems entries).
@@ -148,6 +160,22 @@ int run_pk_normalise(polybin_ctx*, double* d_P);
 // Inverse transform of a box spectrum (the box of wave numbers |n_i| <= m) to a real map on the data grid with the
 // 1/N of the inverse DFT and an optional pointwise multiplier on output; v1 [N0][By][Bz], v2 [N0][N1][Bz].
 template <typename T> int run_inverse_box(polybin_ctx*, const C<T>* box, C<T>* v1, C<T>* v2, T* out, const T* mulout);
+// The same from a box of its own to grid ig, times scale.
+template <typename T>
+int run_inverse_from(polybin_ctx*, const C<T>* box, C<T>* v1, C<T>* v2, T* out, const T* mulout, const InvGrid& ig,
+                     const Box3& keep, double scale);
+// Masked operator (maskop.cu): X -> FT[s IFT[X]] on the box with s = w n, evaluated on the product grid.
+// mask_setup makes s of the given maps; mask_map / mask_grid hand it out; mask_fast: the batched FP32 passes apply.
+template <typename T> int mask_setup(polybin_ctx*, const float* n, const float* w);
+const InvGrid& mask_grid(const polybin_ctx*);
+const void* mask_map(const polybin_ctx*);
+bool mask_fast(const polybin_ctx*);
+int mask_chunk(const polybin_ctx*);              // items of one batch
+// boxes [cnt][box] of s IFT[Theta_b L_ell spec], bins b0 .. b0 + cnt - 1 (cnt <= mask_chunk)
+int mask_shells(polybin_ctx*, const float2* spec, int ell, int b0, int cnt, float2** boxes);
+// the same for the Q-derivative spectra of triplets t0 .. t0 + cnt - 1 combined from the pair spectra
+int mask_triplets(polybin_ctx*, const float2* pairs, int t0, int cnt, float2** boxes);
+void destroy_maskop(polybin_ctx*);
 // Optimal weighting (optimal.cu): out = post (/ n_w) G[Phi pre v (/ n_w)] by preconditioned conjugate gradients, with
 // G the inverse of Phi (IFT[P FT[.]] + n2_w / n_w^2) Phi on the cells with n_w > 0.  pre = null, pre_div = 1 gives
 // S^-1 v; post_div = 1 gives S^-T v; pre = n gives S^-1 P v; post = n with post_div = 1 gives P^T S^-T v.
@@ -260,6 +288,7 @@ struct polybin_ctx {
     // extension slots (unwindowed estimators; optimal weighting)
     void* ext = nullptr;
     void* opt = nullptr;
+    void* maskop = nullptr;
 };
 
 namespace pb {

@@ -72,13 +72,12 @@ __global__ void k_draw(T* __restrict__ out, long N, unsigned long long seed, uin
     }
 }
 
-// Q-derivative spectrum of one triplet (a, b, c) from the pair spectra of two fields (eq. Q-bis-global):
-//   out(k) = fac [ Theta_c (P1_ab - P2_ab) + Theta_a (P1_bc - P2_bc) + Theta_b (P1_ac - P2_ac) ](k),
+// Q-derivative spectrum of one triplet (a, b, c) from the pair spectra (eq. Q-bis-global):
+//   out(k) = fac [ Theta_c P_ab + Theta_a P_bc + Theta_b P_ac ](k),
 // fac = 2 / Delta_abc, over every entry of the box (zero outside bins a, b, c).
 template <typename T>
-__global__ void k_qcomb(const C<T>* __restrict__ P1, const C<T>* __restrict__ P2, long pab, long pbc, long pac,
-                        int a, int b, int c, T fac, AxisRange gx, AxisRange gy, AxisRange gz,
-                        const int16_t* __restrict__ lut, int smax, C<T>* __restrict__ out) {
+__global__ void k_qcomb(const C<T>* __restrict__ P, long pab, long pbc, long pac, int a, int b, int c, T fac, AxisRange gx,
+                        AxisRange gy, AxisRange gz, const int16_t* __restrict__ lut, int smax, C<T>* __restrict__ out) {
     const long nbox = (long)gx.cnt * gy.cnt * gz.cnt;
     for (long o = (long)blockIdx.x * blockDim.x + threadIdx.x; o < nbox; o += (long)gridDim.x * blockDim.x) {
         const int iz = (int)(o % gz.cnt);
@@ -87,21 +86,55 @@ __global__ void k_qcomb(const C<T>* __restrict__ P1, const C<T>* __restrict__ P2
         const int fx = gx.lo + ix, fy = gy.lo + iy, fz = gz.lo + iz;
         const int s = fx * fx + fy * fy + fz * fz;
         const int bin = (s <= smax) ? lut[s] : -1;
-        T re = T(0), im = T(0);
+        C<T> v = mk<T>(T(0), T(0));
         if (bin >= 0) {
-            if (bin == c) { const C<T> u = P1[pab + o], v = P2[pab + o]; re += u.x - v.x; im += u.y - v.y; }
-            if (bin == a) { const C<T> u = P1[pbc + o], v = P2[pbc + o]; re += u.x - v.x; im += u.y - v.y; }
-            if (bin == b) { const C<T> u = P1[pac + o], v = P2[pac + o]; re += u.x - v.x; im += u.y - v.y; }
+            if (bin == c) v = add<T>(v, P[pab + o]);
+            if (bin == a) v = add<T>(v, P[pbc + o]);
+            if (bin == b) v = add<T>(v, P[pac + o]);
         }
-        out[o] = mk<T>(fac * re, fac * im);
+        out[o] = mk<T>(fac * v.x, fac * v.y);
     }
 }
 
-// Compact copy of the binned modes of a box spectrum: out[m] = box[offs[m]] (times wm[m] when wm is not NULL: the
-// half-spectrum weight, 1 or 2, exact in any precision).
+// The same on the compact binned modes (row `blockIdx.y` of the batch): mode m belongs to bin a when it lies in the bin's
+// range of the mode list.  Every mode of the row is written.
+struct QRow {
+    void* out;                    // C<T>* [M]
+    long pab, pbc, pac;
+    int a0, a1, b0, b1, c0, c1;
+    double fac;
+};
+struct QRows {
+    QRow it[kMaxItems];
+};
 template <typename T>
-__global__ void k_gather(const C<T>* __restrict__ box, const int* __restrict__ offs, long M, C<T>* __restrict__ out,
-                         const double* __restrict__ wm = nullptr) {
+__global__ void __launch_bounds__(256) k_qrows(QRows rows, const C<T>* __restrict__ P, const int* __restrict__ offs, int M) {
+    const QRow& q = rows.it[blockIdx.y];
+    const int m = blockIdx.x * 256 + threadIdx.x;
+    if (m >= M) return;
+    const long o = offs[m];
+    C<T> v = mk<T>(T(0), T(0));
+    if (m >= q.c0 && m < q.c1) v = add<T>(v, P[q.pab + o]);
+    if (m >= q.a0 && m < q.a1) v = add<T>(v, P[q.pbc + o]);
+    if (m >= q.b0 && m < q.b1) v = add<T>(v, P[q.pac + o]);
+    const T fac = T(q.fac);
+    static_cast<C<T>*>(q.out)[m] = mk<T>(fac * v.x, fac * v.y);
+}
+
+// out -= v over a box.
+template <typename T>
+__global__ void k_box_sub(C<T>* __restrict__ out, const C<T>* __restrict__ v, long n) {
+    for (long o = (long)blockIdx.x * blockDim.x + threadIdx.x; o < n; o += (long)gridDim.x * blockDim.x)
+        out[o] = sub<T>(out[o], v[o]);
+}
+
+// Compact copy of the binned modes of box spectra: out[y][m] = box[y][offs[m]] (times wm[m] when wm is not NULL: the
+// half-spectrum weight, 1 or 2, exact in any precision), y = blockIdx.y.
+template <typename T>
+__global__ void k_gather(const C<T>* __restrict__ box, long box_stride, const int* __restrict__ offs, long M,
+                         C<T>* __restrict__ out, long out_stride, const double* __restrict__ wm = nullptr) {
+    box += (long)blockIdx.y * box_stride;
+    out += (long)blockIdx.y * out_stride;
     for (long m = (long)blockIdx.x * blockDim.x + threadIdx.x; m < M; m += (long)gridDim.x * blockDim.x) {
         const C<T> v = box[offs[m]];
         out[m] = wm ? mk<T>(v.x * (T)wm[m], v.y * (T)wm[m]) : v;
@@ -366,7 +399,9 @@ struct UwState {
     void* xmap = nullptr;     // one real map [N]
     void* a[2] = {nullptr, nullptr};  // Monte Carlo maps
     void* spec[4] = {nullptr, nullptr, nullptr, nullptr};  // box spectra
-    void* pairs = nullptr;    // pair spectra [4][npairs][box]
+    void* pairs = nullptr;    // pair spectra [2][npairs][box]
+    void *pair1 = nullptr, *pair2 = nullptr;   // intermediates of a batch of pair transforms
+    int pair_chunk = 0;
     void* qbox = nullptr;     // one box spectrum
     void* zc = nullptr;       // compact [nt][M]
     void* yc = nullptr;       // compact [nt][M]
@@ -412,7 +447,7 @@ struct UwState {
 static void uw_free(UwState* u) {
     if (!u) return;
     void* ptrs[] = {u->g2, u->xmap, u->a[0], u->a[1], u->spec[0], u->spec[1], u->spec[2], u->spec[3], u->pairs, u->qbox,
-                    u->zc, u->yc, u->v1, u->v2, u->dF, u->dpart, u->dsum, u->dvec, u->dvec2, u->dinfo, u->dFp_inv, u->dFb_inv,
+                    u->pair1, u->pair2, u->zc, u->yc, u->v1, u->v2, u->dF, u->dpart, u->dsum, u->dvec, u->dvec2, u->dinfo, u->dFp_inv, u->dFb_inv,
                     u->ylc, u->hbox, u->g3, u->dFl_inv, u->dFo_inv, u->bmaps, u->bpart, u->bout,
                     u->dpart_all};
     for (void* p : ptrs)
@@ -457,7 +492,7 @@ static int uw_alloc(polybin_ctx* ctx, bool need_b) {
     if ((rc = need((void**)&u->dvec2, sizeof(double) * 4096))) return rc;
     if (need_b) {
         const size_t nt = ctx->Nabc.size();
-        if ((rc = need(&u->pairs, sizeof(C<T>) * (size_t)4 * np * nbox))) return rc;
+        if ((rc = need(&u->pairs, sizeof(C<T>) * (size_t)2 * np * nbox))) return rc;
         if ((rc = need(&u->qbox, sizeof(C<T>) * nbox))) return rc;
         const long Mp = (std::max(ctx->nmodes, 1L) + 1) / 2 * 2;   // even row stride: 16-byte aligned rows
         const bool fresh = !u->zc;
@@ -475,15 +510,16 @@ static int uw_alloc(polybin_ctx* ctx, bool need_b) {
 
 static unsigned grid1d(long n) { return (unsigned)std::min<long>((n + 255) / 256, 152L * 16); }
 
-// Inverse transform of a box spectrum to a real map: x-pass, y-pass, z-pass (C2R) with the 1/N of the IFT,
-// and an optional pointwise multiplier on output.
+// Inverse transform of a box spectrum to a real map on grid ig: x-pass, y-pass, z-pass (C2R), times scale, and an
+// optional pointwise multiplier on output.
 template <typename T>
-int run_inverse_box(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* out, const T* mulout) {
-    const int N0 = ctx->N[0], N1 = ctx->N[1], N2 = ctx->N[2];
-    const int By = ctx->gy.cnt, Bz = ctx->gz.cnt;
-    const C<T>* tw0 = (const C<T>*)(sizeof(T) == 4 ? ctx->d_tw_f[0] : ctx->d_tw_d[0]);
-    const C<T>* tw1 = (const C<T>*)(sizeof(T) == 4 ? ctx->d_tw_f[1] : ctx->d_tw_d[1]);
-    const C<T>* tw2 = (const C<T>*)(sizeof(T) == 4 ? ctx->d_tw_f[2] : ctx->d_tw_d[2]);
+int run_inverse_from(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* out, const T* mulout, const InvGrid& ig,
+                     const Box3& keep, double scale) {
+    const int N0 = ig.N[0], N1 = ig.N[1], N2 = ig.N[2];
+    const int By = keep.y.cnt, Bz = keep.z.cnt;
+    const C<T>* tw0 = (const C<T>*)(sizeof(T) == 4 ? ig.tw_f[0] : ig.tw_d[0]);
+    const C<T>* tw1 = (const C<T>*)(sizeof(T) == 4 ? ig.tw_f[1] : ig.tw_d[1]);
+    const C<T>* tw2 = (const C<T>*)(sizeof(T) == 4 ? ig.tw_f[2] : ig.tw_d[2]);
     cudaError_t e = cudaSuccess;
     {
         const int tk = cols_per_cta_of<T>(N0);
@@ -493,12 +529,12 @@ int run_inverse_box(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* ou
         const int ncols = By * Bz;
         it.in = box; it.out = v1;
         it.in_os = 0; it.in_es = ncols; it.out_os = 0; it.out_es = ncols;
-        it.ncols = ncols; it.nouter = 1; it.rng = ctx->gx;
+        it.ncols = ncols; it.nouter = 1; it.rng = keep.x;
         if (!(sizeof(T) == 4 && f2::col(N0, +1, b, 1, ncols, 1, ctx->stream))) {
             PB_WITH_NT(N0, NT, {
                 e = cudaFuncSetAttribute((const void*)k_col<T, +1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
                 if (e != cudaSuccess) return fail_cuda(ctx, e, "attr", __FILE__, __LINE__);
-                k_col<T, +1, NT><<<dim3((ncols + tk - 1) / tk, 1, 1), 256, sm, ctx->stream>>>(b, ctx->plan[0], tw0, tk);
+                k_col<T, +1, NT><<<dim3((ncols + tk - 1) / tk, 1, 1), 256, sm, ctx->stream>>>(b, ig.plan[0], tw0, tk);
             })
         }
         ctx->launches++;
@@ -510,12 +546,12 @@ int run_inverse_box(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* ou
         ColItem& it = b.it[0];
         it.in = v1; it.out = v2;
         it.in_os = (long)By * Bz; it.in_es = Bz; it.out_os = (long)N1 * Bz; it.out_es = Bz;
-        it.ncols = Bz; it.nouter = N0; it.rng = ctx->gy;
+        it.ncols = Bz; it.nouter = N0; it.rng = keep.y;
         if (!(sizeof(T) == 4 && f2::col(N1, +1, b, 1, Bz, N0, ctx->stream))) {
             PB_WITH_NT(N1, NT, {
                 e = cudaFuncSetAttribute((const void*)k_col<T, +1, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
                 if (e != cudaSuccess) return fail_cuda(ctx, e, "attr", __FILE__, __LINE__);
-                k_col<T, +1, NT><<<dim3((Bz + tk - 1) / tk, N0, 1), 256, sm, ctx->stream>>>(b, ctx->plan[1], tw1, tk);
+                k_col<T, +1, NT><<<dim3((Bz + tk - 1) / tk, N0, 1), 256, sm, ctx->stream>>>(b, ig.plan[1], tw1, tk);
             })
         }
         ctx->launches++;
@@ -526,9 +562,9 @@ int run_inverse_box(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* ou
         const long nlines = (long)N0 * N1;
         bool done = false;
         if constexpr (std::is_same<T, float>::value)
-            done = f2::inv_z(N2, b, 1, nlines, (float)(1.0 / (double)ctx->ncell), mulout, nullptr, ctx->stream);
+            done = f2::inv_z(N2, b, 1, nlines, (float)scale, mulout, nullptr, ctx->stream);
         if (!done) {
-            const int rc = launch_inv_z<T>(ctx, b, 1, nlines, T(1.0 / (double)ctx->ncell), mulout, ctx->plan[2], tw2);
+            const int rc = launch_inv_z<T>(ctx, b, 1, nlines, T(scale), mulout, ig.plan[2], tw2);
             if (rc) return rc;
         }
         ctx->launches++;
@@ -536,6 +572,12 @@ int run_inverse_box(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* ou
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail_cuda(ctx, e, "run_inverse_box", __FILE__, __LINE__);
     return POLYBIN_OK;
+}
+
+template <typename T>
+int run_inverse_box(polybin_ctx* ctx, const C<T>* box, C<T>* v1, C<T>* v2, T* out, const T* mulout) {
+    return run_inverse_from<T>(ctx, box, v1, v2, out, mulout, ctx->fg, Box3{ctx->gx, ctx->gy, ctx->gz},
+                               1.0 / (double)ctx->ncell);
 }
 
 // Host copy of the segment sums [nell][nb] of the partials dpart.
@@ -587,13 +629,31 @@ static int pk_fisher_draw(polybin_ctx* ctx, const float* n, const float* w, unsi
         u->dpart_all_cap = (size_t)na * (per + na);
     }
     double* const dsums = u->dpart_all + (size_t)na * per;      // [na][nell][nb]
+    const long nbox = (long)ctx->gx.cnt * ctx->gy.cnt * ctx->gz.cnt;
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value) {
+        if (mask_fast(ctx)) {
+            done = true;
+            const int step = mask_chunk(ctx);
+            for (int il = 0; il < nell; ++il)
+                for (int b = 0; b < nb; b += step) {
+                    const int cnt = std::min(step, nb - b);
+                    float2* X = nullptr;
+                    if ((rc = mask_shells(ctx, SA, 2 * il, b, cnt, &X))) return rc;
+                    if ((rc = launch_cross_bin<float>(ctx, X, nbox, cnt, A, u->dpart_all + (size_t)(il * nb + b) * per))) return rc;
+                }
+        }
+    }
+    const InvGrid& pg = mask_grid(ctx);
     T* q = (T*)u->g2;
-    for (int il = 0; il < nell; ++il) {
+    for (int il = 0; il < nell && !done; ++il) {
         if ((rc = ensure_fine_inv<T>(ctx))) return rc;
-        if ((rc = run_shells<T>(ctx, SA, (C<T>*)W.u1f, (C<T>*)W.u2f, q, 2 * il, ctx->fg))) return rc;
+        if ((rc = run_shells<T>(ctx, SA, (C<T>*)W.u1f, (C<T>*)W.u2f, q, 2 * il, pg))) return rc;
         for (int b = 0; b < nb; ++b) {
             C<T>* X = (C<T>*)u->spec[2];
-            if ((rc = run_forward<T, T, float>(ctx, q + (size_t)b * N, w, n, (C<T>*)W.t1, (C<T>*)W.t2, X))) return rc;
+            if ((rc = run_forward<T, T, T>(ctx, q + (size_t)b * pg.ncell, (const T*)mask_map(ctx), (const T*)nullptr,
+                                           (C<T>*)W.t1, (C<T>*)W.t2, X, pg)))
+                return rc;
             if ((rc = launch_cross_bin<T>(ctx, X, 0, 1, A, u->dpart_all + (size_t)(il * nb + b) * per))) return rc;
         }
     }
@@ -944,26 +1004,80 @@ static int pk_fisher_draw_local(polybin_ctx* ctx, const float* n, const float* w
 
 // ---------------------------------------------------------------------------------------------- B Fisher
 
-// Pair spectra P_xy(k) = FT[g_x g_y](k) (x <= y, lexicographic) on the box |n_i| <= m, of the shell maps of one box
-// spectrum.  The product g_x g_y has wave numbers |n_i| <= 2m, so for |k_i| <= m its transform on the contraction grid
-// (more than 3m points per axis: no alias reaches the box) is (N' / N) times the data-grid one: the maps and their
-// products are formed on the contraction grid and the caller multiplies the spectra by cg_ratio = N / N'.
+// Pair spectra of two fields' difference, out[p] = FT[g_x g_y](U1) - FT[g_x g_y](U2) on the box for every pair x <= y, from
+// the shell maps on the contraction grid.  The products have wave numbers |n_i| <= 2m, so for |k_i| <= m their transform
+// there (more than 3m points an axis: no alias reaches the box) is (N' / N) times the data-grid one; the caller multiplies
+// by cg_ratio = N / N'.  The operator is linear in the products, so the FP32 passes subtract them before the transform:
+// one transform a pair, batched.
 template <typename T>
-static int pair_spectra(polybin_ctx* ctx, const C<T>* U, C<T>* out) {
+static int pair_spectra(polybin_ctx* ctx, const C<T>* U1, const C<T>* U2, C<T>* out) {
     UwState* u = static_cast<UwState*>(ctx->ext);
     Work& W = ctx->w;
-    const long Nc = ctx->cg.ncell;
-    const long nbox = (long)ctx->gx.cnt * ctx->gy.cnt * ctx->gz.cnt;
-    const int nb = ctx->nb;
+    const InvGrid& cg = ctx->cg;
+    const long Nc = cg.ncell;
+    const long By = ctx->gy.cnt, Bz = ctx->gz.cnt, nbox = (long)ctx->gx.cnt * By * Bz;
+    const int nb = ctx->nb, np = nb * (nb + 1) / 2;
     int rc;
-    T* g = (T*)u->g2;
-    if ((rc = run_shells<T>(ctx, U, (C<T>*)W.u1, (C<T>*)W.u2, g, 0, ctx->cg))) return rc;
+    T* g1 = (T*)W.g;
+    T* g2 = (T*)u->g2;
+    if ((rc = run_shells<T>(ctx, U1, (C<T>*)W.u1, (C<T>*)W.u2, g1, 0, cg))) return rc;
+    if ((rc = run_shells<T>(ctx, U2, (C<T>*)W.u1, (C<T>*)W.u2, g2, 0, cg))) return rc;
+    if constexpr (std::is_same<T, float>::value) {
+        if (f2::has(cg.N[0]) && f2::has(cg.N[1]) && f2::has(cg.N[2])) {
+            const long nlines = (long)cg.N[0] * cg.N[1], s1 = nlines * Bz, s2 = (long)cg.N[0] * By * Bz;
+            if (!u->pair2) {
+                // intermediates of a batch of pairs near the L2's size
+                u->pair_chunk = (int)std::min<long>(f2::kBatch, std::max<long>(1, (80L << 20) / ((long)sizeof(float2) * (s1 + s2))));
+                if (!u->pair1) PB_CUDA_OK(cudaMalloc(&u->pair1, sizeof(float2) * s1 * u->pair_chunk));
+                PB_CUDA_OK(cudaMalloc(&u->pair2, sizeof(float2) * s2 * u->pair_chunk));
+            }
+            std::vector<int> px, py;
+            for (int x = 0; x < nb; ++x)
+                for (int y = x; y < nb; ++y) { px.push_back(x); py.push_back(y); }
+            for (int p0 = 0; p0 < np; p0 += u->pair_chunk) {
+                const int cnt = std::min(u->pair_chunk, np - p0);
+                f2::ZFwdBatch z;
+                ColBatch c;
+                for (int i = 0; i < cnt; ++i) {
+                    const size_t x = (size_t)px[p0 + i] * Nc, y = (size_t)py[p0 + i] * Nc;
+                    z.it[i] = {g1 + x, g1 + y, nullptr, g2 + x, g2 + y, (float2*)u->pair1 + (size_t)i * s1};
+                }
+                f2::fwd_z(cg.N[2], z, cnt, nlines, (int)Bz, ctx->stream);
+                for (int i = 0; i < cnt; ++i) {
+                    ColItem& it = c.it[i];
+                    it.in = (float2*)u->pair1 + (size_t)i * s1; it.out = (float2*)u->pair2 + (size_t)i * s2;
+                    it.in_os = (long)cg.N[1] * Bz; it.in_es = Bz; it.out_os = By * Bz; it.out_es = Bz;
+                    it.ncols = (int)Bz; it.nouter = cg.N[0]; it.rng = ctx->gy;
+                }
+                f2::col(cg.N[1], -1, c, cnt, (int)Bz, cg.N[0], ctx->stream);
+                for (int i = 0; i < cnt; ++i) {
+                    ColItem& it = c.it[i];
+                    it.in = (float2*)u->pair2 + (size_t)i * s2; it.out = out + (size_t)(p0 + i) * nbox;
+                    it.in_os = 0; it.in_es = By * Bz; it.out_os = 0; it.out_es = By * Bz;
+                    it.ncols = (int)(By * Bz); it.nouter = 1; it.rng = ctx->gx;
+                }
+                f2::col(cg.N[0], -1, c, cnt, (int)(By * Bz), 1, ctx->stream);
+                ctx->launches += 3;
+                PB_CUDA_OK(cudaGetLastError());
+            }
+            return POLYBIN_OK;
+        }
+    }
+    C<T>* tmp = (C<T>*)u->qbox;
     int p = 0;
     for (int x = 0; x < nb; ++x)
-        for (int y = x; y < nb; ++y, ++p)
-            if ((rc = run_forward<T, T, T>(ctx, g + (size_t)x * Nc, g + (size_t)y * Nc, (const T*)nullptr, (C<T>*)W.t1,
-                                           (C<T>*)W.t2, out + (size_t)p * nbox, ctx->cg)))
+        for (int y = x; y < nb; ++y, ++p) {
+            C<T>* o = out + (size_t)p * nbox;
+            if ((rc = run_forward<T, T, T>(ctx, g1 + (size_t)x * Nc, g1 + (size_t)y * Nc, (const T*)nullptr, (C<T>*)W.t1,
+                                           (C<T>*)W.t2, o, cg)))
                 return rc;
+            if ((rc = run_forward<T, T, T>(ctx, g2 + (size_t)x * Nc, g2 + (size_t)y * Nc, (const T*)nullptr, (C<T>*)W.t1,
+                                           (C<T>*)W.t2, tmp, cg)))
+                return rc;
+            uw::k_box_sub<T><<<grid1d(nbox), 256, 0, ctx->stream>>>(o, tmp, nbox);
+            ctx->launches++;
+        }
+    PB_CUDA_OK(cudaGetLastError());
     return POLYBIN_OK;
 }
 
@@ -982,43 +1096,77 @@ static int bk_fisher_draw(polybin_ctx* ctx, const float* n, const float* w, unsi
     const long Mp = (std::max(M, 1L) + 1) / 2 * 2;   // row stride of the compact arrays
     // the split mode takes the Gram on the tensor cores from weighted Z rows; the others weight inside k_gram
     const bool tc_gram = ctx->prec == POLYBIN_SPLIT_TF32X3 && sizeof(T) == 4;
+    const double* zw = tc_gram ? ctx->d_coef : nullptr;
     int rc;
     T* a1 = (T*)u->a[0];
     T* a2 = (T*)u->a[1];
     uw::k_draw<T><<<grid1d((N + 3) / 4), 256, 0, ctx->stream>>>(a1, N, seed, (uint32_t)r, 0u);
     uw::k_draw<T><<<grid1d((N + 3) / 4), 256, 0, ctx->stream>>>(a2, N, seed, (uint32_t)r, 1u);
     ctx->launches += 2;
-    // fields: 0 = s a1, 1 = s a2, 2 = a1, 3 = a2
+    // fields: 0 = s a1, 1 = s a2, 2 = a1, 3 = a2; pair spectra of 0 - 1 and of 2 - 3
     const T* src[4] = {a1, a2, a1, a2};
     C<T>* pairs = (C<T>*)u->pairs;
     for (int f = 0; f < 4; ++f) {
         const float* m1 = f < 2 ? w : nullptr;
         const float* m2 = f < 2 ? n : nullptr;
         if ((rc = run_forward<T, T, float>(ctx, src[f], m1, m2, (C<T>*)W.t1, (C<T>*)W.t2, (C<T>*)u->spec[f]))) return rc;
-        if ((rc = pair_spectra<T>(ctx, (const C<T>*)u->spec[f], pairs + (size_t)f * np * nbox))) return rc;
     }
+    C<T>* const ps = pairs;                           // of the weighted fields
+    C<T>* const pa = pairs + (size_t)np * nbox;
+    if ((rc = pair_spectra<T>(ctx, (const C<T>*)u->spec[0], (const C<T>*)u->spec[1], ps))) return rc;
+    if ((rc = pair_spectra<T>(ctx, (const C<T>*)u->spec[2], (const C<T>*)u->spec[3], pa))) return rc;
     C<T>* Zc = (C<T>*)u->zc;
     C<T>* Yc = (C<T>*)u->yc;
     C<T>* q = (C<T>*)u->qbox;
-    for (int t = 0; t < nt; ++t) {
+    // Y_b: compact binned modes
+    std::vector<int> start(nb + 1);
+    PB_CUDA_OK(cudaMemcpyAsync(start.data(), ctx->d_bin_start, sizeof(int) * (nb + 1), cudaMemcpyDeviceToHost, ctx->stream));
+    PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
+    for (int t0 = 0; t0 < nt; t0 += kMaxItems) {
+        const int cnt = std::min(kMaxItems, nt - t0);
+        uw::QRows rows;
+        for (int i = 0; i < cnt; ++i) {
+            const int a = ctx->trip[3 * (t0 + i)], b = ctx->trip[3 * (t0 + i) + 1], c = ctx->trip[3 * (t0 + i) + 2];
+            const double dl = (a == b && b == c) ? 6.0 : ((a == b || b == c) ? 2.0 : 1.0);
+            rows.it[i] = {Yc + (size_t)(t0 + i) * Mp, (long)pair_index(nb, a, b) * nbox, (long)pair_index(nb, b, c) * nbox,
+                          (long)pair_index(nb, a, c) * nbox, start[a], start[a + 1], start[b], start[b + 1], start[c],
+                          start[c + 1], 2.0 / dl * ctx->cg_ratio};
+        }
+        if (M > 0) uw::k_qrows<T><<<dim3((unsigned)((M + 255) / 256), cnt), 256, 0, ctx->stream>>>(rows, pa, ctx->d_offs, (int)M);
+        ctx->launches++;
+    }
+    PB_CUDA_OK(cudaGetLastError());
+    // Z_a: the masked operator of the weighted fields' combinations -> compact
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value) {
+        if (mask_fast(ctx)) {
+            done = true;
+            const int step = mask_chunk(ctx);
+            for (int t0 = 0; t0 < nt; t0 += step) {
+                const int cnt = std::min(step, nt - t0);
+                float2* X = nullptr;
+                if ((rc = mask_triplets(ctx, ps, t0, cnt, &X))) return rc;
+                uw::k_gather<float><<<dim3(grid1d(M), cnt), 256, 0, ctx->stream>>>(X, nbox, ctx->d_offs, M,
+                                                                                   Zc + (size_t)t0 * Mp, Mp, zw);
+                ctx->launches++;
+            }
+        }
+    }
+    const InvGrid& pg = mask_grid(ctx);
+    for (int t = 0; t < nt && !done; ++t) {
         const int a = ctx->trip[3 * t], b = ctx->trip[3 * t + 1], c = ctx->trip[3 * t + 2];
         const double dl = (a == b && b == c) ? 6.0 : ((a == b || b == c) ? 2.0 : 1.0);
-        const long pab = (long)pair_index(nb, a, b) * nbox, pbc = (long)pair_index(nb, b, c) * nbox,
-                   pac = (long)pair_index(nb, a, c) * nbox;
-        // Y_b: fields a1, a2 (compact binned modes)
-        uw::k_qcomb<T><<<grid1d(nbox), 256, 0, ctx->stream>>>(pairs + (size_t)2 * np * nbox, pairs + (size_t)3 * np * nbox,
-                                                              pab, pbc, pac, a, b, c, T(2.0 / dl * ctx->cg_ratio),
-                                                              ctx->gx, ctx->gy, ctx->gz, ctx->d_lut, ctx->smax, q);
-        uw::k_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(q, ctx->d_offs, M, Yc + (size_t)t * Mp);
-        // Z_a: fields s a1, s a2 -> real map -> times s -> forward -> compact
-        uw::k_qcomb<T><<<grid1d(nbox), 256, 0, ctx->stream>>>(pairs, pairs + (size_t)np * nbox, pab, pbc, pac, a, b, c,
-                                                              T(2.0 / dl * ctx->cg_ratio), ctx->gx, ctx->gy, ctx->gz,
-                                                              ctx->d_lut, ctx->smax, q);
-        ctx->launches += 3;
-        if ((rc = run_inverse_box<T>(ctx, q, (C<T>*)u->v1, (C<T>*)u->v2, (T*)u->xmap, (const T*)nullptr))) return rc;
-        if ((rc = run_forward<T, T, float>(ctx, (const T*)u->xmap, w, n, (C<T>*)W.t1, (C<T>*)W.t2, q))) return rc;
-        uw::k_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(q, ctx->d_offs, M, Zc + (size_t)t * Mp,
-                                                            tc_gram ? ctx->d_coef : nullptr);
+        uw::k_qcomb<T><<<grid1d(nbox), 256, 0, ctx->stream>>>(
+            ps, (long)pair_index(nb, a, b) * nbox, (long)pair_index(nb, b, c) * nbox, (long)pair_index(nb, a, c) * nbox, a, b, c,
+            T(2.0 / dl * ctx->cg_ratio), ctx->gx, ctx->gy, ctx->gz, ctx->d_lut, ctx->smax, q);
+        ctx->launches++;
+        if ((rc = run_inverse_from<T>(ctx, q, (C<T>*)u->v1, (C<T>*)u->v2, (T*)u->xmap, (const T*)nullptr, pg,
+                                      Box3{ctx->gx, ctx->gy, ctx->gz}, 1.0 / (double)N)))
+            return rc;
+        if ((rc = run_forward<T, T, T>(ctx, (const T*)u->xmap, (const T*)mask_map(ctx), (const T*)nullptr, (C<T>*)W.t1,
+                                       (C<T>*)W.t2, q, pg)))
+            return rc;
+        uw::k_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(q, 0, ctx->d_offs, M, Zc + (size_t)t * Mp, 0, zw);
         ctx->launches++;
     }
     if (tc_gram) {
@@ -1146,6 +1294,7 @@ static int fisher_sum(polybin_ctx* ctx, const float* n, const float* w, unsigned
     const int na = which != 1 ? ctx->nell * ctx->nb : (int)ctx->Nabc.size();
     if (sum.size() != (size_t)na * na) sum.assign((size_t)na * na, 0.0);
     std::vector<double> F;
+    if ((which == 0 || which == 1) && r0 < r1 && (rc = mask_setup<T>(ctx, n, w))) return rc;
     for (int r = r0; r < r1; ++r) {
         if (which == 0) {
             if ((rc = pk_fisher_draw<T>(ctx, n, w, seed, r, F))) return rc;
@@ -1385,6 +1534,10 @@ static int bk_multipoles_local_t(polybin_ctx* ctx, const float* delta, int batch
     return POLYBIN_OK;
 }
 
+template int run_inverse_from<float>(polybin_ctx*, const float2*, float2*, float2*, float*, const float*, const InvGrid&,
+                                    const Box3&, double);
+template int run_inverse_from<double>(polybin_ctx*, const double2*, double2*, double2*, double*, const double*, const InvGrid&,
+                                     const Box3&, double);
 template int run_inverse_box<float>(polybin_ctx*, const float2*, float2*, float2*, float*, const float*);
 template int run_inverse_box<double>(polybin_ctx*, const double2*, double2*, double2*, double*, const double*);
 
