@@ -20,6 +20,8 @@
 #include <type_traits>
 #include <vector>
 
+#include "contract.cuh"
+#include "ddmath.cuh"
 #include "fft2.h"
 #include "polybin_internal.h"
 
@@ -44,10 +46,14 @@ __device__ __forceinline__ void philox_round(uint32_t& c0, uint32_t& c1, uint32_
     c0 = n0; c1 = lo1; c2 = n2; c3 = lo0;
 }
 
-// Gaussian white-noise map (Philox4x32-10 + Box-Muller in FP64).
+// Gaussian white-noise map (Philox4x32-10 + Box-Muller): in FP64, or, for FP32 maps, in double-float arithmetic with the
+// product rounded to FP32.  Against FP64 the double-float radii and cosines differ by at most 2e-13 and 2e-10 relative, and
+// of 8 million values all but one in 10^6 round to the same FP32 number.  256^3 cells: 1.16 ms in FP64, bound by the FP64
+// pipe; 0.12 ms.
 template <typename T>
 __global__ void k_draw(T* __restrict__ out, long N, unsigned long long seed, uint32_t draw, uint32_t stream) {
     const long nblk = (N + 3) / 4;
+    const bool wide = reinterpret_cast<uintptr_t>(out) % 16 == 0;   // (a caller's map may lie at any float)
     for (long j = (long)blockIdx.x * blockDim.x + threadIdx.x; j < nblk; j += (long)gridDim.x * blockDim.x) {
         uint32_t c0 = (uint32_t)j, c1 = (uint32_t)((unsigned long long)j >> 32), c2 = draw, c3 = stream;
         uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
@@ -56,18 +62,34 @@ __global__ void k_draw(T* __restrict__ out, long N, unsigned long long seed, uin
             if (r > 0) { k0 += 0x9E3779B9u; k1 += 0xBB67AE85u; }
             philox_round(c0, c1, c2, c3, k0, k1);
         }
-        const double t = 2.3283064365386963e-10;  // 2^-32
-        const double u0 = ((double)c0 + 0.5) * t, u1 = ((double)c1 + 0.5) * t;
-        const double u2 = ((double)c2 + 0.5) * t, u3 = ((double)c3 + 0.5) * t;
-        const double r01 = sqrt(-2.0 * log(u0)), r23 = sqrt(-2.0 * log(u2));
-        double s1, co1, s3, co3;
-        sincospi(2.0 * u1, &s1, &co1);
-        sincospi(2.0 * u3, &s3, &co3);
-        const double z[4] = {r01 * co1, r01 * s1, r23 * co3, r23 * s3};
+        T z[4];
+        if constexpr (sizeof(T) == 4) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const dd::F2 r = dd::radius(2ull * (h ? c2 : c0) + 1ull);
+                dd::F2 co, si;
+                dd::sincos_turn(2ull * (h ? c3 : c1) + 1ull, co, si);
+                z[2 * h] = dd::round_prod(r, co);
+                z[2 * h + 1] = dd::round_prod(r, si);
+            }
+        } else {
+            const double t = 2.3283064365386963e-10;  // 2^-32
+            const double u0 = ((double)c0 + 0.5) * t, u1 = ((double)c1 + 0.5) * t;
+            const double u2 = ((double)c2 + 0.5) * t, u3 = ((double)c3 + 0.5) * t;
+            const double r01 = sqrt(-2.0 * log(u0)), r23 = sqrt(-2.0 * log(u2));
+            double s1, co1, s3, co3;
+            sincospi(2.0 * u1, &s1, &co1);
+            sincospi(2.0 * u3, &s3, &co3);
+            z[0] = r01 * co1; z[1] = r01 * s1; z[2] = r23 * co3; z[3] = r23 * s3;
+        }
+        if (wide && 4 * j + 3 < N) {
+            Vec4<T>::store(out + 4 * j, z);
+            continue;
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const long i = 4 * j + q;
-            if (i < N) out[i] = (T)z[q];
+            if (i < N) out[i] = z[q];
         }
     }
 }
