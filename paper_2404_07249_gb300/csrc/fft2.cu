@@ -11,6 +11,7 @@ namespace f2 {
                      cudaStream_t);                                                                                    \
     bool xq_##G(int, const XqBatch&, int, int, const float2*, AxisRange, AxisRange, AxisRange, cudaStream_t);          \
     bool fwd_z_##G(int, const ZFwdBatch&, int, long, int, cudaStream_t);                                               \
+    bool fwd_z_ylm_##G(int, const YlmBatch&, int, long, int, cudaStream_t);                                            \
     bool inv_z_##G(int, const ZInvBatch&, int, long, float, const float*, uint32_t*, cudaStream_t);                    \
     bool mask_z_##G(int, const ZMaskBatch&, int, long, const float*, int, cudaStream_t);
 PB_F2_DECL(a)
@@ -37,6 +38,10 @@ bool xq(int n, const XqBatch& b, int nitem, int mc, const float2* pairs, AxisRan
 bool fwd_z(int n, const ZFwdBatch& b, int nitem, long nl, int kout, cudaStream_t st) {
     return fwd_z_a(n, b, nitem, nl, kout, st) || fwd_z_b(n, b, nitem, nl, kout, st) || fwd_z_c(n, b, nitem, nl, kout, st) ||
            fwd_z_d(n, b, nitem, nl, kout, st);
+}
+bool fwd_z_ylm(int n, const YlmBatch& b, int nitem, long nl, int kout, cudaStream_t st) {
+    return fwd_z_ylm_a(n, b, nitem, nl, kout, st) || fwd_z_ylm_b(n, b, nitem, nl, kout, st) ||
+           fwd_z_ylm_c(n, b, nitem, nl, kout, st) || fwd_z_ylm_d(n, b, nitem, nl, kout, st);
 }
 bool inv_z(int n, const ZInvBatch& b, int nitem, long nl, float scale, const float* mulout, uint32_t* absmax,
            cudaStream_t st) {

@@ -61,6 +61,19 @@ struct ZFwdItem {
 struct ZFwdBatch {
     ZFwdItem it[kBatch];
 };
+// Forward z-pass of harmonic-weighted fields: field x (w) x Ybar_lm of each cell's direction from the observer.
+struct YlmItem {
+    float2* out;                 // [nlines][kout]
+    // Ybar_lm = (Re or Im of (x + i y)^am) z^odd (d4 z^4 + d2 z^2 + d0) for the unit vector (x, y, z)
+    int am, im, odd;
+    float d4, d2, d0;
+};
+struct YlmBatch {
+    YlmItem it[16];
+    const float *in, *w;         // w may be null
+    int n1;                      // lines: (i, j) = (l / n1, l % n1)
+    float h[3], half, obs[3];    // cell centre (i + 1/2) h - half - obs, in units of the box side
+};
 struct ZMaskItem {
     const float2* in;            // [nlines][kin]
     float2* out;                 // [nlines][kout]
@@ -87,6 +100,7 @@ bool col(int n, int dir, const ColBatch& b, int nitem, int max_cols, int max_out
 bool xfilter(int n, const XInvBatch& b, int nitem, int max_cols, const float2* spec, AxisRange gx, AxisRange gy,
              AxisRange gz, float scale, cudaStream_t st);
 bool fwd_z(int n, const ZFwdBatch& b, int nitem, long nlines, int kout, cudaStream_t st);
+bool fwd_z_ylm(int n, const YlmBatch& b, int nitem, long nlines, int kout, cudaStream_t st);
 bool inv_z(int n, const ZInvBatch& b, int nitem, long nlines, float scale, const float* mulout, uint32_t* absmax,
            cudaStream_t st);
 bool mask_z(int n, const ZMaskBatch& b, int nitem, long nlines, const float* s, int kout, cudaStream_t st);

@@ -39,6 +39,10 @@ template <int N> struct Run {
     static void fwd_z(const ZFwdBatch& b, int nitem, long nlines, int kout, cudaStream_t st) {
         k_fwd_z<N><<<line_grid(nlines, nitem), E::kLineThreads, E::kLineSmem, st>>>(b, nlines, kout);
     }
+    static void fwd_z_ylm(const YlmBatch& b, int nitem, long nlines, int kout, cudaStream_t st) {
+        const dim3 g = line_grid(nlines, nitem);
+        k_fwd_z_ylm<N><<<dim3(g.y, g.x), E::kLineThreads, E::kLineSmem, st>>>(b, nlines, kout);
+    }
     static void inv_z(const ZInvBatch& b, int nitem, long nlines, float scale, const float* mulout, uint32_t* absmax,
                       cudaStream_t st) {
         k_inv_z<N><<<line_grid(nlines, nitem), E::kLineThreads, E::kLineSmem, st>>>(b, nlines, scale, mulout, absmax);
@@ -73,6 +77,10 @@ template <int N> struct Run {
     }                                                                                                                  \
     bool fwd_z_##G(int n, const ZFwdBatch& b, int nitem, long nl, int kout, cudaStream_t st) {                         \
         switch (n) { LENGTHS(fwd_z(b, nitem, nl, kout, st)) }                                                          \
+        return false;                                                                                                  \
+    }                                                                                                                  \
+    bool fwd_z_ylm_##G(int n, const YlmBatch& b, int nitem, long nl, int kout, cudaStream_t st) {                      \
+        switch (n) { LENGTHS(fwd_z_ylm(b, nitem, nl, kout, st)) }                                                      \
         return false;                                                                                                  \
     }                                                                                                                  \
     bool inv_z_##G(int n, const ZInvBatch& b, int nitem, long nl, float scale, const float* mulout, uint32_t* absmax,  \

@@ -354,17 +354,31 @@ __global__ void k_ylm_box_accum(const C<T>* __restrict__ G, C<T>* __restrict__ H
     }
 }
 
-// acc[q] (= or +=) Ybar_lm(k_q) box[offs[q]] over the binned modes (FP64 accumulation).
+// Ybar_lm(k_q) of the binned modes, m = -ell .. ell: tab[m + ell][q] (FP64; laid out once a context).
+static __global__ void k_ylm_table(const int* __restrict__ offs, long M, int ell, AxisRange gx, AxisRange gy, AxisRange gz,
+                                   double* __restrict__ tab) {
+    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < M; q += (long)gridDim.x * blockDim.x) {
+        double x, y, z;
+        const bool ok = box_direction(offs[q], gx, gy, gz, x, y, z);
+        for (int m = -ell; m <= ell; ++m) tab[(long)(m + ell) * M + q] = ok ? ybar<double>(ell, m, x, y, z) : 0.0;
+    }
+}
+
+// acc[q] = sum_i tab[i][q] box[i][offs[q]] over cnt boxes (added to acc when add is set; tab null: weight 1), FP64.
 template <typename T>
-__global__ void k_ylm_gather(const C<T>* __restrict__ box, const int* __restrict__ offs, long M, int ell, int m,
-                             int first, AxisRange gx, AxisRange gy, AxisRange gz, double2* __restrict__ acc) {
+__global__ void k_ylm_gather(const C<T>* __restrict__ box, long box_stride, int cnt, const int* __restrict__ offs, long M,
+                             const double* __restrict__ tab, int add_to, double2* __restrict__ acc) {
     for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < M; q += (long)gridDim.x * blockDim.x) {
         const long o = offs[q];
-        double x, y, z;
-        const double yv = box_direction(o, gx, gy, gz, x, y, z) ? ybar<double>(ell, m, x, y, z) : 0.0;
-        const C<T> g = box[o];
-        const double2 v = make_double2(yv * (double)g.x, yv * (double)g.y);
-        acc[q] = first ? v : make_double2(acc[q].x + v.x, acc[q].y + v.y);
+        double2 v = add_to ? acc[q] : make_double2(0.0, 0.0);
+#pragma unroll 3
+        for (int i = 0; i < cnt; ++i) {
+            const C<T> g = box[(long)i * box_stride + o];
+            const double y = tab ? tab[(long)i * M + q] : 1.0;
+            v.x += y * (double)g.x;
+            v.y += y * (double)g.y;
+        }
+        acc[q] = v;
     }
 }
 
@@ -442,6 +456,9 @@ struct UwState {
     // local line of sight: compact sum_m Ybar_lm(k) FT[Ybar_lm u](k) per ell [3][M]; a box of the same sums; nb maps of
     // one harmonic's inverse transforms; the Fisher matrix and its inverse
     double2* ylc = nullptr;
+    double* yltab = nullptr;      // Ybar_lm of the binned modes, ell = 2 (5 rows) and 4 (9 rows) as lmax has them [..][M]
+    void *yl1 = nullptr, *yl2 = nullptr, *ylbox = nullptr;   // intermediates and boxes of a batch of harmonics
+    int yl_chunk = 0;
     void* hbox = nullptr;
     void* g3 = nullptr;
     std::vector<double> Fl, Fl_inv;
@@ -470,7 +487,7 @@ static void uw_free(UwState* u) {
     if (!u) return;
     void* ptrs[] = {u->g2, u->xmap, u->a[0], u->a[1], u->spec[0], u->spec[1], u->spec[2], u->spec[3], u->pairs, u->qbox,
                     u->pair1, u->pair2, u->zc, u->yc, u->v1, u->v2, u->dF, u->dpart, u->dsum, u->dvec, u->dvec2, u->dinfo, u->dFp_inv, u->dFb_inv,
-                    u->ylc, u->hbox, u->g3, u->dFl_inv, u->dFo_inv, u->bmaps, u->bpart, u->bout,
+                    u->ylc, u->yltab, u->yl1, u->yl2, u->ylbox, u->hbox, u->g3, u->dFl_inv, u->dFo_inv, u->bmaps, u->bpart, u->bout,
                     u->dpart_all};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -893,8 +910,86 @@ static int uw_alloc_local(polybin_ctx* ctx, bool fisher) {
     UwState* u = static_cast<UwState*>(ctx->ext);
     const long nbox = (long)ctx->gx.cnt * ctx->gy.cnt * ctx->gz.cnt;
     if (!u->ylc) PB_CUDA_OK(cudaMalloc(&u->ylc, sizeof(double2) * 3 * std::max(ctx->nmodes, 1L)));
+    if (!u->yltab && ctx->nell > 1 && ctx->nmodes > 0) {
+        const long M = ctx->nmodes;
+        PB_CUDA_OK(cudaMalloc(&u->yltab, sizeof(double) * (ctx->nell > 2 ? 14 : 5) * M));
+        for (int il = 1; il < ctx->nell; ++il) {
+            uw::k_ylm_table<<<grid1d(M), 256, 0, ctx->stream>>>(ctx->d_offs, M, 2 * il, ctx->gx, ctx->gy, ctx->gz,
+                                                                u->yltab + (il == 1 ? 0 : 5 * M));
+            ctx->launches++;
+        }
+        PB_CUDA_OK(cudaGetLastError());
+    }
     if (!u->hbox) PB_CUDA_OK(cudaMalloc(&u->hbox, sizeof(C<T>) * nbox));
     if (fisher && !u->g3) PB_CUDA_OK(cudaMalloc(&u->g3, sizeof(T) * (size_t)ctx->nb * ctx->ncell));
+    return POLYBIN_OK;
+}
+
+// The batched harmonic transforms take the data grid (FP32 two-stage lengths); allocates their workspace on first use.
+static bool ylm_fast(polybin_ctx* ctx) {
+    UwState* u = static_cast<UwState*>(ctx->ext);
+    if (u->yl_chunk) return u->yl_chunk > 0;
+    u->yl_chunk = -1;
+    if (!f2::has(ctx->N[0]) || !f2::has(ctx->N[1]) || !f2::has(ctx->N[2])) return false;
+    const long Bz = ctx->gz.cnt, By = ctx->gy.cnt, nbox = (long)ctx->gx.cnt * By * Bz;
+    const long s1 = (long)ctx->N[0] * ctx->N[1] * Bz, s2 = (long)ctx->N[0] * By * Bz;
+    // intermediates of a batch near the L2's size (at most the nine harmonics of ell = 4)
+    const int c = (int)std::min<long>(9, std::max<long>(1, (112L << 20) / ((long)sizeof(float2) * (s1 + s2))));
+    if (cudaMalloc(&u->yl1, sizeof(float2) * s1 * c) != cudaSuccess || cudaMalloc(&u->yl2, sizeof(float2) * s2 * c) != cudaSuccess ||
+        cudaMalloc(&u->ylbox, sizeof(float2) * nbox * c) != cudaSuccess) {
+        cudaGetLastError();                           // no room for the batch: one harmonic at a time
+        return false;
+    }
+    u->yl_chunk = c;
+    return true;
+}
+
+// boxes[i] = FT[Ybar_l,m0+i in w] on the box for i < cnt (cnt <= yl_chunk); w may be null.
+static int forward_ylm(polybin_ctx* ctx, const float* in, const float* w, int ell, int m0, int cnt, const float2** boxes) {
+    UwState* u = static_cast<UwState*>(ctx->ext);
+    const int N0 = ctx->N[0], N1 = ctx->N[1], N2 = ctx->N[2];
+    const long Bz = ctx->gz.cnt, By = ctx->gy.cnt, nbox = (long)ctx->gx.cnt * By * Bz;
+    const long s1 = (long)N0 * N1 * Bz, s2 = (long)N0 * By * Bz;
+    // d^|m| L_l / dz^|m| c_lm as z^odd (d4 z^4 + d2 z^2 + d0) (see ylm.cuh)
+    static const float d2c[3][4] = {{0, 0, 1.5f, -0.5f}, {1, 0, 0, 1.7320508075688772f}, {0, 0, 0, 0.86602540378443865f}};
+    static const float d4c[5][4] = {{0, 4.375f, -3.75f, 0.375f},
+                                    {1, 0, 5.5339859052946636f, -2.3717082451262845f},
+                                    {0, 0, 3.9131189606246322f, -0.55901699437494742f},
+                                    {1, 0, 0, 2.0916500663351889f},
+                                    {0, 0, 0, 0.73950997288745200f}};
+    f2::YlmBatch z;
+    z.in = in;
+    z.w = w;
+    z.n1 = N1;
+    for (int a = 0; a < 3; ++a) {
+        z.h[a] = 1.f / (float)ctx->N[a];
+        z.obs[a] = (float)(ctx->observer[a] / ctx->L);
+    }
+    z.half = 0.5f;
+    for (int i = 0; i < cnt; ++i) {
+        const int m = m0 + i, am = m < 0 ? -m : m;
+        const float* d = ell == 2 ? d2c[am] : d4c[am];
+        z.it[i] = {(float2*)u->yl1 + (size_t)i * s1, am, m < 0 ? 1 : 0, (int)d[0], d[1], d[2], d[3]};
+    }
+    f2::fwd_z_ylm(N2, z, cnt, (long)N0 * N1, (int)Bz, ctx->stream);
+    ColBatch b;
+    for (int i = 0; i < cnt; ++i) {
+        ColItem& it = b.it[i];
+        it.in = (float2*)u->yl1 + (size_t)i * s1; it.out = (float2*)u->yl2 + (size_t)i * s2;
+        it.in_os = (long)N1 * Bz; it.in_es = Bz; it.out_os = By * Bz; it.out_es = Bz;
+        it.ncols = (int)Bz; it.nouter = N0; it.rng = ctx->gy;
+    }
+    f2::col(N1, -1, b, cnt, (int)Bz, N0, ctx->stream);
+    for (int i = 0; i < cnt; ++i) {
+        ColItem& it = b.it[i];
+        it.in = (float2*)u->yl2 + (size_t)i * s2; it.out = (float2*)u->ylbox + (size_t)i * nbox;
+        it.in_os = 0; it.in_es = By * Bz; it.out_os = 0; it.out_es = By * Bz;
+        it.ncols = (int)(By * Bz); it.nouter = 1; it.rng = ctx->gx;
+    }
+    f2::col(N0, -1, b, cnt, (int)(By * Bz), 1, ctx->stream);
+    ctx->launches += 3;
+    PB_CUDA_OK(cudaGetLastError());
+    *boxes = (const float2*)u->ylbox;
     return POLYBIN_OK;
 }
 
@@ -908,20 +1003,35 @@ static int local_asym(polybin_ctx* ctx, const TIN* in, const float* m1, const fl
     const uw::CellGeom<T> cg = cell_geom<T>(ctx);
     int rc;
     if ((rc = run_forward<T, TIN, float>(ctx, in, m1, m2, (C<T>*)W.t1, (C<T>*)W.t2, ubox))) return rc;
-    uw::k_ylm_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(ubox, ctx->d_offs, M, 0, 0, 1, ctx->gx, ctx->gy, ctx->gz,
-                                                            u->ylc);
+    uw::k_ylm_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(ubox, 0, 1, ctx->d_offs, M, nullptr, 0, u->ylc);
     ctx->launches++;
+    const long nbox = (long)ctx->gx.cnt * ctx->gy.cnt * ctx->gz.cnt;
     C<T>* tmp = (C<T>*)u->spec[2];
     for (int il = 1; il < ctx->nell; ++il) {
         const int ell = 2 * il;
+        const double* tab = u->yltab + (il == 1 ? 0 : 5 * M);
+        double2* acc = u->ylc + (size_t)il * M;
+        if constexpr (std::is_same<T, float>::value && std::is_same<TIN, float>::value) {
+            if (!m2 && ylm_fast(ctx)) {
+                const float2* boxes = nullptr;
+                for (int m = -ell; m <= ell; m += u->yl_chunk) {
+                    const int cnt = std::min(u->yl_chunk, ell - m + 1);
+                    if ((rc = forward_ylm(ctx, in, m1, ell, m, cnt, &boxes))) return rc;
+                    uw::k_ylm_gather<float><<<grid1d(M), 256, 0, ctx->stream>>>(
+                        boxes, nbox, cnt, ctx->d_offs, M, tab + (long)(m + ell) * M, m == -ell ? 0 : 1, acc);
+                    ctx->launches++;
+                }
+                continue;
+            }
+        }
         for (int m = -ell; m <= ell; ++m) {
             uw::k_mul_ylm<T, TIN, float><<<grid1d(N), 256, 0, ctx->stream>>>(in, m1, m2, (T*)u->xmap, ell, m, cg);
             ctx->launches++;
             if ((rc = run_forward<T, T, float>(ctx, (const T*)u->xmap, (const float*)nullptr, (const float*)nullptr,
                                                (C<T>*)W.t1, (C<T>*)W.t2, tmp)))
                 return rc;
-            uw::k_ylm_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(tmp, ctx->d_offs, M, ell, m, m == -ell ? 1 : 0,
-                                                                    ctx->gx, ctx->gy, ctx->gz, u->ylc + (size_t)il * M);
+            uw::k_ylm_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(tmp, 0, 1, ctx->d_offs, M, tab + (long)(m + ell) * M,
+                                                                    m == -ell ? 0 : 1, acc);
             ctx->launches++;
         }
     }
