@@ -466,19 +466,20 @@ __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineTh
     fwd_rest<N>(v, buf, t, act, has2, kout, item.out + l1 * kout);
 }
 
-// The same for the harmonic-weighted fields of a batch: item blockIdx.x of line block blockIdx.y, so that the items that
+// The same for the harmonic-weighted fields of a batch: the items of a line block are consecutive blocks, so that those that
 // read the same lines run together (the field and its weight come from DRAM once for all of them).  Bound by the arithmetic of the harmonic:
 // 68 us a harmonic at 256^3 against 29 for a plain transform; a product pass, 94 us, and a transform a harmonic before.
 template <int N>
 __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineThreads, Geo<N>::TG))
-    k_fwd_z_ylm(YlmBatch batch, long nlines, int kout) {
+    k_fwd_z_ylm(YlmBatch batch, int nitem, long nlines, int kout) {
     extern __shared__ __align__(16) float2 f2_smem[];
     using E = Geo<N>;
     constexpr int P = E::P, Q = E::Q, QP = E::QP;
-    const YlmItem& item = batch.it[blockIdx.x];
+    const unsigned lb = blockIdx.x / (unsigned)nitem;
+    const YlmItem& item = batch.it[blockIdx.x - lb * (unsigned)nitem];
     const int g = threadIdx.x / E::TG, t = threadIdx.x - g * E::TG;
     float2* buf = f2_smem + g * E::GS;
-    const long l1 = 2 * ((long)blockIdx.y * E::G + g);
+    const long l1 = 2 * ((long)lb * E::G + g);
     const bool act = l1 < nlines, has2 = l1 + 1 < nlines;
     float2 v[E::TG];
     if (t < Q && act) {

@@ -40,8 +40,8 @@ template <int N> struct Run {
         k_fwd_z<N><<<line_grid(nlines, nitem), E::kLineThreads, E::kLineSmem, st>>>(b, nlines, kout);
     }
     static void fwd_z_ylm(const YlmBatch& b, int nitem, long nlines, int kout, cudaStream_t st) {
-        const dim3 g = line_grid(nlines, nitem);
-        k_fwd_z_ylm<N><<<dim3(g.y, g.x), E::kLineThreads, E::kLineSmem, st>>>(b, nlines, kout);
+        // one dimension: 1024 x 1024 lines of 512 points are 65536 line blocks, more than a grid's y takes
+        k_fwd_z_ylm<N><<<line_grid(nlines, 1).x * nitem, E::kLineThreads, E::kLineSmem, st>>>(b, nitem, nlines, kout);
     }
     static void inv_z(const ZInvBatch& b, int nitem, long nlines, float scale, const float* mulout, uint32_t* absmax,
                       cudaStream_t st) {
