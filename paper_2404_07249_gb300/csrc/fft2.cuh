@@ -388,10 +388,9 @@ __device__ __forceinline__ void split_lines(const float2* buf, float2* __restric
     }
 }
 
-// Second half of a forward line transform: exchange, second stage, kept coefficients of lines l1, l1 + 1 to out.
+// Second half of a forward line transform: exchange and second stage, the packed result in buf.
 template <int N>
-__device__ __forceinline__ void fwd_rest(float2* v, float2* buf, int t, bool act, bool has2, int kout,
-                                         float2* __restrict__ out) {
+__device__ __forceinline__ void fwd_rest(float2* v, float2* buf, int t, bool act, int kout) {
     constexpr int P = Geo<N>::P, Q = Geo<N>::Q, QP = Geo<N>::QP;
     __syncthreads();
     if (t < P && act) {
@@ -408,7 +407,6 @@ __device__ __forceinline__ void fwd_rest(float2* v, float2* buf, int t, bool act
         }
     }
     __syncthreads();
-    if (act) split_lines<N>(buf, out, out + kout, has2, kout, t);
 }
 
 // z-pass, forward (R2C), the same results as k_fwd_z: lines 2p and 2p + 1 packed as one complex line, multiplied on
@@ -463,12 +461,16 @@ __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineTh
 #pragma unroll
         for (int n1 = 0; n1 < P; ++n1) buf[n1 * QP + t] = v[n1];
     }
-    fwd_rest<N>(v, buf, t, act, has2, kout, item.out + l1 * kout);
+    fwd_rest<N>(v, buf, t, act, kout);
+    if (act) split_lines<N>(buf, item.out + l1 * kout, item.out + (l1 + 1) * kout, has2, kout, t);
 }
 
-// The same for the harmonic-weighted fields of a batch: the items of a line block are consecutive blocks, so that those that
-// read the same lines run together (the field and its weight come from DRAM once for all of them).  Bound by the arithmetic of the harmonic:
-// 68 us a harmonic at 256^3 against 29 for a plain transform; a product pass, 94 us, and a transform a harmonic before.
+// The same for harmonic-weighted fields.  Along a line Ybar_l,m and Ybar_l,-m differ by a constant, Re or Im of
+// e^{i |m| phi}, so an item is one |m|: the field times the part that depends on the polar angle is transformed once and
+// leaves multiplied by either constant.  With u = cos^2, s2 = sin^2 and sc = sin cos of the polar angle (one reciprocal a
+// cell, no root), that part is s2^(|m| / 2) (times sc for odd |m|) times a polynomial in u.  The items of a line block are
+// consecutive blocks, so that those that read the same lines run together (the field and its weight come from DRAM once
+// for all of them).  Bound by instruction issue.
 template <int N>
 __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineThreads, Geo<N>::TG))
     k_fwd_z_ylm(YlmBatch batch, int nitem, long nlines, int kout) {
@@ -481,36 +483,33 @@ __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineTh
     float2* buf = f2_smem + g * E::GS;
     const long l1 = 2 * ((long)lb * E::G + g);
     const bool act = l1 < nlines, has2 = l1 + 1 < nlines;
+    // offset of line l from the observer in the plane
+    auto plane = [&](long l, float& px, float& py) {
+        const int ix = (int)((unsigned)l / (unsigned)batch.n1), iy = (int)l - ix * batch.n1;
+        px = ((float)ix + 0.5f) * batch.h[0] - batch.half - batch.obs[0];
+        py = ((float)iy + 0.5f) * batch.h[1] - batch.half - batch.obs[1];
+    };
     float2 v[E::TG];
     if (t < Q && act) {
-        const long i0 = l1 * N + t;
+        const float c0 = item.am < 2 ? 1.f : 0.f, c1 = (item.am >> 1) == 1 ? 1.f : 0.f, c2 = item.am == 4 ? 1.f : 0.f;
+        const float o0 = item.am & 1 ? 0.f : 1.f, o1 = 1.f - o0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const long l = l1 + (has2 ? h : 0);
-            const long i = i0 + (has2 ? h * N : 0);
-            const int ix = (int)((unsigned)l / (unsigned)batch.n1), iy = (int)l - ix * batch.n1;
-            const float px = ((float)ix + 0.5f) * batch.h[0] - batch.half - batch.obs[0];
-            const float py = ((float)iy + 0.5f) * batch.h[1] - batch.half - batch.obs[1];
-            // (px + i py)^am: constant along the line
-            float re = 1.f, im = 0.f;
-            for (int q = 0; q < item.am; ++q) {
-                const float r2 = re * px - im * py;
-                im = re * py + im * px;
-                re = r2;
-            }
-            const float a = item.im ? im : re, pxy2 = px * px + py * py;
+            const float* __restrict__ in = batch.in + l * N + t;
+            float px, py;
+            plane(l, px, py);
+            const float rho2 = px * px + py * py, rho = sqrtf(rho2);
 #pragma unroll
             for (int j = 0; j < P; ++j) {
                 const float pz = ((float)(t + Q * j) + 0.5f) * batch.h[2] - batch.half - batch.obs[2];
-                const float r2 = pxy2 + pz * pz;
+                const float r2 = rho2 + pz * pz;
                 const bool at = r2 > 0.f;             // the z axis where the centre coincides with the observer
-                const float inv = at ? 1.f / sqrtf(r2) : 0.f;
-                const float z = at ? pz * inv : 1.f, z2 = z * z;
-                float y = a * ((item.d4 * z2 + item.d2) * z2 + item.d0);
-                if (item.odd) y *= z;
-                for (int q = 0; q < item.am; ++q) y *= inv;
-                float f = batch.in[i + Q * j];
-                if (batch.w) f *= batch.w[i + Q * j];
+                const float q = __frcp_rn(at ? r2 : 1.f);
+                const float zq = pz * q, u = at ? pz * zq : 1.f, s2 = rho2 * q, sc = rho * zq;
+                const float y = ((item.d4 * u + item.d2) * u + item.d0) * (c0 + s2 * (c1 + s2 * c2)) * (o0 + o1 * sc);
+                float f = in[Q * j];
+                if (batch.w) f *= batch.w[l * N + t + Q * j];
                 f *= y;
                 if (h == 0) v[j].x = f;
                 else v[j].y = has2 ? f : 0.f;
@@ -520,7 +519,39 @@ __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineTh
 #pragma unroll
         for (int n1 = 0; n1 < P; ++n1) buf[n1 * QP + t] = v[n1];
     }
-    fwd_rest<N>(v, buf, t, act, has2, kout, item.out + l1 * kout);
+    fwd_rest<N>(v, buf, t, act, kout);
+    if (!act) return;
+    float re[2], im[2];                               // e^{i |m| phi} of the two lines (1 on the axis)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float px, py;
+        plane(l1 + h, px, py);
+        const float rho2 = px * px + py * py;
+        const float inv = rho2 > 0.f ? 1.f / sqrtf(rho2) : 0.f;
+        const float cx = rho2 > 0.f ? px * inv : 1.f, cy = py * inv;
+        float a = 1.f, b = 0.f;
+        for (int q = 0; q < item.am; ++q) {
+            const float a2 = a * cx - b * cy;
+            b = a * cy + b * cx;
+            a = a2;
+        }
+        re[h] = a;
+        im[h] = b;
+    }
+    for (int k = t; k < kout; k += E::TG) {
+        const float2 zk = buf[k], zm = buf[k ? N - k : 0];
+        const float2 x1 = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+        const float2 x2 = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+        const long o = l1 * kout + k;
+        if (item.re) {
+            item.re[o] = make_float2(x1.x * re[0], x1.y * re[0]);
+            if (has2) item.re[o + kout] = make_float2(x2.x * re[1], x2.y * re[1]);
+        }
+        if (item.im) {
+            item.im[o] = make_float2(x1.x * im[0], x1.y * im[0]);
+            if (has2) item.im[o + kout] = make_float2(x2.x * im[1], x2.y * im[1]);
+        }
+    }
 }
 
 // z-pass, inverse (C2R), the same results as k_inv_z.  The real lines go through shared memory so that the CTA's 2G lines,

@@ -61,11 +61,12 @@ struct ZFwdItem {
 struct ZFwdBatch {
     ZFwdItem it[kBatch];
 };
-// Forward z-pass of harmonic-weighted fields: field x (w) x Ybar_lm of each cell's direction from the observer.
+// Forward z-pass of harmonic-weighted fields: field x (w) x Ybar_l,m and Ybar_l,-m of each cell's direction from the
+// observer, m = am >= 0, l even.
 struct YlmItem {
-    float2* out;                 // [nlines][kout]
-    // Ybar_lm = (Re or Im of (x + i y)^am) z^odd (d4 z^4 + d2 z^2 + d0) for the unit vector (x, y, z)
-    int am, im, odd;
+    float2 *re, *im;             // [nlines][kout] of m = am and of m = -am (either may be null)
+    // Ybar_lm = (Re or Im of (x + i y)^am) z^(am odd) (d4 z^4 + d2 z^2 + d0) for the unit vector (x, y, z)
+    int am;
     float d4, d2, d0;
 };
 struct YlmBatch {

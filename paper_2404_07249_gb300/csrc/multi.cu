@@ -2,6 +2,11 @@
 // forward transform, the shell maps, the triplet contraction and the copy of its result to pinned host memory --
 // is captured once into a CUDA graph on a private stream and replayed there with a single graph launch, ordered
 // after the work already queued on the contexts' stream.
+//
+// Fields of one context follow one another (they share its workspace); different contexts share nothing that is written,
+// so each is a branch of the graph (kBranches at most).  A small field's kernels leave much of the chip idle: their launch
+// gaps and last waves, and the contraction, which keeps one CTA an SM waiting on its own pipeline while the transforms of
+// another branch run beside it.
 // The graph is cached in the first context, keyed by the context ids and field pointers of the call.
 #include <cuda_runtime.h>
 
@@ -14,12 +19,16 @@
 
 namespace pb {
 
+constexpr int kBranches = 4;                // streams of a capture: the contexts take them in turn
+
 struct MultiCache {
     std::vector<unsigned long long> key;
     cudaStream_t cap = nullptr;             // private stream: capture and replay (the legacy stream cannot capture)
+    cudaStream_t side[kBranches - 1] = {};  // further branches, forked from and joined to cap (capture only)
     cudaEvent_t ev = nullptr;
     cudaGraphExec_t exec = nullptr;
     double* host = nullptr;                 // pinned: contraction results of every field
+    int* err = nullptr;                     // behind them: the error flags of every context
     std::vector<size_t> off;                // per-field offset into host
 };
 
@@ -29,6 +38,8 @@ void destroy_multi(polybin_ctx* ctx) {
     if (m->exec) cudaGraphExecDestroy(m->exec);
     if (m->host) cudaFreeHost(m->host);
     if (m->ev) cudaEventDestroy(m->ev);
+    for (cudaStream_t s : m->side)
+        if (s) cudaStreamDestroy(s);
     if (m->cap) cudaStreamDestroy(m->cap);
     delete m;
     ctx->multi = nullptr;
@@ -64,6 +75,8 @@ extern "C" int polybin_bk_ideal_multi(polybin_ctx* const* ctxs, const float* con
     std::vector<unsigned long long> key;
     key.reserve(2 * (size_t)n_fields + 1);
     key.push_back((unsigned long long)n_fields);
+    std::vector<polybin_ctx*> distinct;
+    std::vector<int> place(n_fields);                 // each field's context among the distinct ones
     for (int i = 0; i < n_fields; ++i) {
         polybin_ctx* c = ctxs[i];
         if (!c || !fields[i] || !bk_out[i]) return fail(c0, POLYBIN_EINVAL, "polybin_bk_ideal_multi: NULL entry %d", i);
@@ -76,6 +89,8 @@ extern "C" int polybin_bk_ideal_multi(polybin_ctx* const* ctxs, const float* con
         }
         if ((rc = ensure_triplets(c))) return rc;
         if ((rc = ensure_err_flag(c))) return rc;
+        place[i] = (int)(std::find(distinct.begin(), distinct.end(), c) - distinct.begin());
+        if (place[i] == (int)distinct.size()) distinct.push_back(c);
         key.push_back(c->uid);
         key.push_back((unsigned long long)(uintptr_t)fields[i]);
     }
@@ -93,12 +108,19 @@ extern "C" int polybin_bk_ideal_multi(polybin_ctx* const* ctxs, const float* con
         }
         {
             polybin_ctx* ctx = c0;
-            PB_CUDA_OK(cudaHostAlloc((void**)&m->host, sizeof(double) * total, cudaHostAllocDefault));
+            const size_t bytes = sizeof(double) * total + sizeof(int) * kErrFlags * distinct.size();
+            PB_CUDA_OK(cudaHostAlloc((void**)&m->host, bytes, cudaHostAllocDefault));
+            m->err = reinterpret_cast<int*>(m->host + total);
         }
         {
             polybin_ctx* ctx = c0;
             PB_CUDA_OK(cudaStreamCreateWithFlags(&m->cap, cudaStreamNonBlocking));
             PB_CUDA_OK(cudaEventCreateWithFlags(&m->ev, cudaEventDisableTiming));
+        }
+        const int nbranch = (int)std::min<size_t>(distinct.size(), kBranches);
+        {
+            polybin_ctx* ctx = c0;
+            for (int k = 1; k < nbranch; ++k) PB_CUDA_OK(cudaStreamCreateWithFlags(&m->side[k - 1], cudaStreamNonBlocking));
         }
         cudaStream_t st = m->cap;
         cudaGraph_t graph = nullptr;
@@ -108,16 +130,35 @@ extern "C" int polybin_bk_ideal_multi(polybin_ctx* const* ctxs, const float* con
             destroy_multi(c0);
             return fail_cuda(c0, e, "cudaStreamBeginCapture", __FILE__, __LINE__);
         }
-        std::vector<cudaStream_t> saved(n_fields);
-        for (int i = 0; i < n_fields; ++i) { saved[i] = ctxs[i]->stream; ctxs[i]->stream = st; ctxs[i]->capturing = true; }
+        for (polybin_ctx* c : distinct) c->capturing = true;
+        const cudaStream_t caller = c0->stream;           // (of every context)
+        for (int i = 0; i < n_fields; ++i) {
+            const int k = place[i] % kBranches;
+            ctxs[i]->stream = k ? m->side[k - 1] : st;
+        }
         rc = POLYBIN_OK;
+        // fork: the capture goes over to the side streams through the event
+        e = cudaEventRecord(m->ev, st);
+        for (int k = 1; k < nbranch && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(m->side[k - 1], m->ev, 0);
+        if (e != cudaSuccess) rc = fail_cuda(c0, e, "cudaStreamWaitEvent", __FILE__, __LINE__);
         for (int i = 0; i < n_fields && !rc; ++i) {
             polybin_ctx* c = ctxs[i];
             rc = c->prec == POLYBIN_FP64 ? capture_field<double>(c, fields[i], m->host + m->off[i])
                                          : capture_field<float>(c, fields[i], m->host + m->off[i]);
             if (rc && c != c0) c0->err = c->err;
         }
-        for (int i = 0; i < n_fields; ++i) { ctxs[i]->capturing = false; ctxs[i]->stream = saved[i]; }
+        for (size_t k = 0; k < distinct.size() && !rc; ++k) {
+            polybin_ctx* c = distinct[k];
+            e = cudaMemcpyAsync(m->err + k * kErrFlags, c->d_err, sizeof(int) * kErrFlags, cudaMemcpyDeviceToHost, c->stream);
+            if (e != cudaSuccess) rc = fail_cuda(c0, e, "capture copy", __FILE__, __LINE__);
+        }
+        // join
+        for (int k = 1; k < nbranch && !rc; ++k) {
+            e = cudaEventRecord(m->ev, m->side[k - 1]);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, m->ev, 0);
+            if (e != cudaSuccess) rc = fail_cuda(c0, e, "cudaStreamWaitEvent", __FILE__, __LINE__);
+        }
+        for (polybin_ctx* c : distinct) { c->capturing = false; c->stream = caller; }
         e = cudaStreamEndCapture(st, &graph);
         if (rc || e != cudaSuccess) cudaGetLastError();
         if (rc) {
@@ -138,11 +179,10 @@ extern "C" int polybin_bk_ideal_multi(polybin_ctx* const* ctxs, const float* con
     if (e != cudaSuccess) return fail_cuda(c0, e, "cudaGraphLaunch", __FILE__, __LINE__);
     for (int i = 0; i < n_fields; ++i) {
         polybin_ctx* c = ctxs[i];
-        int herr[kErrFlags] = {0, 0};
-        {
+        const int* herr = m->err + place[i] * kErrFlags;
+        if (herr[kErrStaging]) {
             polybin_ctx* ctx = c0;
-            PB_CUDA_OK(cudaMemcpy(herr, c->d_err, sizeof(herr), cudaMemcpyDeviceToHost));
-            if (herr[kErrStaging]) PB_CUDA_OK(cudaMemset(c->d_err + kErrStaging, 0, sizeof(int)));
+            PB_CUDA_OK(cudaMemset(c->d_err + kErrStaging, 0, sizeof(int)));
         }
         if (herr[kErrPipeline] || herr[kErrStaging])
             return fail(c0, POLYBIN_ETIMEOUT, "polybin_bk_ideal_multi: a %s wait timed out (field %d)",

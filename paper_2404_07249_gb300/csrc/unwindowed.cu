@@ -354,13 +354,16 @@ __global__ void k_ylm_box_accum(const C<T>* __restrict__ G, C<T>* __restrict__ H
     }
 }
 
-// Ybar_lm(k_q) of the binned modes, m = -ell .. ell: tab[m + ell][q] (FP64; laid out once a context).
+// Place of the harmonic m among the 2 ell + 1: 0, -1, 1, -2, 2, .. (m and -m next to each other).
+__host__ __device__ inline int ylm_row(int m) { return m < 0 ? -2 * m - 1 : 2 * m; }
+
+// Ybar_lm(k_q) of the binned modes: tab[ylm_row(m)][q] (FP64; laid out once a context).
 static __global__ void k_ylm_table(const int* __restrict__ offs, long M, int ell, AxisRange gx, AxisRange gy, AxisRange gz,
                                    double* __restrict__ tab) {
     for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < M; q += (long)gridDim.x * blockDim.x) {
         double x, y, z;
         const bool ok = box_direction(offs[q], gx, gy, gz, x, y, z);
-        for (int m = -ell; m <= ell; ++m) tab[(long)(m + ell) * M + q] = ok ? ybar<double>(ell, m, x, y, z) : 0.0;
+        for (int m = -ell; m <= ell; ++m) tab[(long)ylm_row(m) * M + q] = ok ? ybar<double>(ell, m, x, y, z) : 0.0;
     }
 }
 
@@ -944,19 +947,19 @@ static bool ylm_fast(polybin_ctx* ctx) {
     return true;
 }
 
-// boxes[i] = FT[Ybar_l,m0+i in w] on the box for i < cnt (cnt <= yl_chunk); w may be null.
-static int forward_ylm(polybin_ctx* ctx, const float* in, const float* w, int ell, int m0, int cnt, const float2** boxes) {
+// boxes[i] = FT[Ybar_lm in w] on the box for the harmonics with ylm_row(m) = r0 + i, i < cnt (cnt <= yl_chunk); w may be null.
+static int forward_ylm(polybin_ctx* ctx, const float* in, const float* w, int ell, int r0, int cnt, const float2** boxes) {
     UwState* u = static_cast<UwState*>(ctx->ext);
     const int N0 = ctx->N[0], N1 = ctx->N[1], N2 = ctx->N[2];
     const long Bz = ctx->gz.cnt, By = ctx->gy.cnt, nbox = (long)ctx->gx.cnt * By * Bz;
     const long s1 = (long)N0 * N1 * Bz, s2 = (long)N0 * By * Bz;
-    // d^|m| L_l / dz^|m| c_lm as z^odd (d4 z^4 + d2 z^2 + d0) (see ylm.cuh)
-    static const float d2c[3][4] = {{0, 0, 1.5f, -0.5f}, {1, 0, 0, 1.7320508075688772f}, {0, 0, 0, 0.86602540378443865f}};
-    static const float d4c[5][4] = {{0, 4.375f, -3.75f, 0.375f},
-                                    {1, 0, 5.5339859052946636f, -2.3717082451262845f},
-                                    {0, 0, 3.9131189606246322f, -0.55901699437494742f},
-                                    {1, 0, 0, 2.0916500663351889f},
-                                    {0, 0, 0, 0.73950997288745200f}};
+    // d^|m| L_l / dz^|m| c_lm as z^(|m| odd) (d4 z^4 + d2 z^2 + d0) (see ylm.cuh)
+    static const float d2c[3][3] = {{0, 1.5f, -0.5f}, {0, 0, 1.7320508075688772f}, {0, 0, 0.86602540378443865f}};
+    static const float d4c[5][3] = {{4.375f, -3.75f, 0.375f},
+                                    {0, 5.5339859052946636f, -2.3717082451262845f},
+                                    {0, 3.9131189606246322f, -0.55901699437494742f},
+                                    {0, 0, 2.0916500663351889f},
+                                    {0, 0, 0.73950997288745200f}};
     f2::YlmBatch z;
     z.in = in;
     z.w = w;
@@ -966,12 +969,16 @@ static int forward_ylm(polybin_ctx* ctx, const float* in, const float* w, int el
         z.obs[a] = (float)(ctx->observer[a] / ctx->L);
     }
     z.half = 0.5f;
-    for (int i = 0; i < cnt; ++i) {
-        const int m = m0 + i, am = m < 0 ? -m : m;
+    int nz = 0;
+    for (int i = 0; i < cnt; ++nz) {                  // rows of m = -am and m = am, as far as both are in the batch
+        const int am = (r0 + i + 1) / 2;
         const float* d = ell == 2 ? d2c[am] : d4c[am];
-        z.it[i] = {(float2*)u->yl1 + (size_t)i * s1, am, m < 0 ? 1 : 0, (int)d[0], d[1], d[2], d[3]};
+        f2::YlmItem& it = z.it[nz];
+        it = {nullptr, nullptr, am, d[0], d[1], d[2]};
+        for (; i < cnt && (r0 + i + 1) / 2 == am; ++i)
+            (uw::ylm_row(am) == r0 + i ? it.re : it.im) = (float2*)u->yl1 + (size_t)i * s1;
     }
-    f2::fwd_z_ylm(N2, z, cnt, (long)N0 * N1, (int)Bz, ctx->stream);
+    f2::fwd_z_ylm(N2, z, nz, (long)N0 * N1, (int)Bz, ctx->stream);
     ColBatch b;
     for (int i = 0; i < cnt; ++i) {
         ColItem& it = b.it[i];
@@ -1014,11 +1021,12 @@ static int local_asym(polybin_ctx* ctx, const TIN* in, const float* m1, const fl
         if constexpr (std::is_same<T, float>::value && std::is_same<TIN, float>::value) {
             if (!m2 && ylm_fast(ctx)) {
                 const float2* boxes = nullptr;
-                for (int m = -ell; m <= ell; m += u->yl_chunk) {
-                    const int cnt = std::min(u->yl_chunk, ell - m + 1);
-                    if ((rc = forward_ylm(ctx, in, m1, ell, m, cnt, &boxes))) return rc;
+                for (int r = 0, cnt; r < 2 * ell + 1; r += cnt) {
+                    cnt = std::min(u->yl_chunk, 2 * ell + 1 - r);
+                    if (cnt > 1 && (r + cnt) % 2 == 0) --cnt;   // -m and m share their transform along z
+                    if ((rc = forward_ylm(ctx, in, m1, ell, r, cnt, &boxes))) return rc;
                     uw::k_ylm_gather<float><<<grid1d(M), 256, 0, ctx->stream>>>(
-                        boxes, nbox, cnt, ctx->d_offs, M, tab + (long)(m + ell) * M, m == -ell ? 0 : 1, acc);
+                        boxes, nbox, cnt, ctx->d_offs, M, tab + (long)r * M, r ? 1 : 0, acc);
                     ctx->launches++;
                 }
                 continue;
@@ -1030,8 +1038,8 @@ static int local_asym(polybin_ctx* ctx, const TIN* in, const float* m1, const fl
             if ((rc = run_forward<T, T, float>(ctx, (const T*)u->xmap, (const float*)nullptr, (const float*)nullptr,
                                                (C<T>*)W.t1, (C<T>*)W.t2, tmp)))
                 return rc;
-            uw::k_ylm_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(tmp, 0, 1, ctx->d_offs, M, tab + (long)(m + ell) * M,
-                                                                    m == -ell ? 0 : 1, acc);
+            uw::k_ylm_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(tmp, 0, 1, ctx->d_offs, M,
+                                                                    tab + (long)uw::ylm_row(m) * M, m == -ell ? 0 : 1, acc);
             ctx->launches++;
         }
     }
