@@ -1111,31 +1111,98 @@ static std::vector<std::pair<int, int>> cut_tiles(const std::vector<NeedPair>& P
     return seg;
 }
 
-// Orders the rows [first, last) of a tile, sorted by (j, k), to avoid bank conflicts of the producers' gathers.  A
-// 16-byte load of a warp is served for eight lanes at a time; the slots' swizzle puts chunk c of map m into bank group
-// c ^ (m % 8), so eight consecutive rows are conflict-free when their maps j, and their maps k, are equal or distinct
-// modulo 8.  Greedy: every group of eight takes the first remaining rows that conflict least.
+// Largest number of different maps of one bank group (map % 8) among v.
+static int bank_clash(const std::vector<int>& v) {
+    int most = 0;
+    for (int g = 0; g < 8; ++g) {
+        std::set<int> m;
+        for (int x : v)
+            if ((x & 7) == g) m.insert(x);
+        most = std::max(most, (int)m.size());
+    }
+    return most;
+}
+
+// Orders the rows [first, last) of a tile, sorted by (j, k), for the producers' gathers, which bound the kernel by shared
+// memory.  A 16-byte load of a warp is served for eight lanes at a time, or for sixteen where lanes i and i ^ 1, or i and
+// i ^ 2, read the same address throughout (measured: 4 and 2 cycles a load); the slots' swizzle puts chunk c of map m into
+// bank group c ^ (m % 8), so different maps of one group that are equal modulo 8 clash.
+// Rows therefore come in quads (j1, k1) (j1, k2) (j2, k1) (j2, k2), whose lanes share j by i ^ 1 and k by i ^ 2, and four
+// quads a half-warp are taken to clash least; rows that form no quad follow, eight at a time that clash least.
 static void order_rows(std::vector<NeedPair>& need, int first, int last) {
-    std::vector<NeedPair> rest(need.begin() + first, need.begin() + last), out;
-    std::vector<char> used(rest.size(), 0);
-    while (out.size() < rest.size()) {
-        std::set<int> mj[8], mk[8];          // the group's maps by bank group
-        for (int g = 0; g < 8 && out.size() < rest.size(); ++g) {
-            int best = -1, best_cost = 1 << 30;
-            for (size_t i = 0; i < rest.size(); ++i) {
-                if (used[i]) continue;
-                const std::set<int>&a = mj[rest[i].j & 7], &b = mk[rest[i].k & 7];
-                const int cost = (int)(a.size() - a.count(rest[i].j) + b.size() - b.count(rest[i].k));
-                if (cost < best_cost) { best_cost = cost; best = (int)i; }
-                if (cost == 0) break;
+    const std::vector<NeedPair> rest(need.begin() + first, need.begin() + last);
+    std::map<std::pair<int, int>, int> at;               // (j, k) -> row, of the rows left
+    std::vector<int> js;
+    for (size_t i = 0; i < rest.size(); ++i) {
+        at[{rest[i].j, rest[i].k}] = (int)i;
+        if (js.empty() || js.back() != rest[i].j) js.push_back(rest[i].j);
+    }
+    std::vector<int> order;
+    if (at.size() == rest.size()) {                       // (no pair twice)
+        // quads: of all pairs of j the one with the most k in common first, so that few rows are left over
+        struct Quad { int r[4], j[2], k[2]; };
+        std::vector<Quad> quads;
+        for (;;) {
+            int bj1 = -1, bj2 = -1;
+            std::vector<int> bk;
+            for (size_t x = 0; x < js.size(); ++x)
+                for (size_t y = x + 1; y < js.size(); ++y) {
+                    std::vector<int> ks;
+                    for (auto it = at.lower_bound({js[x], -1}); it != at.end() && it->first.first == js[x]; ++it)
+                        if (at.count({js[y], it->first.second})) ks.push_back(it->first.second);
+                    if (ks.size() / 2 > bk.size() / 2) { bk = ks; bj1 = js[x]; bj2 = js[y]; }
+                }
+            if (bk.size() < 2) break;
+            for (size_t q = 0; q + 1 < bk.size(); q += 2) {
+                Quad d;
+                d.j[0] = bj1; d.j[1] = bj2; d.k[0] = bk[q]; d.k[1] = bk[q + 1];
+                for (int i = 0; i < 4; ++i) {
+                    const std::pair<int, int> key{d.j[i >> 1], d.k[i & 1]};
+                    d.r[i] = at[key];
+                    at.erase(key);
+                }
+                quads.push_back(d);
             }
-            used[best] = 1;
-            mj[rest[best].j & 7].insert(rest[best].j);
-            mk[rest[best].k & 7].insert(rest[best].k);
-            out.push_back(rest[best]);
+        }
+        std::vector<char> used(quads.size(), 0);
+        for (size_t n = 0; n < quads.size();) {
+            std::vector<int> mj, mk;
+            for (int g = 0; g < 4 && n < quads.size(); ++g, ++n) {
+                int best = -1, best_cost = 1 << 30;
+                for (size_t i = 0; i < quads.size(); ++i) {
+                    if (used[i]) continue;
+                    std::vector<int> a = mj, b = mk;
+                    a.insert(a.end(), quads[i].j, quads[i].j + 2);
+                    b.insert(b.end(), quads[i].k, quads[i].k + 2);
+                    const int cost = bank_clash(a) + bank_clash(b);
+                    if (cost < best_cost) { best_cost = cost; best = (int)i; }
+                }
+                used[best] = 1;
+                mj.insert(mj.end(), quads[best].j, quads[best].j + 2);
+                mk.insert(mk.end(), quads[best].k, quads[best].k + 2);
+                order.insert(order.end(), quads[best].r, quads[best].r + 4);
+            }
         }
     }
-    std::copy(out.begin(), out.end(), need.begin() + first);
+    std::vector<char> used(rest.size(), 0);
+    for (int i : order) used[i] = 1;
+    for (std::vector<int> mj, mk; order.size() < rest.size();) {
+        int best = -1, best_cost = 1 << 30;
+        for (size_t i = 0; i < rest.size(); ++i) {
+            if (used[i]) continue;
+            std::vector<int> a = mj, b = mk;
+            a.push_back(rest[i].j);
+            b.push_back(rest[i].k);
+            const int cost = bank_clash(a) + bank_clash(b);
+            if (cost < best_cost) { best_cost = cost; best = (int)i; }
+        }
+        used[best] = 1;
+        mj.push_back(rest[best].j);
+        mk.push_back(rest[best].k);
+        order.push_back(best);
+        if (order.size() % 8 == 0) { mj.clear(); mk.clear(); }
+    }
+    for (size_t i = 0; i < rest.size(); ++i) need[first + i] = rest[order[i]];
 }
 
 // Pure host layout of a plan (no CUDA calls): tiles, row groups, TMEM / shared-memory layout, the row table and the
