@@ -352,27 +352,30 @@ __global__ void __launch_bounds__(Geo<N>::kColThreads, min_ctas(Geo<N>::kColThre
 // ------------------------------------------------------------------------------------------------ lines
 
 // Stage-1 input of thread t of an inverse transform: points k = t + Q j of the packed Hermitian pair Z = X1 + i X2
-// (kz < kin, zero above; imaginary parts of the kz = 0 and N/2 coefficients ignored).
+// (kz < kin, zero above; imaginary parts of the kz = 0 and N/2 coefficients ignored).  Which half of the spectrum a point
+// lies in is known at compile time (but for the middle j of an odd P), so the loads need one comparison each and are issued
+// together.
 template <int N>
 __device__ __forceinline__ void load_hermitian(float2* v, const float2* __restrict__ in1, const float2* __restrict__ in2,
                                                bool has2, int kin, int t) {
     constexpr int P = Geo<N>::P, Q = Geo<N>::Q;
+    float2 a[P], b[P];
 #pragma unroll
     for (int j = 0; j < P; ++j) {
         const int k = t + Q * j;
-        float2 z = make_float2(0.f, 0.f);
-        if (k == 0 || 2 * k == N) {
-            if (k < kin) z = make_float2(in1[k].x, has2 ? in2[k].x : 0.f);
-        } else if (k < kin) {
-            const float2 a = in1[k];
-            const float2 b = has2 ? in2[k] : make_float2(0.f, 0.f);
-            z = make_float2(a.x - b.y, a.y + b.x);
-        } else if (N - k < kin) {
-            const float2 a = in1[N - k];
-            const float2 b = has2 ? in2[N - k] : make_float2(0.f, 0.f);
-            z = make_float2(a.x + b.y, b.x - a.y);
-        }
-        v[j] = z;
+        const bool up = 2 * j + 1 == P ? 2 * k >= N : 2 * j >= P;   // k >= N / 2
+        const int i = up ? N - k : k;
+        const bool in = i < kin;
+        a[j] = in ? in1[i] : make_float2(0.f, 0.f);
+        b[j] = in && has2 ? in2[i] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+        const int k = t + Q * j;
+        const bool up = 2 * j + 1 == P ? 2 * k >= N : 2 * j >= P;
+        float ay = up ? -a[j].y : a[j].y, by = up ? -b[j].y : b[j].y;
+        if ((j == 0 || 2 * j == P || 2 * j + 1 == P) && (k == 0 || 2 * k == N)) ay = by = 0.f;
+        v[j] = make_float2(a[j].x - by, ay + b[j].x);
     }
 }
 
@@ -557,7 +560,9 @@ __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineTh
 // z-pass, inverse (C2R), the same results as k_inv_z.  The real lines go through shared memory so that the CTA's 2G lines,
 // one contiguous block, are written in 16-byte pieces (4-byte stores of P consecutive numbers straight from the registers
 // took 1.54 ms for 30 maps of 288^3 cells).  With absmax, absmax[item] takes the largest magnitude written (bit pattern),
-// which the triplet contraction scales by.
+// which the triplet contraction scales by.  Bound by instruction issue and by the latency of its loads: 30 maps of 288^3
+// cells took 1.25 ms while the branches of the Hermitian input kept its loads apart, and take 0.93 ms (0.57 ms at the copy
+// rate).
 template <int N>
 __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineThreads, Geo<N>::TG))
     k_inv_z(ZInvBatch batch, long nlines, float scale, const float* __restrict__ mulout, uint32_t* __restrict__ absmax) {
@@ -595,27 +600,33 @@ __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineTh
     }
     __syncthreads();
     // lines l0 .. of the CTA, V numbers a store
-    constexpr int V = E::V, NV = N / V;
+    constexpr int V = E::V, NV = N / V, T = E::kLineThreads, STEPS = (2 * E::G * NV + T - 1) / T;
     using VT = typename std::conditional<V == 4, float4, float2>::type;
     const int nl = (int)min((long)2 * E::G, nlines - l0);
     VT* __restrict__ out = reinterpret_cast<VT*>(static_cast<float*>(item.out) + l0 * N);
-    uint32_t top = 0u;
-    for (int q = threadIdx.x; q < nl * NV; q += E::kLineThreads) {
-        const int l = q / NV, e = q - l * NV;
+    float top = 0.f;
+    int l = (int)threadIdx.x / NV, e = (int)threadIdx.x - l * NV;
+#pragma unroll
+    for (int i = 0; i < STEPS; ++i) {
+        if (l >= nl) break;
         VT a = *reinterpret_cast<const VT*>(reinterpret_cast<const float*>(f2_smem) + (l >> 1) * E::OS + (l & 1) * N + V * e);
         float* p = reinterpret_cast<float*>(&a);
+        if (mulout) {
 #pragma unroll
-        for (int i = 0; i < V; ++i) {
-            if (mulout) p[i] *= mulout[l0 * N + (long)q * V + i];
-            top = max(top, __float_as_uint(p[i]) & 0x7fffffffu);
+            for (int c = 0; c < V; ++c) p[c] *= mulout[(l0 + l) * N + V * e + c];
         }
-        out[q] = a;
+#pragma unroll
+        for (int c = 0; c < V; ++c) top = fmaxf(top, fabsf(p[c]));
+        out[l * NV + e] = a;
+        l += T / NV;
+        e += T % NV;
+        if (e >= NV) { e -= NV; ++l; }
     }
     if (absmax) {
         const int lanes = E::kLineThreads - (int)(threadIdx.x & ~31u);     // of this warp (the last one may be partial)
-        top = __reduce_max_sync(lanes >= 32 ? 0xffffffffu : (1u << lanes) - 1u, top);
+        const uint32_t most = __reduce_max_sync(lanes >= 32 ? 0xffffffffu : (1u << lanes) - 1u, __float_as_uint(top));
         // (a look first: of the hundreds of thousands of warps few still raise the maximum)
-        if ((threadIdx.x & 31) == 0 && top > __ldcg(absmax + blockIdx.y)) atomicMax(absmax + blockIdx.y, top);
+        if ((threadIdx.x & 31) == 0 && most > __ldcg(absmax + blockIdx.y)) atomicMax(absmax + blockIdx.y, most);
     }
 }
 
