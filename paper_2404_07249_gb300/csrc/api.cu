@@ -320,8 +320,13 @@ int run_contract(polybin_ctx* ctx, const T* g, int ng, const T* h, int nh, doubl
 // Partials [nx][nb][nseg][nell] of the binned products of nx box spectra X + z x_stride with A.
 template <typename T>
 int launch_cross_bin(polybin_ctx* ctx, const C<T>* X, long x_stride, int nx, const C<T>* A, double* partial) {
-    k_cross_bin<T><<<dim3(ctx->nb, ctx->pk_nseg, nx), 256, 0, ctx->stream>>>(
-        X, A, x_stride, ctx->d_offs, ctx->d_coef, ctx->nmodes, ctx->d_bin_start, ctx->nell, ctx->pk_seg_len, partial);
+    // several spectra a CTA share the mode lists, their weights and A
+    auto launch = [&](auto kernel, int nz) {
+        kernel<<<dim3(ctx->nb, ctx->pk_nseg, (nx + nz - 1) / nz), kXbThreads, 0, ctx->stream>>>(
+            X, A, x_stride, nx, ctx->d_offs, ctx->d_coef, ctx->nmodes, ctx->d_bin_start, ctx->nell, ctx->pk_seg_len, partial);
+    };
+    if (nx == 1) launch(k_cross_bin<T, 1>, 1);
+    else launch(k_cross_bin<T, 3>, 3);
     return launch_check(ctx, "k_cross_bin");
 }
 template int launch_cross_bin<float>(polybin_ctx*, const float2*, long, int, const float2*, double*);
@@ -512,7 +517,7 @@ static int plan_pk(polybin_ctx* ctx) {
     long maxlen = 1;
     for (int b = 0; b < nb; ++b) maxlen = std::max(maxlen, (long)offs[b].size());
     // about four segments of the mode lists an SM (a multiple of the CTA's 256 threads, at most 4096 modes)
-    ctx->pk_seg_len = (int)std::min(4096L, std::max(256L, (M / (4 * 152) + 255) / 256 * 256));
+    ctx->pk_seg_len = (int)std::min(1024L, std::max(256L, (M / (4 * 152) + 255) / 256 * 256));
     ctx->pk_nseg = (int)((maxlen + ctx->pk_seg_len - 1) / ctx->pk_seg_len);
     polybin_ctx* c = ctx;
     PB_CUDA_OK_C(cudaMalloc(&c->d_offs, sizeof(int) * std::max(M, 1L)));

@@ -250,49 +250,80 @@ static __global__ void __launch_bounds__(32 * kRedSlices) k_reduce_partials(cons
 inline unsigned reduce_blocks(long nout) { return (unsigned)((nout + 31) / 32); }
 
 // ------------------------------------------------------------------------------------------------
+// The double of a float.  A conversion instruction takes a slot of the FP64 pipe, which has two lanes a clock an SM on this
+// part; for normal numbers the bits are moved by integer instructions instead.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+    return (double)f;                                 // zeros, subnormal numbers, infinities, NaN
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
 // Binned products over the half spectrum (Sec. 3.4.1, eq. pk-limit; Sec. 3.3.2, eq. fish-from-Q):
 //   partial[z][b][seg][ell] = sum_{modes of segment seg of bin b} coef_ell Re(conj X_z A),
 // coef_ell = w_k L_ell(mu) (w_k = 1 on the kz = 0 and Nyquist planes, 2 elsewhere) precomputed per mode in FP64; with
 // X = A it gives the sums of L_ell |D|^2 over the full k-grid.  X_z = X + z x_stride.  One CTA per (bin, segment of that
-// bin's mode list, z); deterministic tree reduction in FP64.  The FP64 pipe (two lanes a clock an SM on this part) bounds
-// it once every SM has work, so plan_pk cuts the lists into about four segments an SM: with 8192 modes a segment, 20
-// to 40 CTAs took 70 us for 64^3 and for 256^3 alike.
-template <typename T>
-__global__ void __launch_bounds__(256) k_cross_bin(const C<T>* __restrict__ X, const C<T>* __restrict__ A, long x_stride,
-                                                   const int* __restrict__ offs, const double* __restrict__ coef,
-                                                   long nmodes_total, const int* __restrict__ bin_start, int nell,
-                                                   int seg_len, double* __restrict__ partial) {
-    __shared__ double red[256];
-    const int b = blockIdx.x, seg = blockIdx.y;
+// bin's mode list, NZ of the nx spectra); FP64 sums in a fixed order.  Bound by the FP64 pipe (two lanes a clock an SM):
+// two operations a mode and spectrum for the product and one for each ell, after the conversions have left it (four of nine
+// operations) and with one warp a sum at the end instead of a tree over all threads.  plan_pk cuts the lists into about four
+// segments an SM: with 8192 modes a segment, 20 to 40 CTAs took 70 us for 64^3 and for 256^3 alike.
+// Measured, before and after these two: 64^3 FP64 14.0 -> 6.7 us, 24 x 3 spectra on 256^3 (24 bins, three ells) 814 -> 575 us,
+// 512^3 with 30 bins 58 -> 44 us (a segment of at most 1024 modes keeps enough warps in flight there: 87 us with 3072).
+constexpr int kXbThreads = 128;
+template <typename T, int NZ>
+__global__ void __launch_bounds__(kXbThreads) k_cross_bin(const C<T>* __restrict__ X, const C<T>* __restrict__ A, long x_stride,
+                                                          int nx, const int* __restrict__ offs,
+                                                          const double* __restrict__ coef, long nmodes_total,
+                                                          const int* __restrict__ bin_start, int nell, int seg_len,
+                                                          double* __restrict__ partial) {
+    __shared__ double red[NZ * 3][kXbThreads];
+    const int b = blockIdx.x, seg = blockIdx.y, z0 = blockIdx.z * NZ, nz = min(NZ, nx - z0), tid = threadIdx.x;
     const long beg = bin_start[b] + (long)seg * seg_len;
     const long end = min((long)bin_start[b + 1], beg + seg_len);
-    const C<T>* __restrict__ Xz = X + (long)blockIdx.z * x_stride;
-    double* out = partial + (((long)blockIdx.z * gridDim.x + b) * gridDim.y + seg) * nell;
+    const C<T>* __restrict__ Xz = X + (long)z0 * x_stride;
+    auto out = [&](int z) { return partial + (((long)(z0 + z) * gridDim.x + b) * gridDim.y + seg) * nell; };
     if (beg >= end) {
-        if (threadIdx.x < nell) out[threadIdx.x] = 0.0;
+        if (tid < nell)
+            for (int z = 0; z < nz; ++z) out(z)[tid] = 0.0;
         return;
     }
-    double s[3] = {0.0, 0.0, 0.0};
-#pragma unroll 4
-    for (long m = beg + threadIdx.x; m < end; m += 256) {
+    double s[NZ][3] = {};
+#pragma unroll NZ == 1 ? 4 : 2
+    for (long m = beg + tid; m < end; m += kXbThreads) {
         const int o = offs[m];
-        const C<T> x = Xz[o], a = A[o];
-        const double p = (double)x.x * (double)a.x + (double)x.y * (double)a.y;
+        const C<T> a = A[o];
+        C<T> x[NZ];
 #pragma unroll
-        for (int l = 0; l < 3; ++l)
-            if (l < nell) s[l] += coef[(long)l * nmodes_total + m] * p;
+        for (int z = 0; z < NZ; ++z) x[z] = Xz[(long)(z < nz ? z : 0) * x_stride + o];
+        double c[3];
+#pragma unroll
+        for (int l = 0; l < 3; ++l) c[l] = l < nell ? coef[(long)l * nmodes_total + m] : 0.0;
+        const double ax = widen(a.x), ay = widen(a.y);
+#pragma unroll
+        for (int z = 0; z < NZ; ++z) {
+            if (z >= nz) break;
+            const double p = widen(x[z].x) * ax + widen(x[z].y) * ay;
+#pragma unroll
+            for (int l = 0; l < 3; ++l)
+                if (l < nell) s[z][l] += c[l] * p;
+        }
     }
 #pragma unroll
-    for (int l = 0; l < 3; ++l) {
-        if (l >= nell) break;
-        red[threadIdx.x] = s[l];
-        __syncthreads();
-        for (int w = 128; w > 0; w >>= 1) {
-            if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[l] = red[0];
-        __syncthreads();
+    for (int z = 0; z < NZ; ++z)
+#pragma unroll
+        for (int l = 0; l < 3; ++l) red[z * 3 + l][tid] = s[z][l];
+    __syncthreads();
+    const int lane = tid & 31;
+    for (int v = tid >> 5; v < nz * 3; v += kXbThreads / 32) {
+        const int z = v / 3, l = v - z * 3;
+        if (l >= nell) continue;
+        double t = red[v][lane];
+#pragma unroll
+        for (int w = 32; w < kXbThreads; w += 32) t += red[v][lane + w];
+#pragma unroll
+        for (int w = 16; w > 0; w >>= 1) t += __shfl_down_sync(0xffffffffu, t, w);
+        if (lane == 0) out(z)[l] = t;
     }
 }
 
