@@ -62,11 +62,19 @@ inline ContractGeom contract_geom_rows(int nb, int npairs, int nh, long ncell) {
 
 // Dynamic shared memory: products [kCH][rps], singles [kCH][nhp], maps [nb][kGS]; at the end the tiles' sums of one
 // replica (FP64; only with replicas, then at most 128 tiles) in the place of the products.
+constexpr size_t kMaxSmem = 227 * 1024;
+template <typename T> __host__ __device__ inline size_t contract_work(const ContractGeom& G) {
+    return ((size_t)kCH * G.rps + (size_t)kCH * G.nhp + (size_t)G.nb * kGS) * sizeof(T);
+}
+// Behind them a row of zeros and the places of the rows' maps, where shared memory has room for these (it has but for
+// about 800 FP64 rows and more; the pairs are then looked up a product).
+template <typename T> __host__ __device__ inline size_t contract_table(const ContractGeom& G) {
+    const size_t n = kGS * sizeof(T) + (size_t)G.rows_cta * sizeof(int2) + 16;
+    return contract_work<T>(G) + n + 16 <= kMaxSmem ? n : 0;
+}
 template <typename T> inline size_t contract_smem(const ContractGeom& G) {
-    const size_t work = ((size_t)kCH * G.rps + (size_t)kCH * G.nhp + (size_t)(G.nb + 1) * kGS) * sizeof(T) +
-                        (size_t)G.rows_cta * sizeof(int2) + 16;
     const size_t sums = G.kg > 1 ? (size_t)G.rt * G.ct * kTM * kTN * sizeof(double) : 0;
-    return std::max(work, sums) + 16;
+    return std::max(contract_work<T>(G) + contract_table<T>(G), sums) + 16;
 }
 
 template <typename T> struct Vec4;
@@ -105,16 +113,19 @@ __global__ void __launch_bounds__(256, 2) k_contract(const T* __restrict__ g, co
     const int RPS = G.rps, NHP = G.nhp;
     T* sP = reinterpret_cast<T*>(smem_raw);          // [kCH][RPS]
     T* sH = sP + (size_t)kCH * RPS;                   // [kCH][NHP]
-    T* sG = sH + (size_t)kCH * NHP;                   // [nb + 1][kGS], the last row zero
-    // places of the rows' maps in sG (the zero row beyond the last pair)
+    T* sG = sH + (size_t)kCH * NHP;                   // [nb][kGS], and with a table a row of zeros
+    // table: places of the rows' maps in sG (the zeros beyond the last pair)
+    const bool table = contract_table<T>(G) != 0;
     int2* sO = reinterpret_cast<int2*>((reinterpret_cast<uintptr_t>(sG + (G.nb + 1) * kGS) + 15) & ~(uintptr_t)15);
     const int r0 = blockIdx.x * G.rows_cta;
-    for (int i = tid; i < G.rows_cta; i += 256) {
-        const bool in = r0 + i < G.npairs;
-        const short2 jk = in ? pairs[r0 + i] : make_short2(0, 0);
-        sO[i] = in ? make_int2(jk.x * kGS, jk.y * kGS) : make_int2(G.nb * kGS, G.nb * kGS);
+    if (table) {
+        for (int i = tid; i < G.rows_cta; i += 256) {
+            const bool in = r0 + i < G.npairs;
+            const short2 jk = in ? pairs[r0 + i] : make_short2(0, 0);
+            sO[i] = in ? make_int2(jk.x * kGS, jk.y * kGS) : make_int2(G.nb * kGS, G.nb * kGS);
+        }
+        if (tid < kGS) sG[G.nb * kGS + tid] = T(0);
     }
-    if (tid < kGS) sG[G.nb * kGS + tid] = T(0);
     const long cbeg = (long)blockIdx.y * G.cells_cta;
     const long cend = min(ncell, cbeg + G.cells_cta);
     // tile (rt, ct) of replica kq; threads beyond the last replica only stage
@@ -173,15 +184,24 @@ __global__ void __launch_bounds__(256, 2) k_contract(const T* __restrict__ g, co
         }
         __syncthreads();
         if (c0 + kCH < cend) fetch(c0 + kCH);
-        for (int q = warp; q < G.rows_cta / 4; q += 8) {
-            T v[4];
-#pragma unroll
-            for (int u = 0; u < 4; u += 2) {
-                const int4 o = *reinterpret_cast<const int4*>(sO + 4 * q + u);
-                v[u] = sG[o.x + lane] * sG[o.y + lane];
-                v[u + 1] = sG[o.z + lane] * sG[o.w + lane];
+        if (table) {
+            for (int q = warp; q < G.rows_cta / 4; q += 8) {
+                const int4 o = *reinterpret_cast<const int4*>(sO + 4 * q), p = *reinterpret_cast<const int4*>(sO + 4 * q + 2);
+                const T v[4] = {sG[o.x + lane] * sG[o.y + lane], sG[o.z + lane] * sG[o.w + lane],
+                                sG[p.x + lane] * sG[p.y + lane], sG[p.z + lane] * sG[p.w + lane]};
+                Vec4<T>::store(sP + lane * RPS + 4 * q, v);
             }
-            Vec4<T>::store(sP + lane * RPS + 4 * q, v);
+        } else {
+            for (int q = warp; q < G.rows_cta / 4; q += 8) {
+                T v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int gp = r0 + 4 * q + u;
+                    const short2 jk = gp < G.npairs ? pairs[gp] : make_short2(0, 0);
+                    v[u] = gp < G.npairs ? sG[jk.x * kGS + lane] * sG[jk.y * kGS + lane] : T(0);
+                }
+                Vec4<T>::store(sP + lane * RPS + 4 * q, v);
+            }
         }
         if (!h) {
             for (int q = warp; q < G.ct * (kTN / 4); q += 8) {
