@@ -237,20 +237,11 @@ __device__ __forceinline__ void stage_twiddles(C<T>* dst, const C<T>* __restrict
     for (int i = tid; i < n; i += nthr) dst[i] = tw[i];
 }
 
-// One-shot bulk copy global -> shared through the TMA engine (cp.async.bulk: both addresses 16-byte aligned, size a
-// multiple of 16), completing on an mbarrier with the byte count; and the bounded wait on that barrier.
+// Bounded wait on an mbarrier that a bulk copy completes.
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void bulk_bar_init(uint64_t* bar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tfence.mbarrier_init.release.cluster;" ::"r"(smem_addr(bar))
                  : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "fence.proxy.async.shared::cta;\n\t"
-        "mbarrier.arrive.expect_tx.shared::cta.b64 _, [%2], %3;\n\t"
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %3, [%2];" ::"r"(smem_addr(dst)),
-        "l"(src), "r"(smem_addr(bar)), "r"(bytes)
-        : "memory");
 }
 // Waits for phase `parity` of the barrier; false after `limit` polls (the copy never landed).
 __device__ __forceinline__ bool bulk_wait(uint64_t* bar, uint32_t parity, unsigned limit) {
@@ -265,7 +256,6 @@ __device__ __forceinline__ bool bulk_wait(uint64_t* bar, uint32_t parity, unsign
     }
     return false;
 }
-constexpr unsigned kBulkSpinLimit = 1u << 22;
 // Self-test of the staging wait: a barrier armed for 16 bytes that no copy delivers (none is issued); the bounded
 // wait gives up and raises the flag.
 static __global__ void k_bulk_wait_selftest(int* err, unsigned limit) {
@@ -669,245 +659,6 @@ __global__ void __launch_bounds__(256) k_inv_z256(ZInvBatch batch, long nlines, 
 }
 
 // ------------------------------------------------------------------------------------------------
-// z-pass, inverse (C2R), length 288 = 12 x 24, register-resident: the same result as k_inv_z (packing of line pairs,
-// kz = 0 and n/2 treatment) as a two-stage Cooley-Tukey transform.  With k = t + 12 j and n = n1 + 24 n2,
-//   z[n1 + 24 n2] = sum_t w12^(t n2) [ w288^(t n1) sum_j Z[t + 12 j] w24^(j n1) ]      (w_m = e^{+2 pi i / m}),
-// so a group of 12 threads transforms one packed line pair: thread t takes the 24-point DFT over j of its points
-// (in registers, as 3 x 8) and the twiddles w288^(t n1) (read once per thread from the table and kept in registers),
-// the groups exchange through shared memory, and thread t takes the 12-point DFTs (as 3 x 4) of rows n1 = t and
-// t + 12; a last exchange through shared memory makes the two real output lines coalesced (16-byte stores).  A CTA
-// of 192 threads takes 16 line pairs per round and `ppc` line pairs of one item (blockIdx.y) in all.
-
-// e^{i m pi / 12} for m = 0 .. 14 (multiples of 15 degrees; closed forms of cos / sin 15, 30, 45 degrees)
-__host__ __device__ constexpr double root24_re(int m) {
-    constexpr double c15 = 0.96592582628906829, s15 = 0.25881904510252076, c30 = 0.86602540378443865,
-                     c45 = 0.70710678118654752;
-    constexpr double t[15] = {1.0, c15, c30, c45, 0.5, s15, 0.0, -s15, -0.5, -c45, -c30, -c15, -1.0, -c15, -c30};
-    return t[m];
-}
-__host__ __device__ constexpr double root24_im(int m) {
-    constexpr double c15 = 0.96592582628906829, s15 = 0.25881904510252076, c30 = 0.86602540378443865,
-                     c45 = 0.70710678118654752;
-    constexpr double t[15] = {0.0, s15, 0.5, c45, c30, c15, 1.0, c15, c30, c45, 0.5, s15, 0.0, -s15, -0.5};
-    return t[m];
-}
-// a * e^{DIR 2 pi i m / 24}
-template <typename T, int DIR>
-__device__ __forceinline__ C<T> rot24(C<T> a, int m) {
-    const T c = T(root24_re(m)), s = T(DIR * root24_im(m));
-    return mk<T>(a.x * c - a.y * s, a.x * s + a.y * c);
-}
-
-// X[n] = sum_j x[j] e^{DIR 2 pi i j n / 24}, natural order in and out: j = 3a + b, n = c + 8d.
-template <typename T, int DIR>
-__device__ __forceinline__ void dft24(C<T>* x) {
-    C<T> A[3][8];
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-#pragma unroll
-        for (int a = 0; a < 8; ++a) A[b][a] = x[3 * a + b];
-        dft<T, DIR>(A[b], 8);
-    }
-#pragma unroll
-    for (int b = 1; b < 3; ++b)
-#pragma unroll
-        for (int c = 1; c < 8; ++c) A[b][c] = rot24<T, DIR>(A[b][c], b * c);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        C<T> y[3] = {A[0][c], A[1][c], A[2][c]};
-        dft<T, DIR>(y, 3);
-        x[c] = y[0];
-        x[c + 8] = y[1];
-        x[c + 16] = y[2];
-    }
-}
-
-// X[n] = sum_j x[j] e^{DIR 2 pi i j n / 12}, natural order: j = 3a + b, n = c + 4d (w12^m = w24^(2m)).
-template <typename T, int DIR>
-__device__ __forceinline__ void dft12(C<T>* x) {
-    C<T> A[3][4];
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a) A[b][a] = x[3 * a + b];
-        dft<T, DIR>(A[b], 4);
-    }
-#pragma unroll
-    for (int b = 1; b < 3; ++b)
-#pragma unroll
-        for (int c = 1; c < 4; ++c) A[b][c] = rot24<T, DIR>(A[b][c], 2 * b * c);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        C<T> y[3] = {A[0][c], A[1][c], A[2][c]};
-        dft<T, DIR>(y, 3);
-        x[c] = y[0];
-        x[c + 4] = y[1];
-        x[c + 8] = y[2];
-    }
-}
-
-// 16-byte and 8-byte asynchronous global -> shared copies (cp.async; completion by commit / wait_group).
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Copies the `bytes` (a multiple of 8) at src to dst with the CTA's threads: 16-byte pieces, then an 8-byte tail.
-__device__ __forceinline__ void stage_block(unsigned char* dst, const unsigned char* src, long bytes, int tid, int nthr) {
-    const long n16 = bytes >> 4;
-    for (long i = tid; i < n16; i += nthr) cp_async16(dst + 16 * i, src + 16 * i);
-    if ((bytes & 15) && tid == 0) cp_async8(dst + 16 * n16, src + 16 * n16);
-    cp_async_commit();
-}
-
-constexpr int kZ288Threads = 192, kZ288Pairs = 16, kZ288Kmax = 145;
-// exchange buffer of a group: 24 rows of 13 (row stride 13: the 12 threads of a group read 12 rows conflict-free),
-// groups 316 float2 apart (316 = 12 mod 16: the two groups of a half-warp cover the 32 banks exactly)
-constexpr int kZ288Rs = 13, kZ288Gs = 316;
-// dynamic shared memory: twiddle table [288] float2, exchange buffers [16][316] float2, the staging barrier (16
-// bytes), input stage [32 lines][kin] (16-byte aligned: (288 + 16 x 316) x 8 + 16 = 42768 bytes in)
-inline size_t z288_smem(int kin_max) {
-    return (size_t)(288 + kZ288Pairs * kZ288Gs + 2 + 2 * kZ288Pairs * kin_max) * sizeof(float2);
-}
-
-static __global__ void __launch_bounds__(192, 3) k_inv_z288(ZInvBatch batch, long nlines, float scale,
-                                                           const float* __restrict__ mulout,
-                                                           const float2* __restrict__ twg, int ppc, int* err) {
-    constexpr int N = 288, TG = 12, P = 24, G = kZ288Pairs, RS = kZ288Rs, GS = kZ288Gs;
-    static_assert((TG - 1) * (P - 1) < N, "twiddle index t n1 stays below N");
-    extern __shared__ __align__(16) float2 z288_dyn[];
-    float2* stw = z288_dyn;                           // e^{-2 pi i m / 288}
-    float2* sbuf = z288_dyn + N;                      // exchange buffers
-    uint64_t* sbar = reinterpret_cast<uint64_t*>(sbuf + G * GS);   // completion barrier of the staging copies
-    float2* stage = sbuf + G * GS + 2;                // the round's input lines, [2 G][kin]
-    const ZInvItem item = batch.it[blockIdx.y];
-    const float2* __restrict__ in = static_cast<const float2*>(item.in);
-    float* __restrict__ out = static_cast<float*>(item.out);
-    const int kin = item.kin;                         // <= kin_max of the launch (<= 145, the Hermitian half)
-    const int tid = threadIdx.x, g = tid / TG, t = tid - g * TG;
-    float2* buf = sbuf + g * GS;
-    for (int i = tid; i < N; i += kZ288Threads) stw[i] = twg[i];   // visible after the first round's barrier
-    const long npairs = (nlines + 1) / 2;
-    const long p_beg = (long)blockIdx.x * ppc;
-    const long p_end = min(npairs, p_beg + ppc);
-    // A round's input lines, 2q .. min(2 (q + G), nlines) - 1, are one contiguous block: with an even line count
-    // (an even number of lines a round, 16 kin bytes a line pair) and a 16-byte aligned item, one bulk copy by the
-    // TMA engine stages it (completion on sbar); otherwise every thread issues its share of 16-byte cp.async copies.
-    const bool bulk = (nlines % 2 == 0) && (reinterpret_cast<uintptr_t>(in) & 15) == 0;
-    uint32_t phase = 0;
-    if (bulk && tid == 0) bulk_bar_init(sbar);
-    __syncthreads();                                  // the barrier is initialised before its first use
-    auto issue = [&](long q) {
-        const long l0 = 2 * q, l1 = min(2 * min(q + G, p_end), nlines);
-        const long bytes = (l1 - l0) * kin * (long)sizeof(float2);
-        if (bulk) {
-            if (tid == 0) bulk_g2s(stage, in + l0 * kin, (uint32_t)bytes, sbar);
-        } else {
-            stage_block(reinterpret_cast<unsigned char*>(stage), reinterpret_cast<const unsigned char*>(in + l0 * kin),
-                        bytes, tid, kZ288Threads);
-        }
-    };
-    if (p_beg < p_end) issue(p_beg);
-    for (long p0 = p_beg; p0 < p_end; p0 += G) {
-        const long p = p0 + g;
-        const bool act = p < p_end;
-        if (bulk) {
-            // bounded wait for the round's copy; every thread takes the same decision (the barrier below)
-            const bool landed = bulk_wait(sbar, phase, kBulkSpinLimit);
-            phase ^= 1u;
-            if (!__syncthreads_and(landed)) {
-                if (tid == 0) {
-                    atomicExch(err, 1);
-                    bulk_wait(sbar, phase ^ 1u, kBulkSpinLimit);   // let the copy in flight land before exiting
-                }
-                return;
-            }
-        } else {
-            cp_async_wait_all();
-            __syncthreads();                          // the round's lines are in `stage`
-        }
-        float2 v[P];
-        {
-            const bool has2 = act && 2 * p + 1 < nlines;
-            const float2* in1 = stage + (2 * g) * kin;
-            const float2* in2 = in1 + kin;
-#pragma unroll
-            for (int j = 0; j < P; ++j) {
-                const int k = t + TG * j;
-                float2 z = make_float2(0.f, 0.f);
-                if (act) {
-                    if (k == 0 || 2 * k == N) {
-                        if (k < kin) z = make_float2(in1[k].x, has2 ? in2[k].x : 0.f);
-                    } else if (k < kin) {
-                        const float2 a = in1[k];
-                        const float2 b = has2 ? in2[k] : make_float2(0.f, 0.f);
-                        z = make_float2(a.x - b.y, a.y + b.x);
-                    } else if (N - k < kin) {
-                        const float2 a = in1[N - k];
-                        const float2 b = has2 ? in2[N - k] : make_float2(0.f, 0.f);
-                        z = make_float2(a.x + b.y, b.x - a.y);
-                    }
-                }
-                v[j] = z;
-            }
-        }
-        __syncthreads();                              // every thread has its points: refill `stage`
-        if (p0 + G < p_end) issue(p0 + G);
-        // stage 1: 24-point DFT over j, twiddle w288^(t n1); rows n1 of the group's exchange buffer
-        dft24<float, +1>(v);
-        // twiddle w288^(t n1) = conj(tw[t n1]) (t n1 <= 11 x 23 < N: no reduction modulo N)
-#pragma unroll
-        for (int n1 = 1; n1 < P; ++n1) v[n1] = mulc<float>(v[n1], stw[t * n1]);
-#pragma unroll
-        for (int n1 = 0; n1 < P; ++n1) buf[n1 * RS + t] = v[n1];
-        __syncthreads();
-        // stage 2: 12-point DFTs over t of rows n1 = t and t + 12
-        float2 o[2][TG];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-#pragma unroll
-            for (int u = 0; u < TG; ++u) o[h][u] = buf[(t + 12 * h) * RS + u];
-            dft12<float, +1>(o[h]);
-        }
-        __syncthreads();
-        // outputs: z[n1 + 24 n2] -> real parts to line 2p, imaginary parts to line 2p + 1 (staged for coalescing)
-        float* re = reinterpret_cast<float*>(buf);
-        float* im = re + N;
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int n2 = 0; n2 < TG; ++n2) {
-                const int n = t + 12 * h + 24 * n2;
-                re[n] = o[h][n2].x * scale;
-                im[n] = o[h][n2].y * scale;
-            }
-        __syncthreads();
-        constexpr int Q = N / 4;                         // float4 per line
-        for (int q = tid; q < G * 2 * Q; q += kZ288Threads) {
-            const int gg = q / (2 * Q), r = q - gg * 2 * Q;
-            const int side = r / Q, e4 = r - side * Q;
-            const long pp = p0 + gg;
-            const long l = 2 * pp + side;
-            if (pp >= p_end || l >= nlines) continue;
-            float4 a = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(sbuf + gg * GS) + side * N + 4 * e4);
-            if (mulout) {
-                const float* m = mulout + l * N + 4 * e4;
-                a.x *= m[0]; a.y *= m[1]; a.z *= m[2]; a.w *= m[3];
-            }
-            *reinterpret_cast<float4*>(out + l * N + 4 * e4) = a;
-        }
-        // (the next round's first __syncthreads orders these reads of sbuf before its writes)
-    }
-    cp_async_wait_all();
-}
-
-// ------------------------------------------------------------------------------------------------
 // Strided column pass (y or x axis).  Each CTA transforms TK consecutive columns of one outer slab.
 //   forward (DIR = -1): input positions 0..n-1 at in[o*in_os + i*in_es + c]; keeps wave numbers
 //                       f in out_rng, stored at out[o*out_os + (f - lo)*out_es + c].
@@ -1002,63 +753,6 @@ __global__ void __launch_bounds__(256) k_col(ColBatch batch, FftPlan plan, const
             if (c < nc) out[(long)i * item.out_es + c] = z[idx];
         }
     }
-}
-
-// ------------------------------------------------------------------------------------------------
-// Inverse y pass on 288-point columns (FP32), register-resident: the same two-stage transform as k_inv_z288
-// (k = t + 12 j, n = n1 + 24 n2; a 24-point DFT over j, the twiddle w288^(t n1), a 12-point DFT over t), applied to
-// complex columns.  A CTA of 192 threads takes 16 consecutive columns (wave numbers kz) of one x slab of one bin:
-// thread (t, c) = (tid / 16, tid % 16) loads its 24 points straight from the bin's pruned input (rows = the bin's
-// y wave numbers; zero outside them), so a warp reads and writes two rows of 16 consecutive columns (128 bytes
-// each) at a time; the two stages exchange through shared memory (one 24 x 13 buffer a column).
-constexpr int kY288Cols = 16, kY288Threads = 12 * kY288Cols;
-// exchange buffers 313 float2 apart (>= 24 x 13; odd, so the 16 columns a half-warp touches fall on distinct bank
-// pairs: 2 x 313 = 18 mod 32 words)
-constexpr int kY288Gs = 313;
-inline size_t y288_smem() { return (size_t)(288 + kY288Cols * kY288Gs) * sizeof(float2); }
-
-static __global__ void __launch_bounds__(192, 3) k_inv_y288(ColBatch batch, const float2* __restrict__ twg) {
-    constexpr int N = 288, TG = 12, P = 24, TC = kY288Cols, RS = kZ288Rs, GS = kY288Gs;
-    static_assert(P * RS <= GS, "a column's exchange buffer holds 24 rows of 13");
-    static_assert((TG - 1) * (P - 1) < N, "twiddle index t n1 stays below N");
-    extern __shared__ __align__(16) float2 y288_dyn[];
-    float2* stw = y288_dyn;                           // e^{-2 pi i m / 288}
-    const ColItem item = batch.it[blockIdx.z];
-    const int c0 = blockIdx.x * TC, o = blockIdx.y;
-    if (c0 >= item.ncols || o >= item.nouter) return;   // uniform over the CTA
-    const int tid = threadIdx.x, t = tid / TC, c = tid - t * TC;
-    float2* buf = y288_dyn + N + c * GS;              // this column's exchange buffer
-    for (int i = tid; i < N; i += kY288Threads) stw[i] = twg[i];
-    const bool act = c0 + c < item.ncols;
-    const float2* __restrict__ in = static_cast<const float2*>(item.in) + (long)o * item.in_os + c0 + c;
-    float2* __restrict__ out = static_cast<float2*>(item.out) + (long)o * item.out_os + c0 + c;
-    // points k = t + 12 j: wave number f = k (k < 144) or k - 288, input row f - lo when inside the bin's range
-    float2 v[P];
-#pragma unroll
-    for (int j = 0; j < P; ++j) {
-        const int k = t + TG * j;
-        const int i = (k < N / 2 ? k : k - N) - item.rng.lo;
-        v[j] = (act && i >= 0 && i < item.rng.cnt) ? in[(long)i * item.in_es] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();                                  // the twiddle table is in place
-    dft24<float, +1>(v);
-#pragma unroll
-    for (int n1 = 1; n1 < P; ++n1) v[n1] = mulc<float>(v[n1], stw[t * n1]);
-#pragma unroll
-    for (int n1 = 0; n1 < P; ++n1) buf[n1 * RS + t] = v[n1];
-    __syncthreads();
-    float2 w[2][TG];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-#pragma unroll
-        for (int u = 0; u < TG; ++u) w[h][u] = buf[(t + 12 * h) * RS + u];
-        dft12<float, +1>(w[h]);
-    }
-    if (!act) return;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int n2 = 0; n2 < TG; ++n2) out[(long)(t + 12 * h + 24 * n2) * item.out_es] = w[h][n2];
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1168,59 +862,6 @@ __global__ void __launch_bounds__(256) k_inv_x_filter(XInvBatch batch, const C<T
         const int c = idx % TK, i = idx / TK;
         if (c < nc) out[(long)i * ncols + c0 + c] = z[idx];
     }
-}
-
-// The filter + x IFFT on 288-point x lines (FP32), register-resident like k_inv_y288: a CTA of 192 threads takes 16
-// consecutive columns (points (n_y, n_z) of the bin's box, n_z fastest) of one bin; thread (t, c) forms its 24
-// filtered points k = t + 12 j (wave number n_x = k or k - 288, zero outside the bin's x range and the bin) and
-// takes the two-stage 288-point transform; rows of 16 consecutive columns are written (128 bytes).
-static __global__ void __launch_bounds__(192, 3) k_inv_x288_filter(XInvBatch batch, const float2* __restrict__ spec,
-                                                                  AxisRange gx, AxisRange gy, AxisRange gz,
-                                                                  float scale, const float2* __restrict__ twg) {
-    constexpr int N = 288, TG = 12, P = 24, TC = kY288Cols, RS = kZ288Rs, GS = kY288Gs;
-    extern __shared__ __align__(16) float2 x288_dyn[];
-    float2* stw = x288_dyn;                           // e^{-2 pi i m / 288}
-    const XInvItem item = batch.it[blockIdx.y];
-    const int ncols = item.ry.cnt * item.rz.cnt;
-    const int c0 = blockIdx.x * TC;
-    if (c0 >= ncols) return;                          // uniform over the CTA
-    const int tid = threadIdx.x, t = tid / TC, c = tid - t * TC;
-    float2* buf = x288_dyn + N + c * GS;
-    for (int i = tid; i < N; i += kY288Threads) stw[i] = twg[i];
-    const int cc = c0 + c;
-    const bool act = cc < ncols;
-    const int fy = act ? item.ry.lo + cc / item.rz.cnt : 0;
-    const int fz = act ? item.rz.lo + cc % item.rz.cnt : 0;
-    float2 v[P];
-#pragma unroll
-    for (int j = 0; j < P; ++j) {
-        const int k = t + TG * j;
-        const int fx = k < N / 2 ? k : k - N;
-        const int i = fx - item.rx.lo;
-        float2 x = make_float2(0.f, 0.f);          // stays zero outside the bin
-        if (act && i >= 0 && i < item.rx.cnt) x_filter_value<float>(item, spec, gx, gy, gz, scale, fx, fy, fz, x);
-        v[j] = x;
-    }
-    __syncthreads();                                  // the twiddle table is in place
-    dft24<float, +1>(v);
-#pragma unroll
-    for (int n1 = 1; n1 < P; ++n1) v[n1] = mulc<float>(v[n1], stw[t * n1]);
-#pragma unroll
-    for (int n1 = 0; n1 < P; ++n1) buf[n1 * RS + t] = v[n1];
-    __syncthreads();
-    float2 w[2][TG];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-#pragma unroll
-        for (int u = 0; u < TG; ++u) w[h][u] = buf[(t + 12 * h) * RS + u];
-        dft12<float, +1>(w[h]);
-    }
-    if (!act) return;
-    float2* __restrict__ out = static_cast<float2*>(item.out) + cc;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int n2 = 0; n2 < TG; ++n2) out[(long)(t + 12 * h + 24 * n2) * ncols] = w[h][n2];
 }
 
 }  // namespace pb
