@@ -223,7 +223,14 @@ template <int N> struct Geo {
     static constexpr int kLineSmem = kLineSmem0 > kLineSmem1 ? kLineSmem0 : kLineSmem1;
 };
 
-// One column (thread (t, c) of the CTA: column c of TC): load(k) gives point k, store(n, X) takes the results.
+// Wave number of point k = t + step j of N (j of cnt steps): k below N / 2, k - N from there on.  The half is known at compile
+// time but for the middle j of an odd count.
+template <int N> __device__ __forceinline__ int wave(int k, int j, int cnt) {
+    return (2 * j + 1 == cnt ? 2 * k >= N : 2 * j >= cnt) ? k - N : k;
+}
+
+// One column (thread (t, c) of the CTA: column c of TC): load(k, f) gives point k, store(n, f, X) takes the results; f is
+// the point's wave number.
 template <int DIR, int N, class L, class S>
 __device__ __forceinline__ void col_fft(float2* buf, int t, int c, L load, S store) {
     using E = Geo<N>;
@@ -231,7 +238,7 @@ __device__ __forceinline__ void col_fft(float2* buf, int t, int c, L load, S sto
     if (t < Q) {
         float2 v[P];
 #pragma unroll
-        for (int j = 0; j < P; ++j) v[j] = load(t + Q * j);
+        for (int j = 0; j < P; ++j) v[j] = load(t + Q * j, wave<N>(t + Q * j, j, P));
         stage1<DIR, P, Q>(v, t);
 #pragma unroll
         for (int n1 = 0; n1 < P; ++n1) buf[(n1 * QR + t) * TC + c] = v[n1];
@@ -243,7 +250,7 @@ __device__ __forceinline__ void col_fft(float2* buf, int t, int c, L load, S sto
         for (int u = 0; u < Q; ++u) v[u] = buf[(t * QR + u) * TC + c];
         codelet<DIR, Q>(v);
 #pragma unroll
-        for (int n2 = 0; n2 < Q; ++n2) store(t + P * n2, v[n2]);
+        for (int n2 = 0; n2 < Q; ++n2) store(t + P * n2, wave<N>(t + P * n2, n2, Q), v[n2]);
     }
 }
 
@@ -259,21 +266,22 @@ __global__ void __launch_bounds__(Geo<N>::kColThreads, min_ctas(Geo<N>::kColThre
     const bool act = c0 + c < item.ncols;
     const float2* __restrict__ in = static_cast<const float2*>(item.in) + (long)o * item.in_os + c0 + c;
     float2* __restrict__ out = static_cast<float2*>(item.out) + (long)o * item.out_os + c0 + c;
-    const int lo = item.rng.lo, cnt = item.rng.cnt, in_es = (int)item.in_es, out_es = (int)item.out_es;
+    // 32-bit offsets (an outer index spans fewer than 2^31 elements); inactive columns keep nothing
+    const int lo = item.rng.lo;
+    const unsigned cnt = act ? item.rng.cnt : 0, in_es = (unsigned)item.in_es, out_es = (unsigned)item.out_es;
     col_fft<DIR, N>(
         f2_smem, t, c,
-        [&](int k) {
-            if (DIR < 0) return act ? in[(long)k * in_es] : make_float2(0.f, 0.f);
-            const int i = (k < N / 2 ? k : k - N) - lo;   // wave number of position k; zero outside the kept range
-            return act && i >= 0 && i < cnt ? in[(long)i * in_es] : make_float2(0.f, 0.f);
+        [&](int k, int f) {
+            if (DIR < 0) return act ? in[(unsigned)k * in_es] : make_float2(0.f, 0.f);
+            const unsigned i = (unsigned)(f - lo);    // zero outside the kept range
+            return i < cnt ? in[i * in_es] : make_float2(0.f, 0.f);
         },
-        [&](int n, float2 v) {
-            if (!act) return;
+        [&](int n, int f, float2 v) {
             if (DIR > 0) {
-                out[(long)n * out_es] = v;
+                if (act) out[(unsigned)n * out_es] = v;
             } else {
-                const int i = (n < N / 2 ? n : n - N) - lo;
-                if (i >= 0 && i < cnt) out[(long)i * out_es] = v;
+                const unsigned i = (unsigned)(f - lo);
+                if (i < cnt) out[i * out_es] = v;
             }
         });
 }
@@ -294,17 +302,17 @@ __global__ void __launch_bounds__(Geo<N>::kColThreads, min_ctas(Geo<N>::kColThre
     const int fy = act ? item.ry.lo + cc / item.rz.cnt : 0;
     const int fz = act ? item.rz.lo + cc % item.rz.cnt : 0;
     float2* __restrict__ out = static_cast<float2*>(item.out) + cc;
+    const int rlo = item.rx.lo;
+    const unsigned rcnt = act ? item.rx.cnt : 0;
     col_fft<+1, N>(
         f2_smem, t, c,
-        [&](int k) {
-            const int fx = k < N / 2 ? k : k - N;
-            const int i = fx - item.rx.lo;
+        [&](int, int fx) {
             float2 v = make_float2(0.f, 0.f);          // stays zero outside the bin
-            if (act && i >= 0 && i < item.rx.cnt) x_filter_value<float>(item, spec, gx, gy, gz, scale, fx, fy, fz, v);
+            if ((unsigned)(fx - rlo) < rcnt) x_filter_value<float>(item, spec, gx, gy, gz, scale, fx, fy, fz, v);
             return v;
         },
-        [&](int n, float2 v) {
-            if (act) out[(long)n * ncols] = v;
+        [&](int n, int, float2 v) {
+            if (act) out[(unsigned)(n * ncols)] = v;
         });
 }
 
@@ -327,13 +335,13 @@ __global__ void __launch_bounds__(Geo<N>::kColThreads, min_ctas(Geo<N>::kColThre
     const float2* __restrict__ p = pairs + (fy - gy.lo) * gz.cnt + (fz - gz.lo);
     const int xs = gy.cnt * gz.cnt;
     float2* __restrict__ out = item.out + cc;
+    const int rlo = item.rx.lo;
+    const unsigned rcnt = act ? item.rx.cnt : 0;
     col_fft<+1, N>(
         f2_smem, t, c,
-        [&](int k) {
-            const int fx = k < N / 2 ? k : k - N;
-            const int i = fx - item.rx.lo;
+        [&](int, int fx) {
             float2 v = make_float2(0.f, 0.f);
-            if (act && i >= 0 && i < item.rx.cnt) {
+            if ((unsigned)(fx - rlo) < rcnt) {
                 const int s = fx * fx + syz;
                 const long o = (long)(fx - gx.lo) * xs;
                 if (s >= item.clo && s <= item.chi) v = add<float>(v, p[item.pab + o]);
@@ -344,8 +352,8 @@ __global__ void __launch_bounds__(Geo<N>::kColThreads, min_ctas(Geo<N>::kColThre
             }
             return v;
         },
-        [&](int n, float2 v) {
-            if (act) out[(long)n * ncols] = v;
+        [&](int n, int, float2 v) {
+            if (act) out[(unsigned)(n * ncols)] = v;
         });
 }
 
