@@ -497,12 +497,13 @@ __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineTh
     // offset of line l from the observer in the plane
     auto plane = [&](long l, float& px, float& py) {
         const int ix = (int)((unsigned)l / (unsigned)batch.n1), iy = (int)l - ix * batch.n1;
-        px = ((float)ix + 0.5f) * batch.h[0] - batch.half - batch.obs[0];
-        py = ((float)iy + 0.5f) * batch.h[1] - batch.half - batch.obs[1];
+        px = ((float)(ix - batch.cell[0]) - batch.frac[0]) * batch.h[0];
+        py = ((float)(iy - batch.cell[1]) - batch.frac[1]) * batch.h[1];
     };
     float2 v[E::TG];
     if (t < Q && act) {
         const float c0 = item.am < 2 ? 1.f : 0.f, c1 = (item.am >> 1) == 1 ? 1.f : 0.f, c2 = item.am == 4 ? 1.f : 0.f;
+        const float tz = (float)(t - batch.cell[2]);
         const float o0 = item.am & 1 ? 0.f : 1.f, o1 = 1.f - o0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -513,7 +514,7 @@ __global__ void __launch_bounds__(Geo<N>::kLineThreads, min_ctas(Geo<N>::kLineTh
             const float rho2 = px * px + py * py, rho = sqrtf(rho2);
 #pragma unroll
             for (int j = 0; j < P; ++j) {
-                const float pz = ((float)(t + Q * j) + 0.5f) * batch.h[2] - batch.half - batch.obs[2];
+                const float pz = (tz + (float)(Q * j) - batch.frac[2]) * batch.h[2];
                 const float r2 = rho2 + pz * pz;
                 const bool at = r2 > 0.f;             // the z axis where the centre coincides with the observer
                 const float q = __frcp_rn(at ? r2 : 1.f);

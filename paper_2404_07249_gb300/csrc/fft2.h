@@ -73,7 +73,9 @@ struct YlmBatch {
     YlmItem it[16];
     const float *in, *w;         // w may be null
     int n1;                      // lines: (i, j) = (l / n1, l % n1)
-    float h[3], half, obs[3];    // cell centre (i + 1/2) h - half - obs, in units of the box side
+    // cell centre from the observer (i - cell - frac) h, in units of the box side: exact to FP32's last bit near the observer
+    float h[3], frac[3];
+    int cell[3];
 };
 struct ZMaskItem {
     const float2* in;            // [nlines][kin]

@@ -966,9 +966,12 @@ static int forward_ylm(polybin_ctx* ctx, const float* in, const float* w, int el
     z.n1 = N1;
     for (int a = 0; a < 3; ++a) {
         z.h[a] = 1.f / (float)ctx->N[a];
-        z.obs[a] = (float)(ctx->observer[a] / ctx->L);
+        // the observer in cell units, FP64's last digits dropped where it is a cell's centre
+        const double c = (ctx->observer[a] / ctx->L + 0.5) * ctx->N[a] - 0.5;
+        const double near = std::fabs(c) < 1e6 ? std::nearbyint(c) : 0.0, f = c - near;
+        z.cell[a] = (int)near;
+        z.frac[a] = std::fabs(f) < 1e-9 ? 0.f : (float)f;
     }
-    z.half = 0.5f;
     int nz = 0;
     for (int i = 0; i < cnt; ++nz) {                  // rows of m = -am and m = am, as far as both are in the batch
         const int am = (r0 + i + 1) / 2;
