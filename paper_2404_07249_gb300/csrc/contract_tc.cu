@@ -23,8 +23,8 @@
 // SM.  What bounds the kernel is shared memory: the producers' gathers (two 16-byte loads for every four products) and the
 // B operand's conversion; before, with 32-cell stages and one accumulator buffer, it was the barrier round trips of its
 // stages.  A stage is therefore 64 cells and the accumulators are double-buffered, so that no MMA waits for the epilogue.
-// Measured at 30 maps of 288^3 cells (two tiles): 3.88 ms with TF32 parts, 2.81 ms (and 0.39 ms for the maxima where the
-// maps come without them).  Tensor memory (512 columns) holds two accumulator buffers (2W columns a tile) and a ring of A
+// Measured at 30 maps of 288^3 cells (two tiles): 3.88 ms with TF32 parts, 2.81 ms with FP16 ones, 2.64 ms with the rows in
+// quads that share their loads (and 0.39 ms for the maxima where the maps come without them).  Tensor memory (512 columns) holds two accumulator buffers (2W columns a tile) and a ring of A
 // stages (64 columns a tile a stage).
 //
 // One CTA per SM over a contiguous range of cells, in stages of 64 cells (two TMA ring slots).  Warp roles, by
@@ -1111,16 +1111,26 @@ static std::vector<std::pair<int, int>> cut_tiles(const std::vector<NeedPair>& P
     return seg;
 }
 
-// Largest number of different maps of one bank group (map % 8) among v.
-static int bank_clash(const std::vector<int>& v) {
-    int most = 0;
-    for (int g = 0; g < 8; ++g) {
-        std::set<int> m;
-        for (int x : v)
-            if ((x & 7) == g) m.insert(x);
-        most = std::max(most, (int)m.size());
+// A set of maps (slot rows, at most 128), and the largest number of them in one bank group (map % 8).
+struct MapSet {
+    uint64_t w[2] = {0, 0};
+    void add(int m) { w[m >> 6] |= 1ull << (m & 63); }
+    void drop(int m) { w[m >> 6] &= ~(1ull << (m & 63)); }
+    bool has(int m) const { return (w[m >> 6] >> (m & 63)) & 1; }
+    int size() const { return __builtin_popcountll(w[0]) + __builtin_popcountll(w[1]); }
+    int clash() const {
+        int most = 0;
+        for (int g = 0; g < 8; ++g) {
+            const uint64_t m = 0x0101010101010101ull << g;
+            most = std::max(most, __builtin_popcountll(w[0] & m) + __builtin_popcountll(w[1] & m));
+        }
+        return most;
     }
-    return most;
+};
+static MapSet operator&(MapSet a, const MapSet& b) {
+    a.w[0] &= b.w[0];
+    a.w[1] &= b.w[1];
+    return a;
 }
 
 // Orders the rows [first, last) of a tile, sorted by (j, k), for the producers' gathers, which bound the kernel by shared
@@ -1131,78 +1141,82 @@ static int bank_clash(const std::vector<int>& v) {
 // quads a half-warp are taken to clash least; rows that form no quad follow, eight at a time that clash least.
 static void order_rows(std::vector<NeedPair>& need, int first, int last) {
     const std::vector<NeedPair> rest(need.begin() + first, need.begin() + last);
-    std::map<std::pair<int, int>, int> at;               // (j, k) -> row, of the rows left
-    std::vector<int> js;
-    for (size_t i = 0; i < rest.size(); ++i) {
-        at[{rest[i].j, rest[i].k}] = (int)i;
-        if (js.empty() || js.back() != rest[i].j) js.push_back(rest[i].j);
+    const int n = (int)rest.size();
+    std::vector<short> at(128 * 128, -1);                 // row of (j, k)
+    MapSet ks[128];                                       // the k of the rows left of every j
+    MapSet jset;
+    bool plain = true;                                    // maps in range and no pair twice
+    for (int i = 0; i < n; ++i) {
+        const int j = rest[i].j, k = rest[i].k;
+        if (j < 0 || k < 0 || j >= 128 || k >= 128) return;
+        plain = plain && !ks[j].has(k);
+        ks[j].add(k);
+        jset.add(j);
+        at[j * 128 + k] = (short)i;
     }
-    std::vector<int> order;
-    if (at.size() == rest.size()) {                       // (no pair twice)
+    std::vector<int> js, order;
+    for (int j = 0; j < 128; ++j)
+        if (jset.has(j)) js.push_back(j);
+    if (plain) {
         // quads: of all pairs of j the one with the most k in common first, so that few rows are left over
         struct Quad { int r[4], j[2], k[2]; };
         std::vector<Quad> quads;
         for (;;) {
-            int bj1 = -1, bj2 = -1;
-            std::vector<int> bk;
+            int b1 = -1, b2 = -1, most = 0;
             for (size_t x = 0; x < js.size(); ++x)
                 for (size_t y = x + 1; y < js.size(); ++y) {
-                    std::vector<int> ks;
-                    for (auto it = at.lower_bound({js[x], -1}); it != at.end() && it->first.first == js[x]; ++it)
-                        if (at.count({js[y], it->first.second})) ks.push_back(it->first.second);
-                    if (ks.size() / 2 > bk.size() / 2) { bk = ks; bj1 = js[x]; bj2 = js[y]; }
+                    const int c = (ks[js[x]] & ks[js[y]]).size() / 2;
+                    if (c > most) { most = c; b1 = js[x]; b2 = js[y]; }
                 }
-            if (bk.size() < 2) break;
-            for (size_t q = 0; q + 1 < bk.size(); q += 2) {
-                Quad d;
-                d.j[0] = bj1; d.j[1] = bj2; d.k[0] = bk[q]; d.k[1] = bk[q + 1];
-                for (int i = 0; i < 4; ++i) {
-                    const std::pair<int, int> key{d.j[i >> 1], d.k[i & 1]};
-                    d.r[i] = at[key];
-                    at.erase(key);
-                }
-                quads.push_back(d);
+            if (!most) break;
+            const MapSet both = ks[b1] & ks[b2];
+            for (int k = 0, k1 = -1, c = 0; c < 2 * most; ++k) {
+                if (!both.has(k)) continue;
+                ++c;
+                if (k1 < 0) { k1 = k; continue; }
+                quads.push_back({{at[b1 * 128 + k1], at[b1 * 128 + k], at[b2 * 128 + k1], at[b2 * 128 + k]}, {b1, b2}, {k1, k}});
+                for (int q : {k1, k}) { ks[b1].drop(q); ks[b2].drop(q); }
+                k1 = -1;
             }
         }
         std::vector<char> used(quads.size(), 0);
-        for (size_t n = 0; n < quads.size();) {
-            std::vector<int> mj, mk;
-            for (int g = 0; g < 4 && n < quads.size(); ++g, ++n) {
+        for (size_t done = 0; done < quads.size();) {
+            MapSet mj, mk;                                // of a half-warp
+            for (int g = 0; g < 4 && done < quads.size(); ++g, ++done) {
                 int best = -1, best_cost = 1 << 30;
-                for (size_t i = 0; i < quads.size(); ++i) {
+                for (size_t i = 0; i < quads.size() && best_cost > 2; ++i) {
                     if (used[i]) continue;
-                    std::vector<int> a = mj, b = mk;
-                    a.insert(a.end(), quads[i].j, quads[i].j + 2);
-                    b.insert(b.end(), quads[i].k, quads[i].k + 2);
-                    const int cost = bank_clash(a) + bank_clash(b);
+                    MapSet a = mj, b = mk;
+                    for (int q = 0; q < 2; ++q) { a.add(quads[i].j[q]); b.add(quads[i].k[q]); }
+                    const int cost = a.clash() + b.clash();
                     if (cost < best_cost) { best_cost = cost; best = (int)i; }
                 }
                 used[best] = 1;
-                mj.insert(mj.end(), quads[best].j, quads[best].j + 2);
-                mk.insert(mk.end(), quads[best].k, quads[best].k + 2);
+                for (int q = 0; q < 2; ++q) { mj.add(quads[best].j[q]); mk.add(quads[best].k[q]); }
                 order.insert(order.end(), quads[best].r, quads[best].r + 4);
             }
         }
     }
-    std::vector<char> used(rest.size(), 0);
+    std::vector<char> used(n, 0);
     for (int i : order) used[i] = 1;
-    for (std::vector<int> mj, mk; order.size() < rest.size();) {
+    MapSet mj, mk;                                        // of eight lanes
+    while ((int)order.size() < n) {
         int best = -1, best_cost = 1 << 30;
-        for (size_t i = 0; i < rest.size(); ++i) {
+        for (int i = 0; i < n && best_cost > 2; ++i) {
             if (used[i]) continue;
-            std::vector<int> a = mj, b = mk;
-            a.push_back(rest[i].j);
-            b.push_back(rest[i].k);
-            const int cost = bank_clash(a) + bank_clash(b);
-            if (cost < best_cost) { best_cost = cost; best = (int)i; }
+            MapSet a = mj, b = mk;
+            a.add(rest[i].j);
+            b.add(rest[i].k);
+            const int cost = a.clash() + b.clash();
+            if (cost < best_cost) { best_cost = cost; best = i; }
         }
         used[best] = 1;
-        mj.push_back(rest[best].j);
-        mk.push_back(rest[best].k);
+        mj.add(rest[best].j);
+        mk.add(rest[best].k);
         order.push_back(best);
-        if (order.size() % 8 == 0) { mj.clear(); mk.clear(); }
+        if (order.size() % 8 == 0) { mj = MapSet{}; mk = MapSet{}; }
     }
-    for (size_t i = 0; i < rest.size(); ++i) need[first + i] = rest[order[i]];
+    for (int i = 0; i < n; ++i) need[first + i] = rest[order[i]];
 }
 
 // Pure host layout of a plan (no CUDA calls): tiles, row groups, TMEM / shared-memory layout, the row table and the
