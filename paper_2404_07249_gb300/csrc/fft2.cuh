@@ -141,9 +141,10 @@ template <int DIR, int P, int Q> __device__ __forceinline__ void stage1(float2* 
 
 // ------------------------------------------------------------------------------------------------ columns
 
-// CTAs per SM asked of the compiler: registers for about 2.5 max(P, Q) complex values a thread.
+// CTAs per SM asked of the compiler: registers for about 2.5 max(P, Q) complex values a thread (17 and 18 points: 72, so that
+// three column CTAs of 288 threads fit an SM; with 80, two did, and the maps of 30 bins on 288^3 took 1.50 ms instead of 1.41).
 __host__ __device__ constexpr int min_ctas(int threads, int pts) {
-    const int regs = pts <= 12 ? 56 : (pts <= 16 ? 64 : (pts <= 20 ? 80 : 128));
+    const int regs = pts <= 12 ? 56 : (pts <= 16 ? 64 : (pts <= 18 ? 72 : (pts <= 20 ? 80 : 128)));
     const int n = 65536 / (threads * regs);
     return n < 1 ? 1 : n;
 }
