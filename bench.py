@@ -530,7 +530,7 @@ def main():
     nb = len(edges) - 1
     # dominant kernel: the triplet contraction over the cells of the alias-free contraction grid.  Algorithmic
     # work per launch: 2 flops per closed triplet per cell; algorithmic bytes: the n_b float32 maps read once.  The
-    # intensity (2 ntrip / (4 n_b) flop per byte, ~47 at 30 bins) is below the FP16 ridge (peak TF/s over peak
+    # intensity (2 ntrip / (4 n_b) flop per byte, ~47 at 30 bins) is below the BF16 ridge (peak TF/s over peak
     # TB/s, ~253), so the binding roof is HBM; the tensor-side rate is reported next to it.
     algo_flops = 2.0 * ntrip * Nc
     algo_bytes = 4.0 * nb * Nc
@@ -541,10 +541,10 @@ def main():
     roof["achieved"] = algo_bytes / t_con / 1e9 if t_con > 0 else None
     roof["frac"] = roof["achieved"] / roof["peak"] if roof["achieved"] else None
     if args.prec == "split":
-        peak_tf = float(peaks["bf16_tflops_sustained"])              # the split parts are FP16: the bf16 rate
+        peak_tf = float(peaks["bf16_tflops_sustained"])              # the split parts are BF16
         roof["tensor_side"] = {"achieved_tflops": algo_flops / t_con / 1e12 if t_con > 0 else None,
                                "peak_tflops": peak_tf,
-                               "peak_source": f"{peak_src} bf16 sustained (FP16 parts run at its rate)"}
+                               "peak_source": f"{peak_src} bf16 sustained"}
     else:
         alu = 152 * 128 * 2 * sm_max * 1e6 / 1e12 if args.prec == "fp32" else 152 * 2 * 2 * sm_max * 1e6 / 1e12
         roof["alu_side"] = {"achieved_tflops": algo_flops / t_con / 1e12 if t_con > 0 else None, "peak_tflops": alu}
@@ -565,7 +565,7 @@ def main():
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": {"split": "fp16 hi + lo (22 bits), fp32 and fp64 sums", "fp32": "f32", "fp64": "f64"}[args.prec],
+            "vs_baseline": None, "dtype": {"split": "bf16 x 3 (24 bits), fp32 and fp64 sums", "fp32": "f32", "fp64": "f64"}[args.prec],
             "data": "synthetic",
             "config": {"workload": w.name + ("_grid_override" if args.grid else ""), "grid": list(grid), "box": box,
                        "n_kbins": nb, "n_triplets": ntrip, "contraction_grid": list(cgrid),

@@ -44,7 +44,7 @@ typedef enum {
 typedef enum {
     POLYBIN_FP64 = 0,         /* FP64 FFTs and FP64 contraction: the plain double-precision GPU path        */
     POLYBIN_FP32 = 1,         /* FP32 FFTs, FP32 SIMT contraction with FP64 flushes and FP64 cross-CTA sums  */
-    POLYBIN_SPLIT_TF32X3 = 2  /* FP32 FFTs, tensor-core contraction of values split into two 11-bit parts     */
+    POLYBIN_SPLIT_TF32X3 = 2  /* FP32 FFTs, tensor-core contraction of values split into three BF16 parts     */
 } polybin_prec;
 
 /* Create a context for one grid and one set of k-bins.

@@ -1,4 +1,4 @@
-// Tensor-core (tcgen05, sm_103a) triplet contraction with two-term split products.
+// Tensor-core (tcgen05, sm_103a) triplet contraction with three-term split products.
 //
 // Computes sums M[(j, k)][i] = sum_x g_j(x) g_k(x) h_i(x) over the cells x (Sec. 4.3.1, eq. beta-def: the
 // real-space sum of the separable bispectrum; with h = g the entry of pair (b, c) and single a is S_abc).  The work
@@ -7,25 +7,30 @@
 // the triplet a <= b <= c is read from pair (b, c) and single a, which prunes the 465 pairs x 30 singles of a
 // 30-bin binning to 255 pairs in two tiles with windows of 16 and 32 singles.
 //
-// Arithmetic: the pair products A = g_j g_k (FP32) and the singles B are split as hi + lo with hi the value rounded to
-// 11 bits and lo the rounded remainder, 22 bits in all.  Both parts are FP16, which has TF32's 11 bits at twice its
-// tensor rate and half its storage.  FP16's short exponent is met by powers of two taken from the maps' maxima
-// (found by the z-pass that writes them, or by k_absmax): a row's products are scaled below 2^15, a single's values below 2^15, and the final FP64 sums scaled
-// back.  Values far below a map's maximum lose bits only below 2^-40 of it.  Per tile and K = 16 cells two MMAs of
-// N = 2W run, D[:, hi | lo] += A_lo . [B_hi | B_lo]^T and then A_hi . [B_hi | B_lo]^T: all four partial products.  The
-// tensor core's internal accumulation is not round-to-nearest, so D restarts every 64 cells, the A_lo terms first
-// (they add to a small sum); the epilogue adds D into FP32 registers (round-to-nearest) and those into FP64 shared
-// memory every 2048 cells.  Cross-CTA sums are FP64 in a fixed order (deterministic).
+// Arithmetic: the pair products A = g_j g_k (FP32) and the singles B are split into three BF16 parts of 8 bits each,
+// v = v1 + v2 + v3 (v1 and v2 rounded to nearest, v3 what is left): all 24 bits, with FP32's exponent, so that a value
+// keeps them however far it lies below the largest of its map.  (Two FP16 parts take fewer instructions and less storage,
+// but their exponent ends 2^-40 below a scale that has to be taken from the maps' maxima: two maps with a peak of 2^12 in
+// different cells left their products, and the sums, with an error of 3e-5.)  Per tile and K = 16 cells six MMAs of N = W run, smallest terms
+// first: A1 B3, A3 B1, A2 B2, A1 B2, A2 B1, A1 B1; the three left out are below 2^-26 of the product.  The
+// tensor core's internal accumulation is not round-to-nearest, so D restarts every 64 cells; the epilogue adds D into FP32
+// registers (round-to-nearest) and those into FP64 shared memory every 2048 cells.  Cross-CTA sums are FP64 in a fixed
+// order (deterministic).  Rows whose products' magnitude lies outside 2^-40 .. 2^40, and all singles, are scaled by powers of
+// two from the maps' maxima (found by the z-pass that writes them, or by k_absmax), which the final sums undo: products of
+// three maps of any magnitude then stay in FP32's range.
 //
 // Measured on this part (and shaping the design): an MMA issued from warp-uniform code with its operands in uniform
 // registers costs ~16-20 cycles at N = 32 (the tensor pipe's rate), but ~200 cycles from a one-lane branch, so the
 // issuing loop is warp-uniform (elect.sync inside the asm) and divide-free; tensor memory stores reach ~650 B/clk an
-// SM.  What bounds the kernel is shared memory: the producers' gathers (two 16-byte loads for every four products) and the
-// B operand's conversion; before, with 32-cell stages and one accumulator buffer, it was the barrier round trips of its
-// stages.  A stage is therefore 64 cells and the accumulators are double-buffered, so that no MMA waits for the epilogue.
-// Measured at 30 maps of 288^3 cells (two tiles): 3.88 ms with TF32 parts, 2.81 ms with FP16 ones, 2.64 ms with the rows in
-// quads that share their loads (and 0.39 ms for the maxima where the maps come without them).  Tensor memory (512 columns) holds two accumulator buffers (2W columns a tile) and a ring of A
-// stages (64 columns a tile a stage).
+// SM.  What bounds the kernel is instruction issue and the latency of the producers' chains (gathers, two 16-byte loads for
+// every four products, and eleven instructions of split for two products); the MMAs are not it (half of them: 5 % less).
+// So four producer groups, 16 cells at a time in few registers, and B warps that take every other stage; a stage is 64
+// cells and the accumulators are double-buffered, so that no MMA waits for the epilogue.  Measured, ms, at 30 maps
+// of 288^3 cells (two tiles) and at 20 maps of 192^3 (one tile): two TF32 parts in 32-cell stages 3.90 and 0.778, two
+// FP16 parts 2.64 and 0.459, three BF16 parts with two producer groups and 32 cells at a time 3.39 and 0.549 (3.22 and
+// 0.522 without a row scale of 1), with three groups and 16 cells 2.87 and 0.527, four groups 2.77 and 0.546, and B warps on
+// alternate stages 2.71 and 0.498.  Tensor memory (512 columns) holds two accumulator buffers (W columns a tile each) and
+// a ring of A stages (96 columns a tile a stage).
 //
 // One CTA per SM over a contiguous range of cells, in stages of 64 cells (two TMA ring slots).  Warp roles, by
 // warpgroup (setmaxnreg moves registers from warpgroup 0 to the producers):
@@ -33,15 +38,15 @@
 //                load, 128-byte swizzle) into an 8-slot shared-memory ring.
 //   warp 1       MMA issue: waits for the stage (converged), issues every tile's MMAs and commits them to the A
 //                stage's release barrier and the accumulator barrier.
-//   warps 4-7    the B operand: scale and split the singles of every stage into FP16 rows of 64 cells (128-byte swizzle),
-//                8 rows of hi and 8 of lo alternating.
+//   warps 4-7    the B operand: scale and split the singles into BF16 rows of 64 cells (128-byte swizzle), one block of
+//                rows a part; two warps a stage, one a slot.
 //   producers    groups of four warps; group g makes the 32 cells of slots g, g + kProdGroups, ..  A thread owns one TMEM
-//                lane, i.e. one row of every tile: it forms the pair products, splits them and writes hi / lo straight
+//                lane, i.e. one row of every tile: it forms the pair products, splits them and writes the parts straight
 //                into tensor memory (tcgen05.st: the A operand never touches shared memory).
 //   epilogue     four warps: after every stage read D with tcgen05.ld (each warp its TMEM lane quarter), release it to
 //                the issuer, accumulate.
 #include <cuda.h>
-#include <cuda_fp16.h>
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -63,12 +68,14 @@ constexpr int kRingSlots = 8;
 constexpr int kKC = 64;            // cells per A stage = two ring slots (four K = 16 MMA steps)
 constexpr int kMaxAStages = 6;
 constexpr int kSpill = 32;         // stages per FP32 register sum (2048 cells)
-constexpr int kDBuf = 2;           // accumulator buffers (the epilogue reads one while the MMAs fill the other)
-constexpr int kAcols = 64;         // tensor memory columns of a tile's A stage: hi and lo of 64 cells, two a column
-constexpr int kMaxTiles = 3;       // tiles per CTA
+constexpr int kParts = 3;          // BF16 parts of a value
+constexpr int kAccBufs = 2;        // accumulator buffers (the epilogue reads one while the MMAs fill the other)
+constexpr int kDBuf = 1;           // blocks of d_cols accumulator columns: a tile's 2W columns there hold both its buffers
+constexpr int kAcols = 32 * kParts;   // tensor memory columns of a tile's A stage: the parts of 64 cells, two a column
+constexpr int kMaxTiles = 2;       // tiles per CTA (three leave no room for two A stages)
 constexpr int kMaxUnits = 3;       // 16-column output units per CTA (16 FP32 sums each, in registers)
 constexpr int kMaxGroups = 4;      // row groups (grid.y)
-constexpr int kProdGroups = 2;     // producer warp groups; group g makes slots g, g + kProdGroups, .. (32 cells each)
+constexpr int kProdGroups = 4;     // producer warp groups; group g makes slots g, g + kProdGroups, .. (32 cells each)
 constexpr int kProdWarps = 4 * kProdGroups;
 constexpr int kEpiWarps = 4;
 // Warpgroup 0: TMA (warp 0), MMA issue (warp 1), two idle warps; then the B operand (four warps), the producers and the
@@ -76,10 +83,10 @@ constexpr int kEpiWarps = 4;
 constexpr int kBWarp0 = 4, kBWarps = 4;
 constexpr int kProdWarp0 = kBWarp0 + kBWarps;
 constexpr int kWarps = kProdWarp0 + kProdWarps + kEpiWarps;
-// Register split (setmaxnreg, per warpgroup): the CTA is launched with kRegsLaunch registers a thread; warpgroup 0 gives
-// registers back, the producers take them, the B warps and the epilogue keep what they have.
-constexpr int kRegsLaunch = 96, kRegsCtl = 40, kRegsB = 96, kRegsProd = 120;
-static_assert((kRegsCtl + kRegsB) * 128 + kRegsProd * 32 * kProdWarps + kRegsLaunch * 32 * kEpiWarps <= kRegsLaunch * 32 * kWarps,
+// Register split (setmaxnreg, per warpgroup): the CTA is launched with kRegsLaunch registers a thread; warpgroup 0 and the B
+// warps give registers back, the producers and the epilogue take them.
+constexpr int kRegsLaunch = 72, kRegsCtl = 24, kRegsB = 64, kRegsProd = 80, kRegsEpi = 88;
+static_assert((kRegsCtl + kRegsB) * 128 + kRegsProd * 32 * kProdWarps + kRegsEpi * 32 * kEpiWarps <= kRegsLaunch * 32 * kWarps,
               "register split exceeds the launch allocation");
 constexpr int kThreads = 32 * kWarps;
 constexpr int kMinSmem = 120 * 1024;   // one CTA per SM (the CTA allocates all 512 TMEM columns)
@@ -90,11 +97,11 @@ struct GroupDesc {
     int tile0;                 // first tile (row table index / 128)
     int ntiles, nunits, nA;    // tiles, 16-column units, A stages
     int unit_base;             // first unit of this group in the partial layout
-    int d_cols;                // TMEM columns of one accumulator buffer (kDBuf buffers at 0, d_cols, ...)
+    int d_cols;                // TMEM columns of the accumulators
     int a_col0;                // first TMEM column of the A ring
-    int bstage_bytes;          // bytes of one part (hi or lo) of a B stage: 128 for each row of the singles region
+    int bstage_bytes;          // bytes of one part of a B stage: 128 for each row of the singles region
     int tile_w[kMaxTiles];
-    int dm_col[kMaxTiles];     // TMEM column of tile t's accumulator: [B_hi 8 | B_lo 8] for every 8 singles (2W columns)
+    int dm_col[kMaxTiles];     // TMEM column of tile t's accumulators: two buffers of W columns
     int tile_s0[kMaxTiles];    // first single of tile t's window
     int unit_tile[kMaxUnits], unit_c[kMaxUnits];
 };
@@ -204,20 +211,26 @@ __device__ __forceinline__ void split_x2(uint64_t v, uint64_t& hi, uint64_t& lo)
     hi = (uint64_t)h0 | ((uint64_t)h1 << 32);
     lo = sub_x2(v, hi);
 }
-// Two values at once: v = hi + lo + (a remainder below 2^-22 |v|), hi and lo packed FP16 pairs rounded to nearest (the
-// first value in the low half); hi is 11 bits of v and v - hi is exact in FP32.
-__device__ __forceinline__ void split_h2(uint64_t v, uint32_t& hi, uint32_t& lo) {
-    const float v0 = __uint_as_float((uint32_t)v), v1 = __uint_as_float((uint32_t)(v >> 32));
-    const __half2 h = __floats2half2_rn(v0, v1);
-    hi = *reinterpret_cast<const uint32_t*>(&h);
-    const float2 f = __half22float2(h);
-    const uint64_t r = sub_x2(v, f2pack(f.x, f.y));
-    const __half2 l = __floats2half2_rn(__uint_as_float((uint32_t)r), __uint_as_float((uint32_t)(r >> 32)));
-    lo = *reinterpret_cast<const uint32_t*>(&l);
+// Two values at once: v = p1 + p2 + p3 exactly (24 bits of a normal number), packed BF16 pairs (the first value in the low
+// half): p1 and p2 rounded to nearest, each remainder exact in FP32; what is left then has at most 8 bits, so that p3 is its
+// upper half.
+__device__ __forceinline__ uint32_t bf16x2_rn(uint64_t v) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(__uint_as_float((uint32_t)(v >> 32))), "f"(__uint_as_float((uint32_t)v)));
+    return r;
+}
+__device__ __forceinline__ uint64_t bf16x2_value(uint32_t p) { return (uint64_t)(p << 16) | ((uint64_t)(p & 0xFFFF0000u) << 32); }
+__device__ __forceinline__ void split_b3(uint64_t v, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
+    p1 = bf16x2_rn(v);
+    const uint64_t r = sub_x2(v, bf16x2_value(p1));
+    p2 = bf16x2_rn(r);
+    const uint64_t q = sub_x2(r, bf16x2_value(p2));
+    p3 = __byte_perm((uint32_t)q, (uint32_t)(q >> 32), 0x7632);
 }
 // Scale exponents.  map_exp(m): the smallest e with m < 2^e for a map's largest magnitude m (bit pattern; 0 for a map
-// with infinities or NaN, whose sums are not finite at any scale).  A row (j, k) is scaled by 2^row_exp, a single by
-// 2^single_exp, which puts every product and every single below 2^15 (half the largest FP16 number).
+// with infinities or NaN, whose sums are not finite at any scale).  A row (j, k) is scaled by 2^row_exp: not at all (the
+// producers then save a multiplication) where its products lie below 2^40 and not all below 2^-40, else to below 2^15; a
+// single by 2^single_exp, to below 2^15.
 __host__ __device__ inline int map_exp(uint32_t m) {
     const int e = (int)((m >> 23) & 255u);
     return e == 255 ? 0 : (e < 1 ? 1 : e) - 126;
@@ -227,7 +240,10 @@ __device__ __forceinline__ uint32_t row_max(const uint32_t* gmax, const uint32_t
     return r < h_row0 ? gmax[r] : hmax[r - h_row0];
 }
 __host__ __device__ inline int clamp_exp(int e) { return e < -126 ? -126 : (e > 127 ? 127 : e); }
-__host__ __device__ inline int row_exp(uint32_t mj, uint32_t mk) { return clamp_exp(15 - map_exp(mj) - map_exp(mk)); }
+__host__ __device__ inline int row_exp(uint32_t mj, uint32_t mk) {
+    const int e = map_exp(mj) + map_exp(mk);
+    return e >= -40 && e <= 40 ? 0 : clamp_exp(15 - e);
+}
 __host__ __device__ inline int single_exp(uint32_t ma) { return clamp_exp(15 - map_exp(ma)); }
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }   // -126 <= e <= 127
 
@@ -240,6 +256,10 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* v) {
         "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]),
         "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]));
 }
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* v) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(v[0]),
+                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]));
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
@@ -249,7 +269,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
         : "r"(taddr)
         : "memory");
 }
-// tcgen05.wait::ld tied to two 16-register loads (32 operands).
+// tcgen05.wait::ld tied to a 16-register load, and to two.
+__device__ __forceinline__ void tmem_wait_ld16(uint32_t* a) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
+                   "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15])
+                 :
+                 : "memory");
+}
 __device__ __forceinline__ void tmem_wait_ld32(uint32_t* a, uint32_t* b) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
@@ -278,9 +305,9 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// The same for kind::f16 with FP16 operands (D = F32, A = B = F16, both K-major).
-__host__ __device__ constexpr uint32_t idesc_f16(int M, int N) {
-    return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// The same for kind::f16 with BF16 operands (D = F32, A = B = BF16, both K-major).
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 // The MMA and its commit are executed by a whole converged warp and issued by the one lane that elect.sync picks
@@ -336,10 +363,12 @@ __device__ __forceinline__ void epilogue(const GroupDesc& G, const Params& P, ui
     const int q = warp & 3;
     const int row = 32 * q + lane;
     const uint32_t lane_base = (uint32_t)(32 * q) << 16;
-    uint32_t cols[NU];        // unit u: 32 columns [hi 8 | lo 8 | hi 8 | lo 8]
+    uint32_t cols[NU], bufw[NU];        // unit u: 16 columns of its tile's buffer (W columns from one buffer to the other)
 #pragma unroll
-    for (int u = 0; u < NU; ++u) cols[u] = (uint32_t)(G.dm_col[G.unit_tile[u]] + 2 * G.unit_c[u]);
-    const uint32_t d_cols = (uint32_t)G.d_cols;
+    for (int u = 0; u < NU; ++u) {
+        cols[u] = (uint32_t)(G.dm_col[G.unit_tile[u]] + G.unit_c[u]);
+        bufw[u] = (uint32_t)G.tile_w[G.unit_tile[u]];
+    }
     int* const err = P.err;
     double* const out = P.partial + ((size_t)blockIdx.x * P.total_units + G.unit_base) * 2048;
 
@@ -352,19 +381,14 @@ __device__ __forceinline__ void epilogue(const GroupDesc& G, const Params& P, ui
         const int db = st & 1;
         if (!warp_wait(&d_full[db], (uint32_t)((st >> 1) & 1), abort_flag, err)) break;
         tc_fence_after();
-        const uint32_t dbase = tmem + lane_base + (uint32_t)db * d_cols;
+        const uint32_t dbase = tmem + lane_base;
 #pragma unroll
         for (int u = 0; u < NU; ++u) {
-            // both halves in flight together, one wait
-            uint32_t v0[16], v1[16];
-            tmem_ld16(dbase + cols[u], v0);
-            tmem_ld16(dbase + cols[u] + 16u, v1);
-            tmem_wait_ld32(v0, v1);
+            uint32_t v[16];
+            tmem_ld16(dbase + cols[u] + (db ? bufw[u] : 0u), v);
+            tmem_wait_ld16(v);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                acc[u][j] += __uint_as_float(v0[j]) + __uint_as_float(v0[8 + j]);
-                acc[u][8 + j] += __uint_as_float(v1[j]) + __uint_as_float(v1[8 + j]);
-            }
+            for (int j = 0; j < 16; ++j) acc[u][j] += __uint_as_float(v[j]);
         }
         tc_fence_before();
         __syncwarp();
@@ -387,14 +411,14 @@ __device__ __forceinline__ void epilogue(const GroupDesc& G, const Params& P, ui
 }
 
 
-// Producer warp of group gp: the 32 cells of slots gp, gp + 3, .. (two slots a 64-cell stage), for NT tiles.  A thread owns TMEM
-// lane 32 (warp % 4) + lane, i.e. row `row` of every tile.  The 64 columns of a tile's stage block are [hi 16 | lo 16]
-// of slot 0, then of slot 1 (two cells a column); a thread writes its slot's part with one 32-column TMEM store per
-// tile.
-template <int NT>
-__device__ __forceinline__ void producer(const GroupDesc& G, const Params& P, uint32_t tmem, const unsigned char* ring,
-                                         uint64_t* slot_full, uint64_t* slot_empty, uint64_t* a_full, uint64_t* a_empty,
-                                         volatile int* abort_flag, int nstages, int warp, int lane) {
+// Producer warp of group gp: the 32 cells of slots gp, gp + kProdGroups, .. (two slots a 64-cell stage), for NT tiles (SC: some
+// row of the warp is scaled).  A thread owns TMEM lane 32 (warp % 4) + lane, i.e. row `row` of every tile.  The 96
+// columns of a tile's stage block are the parts [A1 8 | A2 8 | A3 8] (two cells a column) of each K step of 16 cells; a
+// thread makes a step at a time and writes it with three 8-column TMEM stores (24 values in registers instead of 48).
+template <int NT, bool SC>
+__device__ __forceinline__ void produce(const GroupDesc& G, const Params& P, uint32_t tmem, const unsigned char* ring,
+                                        uint64_t* slot_full, uint64_t* slot_empty, uint64_t* a_full, uint64_t* a_empty,
+                                        volatile int* abort_flag, int nstages, int warp, int lane) {
     const int gp = (warp - kProdWarp0) >> 2;
     const int q = warp & 3;
     const int row = 32 * q + lane;
@@ -432,26 +456,40 @@ __device__ __forceinline__ void producer(const GroupDesc& G, const Params& P, ui
         bool ok = true;
 #pragma unroll
         for (int t = 0; t < NT; ++t) {
-            uint32_t v[32];
             const unsigned char* rj = slot + oj[t];
             const unsigned char* rk = slot + ok_[t];
+            const uint32_t dst = lane_base + a_stage + (uint32_t)(kAcols * t) + (uint32_t)(kAcols / 2) * half;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                const float4 x = *reinterpret_cast<const float4*>(rj + ((c << 4) ^ xj[t]));
-                const float4 y = *reinterpret_cast<const float4*>(rk + ((c << 4) ^ xk[t]));
-                split_h2(mul_x2(mul_x2(f2pack(x.x, x.y), f2pack(y.x, y.y)), scale[t]), v[2 * c], v[16 + 2 * c]);
-                split_h2(mul_x2(mul_x2(f2pack(x.z, x.w), f2pack(y.z, y.w)), scale[t]), v[2 * c + 1], v[16 + 2 * c + 1]);
-            }
-            if (pad[t]) {
+            for (int ks = 0; ks < 2; ++ks) {
+                uint32_t v[kParts][8];
 #pragma unroll
-                for (int c = 0; c < 32; ++c) v[c] = 0u;
+                for (int c = 0; c < 4; ++c) {
+                    const float4 x = *reinterpret_cast<const float4*>(rj + (((4 * ks + c) << 4) ^ xj[t]));
+                    const float4 y = *reinterpret_cast<const float4*>(rk + (((4 * ks + c) << 4) ^ xk[t]));
+                    uint64_t a = mul_x2(f2pack(x.x, x.y), f2pack(y.x, y.y)), b = mul_x2(f2pack(x.z, x.w), f2pack(y.z, y.w));
+                    if (SC) {
+                        a = mul_x2(a, scale[t]);
+                        b = mul_x2(b, scale[t]);
+                    }
+                    split_b3(a, v[0][2 * c], v[1][2 * c], v[2][2 * c]);
+                    split_b3(b, v[0][2 * c + 1], v[1][2 * c + 1], v[2][2 * c + 1]);
+                }
+                if (pad[t]) {
+#pragma unroll
+                    for (int p = 0; p < kParts; ++p)
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) v[p][c] = 0u;
+                }
+                if (t == 0 && ks == 0) {
+                    // tensor memory A stage `as` is free once the MMAs of stage st - nA completed
+                    if (st >= nA) ok = warp_wait(&a_empty[as], aph, abort_flag, err);
+                    tc_fence_after();
+                }
+                if (ok) {
+#pragma unroll
+                    for (int p = 0; p < kParts; ++p) tmem_st8(dst + (uint32_t)(8 * (kParts * ks + p)), v[p]);
+                }
             }
-            if (t == 0) {
-                // tensor memory A stage `as` is free once the MMAs of stage st - nA completed
-                if (st >= nA) ok = warp_wait(&a_empty[as], aph, abort_flag, err);
-                tc_fence_after();
-            }
-            if (ok) tmem_st32(lane_base + a_stage + (uint32_t)(kAcols * t) + 32u * half, v);
         }
         if (!ok) break;
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
@@ -474,10 +512,27 @@ __device__ __forceinline__ void producer(const GroupDesc& G, const Params& P, ui
     }
 }
 
-// B warp w (0 .. 3): half of the singles (8-row groups w / 2, w / 2 + 2, ..) of ring slot b = w % 2 of every stage -> FP16
-// hi and lo rows of 64 cells (128 bytes, 128-byte swizzle), cells 32 b .. 32 b + 31.  Rows r of the singles region, in
-// groups of eight: hi rows of group i at 2 i x 1024 bytes, lo rows at (2 i + 1) x 1024, so that a window of W singles is
-// 2W consecutive B rows.  A warp makes a group of eight rows at a time, lane (r, piece) = (lane / 4, lane % 4) eight cells
+// (the choice is the same for the 32 rows of a warp)
+template <int NT>
+__device__ __forceinline__ void producer(const GroupDesc& G, const Params& P, uint32_t tmem, const unsigned char* ring,
+                                         uint64_t* slot_full, uint64_t* slot_empty, uint64_t* a_full, uint64_t* a_empty,
+                                         volatile int* abort_flag, int nstages, int warp, int lane) {
+    const int row = 32 * (warp & 3) + lane;
+    bool sc = false;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+        const short2 jk = P.rows[(size_t)(G.tile0 + t) * 128 + row];
+        if (jk.x >= 0) sc |= row_exp(row_max(P.gmax, P.hmax, P.h_row0, jk.x), row_max(P.gmax, P.hmax, P.h_row0, jk.y)) != 0;
+    }
+    if (__any_sync(0xffffffffu, sc))
+        produce<NT, true>(G, P, tmem, ring, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane);
+    else
+        produce<NT, false>(G, P, tmem, ring, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane);
+}
+
+// B warp w (0 .. 3): the singles of ring slot b = w % 2 of stages w / 2, w / 2 + 2, .. -> BF16 rows of 64 cells (128
+// bytes, 128-byte swizzle), cells 32 b .. 32 b + 31, one block of all rows a part (bstage_bytes), so
+// that a window of W singles is W consecutive rows of a block.  A warp makes a group of eight rows at a time, lane (r, piece) = (lane / 4, lane % 4) eight cells
 // of row r; the rows' scales wait in shared memory.  (Two warps with the scales read from global memory set the pace of the
 // whole kernel.)
 __device__ __forceinline__ void make_b(const GroupDesc& G, const Params& P, const unsigned char* ring,
@@ -485,32 +540,33 @@ __device__ __forceinline__ void make_b(const GroupDesc& G, const Params& P, cons
                                        uint64_t* a_full, uint64_t* a_empty, volatile int* abort_flag, int nstages, int w,
                                        int lane) {
     const int b = w & 1;
-    const int nA = G.nA, slot_bytes = P.slot_bytes, stage_bytes = 2 * G.bstage_bytes;
+    const int nA = G.nA, slot_bytes = P.slot_bytes, part_bytes = G.bstage_bytes, stage_bytes = kParts * part_bytes;
     const int ngrp = P.s_chunks / 64;               // groups of eight rows (eight chunks a row)
     int* const err = P.err;
     const int r = lane >> 2, pc = lane & 3, x = r << 4;
     const int src0 = P.s_off + r * 128 + ((pc << 5) ^ x), src1 = P.s_off + r * 128 + (((pc << 5) + 16) ^ x);
     const int dst0 = r * 128 + (((4 * b + pc) << 4) ^ x);
-    int s = b, as = 0;
+    int s = w, as = w >> 1;
     uint32_t sph = 0u, aph = 1u;
-    for (int st = 0; st < nstages; ++st) {
+    for (int st = w >> 1; st < nstages; st += 2) {
         if (!warp_wait(&slot_full[s], sph, abort_flag, err)) break;
         if (st >= nA && !warp_wait(&a_empty[as], aph, abort_flag, err)) break;
         const unsigned char* src = ring + (size_t)s * slot_bytes;
         unsigned char* dst = bst + (size_t)as * stage_bytes + dst0;
 #pragma unroll 2
-        for (int g = w >> 1; g < ngrp; g += 2) {
+        for (int g = 0; g < ngrp; ++g) {
             const float f = bscale[8 * g + r];
             const uint64_t f2 = f2pack(f, f);
             const float4 u = *reinterpret_cast<const float4*>(src + src0 + g * 1024);
             const float4 v = *reinterpret_cast<const float4*>(src + src1 + g * 1024);
-            uint4 h, l;
-            split_h2(mul_x2(f2pack(u.x, u.y), f2), h.x, l.x);
-            split_h2(mul_x2(f2pack(u.z, u.w), f2), h.y, l.y);
-            split_h2(mul_x2(f2pack(v.x, v.y), f2), h.z, l.z);
-            split_h2(mul_x2(f2pack(v.z, v.w), f2), h.w, l.w);
-            *reinterpret_cast<uint4*>(dst + g * 2048) = h;
-            *reinterpret_cast<uint4*>(dst + g * 2048 + 1024) = l;
+            uint4 p, q, o;
+            split_b3(mul_x2(f2pack(u.x, u.y), f2), p.x, q.x, o.x);
+            split_b3(mul_x2(f2pack(u.z, u.w), f2), p.y, q.y, o.y);
+            split_b3(mul_x2(f2pack(v.x, v.y), f2), p.z, q.z, o.z);
+            split_b3(mul_x2(f2pack(v.z, v.w), f2), p.w, q.w, o.w);
+            *reinterpret_cast<uint4*>(dst + g * 1024) = p;
+            *reinterpret_cast<uint4*>(dst + part_bytes + g * 1024) = q;
+            *reinterpret_cast<uint4*>(dst + 2 * part_bytes + g * 1024) = o;
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // B stores -> tensor core
         __syncwarp();
@@ -518,9 +574,10 @@ __device__ __forceinline__ void make_b(const GroupDesc& G, const Params& P, cons
             mbar_arrive(&a_full[as]);
             mbar_arrive(&slot_empty[s]);
         }
-        s += 2;
-        if (s >= kRingSlots) { s = b; sph ^= 1u; }
-        if (++as == nA) { as = 0; aph ^= 1u; }
+        s += 4;
+        if (s >= kRingSlots) { s -= kRingSlots; sph ^= 1u; }
+        as += 2;
+        if (as >= nA) { as -= nA; aph ^= 1u; }
     }
 }
 
@@ -538,9 +595,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint64_t* slot_empty = bars + kRingSlots;          // [kRingSlots]  producers, B warps -> TMA
     uint64_t* a_full = bars + 2 * kRingSlots;          // [kMaxAStages] producers, B warps -> issuer
     uint64_t* a_empty = a_full + kMaxAStages;          // [kMaxAStages] MMA commit -> producers, B warps
-    uint64_t* d_full = a_empty + kMaxAStages;          // [kDBuf]       MMA commit -> epilogue
-    uint64_t* d_empty = d_full + kDBuf;                // [kDBuf]       epilogue -> issuer
-    uint64_t* fin = d_empty + kDBuf;
+    uint64_t* d_full = a_empty + kMaxAStages;          // [kAccBufs]    MMA commit -> epilogue
+    uint64_t* d_empty = d_full + kAccBufs;             // [kAccBufs]    epilogue -> issuer
+    uint64_t* fin = d_empty + kAccBufs;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(fin + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     float* bscale = reinterpret_cast<float*>(tmem_slot + 2);                    // [64] scales of the singles region's rows
@@ -563,13 +620,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (tid == 0) {
         for (int s = 0; s < kRingSlots; ++s) {
             mbar_init(&slot_full[s], 1);
-            mbar_init(&slot_empty[s], 4 + 2);          // the slot's producer group and its two B warps
+            mbar_init(&slot_empty[s], 4 + 1);          // the slot's producer group and its B warp
         }
         for (int s = 0; s < kMaxAStages; ++s) {
-            mbar_init(&a_full[s], 4 * 2 + kBWarps);    // four producer warps a slot, two slots; the B warps
+            mbar_init(&a_full[s], 4 * 2 + 2);          // two slots a stage: four producer warps and a B warp each
             mbar_init(&a_empty[s], 1);
         }
-        for (int i = 0; i < kDBuf; ++i) {
+        for (int i = 0; i < kAccBufs; ++i) {
             mbar_init(&d_full[i], 1);
             mbar_init(&d_empty[i], kEpiWarps);
         }
@@ -587,7 +644,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem = *tmem_slot;
 
     if (warp < kBWarp0) {
-        // warpgroup 0 hands registers to the producers (all four warps, one instruction)
+        // warpgroup 0 hands registers on (all four warps, one instruction)
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsCtl));
         if (warp == 0) {
             // ------------------------------------------------------------------ TMA producer
@@ -624,41 +681,47 @@ __global__ void __launch_bounds__(kThreads, 1)
                 *abort_flag = 1;
                 atomicExch(err, 1);
             }
-            // tile t's window of singles: 2W rows of the B stage from group s0 / 8 (2048 bytes a group of eight)
-            uint32_t idesc[kMaxTiles], dcol[kMaxTiles];
+            // tile t's window of singles: W rows of each part of the B stage from row s0
+            uint32_t idesc[kMaxTiles], dcol[kMaxTiles], dbuf[kMaxTiles];
             uint64_t bwin[kMaxTiles];
 #pragma unroll
             for (int t = 0; t < kMaxTiles; ++t) {
                 const int tt = t < ntiles ? t : 0;
-                idesc[t] = idesc_f16(128, 2 * G.tile_w[tt]);
+                idesc[t] = idesc_bf16(128, G.tile_w[tt]);
                 dcol[t] = (uint32_t)G.dm_col[tt];
-                bwin[t] = sdesc_sw128(smem_u32(bst) + (uint32_t)(256 * G.tile_s0[tt]));
+                dbuf[t] = (uint32_t)G.tile_w[tt];
+                bwin[t] = sdesc_sw128(smem_u32(bst) + (uint32_t)(128 * G.tile_s0[tt]));
             }
-            const uint32_t a_step = (uint32_t)(kAcols * ntiles), d_cols = (uint32_t)G.d_cols;
-            // descriptor address step (16-byte units; no carry out of the 14-bit field: shared memory < 2^18 bytes)
-            const uint64_t b_step = (uint64_t)(2 * G.bstage_bytes >> 4);
+            const uint32_t a_step = (uint32_t)(kAcols * ntiles);
+            // descriptor address steps (16-byte units; no carry out of the 14-bit field: shared memory < 2^18 bytes)
+            const uint64_t b_part = (uint64_t)(G.bstage_bytes >> 4), b_step = kParts * b_part;
             int as = 0;
             uint32_t aph = 0, aa = (uint32_t)a_col0, db = 0, dph = 1;
             uint64_t bo = 0;
             for (int st = 0; st < nstages && tmem_ok; ++st) {
                 // the epilogue has read this accumulator buffer's previous sums
-                if (st >= kDBuf && !warp_wait(&d_empty[db], dph, abort_flag, err)) break;
+                if (st >= kAccBufs && !warp_wait(&d_empty[db], dph, abort_flag, err)) break;
                 if (!warp_wait(&a_full[as], aph, abort_flag, err)) break;
                 tc_fence_after();
 #pragma unroll
                 for (int t = 0; t < kMaxTiles; ++t) {
                     if (t < ntiles) {
-                        const uint32_t d = dcol[t] + db * d_cols, a = aa + (uint32_t)(kAcols * t);
+                        const uint32_t d = dcol[t] + (db ? dbuf[t] : 0u), a = aa + (uint32_t)(kAcols * t);
                         const uint64_t bd = bwin[t] + bo;
-                        // K step ks: cells 16 ks .. 16 ks + 15; A_hi at slot block ks / 2, column 8 (ks % 2); A_lo at
-                        // +16.  B advances 32 bytes a step within the swizzle atom (2 in the descriptor)
+                        // K step ks: cells 16 ks .. 16 ks + 15, A part p at column 24 ks + 8 p.  B advances 32 bytes a
+                        // step within the swizzle atom (2 in the descriptor)
+                        auto products = [&](int pa, int pb) {
 #pragma unroll
-                        for (int ks = 0; ks < kKC / 16; ++ks)
-                            mma_f16(d, a + 16u + 32u * (ks >> 1) + 8u * (ks & 1), bd + (uint64_t)(2 * ks), idesc[t],
-                                    ks ? 1u : 0u);
-#pragma unroll
-                        for (int ks = 0; ks < kKC / 16; ++ks)
-                            mma_f16(d, a + 32u * (ks >> 1) + 8u * (ks & 1), bd + (uint64_t)(2 * ks), idesc[t], 1u);
+                            for (int ks = 0; ks < kKC / 16; ++ks)
+                                mma_f16(d, a + (uint32_t)(8 * (kParts * ks + pa)),
+                                        bd + pb * b_part + (uint64_t)(2 * ks), idesc[t], pa == 0 && pb == 2 && ks == 0 ? 0u : 1u);
+                        };
+                        products(0, 2);
+                        products(2, 0);
+                        products(1, 1);
+                        products(0, 1);
+                        products(1, 0);
+                        products(0, 0);
                     }
                 }
                 mma_commit(&a_empty[as]);
@@ -674,17 +737,17 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp < kProdWarp0) {
         // ------------------------------------------------------------------ the B operand
-        if (kRegsB < kRegsLaunch) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsB));
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsB));
         make_b(G, P, ring, bst, bscale, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp - kBWarp0, lane);
     } else if (warp < kProdWarp0 + kProdWarps) {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsProd));
         // ------------------------------------------------------------------ producers
         switch (ntiles) {
             case 1: producer<1>(G, P, tmem, ring, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
-            case 2: producer<2>(G, P, tmem, ring, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
-            default: producer<3>(G, P, tmem, ring, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
+            default: producer<2>(G, P, tmem, ring, slot_full, slot_empty, a_full, a_empty, abort_flag, nstages, warp, lane); break;
         }
     } else {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
         // ------------------------------------------------------------------ epilogue
         switch (G.nunits) {
             case 1: epilogue<1>(G, P, tmem, acc64, d_full, d_empty, abort_flag, nstages, warp, lane); break;
@@ -760,10 +823,6 @@ __global__ void k_wait_selftest(int* err, unsigned limit) {
 // 128-byte swizzle) has B[0][0] = 1 + 3 2^-12, three quarters of a TF32 unit above 1.  Truncation gives D[0][0] = 1
 // and D[1][0] = 1 + 2^-10; rounding to nearest would give 1 + 2^-10 and (1 + 2^-10)^2.  res: D[0][0], D[1][0] (FP32
 // bit patterns) and a timeout flag.
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(v[0]),
-                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]));
-}
 
 __global__ void __launch_bounds__(128, 1) k_tf32_selfcheck(uint32_t* res) {
     __shared__ __align__(1024) unsigned char sB[16 * 128];
@@ -1056,7 +1115,7 @@ struct NeedPair {
 // per group; 2: two CTAs per SM and row group, shorter cell ranges).
 struct PlanOpts {
     int tile_cost = 8;
-    int group_cap = 3;
+    int group_cap = kMaxTiles;
     int cta_mode = 0;
 };
 
@@ -1248,7 +1307,7 @@ static const char* layout_plan(Plan& pl, long ncell, int nsm, int ng, int nh, in
         tiles.push_back({sg.first, sg.second, s0, round_w(hi + 1 - s0)});
     }
     if (tiles.empty()) tiles.push_back({0, 0, 0, 16});
-    // row groups: consecutive tiles while TMEM (two accumulator buffers + two A stages) and the 3 output units allow
+    // row groups: consecutive tiles while TMEM (the accumulators + two A stages) and the 3 output units allow
     std::vector<std::pair<int, int>> groups;
     for (int t = 0; t < (int)tiles.size();) {
         int e = t, dcols = 0, units = 0;
@@ -1284,7 +1343,7 @@ static const char* layout_plan(Plan& pl, long ncell, int nsm, int ng, int nh, in
         D = GroupDesc{};
         const int t0 = groups[gi].first, nt = groups[gi].second - t0;
         D.tile0 = t0; D.ntiles = nt; D.unit_base = unit_base;
-        // accumulators (2W columns) of every tile, largest first, so each is aligned to its size
+        // accumulators (two buffers of W columns) of every tile, largest first, so each is aligned to its size
         std::vector<std::pair<int, int>> dl;   // (size, tile)
         for (int t = 0; t < nt; ++t) dl.push_back({2 * tiles[t0 + t].W, t});
         std::stable_sort(dl.begin(), dl.end(), [](auto& a, auto& b) { return a.first > b.first; });
@@ -1296,14 +1355,14 @@ static const char* layout_plan(Plan& pl, long ncell, int nsm, int ng, int nh, in
         D.d_cols = (col + 31) / 32 * 32;
         D.a_col0 = kDBuf * D.d_cols;
         D.nA = std::min(kMaxAStages, (512 - D.a_col0) / (kAcols * nt));
-        // windows of singles; B stages hold a slot's whole singles region, hi and lo
+        // windows of singles; B stages hold a slot's whole singles region, in parts
         for (int t = 0; t < nt; ++t) {
             const TileH& T = tiles[t0 + t];
             D.tile_w[t] = T.W;
             D.tile_s0[t] = T.s0;
         }
         D.bstage_bytes = srows * 128;
-        max_b = std::max(max_b, D.nA * 2 * D.bstage_bytes);
+        max_b = std::max(max_b, D.nA * kParts * D.bstage_bytes);
         // output units
         int u = 0;
         for (int t = 0; t < nt; ++t)
@@ -1504,7 +1563,7 @@ static int launch(polybin_ctx* ctx, Plan& pl, const float* g, const float* h, do
 }
 
 // Autotuner.  On the first launch of a plan outside stream capture (unless POLYBIN_AUTOTUNE=0), every distinct valid
-// candidate of the option grid {tile cost 8, 24} x {3 or 1 tiles a group} x {cell splits 0, 1, 2} runs on the
+// candidate of the option grid {tile cost 8, 24} x {2 or 1 tiles a group} x {cell splits 0, 1, 2} runs on the
 // caller's own inputs, timed with CUDA events on the context stream (one launch to warm up, two timed); the fastest
 // replaces the plan in the cache.  Candidates differ only in how cells and rows are split, so their results agree to
 // FP32 rounding of the partial sums; after tuning every call takes the chosen plan.
