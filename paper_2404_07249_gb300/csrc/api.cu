@@ -477,6 +477,7 @@ static double leg(int ell, double mu2) {
     return (35.0 * mu2 * mu2 - 30.0 * mu2 + 3.0) / 8.0;
 }
 
+constexpr long kPkMaxSegments = 8192;
 static int plan_pk(polybin_ctx* ctx) {
     const int nb = ctx->nb, nell = ctx->nell;
     const int Bx = ctx->gx.cnt, By = ctx->gy.cnt, Bz = ctx->gz.cnt;
@@ -516,8 +517,10 @@ static int plan_pk(polybin_ctx* ctx) {
     }
     long maxlen = 1;
     for (int b = 0; b < nb; ++b) maxlen = std::max(maxlen, (long)offs[b].size());
-    // about four segments of the mode lists an SM (a multiple of the CTA's 256 threads, at most 4096 modes)
-    ctx->pk_seg_len = (int)std::min(1024L, std::max(256L, (M / (4 * 152) + 255) / 256 * 256));
+    // about four segments of the mode lists an SM, of 256 to 1024 modes; no bin more than kPkMaxSegments of them (longer ones
+    // then): the segments are a grid's y dimension, 65535 at most, and a bin of a 1024^3 grid can hold 2.8e8 modes
+    const long most = (maxlen + kPkMaxSegments - 1) / kPkMaxSegments;
+    ctx->pk_seg_len = (int)std::max(std::min(1024L, std::max(256L, (M / (4 * 152) + 255) / 256 * 256)), (most + 255) / 256 * 256);
     ctx->pk_nseg = (int)((maxlen + ctx->pk_seg_len - 1) / ctx->pk_seg_len);
     polybin_ctx* c = ctx;
     PB_CUDA_OK_C(cudaMalloc(&c->d_offs, sizeof(int) * std::max(M, 1L)));

@@ -308,7 +308,7 @@ __device__ __forceinline__ double widen(double f) { return f; }
 // bin's mode list, NZ of the nx spectra); FP64 sums in a fixed order.  Bound by the FP64 pipe (two lanes a clock an SM):
 // two operations a mode and spectrum for the product and one for each ell, after the conversions have left it (four of nine
 // operations) and with one warp a sum at the end instead of a tree over all threads.  plan_pk cuts the lists into about four
-// segments an SM: with 8192 modes a segment, 20 to 40 CTAs took 70 us for 64^3 and for 256^3 alike.
+// segments an SM, at most 8192 a bin: with 8192 modes a segment, 20 to 40 CTAs took 70 us for 64^3 and for 256^3 alike.
 // Measured, before and after these two: 64^3 FP64 14.0 -> 6.7 us, 24 x 3 spectra on 256^3 (24 bins, three ells) 814 -> 575 us,
 // 512^3 with 30 bins 58 -> 44 us (a segment of at most 1024 modes keeps enough warps in flight there: 87 us with 3072).
 constexpr int kXbThreads = 128;
