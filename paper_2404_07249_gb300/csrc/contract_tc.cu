@@ -1518,7 +1518,8 @@ static int launch(polybin_ctx* ctx, Plan& pl, const float* g, const float* h, do
         mh = mg;
     }
     if ((rc = ensure_err_flag(ctx))) return rc;
-    cudaError_t e = cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream);
+    // (under capture the flag stays set for the rest of the graph, which clears it at its head and hands it out at its end)
+    cudaError_t e = ctx->capturing ? cudaSuccess : cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream);
     if (e != cudaSuccess) return fail_cuda(ctx, e, "cudaMemsetAsync", __FILE__, __LINE__);
     e = cudaFuncSetAttribute((const void*)k_contract_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
     if (e != cudaSuccess) return fail_cuda(ctx, e, "cudaFuncSetAttribute(k_contract_tc)", __FILE__, __LINE__);

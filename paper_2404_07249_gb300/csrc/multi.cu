@@ -142,6 +142,12 @@ extern "C" int polybin_bk_ideal_multi(polybin_ctx* const* ctxs, const float* con
         e = cudaEventRecord(m->ev, st);
         for (int k = 1; k < nbranch && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(m->side[k - 1], m->ev, 0);
         if (e != cudaSuccess) rc = fail_cuda(c0, e, "cudaStreamWaitEvent", __FILE__, __LINE__);
+        // a wait that gives up in any field of a context raises its flag for good: cleared here, read behind the last field
+        for (size_t k = 0; k < distinct.size() && !rc; ++k) {
+            polybin_ctx* c = distinct[k];
+            e = cudaMemsetAsync(c->d_err, 0, sizeof(int) * kErrFlags, c->stream);
+            if (e != cudaSuccess) rc = fail_cuda(c0, e, "capture memset", __FILE__, __LINE__);
+        }
         for (int i = 0; i < n_fields && !rc; ++i) {
             polybin_ctx* c = ctxs[i];
             rc = c->prec == POLYBIN_FP64 ? capture_field<double>(c, fields[i], m->host + m->off[i])
@@ -186,7 +192,7 @@ extern "C" int polybin_bk_ideal_multi(polybin_ctx* const* ctxs, const float* con
             PB_CUDA_OK(cudaMemset(c->d_err + kErrStaging, 0, sizeof(int)));
         }
         if (herr[kErrPipeline] || herr[kErrStaging])
-            return fail(c0, POLYBIN_ETIMEOUT, "polybin_bk_ideal_multi: a %s wait timed out (field %d)",
+            return fail(c0, POLYBIN_ETIMEOUT, "polybin_bk_ideal_multi: a %s wait timed out (a field of the context of field %d)",
                         herr[kErrStaging] ? "bulk staging" : "pipeline", i);
         const double* B = m->host + m->off[i];
         std::memcpy(bk_out[i], B, sizeof(double) * c->Nabc.size());
