@@ -34,6 +34,7 @@ int fail(polybin_ctx* ctx, int status, const char* fmt, ...) {
 }
 
 int fail_cuda(polybin_ctx* ctx, cudaError_t e, const char* what, const char* file, int line) {
+    cudaGetLastError();                               // reported here: the next launch's check does not find it again
     return fail(ctx, e == cudaErrorMemoryAllocation ? POLYBIN_ENOMEM : POLYBIN_ECUDA, "%s failed: %s (%s:%d)", what,
                 cudaGetErrorString(e), file, line);
 }

@@ -6,6 +6,9 @@
 // any grid of more than 4m points is that of the data grid, up to rounding: 144^3 instead of 256^3 (5.6 times fewer cells)
 // for 16 bispectrum bins up to 33 k_F, 192^3 for 24 power spectrum bins up to 48 k_F.
 //
+// Memory.  The transforms of s run in the caller's scratch; what stays is s and one batch's intermediates.  Where these do not
+// fit, the operator runs on the data grid with the maps n and w (mask_direct), which takes no memory of its own.
+//
 // Batches.  The FP32 passes run over a chunk of bins or triplets a launch (as many as keep the intermediates near the
 // L2's size), the first one filters or combines on load, and the z passes around the product are one kernel (f2::mask_z),
 // so the real maps are never stored.
@@ -28,8 +31,8 @@ struct MaskOp {
     void* tw[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     bool reduced = false;         // the product grid is smaller than the data grid
     bool fast = false;
+    bool direct = false;          // no map of s: the data grid, multiplied by w and n
     void* smap = nullptr;         // s N / N' on the product grid
-    void *f1 = nullptr, *f2 = nullptr, *sbox = nullptr, *v1 = nullptr, *v2 = nullptr;   // transforms of s
     // batches of `chunk` items: x passes [N0][By][Bz], y passes [N0][N1][Bz] before and after the product, boxes
     int chunk = 0;
     float2 *bx = nullptr, *by = nullptr, *bz = nullptr, *boxes = nullptr;
@@ -38,15 +41,32 @@ struct MaskOp {
 static MaskOp* op_of(const polybin_ctx* ctx) { return static_cast<MaskOp*>(ctx->maskop); }
 const InvGrid& mask_grid(const polybin_ctx* ctx) { return op_of(ctx)->pg; }
 const void* mask_map(const polybin_ctx* ctx) { return op_of(ctx)->smap; }
-bool mask_fast(const polybin_ctx* ctx) { return op_of(ctx)->fast; }
+bool mask_direct(const polybin_ctx* ctx) { return op_of(ctx)->direct; }
+bool mask_fast(const polybin_ctx* ctx) { return op_of(ctx)->fast && !op_of(ctx)->direct; }
 int mask_chunk(const polybin_ctx* ctx) { return op_of(ctx)->chunk; }
+
+// (their places are null afterwards: they may be allocated again)
+static void free_maps(MaskOp* o) {
+    void** ptrs[] = {&o->smap, (void**)&o->bx, (void**)&o->by, (void**)&o->bz, (void**)&o->boxes};
+    for (void** p : ptrs) {
+        if (*p) cudaFree(*p);
+        *p = nullptr;
+    }
+}
+
+bool mask_release(polybin_ctx* ctx) {
+    MaskOp* o = op_of(ctx);
+    if (!o || !o->smap) return false;
+    free_maps(o);
+    o->direct = true;
+    return true;
+}
 
 void destroy_maskop(polybin_ctx* ctx) {
     MaskOp* o = op_of(ctx);
     if (!o) return;
-    void* ptrs[] = {o->tw[0], o->tw[1], o->tw[2], o->tw[3], o->tw[4], o->tw[5], o->smap, o->f1, o->f2, o->sbox, o->v1, o->v2,
-                    o->bx, o->by, o->bz, o->boxes};
-    for (void* p : ptrs)
+    free_maps(o);
+    for (void* p : o->tw)
         if (p) cudaFree(p);
     delete o;
     ctx->maskop = nullptr;
@@ -59,26 +79,35 @@ __global__ void k_weight(const float* __restrict__ n, const float* __restrict__ 
         out[i] = T(w[i]) * T(n[i]);
 }
 
+static unsigned map_blocks(long n) { return (unsigned)std::min<long>((n + 255) / 256, 152L * 16); }
+
+static int checked(polybin_ctx* ctx, const char* what) {
+    ctx->launches++;
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? POLYBIN_OK : fail_cuda(ctx, e, what, __FILE__, __LINE__);
+}
+
+// The grid, and on first use (or after a call that found no room) the maps.
 template <typename T>
 static int mask_plan(polybin_ctx* ctx) {
-    MaskOp* o = new (std::nothrow) MaskOp();
-    if (!o) return fail(ctx, POLYBIN_ENOMEM, "masked operator: out of host memory");
-    ctx->maskop = o;
+    MaskOp* o = op_of(ctx);
     int rc;
-    if ((rc = plan_product_grid(ctx, o->pg, o->keep, o->tw))) return rc;
-    o->reduced = o->pg.ncell < ctx->ncell;
-    o->fast = sizeof(T) == 4 && f2::has(o->pg.N[0]) && f2::has(o->pg.N[1]) && f2::has(o->pg.N[2]);
+    if (!o) {
+        o = new (std::nothrow) MaskOp();
+        if (!o) return fail(ctx, POLYBIN_ENOMEM, "masked operator: out of host memory");
+        ctx->maskop = o;
+        if ((rc = plan_product_grid(ctx, o->pg, o->keep, o->tw))) {
+            destroy_maskop(ctx);
+            return rc;
+        }
+        o->reduced = o->pg.ncell < ctx->ncell;
+        o->fast = sizeof(T) == 4 && f2::has(o->pg.N[0]) && f2::has(o->pg.N[1]) && f2::has(o->pg.N[2]);
+    }
+    o->direct = !o->reduced && !o->fast;
+    if (o->direct || o->smap) return POLYBIN_OK;
     const long By = ctx->gy.cnt, Bz = ctx->gz.cnt, nbox = (long)ctx->gx.cnt * By * Bz;
     const long P0 = o->pg.N[0], P1 = o->pg.N[1];
     PB_CUDA_OK(cudaMalloc(&o->smap, sizeof(T) * o->pg.ncell));
-    if (o->reduced) {
-        const long sy = o->keep.y.cnt, sz = o->keep.z.cnt;
-        PB_CUDA_OK(cudaMalloc(&o->f1, sizeof(C<T>) * ctx->N[0] * ctx->N[1] * sz));
-        PB_CUDA_OK(cudaMalloc(&o->f2, sizeof(C<T>) * ctx->N[0] * sy * sz));
-        PB_CUDA_OK(cudaMalloc(&o->sbox, sizeof(C<T>) * o->keep.x.cnt * sy * sz));
-        PB_CUDA_OK(cudaMalloc(&o->v1, sizeof(C<T>) * P0 * sy * sz));
-        PB_CUDA_OK(cudaMalloc(&o->v2, sizeof(C<T>) * P0 * P1 * sz));
-    }
     if (o->fast) {
         // intermediates of a chunk near the L2's 129 MB
         const long item = (long)sizeof(float2) * (P0 * By * Bz + 2 * P0 * P1 * Bz + nbox);
@@ -91,36 +120,51 @@ static int mask_plan(polybin_ctx* ctx) {
     return POLYBIN_OK;
 }
 
+// s = w n low-passed to the product grid.  The steps lie in `scratch`, two regions that they use in turn.
 template <typename T>
-int mask_setup(polybin_ctx* ctx, const float* n, const float* w) {
-    int rc;
-    if (!ctx->maskop && (rc = mask_plan<T>(ctx))) {
-        destroy_maskop(ctx);
-        return rc;
-    }
+static int mask_lowpass(polybin_ctx* ctx, const float* n, const float* w, void* scratch, size_t bytes) {
     MaskOp* o = op_of(ctx);
-    if (!o->reduced) {
-        k_weight<T><<<(unsigned)std::min<long>((ctx->ncell + 255) / 256, 152L * 16), 256, 0, ctx->stream>>>(n, w, ctx->ncell,
-                                                                                                       (T*)o->smap);
-        ctx->launches++;
-        PB_CUDA_OK(cudaGetLastError());
-        return POLYBIN_OK;
+    const long sx = o->keep.x.cnt, sy = o->keep.y.cnt, sz = o->keep.z.cnt, P0 = o->pg.N[0], P1 = o->pg.N[1];
+    // t1 [N0][N1][sz], then box [sx][sy][sz], then v2 [P0][P1][sz]; t2 [N0][sy][sz], then v1 [P0][sy][sz]
+    const size_t one = sizeof(C<T>) * std::max({(long)ctx->N[0] * ctx->N[1] * sz, sx * sy * sz, P0 * P1 * sz});
+    const size_t two = sizeof(C<T>) * std::max(ctx->N[0] * sy * sz, P0 * sy * sz);
+    void* own = nullptr;
+    if (one + two > bytes) {
+        PB_CUDA_OK(cudaMalloc(&own, one + two));
+        scratch = own;
     }
-    if ((rc = run_forward_box<T, float, float>(ctx, n, w, (const float*)nullptr, (C<T>*)o->f1, (C<T>*)o->f2, (C<T>*)o->sbox,
-                                               ctx->fg, o->keep)))
-        return rc;
+    C<T>* const r1 = (C<T>*)scratch;
+    C<T>* const r2 = (C<T>*)((char*)scratch + one);
+    int rc = run_forward_box<T, float, float>(ctx, n, w, (const float*)nullptr, r1, r2, r1, ctx->fg, o->keep);
     // 1/N' instead of 1/N: the sums over the product grid's cells then have the data grid's normalisation
-    return run_inverse_from<T>(ctx, (const C<T>*)o->sbox, (C<T>*)o->v1, (C<T>*)o->v2, (T*)o->smap, (const T*)nullptr, o->pg,
-                               o->keep, 1.0 / (double)o->pg.ncell);
+    if (!rc)
+        rc = run_inverse_from<T>(ctx, r1, r2, r1, (T*)o->smap, (const T*)nullptr, o->pg, o->keep, 1.0 / (double)o->pg.ncell);
+    if (own) cudaFree(own);                           // (waits for the steps)
+    return rc;
 }
-template int mask_setup<float>(polybin_ctx*, const float*, const float*);
-template int mask_setup<double>(polybin_ctx*, const float*, const float*);
 
-static int checked(polybin_ctx* ctx, const char* what) {
-    ctx->launches++;
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? POLYBIN_OK : fail_cuda(ctx, e, what, __FILE__, __LINE__);
+template <typename T>
+int mask_setup(polybin_ctx* ctx, const float* n, const float* w, void* scratch, size_t bytes) {
+    int rc = mask_plan<T>(ctx);
+    MaskOp* o = op_of(ctx);
+    if (!rc && !o->direct) {
+        if (o->reduced) {
+            rc = mask_lowpass<T>(ctx, n, w, scratch, bytes);
+        } else {
+            k_weight<T><<<map_blocks(ctx->ncell), 256, 0, ctx->stream>>>(n, w, ctx->ncell, (T*)o->smap);
+            rc = checked(ctx, "k_weight");
+        }
+    }
+    if (rc == POLYBIN_ENOMEM && o) {
+        cudaGetLastError();                           // no room: the data grid
+        free_maps(o);
+        o->direct = true;
+        rc = POLYBIN_OK;
+    }
+    return rc;
 }
+template int mask_setup<float>(polybin_ctx*, const float*, const float*, void*, size_t);
+template int mask_setup<double>(polybin_ctx*, const float*, const float*, void*, size_t);
 
 // The passes after the first: item i (its box ry, rz) from bx to boxes.
 static int finish(polybin_ctx* ctx, int cnt, const AxisRange* ry, const AxisRange* rz) {

@@ -165,8 +165,12 @@ template <typename T>
 int run_inverse_from(polybin_ctx*, const C<T>* box, C<T>* v1, C<T>* v2, T* out, const T* mulout, const InvGrid& ig,
                      const Box3& keep, double scale);
 // Masked operator (maskop.cu): X -> FT[s IFT[X]] on the box with s = w n, evaluated on the product grid.
-// mask_setup makes s of the given maps; mask_map / mask_grid hand it out; mask_fast: the batched FP32 passes apply.
-template <typename T> int mask_setup(polybin_ctx*, const float* n, const float* w);
+// mask_setup makes s of the given maps (in `bytes` of scratch that nothing else uses meanwhile); mask_map / mask_grid hand
+// it out; mask_fast: the batched FP32 passes apply; mask_direct: there is no s, the operator is the data grid's with n and w.
+template <typename T> int mask_setup(polybin_ctx*, const float* n, const float* w, void* scratch, size_t bytes);
+bool mask_direct(const polybin_ctx*);
+// Gives the maps back (mask_direct from here on, until the next mask_setup); false if there are none.
+bool mask_release(polybin_ctx*);
 const InvGrid& mask_grid(const polybin_ctx*);
 const void* mask_map(const polybin_ctx*);
 bool mask_fast(const polybin_ctx*);

@@ -365,6 +365,7 @@ __global__ void k_ylm_box_accum(const C<T>* __restrict__ G, C<T>* __restrict__ H
 
 // Place of the harmonic m among the 2 ell + 1: 0, -1, 1, -2, 2, .. (m and -m next to each other).
 __host__ __device__ inline int ylm_row(int m) { return m < 0 ? -2 * m - 1 : 2 * m; }
+__host__ __device__ inline int ylm_m(int row) { return row & 1 ? -(row + 1) / 2 : row / 2; }
 
 // Ybar_lm(k_q) of the binned modes: tab[ylm_row(m)][q] (FP64; laid out once a context).
 static __global__ void k_ylm_table(const int* __restrict__ offs, long M, int ell, AxisRange gx, AxisRange gy, AxisRange gz,
@@ -376,17 +377,24 @@ static __global__ void k_ylm_table(const int* __restrict__ offs, long M, int ell
     }
 }
 
-// acc[q] = sum_i tab[i][q] box[i][offs[q]] over cnt boxes (added to acc when add is set; tab null: weight 1), FP64.
-template <typename T>
+// acc[q] = sum_i Ybar_lm(k_q) box[i][offs[q]] over the cnt harmonics of ell of rows r0, r0 + 1, .. (added to acc when add_to is
+// set), FP64.  Ybar_lm from the table (row r0 first), worked out here, or 1.
+enum YlmWeight { kYlmOne, kYlmTable, kYlmHere };
+template <typename T, YlmWeight W>
 __global__ void k_ylm_gather(const C<T>* __restrict__ box, long box_stride, int cnt, const int* __restrict__ offs, long M,
-                             const double* __restrict__ tab, int add_to, double2* __restrict__ acc) {
+                             const double* __restrict__ tab, int ell, int r0, AxisRange gx, AxisRange gy, AxisRange gz,
+                             int add_to, double2* __restrict__ acc) {
     for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < M; q += (long)gridDim.x * blockDim.x) {
         const long o = offs[q];
         double2 v = add_to ? acc[q] : make_double2(0.0, 0.0);
+        double kx = 0.0, ky = 0.0, kz = 0.0;
+        const bool ok = W == kYlmHere && box_direction(o, gx, gy, gz, kx, ky, kz);
 #pragma unroll 3
         for (int i = 0; i < cnt; ++i) {
             const C<T> g = box[(long)i * box_stride + o];
-            const double y = tab ? tab[(long)i * M + q] : 1.0;
+            double y = 1.0;
+            if (W == kYlmTable) y = tab[(long)i * M + q];
+            if (W == kYlmHere) y = ok ? ybar<double>(ell, ylm_m(r0 + i), kx, ky, kz) : 0.0;
             v.x += y * (double)g.x;
             v.y += y * (double)g.y;
         }
@@ -449,7 +457,7 @@ struct UwState {
     void* spec[4] = {nullptr, nullptr, nullptr, nullptr};  // box spectra
     void* pairs = nullptr;    // pair spectra [2][npairs][box]
     void *pair1 = nullptr, *pair2 = nullptr;   // intermediates of a batch of pair transforms
-    int pair_chunk = 0;
+    int pair_chunk = 0;       // (-1: no room for a batch)
     void* qbox = nullptr;     // one box spectrum
     void* zc = nullptr;       // compact [nt][M]
     void* yc = nullptr;       // compact [nt][M]
@@ -470,7 +478,8 @@ struct UwState {
     double2* ylc = nullptr;
     double* yltab = nullptr;      // Ybar_lm of the binned modes, ell = 2 (5 rows) and 4 (9 rows) as lmax has them [..][M]
     void *yl1 = nullptr, *yl2 = nullptr, *ylbox = nullptr;   // intermediates and boxes of a batch of harmonics
-    int yl_chunk = 0;
+    int yl_chunk = 0;             // (-1: no room for a batch)
+    bool yltab_off = false;       // no room for the table
     void* hbox = nullptr;
     void* g3 = nullptr;
     std::vector<double> Fl, Fl_inv;
@@ -695,16 +704,18 @@ static int pk_fisher_draw(polybin_ctx* ctx, const float* n, const float* w, unsi
                 }
         }
     }
-    const InvGrid& pg = mask_grid(ctx);
+    const bool direct = mask_direct(ctx);
+    const InvGrid& pg = direct ? ctx->fg : mask_grid(ctx);
     T* q = (T*)u->g2;
     for (int il = 0; il < nell && !done; ++il) {
         if ((rc = ensure_fine_inv<T>(ctx))) return rc;
         if ((rc = run_shells<T>(ctx, SA, (C<T>*)W.u1f, (C<T>*)W.u2f, q, 2 * il, pg))) return rc;
         for (int b = 0; b < nb; ++b) {
             C<T>* X = (C<T>*)u->spec[2];
-            if ((rc = run_forward<T, T, T>(ctx, q + (size_t)b * pg.ncell, (const T*)mask_map(ctx), (const T*)nullptr,
-                                           (C<T>*)W.t1, (C<T>*)W.t2, X, pg)))
-                return rc;
+            const T* qb = q + (size_t)b * pg.ncell;
+            rc = direct ? run_forward<T, T, float>(ctx, qb, w, n, (C<T>*)W.t1, (C<T>*)W.t2, X)
+                        : run_forward<T, T, T>(ctx, qb, (const T*)mask_map(ctx), (const T*)nullptr, (C<T>*)W.t1, (C<T>*)W.t2, X, pg);
+            if (rc) return rc;
             if ((rc = launch_cross_bin<T>(ctx, X, 0, 1, A, u->dpart_all + (size_t)(il * nb + b) * per))) return rc;
         }
     }
@@ -922,19 +933,51 @@ static int uw_alloc_local(polybin_ctx* ctx, bool fisher) {
     UwState* u = static_cast<UwState*>(ctx->ext);
     const long nbox = (long)ctx->gx.cnt * ctx->gy.cnt * ctx->gz.cnt;
     if (!u->ylc) PB_CUDA_OK(cudaMalloc(&u->ylc, sizeof(double2) * 3 * std::max(ctx->nmodes, 1L)));
-    if (!u->yltab && ctx->nell > 1 && ctx->nmodes > 0) {
-        const long M = ctx->nmodes;
-        PB_CUDA_OK(cudaMalloc(&u->yltab, sizeof(double) * (ctx->nell > 2 ? 14 : 5) * M));
-        for (int il = 1; il < ctx->nell; ++il) {
-            uw::k_ylm_table<<<grid1d(M), 256, 0, ctx->stream>>>(ctx->d_offs, M, 2 * il, ctx->gx, ctx->gy, ctx->gz,
-                                                                u->yltab + (il == 1 ? 0 : 5 * M));
-            ctx->launches++;
-        }
-        PB_CUDA_OK(cudaGetLastError());
-    }
     if (!u->hbox) PB_CUDA_OK(cudaMalloc(&u->hbox, sizeof(C<T>) * nbox));
     if (fisher && !u->g3) PB_CUDA_OK(cudaMalloc(&u->g3, sizeof(T) * (size_t)ctx->nb * ctx->ncell));
     return POLYBIN_OK;
+}
+
+// The table of Ybar_lm, on first use; without room for it the weights are worked out where they are used.
+static int ensure_yltab(polybin_ctx* ctx) {
+    UwState* u = static_cast<UwState*>(ctx->ext);
+    const long M = ctx->nmodes;
+    if (u->yltab || u->yltab_off || ctx->nell < 2 || M < 1) return POLYBIN_OK;
+    if (cudaMalloc(&u->yltab, sizeof(double) * (ctx->nell > 2 ? 14 : 5) * M) != cudaSuccess) {
+        cudaGetLastError();
+        u->yltab = nullptr;
+        u->yltab_off = true;
+        return POLYBIN_OK;
+    }
+    for (int il = 1; il < ctx->nell; ++il) {
+        uw::k_ylm_table<<<grid1d(M), 256, 0, ctx->stream>>>(ctx->d_offs, M, 2 * il, ctx->gx, ctx->gy, ctx->gz,
+                                                            u->yltab + (il == 1 ? 0 : 5 * M));
+        ctx->launches++;
+    }
+    PB_CUDA_OK(cudaGetLastError());
+    return POLYBIN_OK;
+}
+
+// Gives back what only makes calls faster: the batches' intermediates, the table, the masked operator's maps.  False if there
+// is nothing to give back.
+static bool drop_batches(polybin_ctx* ctx) {
+    UwState* u = static_cast<UwState*>(ctx->ext);
+    bool any = mask_release(ctx);
+    void** ptrs[] = {&u->pair1, &u->pair2, &u->yl1, &u->yl2, &u->ylbox, (void**)&u->yltab};
+    for (void** p : ptrs) {
+        if (!*p) continue;
+        cudaFree(*p);
+        *p = nullptr;
+        any = true;
+    }
+    u->pair_chunk = u->yl_chunk = -1;
+    u->yltab_off = true;
+    return any;
+}
+// Runs f, and where an allocation fails that f cannot do without, once more without these.
+template <class F> static int with_room(polybin_ctx* ctx, F f) {
+    const int rc = f();
+    return rc == POLYBIN_ENOMEM && drop_batches(ctx) ? f() : rc;
 }
 
 // The batched harmonic transforms take the data grid (FP32 two-stage lengths); allocates their workspace on first use.
@@ -950,6 +993,10 @@ static bool ylm_fast(polybin_ctx* ctx) {
     if (cudaMalloc(&u->yl1, sizeof(float2) * s1 * c) != cudaSuccess || cudaMalloc(&u->yl2, sizeof(float2) * s2 * c) != cudaSuccess ||
         cudaMalloc(&u->ylbox, sizeof(float2) * nbox * c) != cudaSuccess) {
         cudaGetLastError();                           // no room for the batch: one harmonic at a time
+        for (void** p : {&u->yl1, &u->yl2, &u->ylbox}) {
+            if (*p) cudaFree(*p);
+            *p = nullptr;
+        }
         return false;
     }
     u->yl_chunk = c;
@@ -1022,13 +1069,24 @@ static int local_asym(polybin_ctx* ctx, const TIN* in, const float* m1, const fl
     const uw::CellGeom<T> cg = cell_geom<T>(ctx);
     int rc;
     if ((rc = run_forward<T, TIN, float>(ctx, in, m1, m2, (C<T>*)W.t1, (C<T>*)W.t2, ubox))) return rc;
-    uw::k_ylm_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(ubox, 0, 1, ctx->d_offs, M, nullptr, 0, u->ylc);
-    ctx->launches++;
+    if ((rc = ensure_yltab(ctx))) return rc;
+    // (boxes: cnt harmonics of ell from row r0 on)
+    auto gather = [&](const C<T>* boxes, long stride, int cnt, int ell, int r0, double2* acc) {
+        const double* tab = ell && u->yltab ? u->yltab + (ell == 2 ? 0 : 5 * M) + (long)r0 * M : nullptr;
+        auto launch = [&](auto kernel) {
+            kernel<<<grid1d(M), 256, 0, ctx->stream>>>(boxes, stride, cnt, ctx->d_offs, M, tab, ell, r0, ctx->gx, ctx->gy, ctx->gz,
+                                                       r0 ? 1 : 0, acc);
+        };
+        if (!ell) launch(uw::k_ylm_gather<T, uw::kYlmOne>);
+        else if (tab) launch(uw::k_ylm_gather<T, uw::kYlmTable>);
+        else launch(uw::k_ylm_gather<T, uw::kYlmHere>);
+        ctx->launches++;
+    };
+    gather(ubox, 0, 1, 0, 0, u->ylc);
     const long nbox = (long)ctx->gx.cnt * ctx->gy.cnt * ctx->gz.cnt;
     C<T>* tmp = (C<T>*)u->spec[2];
     for (int il = 1; il < ctx->nell; ++il) {
         const int ell = 2 * il;
-        const double* tab = u->yltab + (il == 1 ? 0 : 5 * M);
         double2* acc = u->ylc + (size_t)il * M;
         if constexpr (std::is_same<T, float>::value && std::is_same<TIN, float>::value) {
             if (!m2 && ylm_fast(ctx)) {
@@ -1037,22 +1095,18 @@ static int local_asym(polybin_ctx* ctx, const TIN* in, const float* m1, const fl
                     cnt = std::min(u->yl_chunk, 2 * ell + 1 - r);
                     if (cnt > 1 && (r + cnt) % 2 == 0) --cnt;   // -m and m share their transform along z
                     if ((rc = forward_ylm(ctx, in, m1, ell, r, cnt, &boxes))) return rc;
-                    uw::k_ylm_gather<float><<<grid1d(M), 256, 0, ctx->stream>>>(
-                        boxes, nbox, cnt, ctx->d_offs, M, tab + (long)r * M, r ? 1 : 0, acc);
-                    ctx->launches++;
+                    gather(boxes, nbox, cnt, ell, r, acc);
                 }
                 continue;
             }
         }
-        for (int m = -ell; m <= ell; ++m) {
-            uw::k_mul_ylm<T, TIN, float><<<grid1d(N), 256, 0, ctx->stream>>>(in, m1, m2, (T*)u->xmap, ell, m, cg);
+        for (int r = 0; r < 2 * ell + 1; ++r) {
+            uw::k_mul_ylm<T, TIN, float><<<grid1d(N), 256, 0, ctx->stream>>>(in, m1, m2, (T*)u->xmap, ell, uw::ylm_m(r), cg);
             ctx->launches++;
             if ((rc = run_forward<T, T, float>(ctx, (const T*)u->xmap, (const float*)nullptr, (const float*)nullptr,
                                                (C<T>*)W.t1, (C<T>*)W.t2, tmp)))
                 return rc;
-            uw::k_ylm_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(tmp, 0, 1, ctx->d_offs, M,
-                                                                    tab + (long)uw::ylm_row(m) * M, m == -ell ? 0 : 1, acc);
-            ctx->launches++;
+            gather(tmp, 0, 1, ell, r, acc);
         }
     }
     PB_CUDA_OK(cudaGetLastError());
@@ -1175,14 +1229,20 @@ static int pair_spectra(polybin_ctx* ctx, const C<T>* U1, const C<T>* U2, C<T>* 
     if ((rc = run_shells<T>(ctx, U1, (C<T>*)W.u1, (C<T>*)W.u2, g1, 0, cg))) return rc;
     if ((rc = run_shells<T>(ctx, U2, (C<T>*)W.u1, (C<T>*)W.u2, g2, 0, cg))) return rc;
     if constexpr (std::is_same<T, float>::value) {
-        if (f2::has(cg.N[0]) && f2::has(cg.N[1]) && f2::has(cg.N[2])) {
-            const long nlines = (long)cg.N[0] * cg.N[1], s1 = nlines * Bz, s2 = (long)cg.N[0] * By * Bz;
-            if (!u->pair2) {
-                // intermediates of a batch of pairs near the L2's size
-                u->pair_chunk = (int)std::min<long>(f2::kBatch, std::max<long>(1, (80L << 20) / ((long)sizeof(float2) * (s1 + s2))));
-                if (!u->pair1) PB_CUDA_OK(cudaMalloc(&u->pair1, sizeof(float2) * s1 * u->pair_chunk));
-                PB_CUDA_OK(cudaMalloc(&u->pair2, sizeof(float2) * s2 * u->pair_chunk));
+        const long nlines = (long)cg.N[0] * cg.N[1], s1 = nlines * Bz, s2 = (long)cg.N[0] * By * Bz;
+        if (f2::has(cg.N[0]) && f2::has(cg.N[1]) && f2::has(cg.N[2]) && !u->pair_chunk) {
+            // intermediates of a batch of pairs near the L2's size
+            const int c = (int)std::min<long>(std::min(f2::kBatch, np), std::max<long>(1, (80L << 20) / ((long)sizeof(float2) * (s1 + s2))));
+            if (cudaMalloc(&u->pair1, sizeof(float2) * s1 * c) == cudaSuccess && cudaMalloc(&u->pair2, sizeof(float2) * s2 * c) == cudaSuccess) {
+                u->pair_chunk = c;
+            } else {
+                cudaGetLastError();                   // no room: one pair at a time
+                if (u->pair1) cudaFree(u->pair1);
+                u->pair1 = u->pair2 = nullptr;
+                u->pair_chunk = -1;
             }
+        }
+        if (u->pair_chunk > 0) {
             std::vector<int> px, py;
             for (int x = 0; x < nb; ++x)
                 for (int y = x; y < nb; ++y) { px.push_back(x); py.push_back(y); }
@@ -1304,7 +1364,8 @@ static int bk_fisher_draw(polybin_ctx* ctx, const float* n, const float* w, unsi
             }
         }
     }
-    const InvGrid& pg = mask_grid(ctx);
+    const bool direct = mask_direct(ctx);
+    const InvGrid& pg = direct ? ctx->fg : mask_grid(ctx);
     for (int t = 0; t < nt && !done; ++t) {
         const int a = ctx->trip[3 * t], b = ctx->trip[3 * t + 1], c = ctx->trip[3 * t + 2];
         const double dl = (a == b && b == c) ? 6.0 : ((a == b || b == c) ? 2.0 : 1.0);
@@ -1315,9 +1376,10 @@ static int bk_fisher_draw(polybin_ctx* ctx, const float* n, const float* w, unsi
         if ((rc = run_inverse_from<T>(ctx, q, (C<T>*)u->v1, (C<T>*)u->v2, (T*)u->xmap, (const T*)nullptr, pg,
                                       Box3{ctx->gx, ctx->gy, ctx->gz}, 1.0 / (double)N)))
             return rc;
-        if ((rc = run_forward<T, T, T>(ctx, (const T*)u->xmap, (const T*)mask_map(ctx), (const T*)nullptr, (C<T>*)W.t1,
-                                       (C<T>*)W.t2, q, pg)))
-            return rc;
+        rc = direct ? run_forward<T, T, float>(ctx, (const T*)u->xmap, w, n, (C<T>*)W.t1, (C<T>*)W.t2, q)
+                    : run_forward<T, T, T>(ctx, (const T*)u->xmap, (const T*)mask_map(ctx), (const T*)nullptr, (C<T>*)W.t1,
+                                           (C<T>*)W.t2, q, pg);
+        if (rc) return rc;
         uw::k_gather<T><<<grid1d(M), 256, 0, ctx->stream>>>(q, 0, ctx->d_offs, M, Zc + (size_t)t * Mp, 0, zw);
         ctx->launches++;
     }
@@ -1446,12 +1508,14 @@ static int fisher_sum(polybin_ctx* ctx, const float* n, const float* w, unsigned
     const int na = which != 1 ? ctx->nell * ctx->nb : (int)ctx->Nabc.size();
     if (sum.size() != (size_t)na * na) sum.assign((size_t)na * na, 0.0);
     std::vector<double> F;
-    if ((which == 0 || which == 1) && r0 < r1 && (rc = mask_setup<T>(ctx, n, w))) return rc;
+    if ((which == 0 || which == 1) && r0 < r1 &&
+        (rc = mask_setup<T>(ctx, n, w, u->g2, sizeof(T) * (size_t)ctx->nb * ctx->ncell)))
+        return rc;
     for (int r = r0; r < r1; ++r) {
         if (which == 0) {
-            if ((rc = pk_fisher_draw<T>(ctx, n, w, seed, r, F))) return rc;
+            if ((rc = with_room(ctx, [&] { return pk_fisher_draw<T>(ctx, n, w, seed, r, F); }))) return rc;
         } else if (which == 2) {
-            if ((rc = pk_fisher_draw_local<T>(ctx, n, w, seed, r, F))) return rc;
+            if ((rc = with_room(ctx, [&] { return pk_fisher_draw_local<T>(ctx, n, w, seed, r, F); }))) return rc;
         } else if (which == 3) {
             if ((rc = pk_fisher_draw_opt<T>(ctx, n, seed, r, F))) return rc;
         } else {
@@ -1459,8 +1523,11 @@ static int fisher_sum(polybin_ctx* ctx, const float* n, const float* w, unsigned
                 cudaError_t e = cudaMalloc(&u->dF, sizeof(double) * (size_t)na * na);
                 if (e != cudaSuccess) return fail_cuda(ctx, e, "cudaMalloc Fisher", __FILE__, __LINE__);
             }
-            PB_CUDA_OK(cudaMemsetAsync(u->dF, 0, sizeof(double) * (size_t)na * na, ctx->stream));
-            if ((rc = bk_fisher_draw<T>(ctx, n, w, seed, r))) return rc;
+            auto draw = [&]() -> int {
+                PB_CUDA_OK(cudaMemsetAsync(u->dF, 0, sizeof(double) * (size_t)na * na, ctx->stream));
+                return bk_fisher_draw<T>(ctx, n, w, seed, r);
+            };
+            if ((rc = with_room(ctx, draw))) return rc;
             F.resize((size_t)na * na);
             PB_CUDA_OK(cudaMemcpyAsync(F.data(), u->dF, sizeof(double) * F.size(), cudaMemcpyDeviceToHost, ctx->stream));
             PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
@@ -1829,7 +1896,7 @@ static int pk_unwindowed_local_t(polybin_ctx* ctx, const float* d, const float* 
     UwState* u = static_cast<UwState*>(ctx->ext);
     const int na = ctx->nell * ctx->nb;
     std::vector<double> pnum;
-    if ((rc = pk_numerator_local_t<T>(ctx, d, w, pnum))) return rc;
+    if ((rc = with_room(ctx, [&] { return pk_numerator_local_t<T>(ctx, d, w, pnum); }))) return rc;
     if (pnum_out) std::memcpy(pnum_out, pnum.data(), sizeof(double) * na);
     if (!pk_out) return POLYBIN_OK;
     if (!u->have_l)
