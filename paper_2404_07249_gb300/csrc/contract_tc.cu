@@ -880,12 +880,13 @@ __global__ void __launch_bounds__(128, 1) k_tf32_selfcheck(uint32_t* res) {
 // Tensor-core Gram matrix of the bispectrum Fisher (Sec. 4.3.4, eq. bk-fish-def in Fourier space):
 //   part[s][i][j] = sum_{k in split s} A[i][k] B[j][k],  A = Z (weighted), B = Y as float32 rows [n][K], K = 2 M
 // (real and imaginary parts of the binned modes interleaved: re*re + im*im is the real part of conj(Z) Y).
-// A CTA takes a 128 x 32 output tile and a contiguous range of K.  Arithmetic as in the triplet contraction:
-// A = A_hi + A_lo (A_hi rounded to TF32 by the producers, written to tensor memory), B_hi = the raw TMA tile (read as
+// A CTA takes a 128 x 32 output tile and a contiguous range of K.  Arithmetic: A = A_hi + A_lo (A_hi rounded to TF32 by the producers, written to tensor memory), B_hi = the raw TMA tile (read as
 // TF32 by truncation), B_lo = (B - trunc B) rounded to TF32; D_hh += A_hi B_hi, D_c += A_hi B_lo + A_lo B_hi; D restarts
-// every 64 K (8 MMAs a column), FP32 register sums, FP64 register sums every 2048 K; FP64 partials per K split.
+// every 32 K (4 MMAs a column: the tensor core cuts each partial sum towards zero, and with 64 K the bispectrum Fisher term of
+// 564 triplets came out 1.2e-7 too small instead of 4e-8; 10.72 -> 10.85 ms), FP32 register sums, FP64 register sums every
+// 2048 K; FP64 partials per K split.
 namespace gram {
-constexpr int kBM = 128, kBN = 32, kKC = 32, kStages = 6, kPeriod = 2, kSpill = 32;
+constexpr int kBM = 128, kBN = 32, kKC = 32, kStages = 6, kPeriod = 1, kSpill = 64;
 constexpr int kThreads = 384;   // warps 0 TMA/TMEM, 1 MMA, 2 B_lo, 3 idle, 4-7 A producers, 8-11 epilogue
 constexpr int kAStage = kBM * 128, kBStage = kBN * 128;   // raw tiles: 32 floats (128 B) a row
 constexpr int kSmem = kStages * (kAStage + 2 * kBStage) + 1024 + 256;
