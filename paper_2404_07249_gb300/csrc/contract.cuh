@@ -14,8 +14,9 @@
 // Measured at 13 bins (55 rows x 13 singles) on 100^3 cells: 845 us before the replicas, 359 us with them, 270 us now;
 // instruction issue bounds it.
 //
-// Precision (float): products and chunk sums in FP32, flushed every FLUSH chunks into FP64 registers (double: FP64
-// throughout); per-CTA FP64 partials are reduced across CTAs in a fixed order (deterministic).
+// Precision: products and sums of kFlush chunks in the maps' precision, added to FP64 totals (FP32: the sums are short enough
+// for 24 bits; FP64: no sum is longer than 512 terms however many cells a CTA takes); per-CTA FP64 partials are reduced
+// across CTAs in a fixed order (deterministic).
 #pragma once
 #include <algorithm>
 
@@ -26,7 +27,7 @@ namespace pb {
 constexpr int kCH = 32;       // cells per chunk (one a lane when products are formed)
 constexpr int kTM = 4;        // pair rows per thread
 constexpr int kTN = 8;        // singles per thread
-constexpr int kFlush = 16;    // chunks per FP32 partial sum (512 cells)
+constexpr int kFlush = 16;    // chunks per partial sum (512 cells)
 constexpr int kGS = kCH + 1;  // row stride of the staged maps
 
 struct ContractGeom {
@@ -136,20 +137,32 @@ __global__ void __launch_bounds__(256, 2) k_contract(const T* __restrict__ g, co
 
     // FP32 sums two a register pair: one f32x2 instruction is two fused multiply-adds
     uint64_t acc[kTM][kTN / 2];
-    double acc64[kTM][kTN];
+    double acc64[kTM][kTN];                           // totals; FP64: the sums
 #pragma unroll
     for (int u = 0; u < kTM; ++u)
 #pragma unroll
         for (int v = 0; v < kTN; ++v) { acc[u][v / 2] = 0; acc64[u][v] = 0.0; }
+    // FP64 totals lie in local memory, touched every 512 cells: with both in registers an SM holds one CTA, and the bispectrum
+    // of 8 bins on 64^3 cells took 462 us instead of 337 (334 with one running sum)
+    volatile double total[sizeof(T) == 8 ? kTM * kTN : 1];
+    bool have_total = false;
     auto flush = [&]() {
 #pragma unroll
         for (int u = 0; u < kTM; ++u)
 #pragma unroll
             for (int v = 0; v < kTN; v += 2) {
-                acc64[u][v] += (double)__uint_as_float((unsigned)acc[u][v / 2]);
-                acc64[u][v + 1] += (double)__uint_as_float((unsigned)(acc[u][v / 2] >> 32));
-                acc[u][v / 2] = 0;
+                if constexpr (sizeof(T) == 8) {
+                    for (int q = v; q < v + 2; ++q) {
+                        total[u * kTN + q] = have_total ? total[u * kTN + q] + acc64[u][q] : acc64[u][q];
+                        acc64[u][q] = 0.0;
+                    }
+                } else {
+                    acc64[u][v] += (double)__uint_as_float((unsigned)acc[u][v / 2]);
+                    acc64[u][v + 1] += (double)__uint_as_float((unsigned)(acc[u][v / 2] >> 32));
+                    acc[u][v / 2] = 0;
+                }
             }
+        have_total = true;
     };
 
     // warp w stages maps w, w + 8, .. (at most 8 of g, 8 of h), lane = cell
@@ -233,10 +246,17 @@ __global__ void __launch_bounds__(256, 2) k_contract(const T* __restrict__ g, co
                         }
                     }
             }
-            if (sizeof(T) == 4 && (chunk + 1) % kFlush == 0) flush();
+            if ((chunk + 1) % kFlush == 0) flush();
         }
     }
-    if constexpr (sizeof(T) == 4) flush();
+    if constexpr (sizeof(T) == 4) {
+        flush();
+    } else if (have_total) {
+#pragma unroll
+        for (int u = 0; u < kTM; ++u)
+#pragma unroll
+            for (int v = 0; v < kTN; ++v) acc64[u][v] += total[u * kTN + v];
+    }
     // replicas 1, 2, .. are added to replica 0 in order
     double* red = reinterpret_cast<double*>(smem_raw);   // [kTM * kTN][ntile]
     for (int q = 1; q < G.kg; ++q) {
