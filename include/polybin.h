@@ -54,9 +54,9 @@ typedef enum {
  * l_max        : largest even Legendre order of the power spectrum (0, 2 or 4).
  * prec         : a polybin_prec value.
  * cuda_stream  : cudaStream_t to run on (NULL = legacy default stream).
- * The first POLYBIN_SPLIT_TF32X3 context on a device runs a one-MMA self-check on known operands: the split scheme
- * takes the tensor core's reading of an FP32 operand (its 13 low bits dropped) as the high part of the maps; if the
- * device reads it otherwise, polybin_init returns POLYBIN_ETOL (for this and every later split context there).
+ * The first POLYBIN_SPLIT_TF32X3 context on a device runs a one-MMA self-check on known operands: the bispectrum Fisher
+ * matrix takes the tensor core's reading of an FP32 operand (its 13 low bits dropped) as the high part of its rows; if
+ * the device reads it otherwise, polybin_init returns POLYBIN_ETOL (for this and every later split context there).
  * On success *out receives the context (destroy with polybin_destroy); on failure *out is NULL and
  * polybin_last_error(NULL) describes the error. */
 int polybin_init(polybin_ctx** out, const int grid[3], const double boxsize[3], const double* k_edges,
@@ -331,11 +331,10 @@ int polybin_last_path(const polybin_ctx* ctx, int* path);
  * polybin_contract stay on the data grid. */
 int polybin_contraction_grid(const polybin_ctx* ctx, int dims[3]);
 
-/* Failure-detection self-test: one kernel waits on an mbarrier phase that nothing completes, using the same bounded
- * poll as the tensor-core pipeline, and another on a barrier armed for a bulk staging copy that is never issued,
- * using the bounded wait of the transform passes' staging; each wait gives up after 2^14 polls and sets its device
- * error flag, the kernels return and the context stays usable (the flags are cleared afterwards).
- * *timed_out = 1 when both bounded waits gave up (the expected outcome). */
+/* Failure-detection self-test: a kernel waits on an mbarrier phase that nothing completes, using the same bounded
+ * poll as the tensor-core pipeline; the wait gives up after 2^14 polls and sets the device error flag, the kernel
+ * returns and the context stays usable (the flag is cleared afterwards).
+ * *timed_out = 1 when the bounded wait gave up (the expected outcome). */
 int polybin_selftest_wait(polybin_ctx* ctx, int* timed_out);
 
 /* ---- individual steps, for testing and composition (device pointers only) --------------------------------- */

@@ -80,10 +80,6 @@ static int launch_check(polybin_ctx* ctx, const char* what) {
 template <typename T> static int lines_per_cta(int n) { return lines_per_cta_of<T>(n); }
 template <typename T> static int cols_per_cta(int n) { return cols_per_cta_of<T>(n); }
 
-template <typename T> static const C<T>* twiddles(polybin_ctx* ctx, int axis);
-template <> const float2* twiddles<float>(polybin_ctx* ctx, int axis) { return (const float2*)ctx->d_tw_f[axis]; }
-template <> const double2* twiddles<double>(polybin_ctx* ctx, int axis) { return (const double2*)ctx->d_tw_d[axis]; }
-
 // ----------------------------------------------------------------------------------------------- pipelines
 
 // a1: pruned forward transform of one real field on grid ig (optionally times m1 * m2) into the box of the wave
@@ -290,12 +286,6 @@ int run_shells_m(polybin_ctx* ctx, const C<T>* box, C<T>* u1, C<T>* u2, T* g, in
         if ((rc = launch_check(ctx, "k_inv_z"))) return rc;
     }
     return POLYBIN_OK;
-}
-
-// Launches the staging-wait self-test into the staging error flag (the caller clears and reads it).
-int run_bulk_wait_selftest(polybin_ctx* ctx, unsigned limit) {
-    k_bulk_wait_selftest<<<1, 32, 0, ctx->stream>>>(ctx->d_err + kErrStaging, limit);
-    return launch_check(ctx, "k_bulk_wait_selftest");
 }
 
 ContractGeom contract_geom(int nb, int nh, long ncell) { return contract_geom_rows(nb, nb * (nb + 1) / 2, nh, ncell); }

@@ -817,8 +817,8 @@ __global__ void k_wait_selftest(int* err, unsigned limit) {
 }
 
 // ------------------------------------------------------------------------------------------------ self-check
-// What the split-TF32 scheme assumes of the tensor core, checked on known operands: an FP32 B operand is read as TF32
-// by dropping its 13 low bits (B_hi = the raw map), and a TF32 value written to tensor memory as the A operand is
+// What the Gram matrix assumes of the tensor core, checked on known operands: an FP32 B operand is read as TF32
+// by dropping its 13 low bits (B_hi = the raw row), and a TF32 value written to tensor memory as the A operand is
 // used exactly.  A (tensor memory, M = 128, K = 8) has A[0][0] = 1 and A[1][0] = 1 + 2^-10; B (shared memory, N = 16,
 // 128-byte swizzle) has B[0][0] = 1 + 3 2^-12, three quarters of a TF32 unit above 1.  Truncation gives D[0][0] = 1
 // and D[1][0] = 1 + 2^-10; rounding to nearest would give 1 + 2^-10 and (1 + 2^-10)^2.  res: D[0][0], D[1][0] (FP32
@@ -880,8 +880,8 @@ __global__ void __launch_bounds__(128, 1) k_tf32_selfcheck(uint32_t* res) {
 // Tensor-core Gram matrix of the bispectrum Fisher (Sec. 4.3.4, eq. bk-fish-def in Fourier space):
 //   part[s][i][j] = sum_{k in split s} A[i][k] B[j][k],  A = Z (weighted), B = Y as float32 rows [n][K], K = 2 M
 // (real and imaginary parts of the binned modes interleaved: re*re + im*im is the real part of conj(Z) Y).
-// A CTA takes a 128 x 32 output tile and a contiguous range of K.  Arithmetic: A = A_hi + A_lo (A_hi rounded to TF32 by the producers, written to tensor memory), B_hi = the raw TMA tile (read as
-// TF32 by truncation), B_lo = (B - trunc B) rounded to TF32; D_hh += A_hi B_hi, D_c += A_hi B_lo + A_lo B_hi; D restarts
+// A CTA takes a 128 x 32 output tile and a contiguous range of K.  Arithmetic: A = A_hi + A_lo (A_hi rounded to TF32 by
+// the producers, written to tensor memory), B_hi = the raw TMA tile (read as TF32 by truncation), B_lo = (B - trunc B) rounded to TF32; D_hh += A_hi B_hi, D_c += A_hi B_lo + A_lo B_hi; D restarts
 // every 32 K (4 MMAs a column: the tensor core cuts each partial sum towards zero, and with 64 K the bispectrum Fisher term of
 // 564 triplets came out 1.2e-7 too small instead of 4e-8; 10.72 -> 10.85 ms), FP32 register sums, FP64 register sums every
 // 2048 K; FP64 partials per K split.
@@ -1734,7 +1734,7 @@ static int ell_plan(polybin_ctx* ctx, Plan** out) {
 bool split_tc_available() { return true; }
 
 // Runs k_tf32_selfcheck once per device (the first split-TF32 context on it); POLYBIN_ETOL if the tensor core does
-// not read FP32 operands as the split scheme assumes.
+// not read FP32 operands as the Gram matrix assumes.
 int tf32_selfcheck(polybin_ctx* ctx) {
     static std::mutex mu;
     static int state[256] = {};   // 0 unchecked, 1 ok, -1 failed
@@ -1784,18 +1784,12 @@ int ensure_err_flag(polybin_ctx* ctx) {
     return POLYBIN_OK;
 }
 
-// Reads both error flags after the work queued on the stream (synchronising it).  The staging flag is raised by the
-// transform passes that run before the contraction on the same stream and is cleared once reported.
+// Reads the error flags after the work queued on the stream (synchronising it).
 int read_err_flags(polybin_ctx* ctx, const char* what) {
-    int herr[kErrFlags] = {0, 0};
+    int herr[kErrFlags] = {};
     cudaError_t e = cudaMemcpyAsync(herr, ctx->d_err, sizeof(herr), cudaMemcpyDeviceToHost, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) return fail_cuda(ctx, e, "error flags", __FILE__, __LINE__);
-    if (herr[kErrStaging]) {
-        e = cudaMemset(ctx->d_err + kErrStaging, 0, sizeof(int));
-        if (e != cudaSuccess) return fail_cuda(ctx, e, "cudaMemset err flag", __FILE__, __LINE__);
-        return fail(ctx, POLYBIN_ETIMEOUT, "%s: a bulk staging copy of a transform pass did not complete", what);
-    }
     if (herr[kErrPipeline]) return fail(ctx, POLYBIN_ETIMEOUT, "%s: a pipeline wait timed out", what);
     return POLYBIN_OK;
 }
@@ -1913,12 +1907,11 @@ extern "C" int polybin_selftest_wait(polybin_ctx* ctx, int* timed_out) {
     pb::tc::k_wait_selftest<<<1, 32, 0, ctx->stream>>>(ctx->d_err + pb::kErrPipeline, 1u << 14);
     ctx->launches++;
     PB_CUDA_OK(cudaGetLastError());
-    if ((rc = pb::run_bulk_wait_selftest(ctx, 1u << 14))) return rc;
-    int h[pb::kErrFlags] = {0, 0};
+    int h[pb::kErrFlags] = {};
     PB_CUDA_OK(cudaMemcpyAsync(h, ctx->d_err, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream));
     PB_CUDA_OK(cudaStreamSynchronize(ctx->stream));
     PB_CUDA_OK(cudaMemsetAsync(ctx->d_err, 0, pb::kErrFlags * sizeof(int), ctx->stream));
-    *timed_out = (h[pb::kErrPipeline] && h[pb::kErrStaging]) ? 1 : 0;
+    *timed_out = h[pb::kErrPipeline] ? 1 : 0;
     return POLYBIN_OK;
 }
 

@@ -237,36 +237,6 @@ __device__ __forceinline__ void stage_twiddles(C<T>* dst, const C<T>* __restrict
     for (int i = tid; i < n; i += nthr) dst[i] = tw[i];
 }
 
-// Bounded wait on an mbarrier that a bulk copy completes.
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void bulk_bar_init(uint64_t* bar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tfence.mbarrier_init.release.cluster;" ::"r"(smem_addr(bar))
-                 : "memory");
-}
-// Waits for phase `parity` of the barrier; false after `limit` polls (the copy never landed).
-__device__ __forceinline__ bool bulk_wait(uint64_t* bar, uint32_t parity, unsigned limit) {
-    for (unsigned it = 0; it < limit; ++it) {
-        uint32_t ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(ok)
-            : "r"(smem_addr(bar)), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-// Self-test of the staging wait: a barrier armed for 16 bytes that no copy delivers (none is issued); the bounded
-// wait gives up and raises the flag.
-static __global__ void k_bulk_wait_selftest(int* err, unsigned limit) {
-    __shared__ uint64_t bar;
-    if (threadIdx.x == 0) {
-        bulk_bar_init(&bar);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], 16;" ::"r"(smem_addr(&bar)) : "memory");
-        if (!bulk_wait(&bar, 0u, limit)) atomicExch(err, 1);
-    }
-}
-
 // ------------------------------------------------------------------------------------------------
 // z-pass, forward: pairs of real lines (lines 2p, 2p+1 of the flattened (x, y) index) packed as one
 // complex line, transformed, then split into the two Hermitian half-spectra; only kz < kout is stored.

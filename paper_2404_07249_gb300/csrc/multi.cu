@@ -187,13 +187,9 @@ extern "C" int polybin_bk_ideal_multi(polybin_ctx* const* ctxs, const float* con
     for (int i = 0; i < n_fields; ++i) {
         polybin_ctx* c = ctxs[i];
         const int* herr = m->err + place[i] * kErrFlags;
-        if (herr[kErrStaging]) {
-            polybin_ctx* ctx = c0;
-            PB_CUDA_OK(cudaMemset(c->d_err + kErrStaging, 0, sizeof(int)));
-        }
-        if (herr[kErrPipeline] || herr[kErrStaging])
-            return fail(c0, POLYBIN_ETIMEOUT, "polybin_bk_ideal_multi: a %s wait timed out (a field of the context of field %d)",
-                        herr[kErrStaging] ? "bulk staging" : "pipeline", i);
+        if (herr[kErrPipeline])
+            return fail(c0, POLYBIN_ETIMEOUT, "polybin_bk_ideal_multi: a pipeline wait timed out (a field of the context of field %d)",
+                        i);
         const double* B = m->host + m->off[i];
         std::memcpy(bk_out[i], B, sizeof(double) * c->Nabc.size());
     }

@@ -193,11 +193,10 @@ void destroy_extras(polybin_ctx*);
 void destroy_unwindowed(polybin_ctx*);
 void destroy_multi(polybin_ctx*);
 // Device error flags of a context: [kErrPipeline] the tensor-core kernels' bounded waits (cleared before each of
-// their launches, in a captured graph once at its head), [kErrStaging] the bulk staging copies of the transform passes (cleared when reported).
-constexpr int kErrPipeline = 0, kErrStaging = 1, kErrFlags = 2;
+// their launches, in a captured graph once at its head).
+constexpr int kErrPipeline = 0, kErrFlags = 1;
 int ensure_err_flag(polybin_ctx*);
 int read_err_flags(polybin_ctx*, const char* what);
-int run_bulk_wait_selftest(polybin_ctx*, unsigned limit);
 
 }  // namespace pb
 
