@@ -39,8 +39,8 @@ UNIT = "estimates/s"
 E2E_BATCH = 8   # fields a call in the end-to-end measurement (pinned host memory: 8 x 537 MB at 512^3)
 
 CAPTURED_TRAFFIC = {
-    ("18603d1966df9004b943ba7430f520fed9d35ea5170fab736749ecde1e06c671", "lognormal_kaiser512", "split"):
-        2868029000 + 3736000,
+    ("9a9872e07185046ecafec7e611a052a55088ba8e236891b62fc2fb037718e1cc", "lognormal_kaiser512", "split"):
+        2867759000 + 3895552,
 }
 
 

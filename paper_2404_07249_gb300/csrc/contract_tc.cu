@@ -22,9 +22,10 @@
 // Measured on this part (and shaping the design): an MMA issued from warp-uniform code with its operands in uniform
 // registers costs ~16-20 cycles at N = 32 (the tensor pipe's rate), but ~200 cycles from a one-lane branch, so the
 // issuing loop is warp-uniform (elect.sync inside the asm) and divide-free; tensor memory stores reach ~650 B/clk an
-// SM.  What bounds the kernel is instruction issue and the latency of the producers' chains (gathers, two 16-byte loads for
-// every four products, and eleven instructions of split for two products); the MMAs are not it (half of them: 5 % less).
-// So four producer groups, 16 cells at a time in few registers, and B warps that take every other stage; a stage is 64
+// SM.  What bounds the kernel is the producers: their gathers (two 16-byte loads for every four products; the shared-memory
+// pipe is busy 76 % of the time, nearly half of it with bank conflicts) and ten instructions of split for two products (2.64
+// of 4 instructions a clock); the tensor pipe is busy 27 % (half of the MMAs: 5 % less time).  So four producer groups,
+// 16 cells at a time in few registers, and B warps that take every other stage; a stage is 64
 // cells and the accumulators are double-buffered, so that no MMA waits for the epilogue.  Measured, ms, at 30 maps
 // of 288^3 cells (two tiles) and at 20 maps of 192^3 (one tile): two TF32 parts in 32-cell stages 3.90 and 0.778, two
 // FP16 parts 2.64 and 0.459, three BF16 parts with two producer groups and 32 cells at a time 3.39 and 0.549 (3.22 and
